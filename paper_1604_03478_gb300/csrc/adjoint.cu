@@ -49,7 +49,8 @@ namespace lbm {
 // level before, which differ by at most one.
 template <typename ST, int FACE>
 __global__ void __launch_bounds__(128) k_snapshot(const __grid_constant__ KP p, const ST *__restrict__ F, const ST *__restrict__ G,
-                                                  const int *__restrict__ js, const int *__restrict__ nb,
+                                                  const int *__restrict__ js, const int *__restrict__ js_old,
+                                                  const int *__restrict__ nb,
                                                   const double *__restrict__ s, const float *__restrict__ thw,
                                                   int inflight, float *__restrict__ out, double *__restrict__ out_s,
                                                   int *__restrict__ out_js, int *__restrict__ out_nb) {
@@ -69,7 +70,7 @@ __global__ void __launch_bounds__(128) k_snapshot(const __grid_constant__ KP p, 
     float g[7], f[19];
     gather_g<ST, FACE>(p, G, x, y, z, inflight != 0, thw, g);
     const bool liq = a < js[col];
-    if (liq) gather_f<ST, FACE>(p, F, js, x, y, z, inflight != 0, f);
+    if (liq) gather_f_now<ST, FACE>(p, F, js, js_old, x, y, z, inflight != 0, f);
 #pragma unroll
     for (int i = 0; i < 19; ++i) out[i * p.N + c] = liq ? f[i] : 0.0f;
 #pragma unroll
@@ -1054,16 +1055,16 @@ LBM_API lbm_status lbm_melt_tape_backward(lbm_melt *h, const double *seed, doubl
             float *out = snap + (size_t)j * 26 * N;
             double *os = snap_s + (size_t)j * nc;
             int *ojs = snap_js + (size_t)j * nc, *onb = snap_nb + (size_t)j * nc;
-            const int *js = h->js[cur], *nbv = h->nb[cur];
+            const int *js = h->js[cur], *jso = h->js[1 - cur], *nbv = h->nb[cur];
             const double *sv = h->s[cur];
             if (h->precision == 1) {
                 const __half *F = (const __half *)h->F, *G = (const __half *)h->G;
-                if (h->face == 0) lbm::k_snapshot<__half, 0><<<grd, blk, 0, sm>>>(p, F, G, js, nbv, sv, thw, inflight, out, os, ojs, onb);
-                else lbm::k_snapshot<__half, 1><<<grd, blk, 0, sm>>>(p, F, G, js, nbv, sv, thw, inflight, out, os, ojs, onb);
+                if (h->face == 0) lbm::k_snapshot<__half, 0><<<grd, blk, 0, sm>>>(p, F, G, js, jso, nbv, sv, thw, inflight, out, os, ojs, onb);
+                else lbm::k_snapshot<__half, 1><<<grd, blk, 0, sm>>>(p, F, G, js, jso, nbv, sv, thw, inflight, out, os, ojs, onb);
             } else {
                 const float *F = (const float *)h->F, *G = (const float *)h->G;
-                if (h->face == 0) lbm::k_snapshot<float, 0><<<grd, blk, 0, sm>>>(p, F, G, js, nbv, sv, thw, inflight, out, os, ojs, onb);
-                else lbm::k_snapshot<float, 1><<<grd, blk, 0, sm>>>(p, F, G, js, nbv, sv, thw, inflight, out, os, ojs, onb);
+                if (h->face == 0) lbm::k_snapshot<float, 0><<<grd, blk, 0, sm>>>(p, F, G, js, jso, nbv, sv, thw, inflight, out, os, ojs, onb);
+                else lbm::k_snapshot<float, 1><<<grd, blk, 0, sm>>>(p, F, G, js, jso, nbv, sv, thw, inflight, out, os, ojs, onb);
             }
             return cudaGetLastError();
         };

@@ -135,29 +135,32 @@ ENS_FN void ens_even(const CavDesc &d, int cur, int x, int y, int z) {
 }
 template <typename ST, int FACE>
 ENS_FN void ens_odd(const CavDesc &d, int cur, const float *trd, int x, int y, int z) {
-    odd_node<ST, FACE, false>(d.p, nullptr, (ST *)d.F, (ST *)d.G, d.js[cur], d.nb[cur], d.gpost, trd, d.thw, x, y, z);
+    odd_node<ST, FACE, false>(d.p, nullptr, (ST *)d.F, (ST *)d.G, d.js[cur], d.js[1 - cur], d.nb[cur], d.gpost, trd, d.thw, x, y, z);
 }
 
-// One column of phase 2 (front update; returns the new liquid count) or 3
-// (flip; returns -1).  The front update does not load the ghost's likely
-// source node with the gradient stencil (as k_front does): under this
-// kernel's register cap that spilled 1.3 KB a thread and slowed every phase
-// (19.8 k against 23.2 k MLUPS on the 48-cavity workload).
+// One column of phase 2 (front update; returns the new liquid count).  It
+// does not load the ghost's likely source node with the gradient stencil (as
+// k_front does): under this kernel's register cap that spilled 1.3 KB a
+// thread and slowed every phase (19.8 k against 23.2 k MLUPS on the
+// 48-cavity workload).
 template <typename ST>
-ENS_FN int ens_column(const CavDesc &d, int cur, int inflight, int phase, int col) {
-    if (phase == 2) {
-        const ST *F = (const ST *)d.F, *G = (const ST *)d.G;
-        if (d.face == 0)
-            return front_column<ST, 0, false>(d.p, F, G, d.js[cur], d.js[1 - cur], d.s[cur], d.s[1 - cur], d.gpost, d.thw,
-                                       inflight, 1, d.status, col);
-        return front_column<ST, 1, false>(d.p, F, G, d.js[cur], d.js[1 - cur], d.s[cur], d.s[1 - cur], d.gpost, d.thw,
-                                   inflight, 1, d.status, col);
-    } else {
-        ST *F = (ST *)d.F;
-        if (d.face == 0) flip_column<ST, 0>(d.p, F, d.js[cur], d.js[1 - cur], d.nb[1 - cur], inflight, 1, col);
-        else flip_column<ST, 1>(d.p, F, d.js[cur], d.js[1 - cur], d.nb[1 - cur], inflight, 1, col);
-        return -1;
-    }
+ENS_FN int ens_front(const CavDesc &d, int cur, int inflight, int col) {
+    ST *F = (ST *)d.F;
+    const ST *G = (const ST *)d.G;
+    if (d.face == 0)
+        return front_column<ST, 0, false>(d.p, F, G, d.js[cur], d.js[1 - cur], d.nb[1 - cur], d.s[cur], d.s[1 - cur],
+                                          d.gpost, d.thw, inflight, 1, d.status, col);
+    return front_column<ST, 1, false>(d.p, F, G, d.js[cur], d.js[1 - cur], d.nb[1 - cur], d.s[cur], d.s[1 - cur],
+                                      d.gpost, d.thw, inflight, 1, d.status, col);
+}
+
+// One column of phase 3: the flip of its nodes (liquid counts jo, jn).
+template <typename ST>
+ENS_FN void ens_flip(const CavDesc &d, int cur, int inflight, int col) {
+    ST *F = (ST *)d.F;
+    const int jo = d.js[cur][col], jn = d.js[1 - cur][col];
+    if (d.face == 0) flip_column<ST, 0>(d.p, F, d.js[cur], inflight != 0, col, jo, jn);
+    else flip_column<ST, 1>(d.p, F, d.js[cur], inflight != 0, col, jo, jn);
 }
 
 template <typename ST, int K>
@@ -226,30 +229,46 @@ __global__ void ENS_BOUNDS k_ensemble(const __grid_constant__ EnsWork w, int nst
         if (blockIdx.x == 0 && threadIdx.x == 0) ctr[(t + 1) & 1] = 0ull;
         if (!grid_barrier(w, gridDim.x)) return;
         if (timer) { const unsigned long long tn = global_ns(); phase_ns[0] += tn - tp; tp = tn; }
-        // phases 2 and 3: front update (Eq. 6), then flip, of every column.
-        // Items are dealt round-robin: consecutive items, which hold
-        // neighbouring columns and so much the same amount of flip work, go
-        // to different blocks (one contiguous range per block ran the flip
-        // phase 67 against 37 us a step on the 48-cavity workload).
-        for (int phase = 2; phase <= 3; ++phase) {
-            for (long long it = blockIdx.x; it < items2; it += gridDim.x) {
-                const int k = find_cavity(w.col_begin, w.ncav, it);
-                const CavDesc &d = w.desc[k];
-                const int cur = d.cur0 ^ (t & 1), inflight = 1 - (d.inflight0 ^ (t & 1));
-                const int col = (int)((it - w.col_begin[k]) * blockDim.x + threadIdx.x);
-                const int jn = col < d.p.ncols ? ens_column<ST>(d, cur, inflight, phase, col) : -1;
-                if (phase == 2) {  // an item is one cavity's columns: whole warps
-                    const int m = __reduce_max_sync(0xffffffffu, jn);
-                    if ((threadIdx.x & 31) == 0 && m >= 0) atomicMax(d.jmax, m);
+        // phase 2: front update (Eq. 6) of every column; phase 3: flip of the
+        // columns whose liquid count changed, by the thread that updated
+        // them.  No barrier between the two (see flip_column).  Items are
+        // dealt round-robin: consecutive items, which hold neighbouring
+        // columns and so much the same amount of flip work, go to different
+        // blocks.
+        unsigned long long changed = 0;  // bit n: this thread's column of its n-th item since `first`
+        long long first = blockIdx.x;
+        for (long long it = blockIdx.x;; it += gridDim.x) {
+            const bool more = it < items2;
+            if (!more || it - first == 64ll * gridDim.x) {
+                if (!more && timer) { const unsigned long long tn = global_ns(); phase_ns[1] += tn - tp; tp = tn; }
+                for (; changed; changed &= changed - 1) {
+                    const long long jt = first + (__ffsll((long long)changed) - 1) * (long long)gridDim.x;
+                    const int k = find_cavity(w.col_begin, w.ncav, jt);
+                    const CavDesc &d = w.desc[k];
+                    ens_flip<ST>(d, d.cur0 ^ (t & 1), 1 - (d.inflight0 ^ (t & 1)),
+                                 (int)((jt - w.col_begin[k]) * blockDim.x + threadIdx.x));
                 }
+                first = it;
             }
-            if (!grid_barrier(w, gridDim.x)) return;
-            if (timer) {
-                const unsigned long long tn = global_ns();
-                phase_ns[phase - 1] += tn - tp;
-                tp = tn;
-                if (phase == 3) phase_ns[3] += 1ull;
+            if (!more) break;
+            const int k = find_cavity(w.col_begin, w.ncav, it);
+            const CavDesc &d = w.desc[k];
+            const int cur = d.cur0 ^ (t & 1), inflight = 1 - (d.inflight0 ^ (t & 1));
+            const int col = (int)((it - w.col_begin[k]) * blockDim.x + threadIdx.x);
+            int jn = -1;
+            if (col < d.p.ncols) {
+                jn = ens_front<ST>(d, cur, inflight, col);
+                if (jn != d.js[cur][col]) changed |= 1ull << (int)((it - first) / gridDim.x);
             }
+            const int m = __reduce_max_sync(0xffffffffu, jn);  // an item is one cavity's columns: whole warps
+            if ((threadIdx.x & 31) == 0 && m >= 0) atomicMax(d.jmax, m);
+        }
+        if (!grid_barrier(w, gridDim.x)) return;
+        if (timer) {
+            const unsigned long long tn = global_ns();
+            phase_ns[2] += tn - tp;
+            tp = tn;
+            phase_ns[3] += 1ull;
         }
     }
 }

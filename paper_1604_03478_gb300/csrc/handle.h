@@ -99,7 +99,7 @@ struct lbm_melt {
 // Release a handle's recorded run and the adjoint's buffers (defined with
 // the adjoint).
 void lbm_tape_free(lbm_melt *h);
-// Enqueue one step (stream-collide, front, flip) from phase (cur, inflight)
+// Enqueue one step (stream-collide, front with flip) from phase (cur, inflight)
 // on stream st, the stream-collide grid cut at `height`; advances cur and
 // inflight.  No host bookkeeping (step counters, read-backs, report rows).
 cudaError_t lbm_enqueue_step(lbm_melt *h, int &cur, int &inflight, int height, cudaStream_t st);

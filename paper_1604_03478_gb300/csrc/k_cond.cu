@@ -33,6 +33,21 @@ __device__ __forceinline__ void collide_solid2(const KP &p, float2 (&g)[7]) {
     g[6] = add2(g[6], sub2(ez, c3));
 }
 
+// Smallest and largest liquid count of the pair's 3x3 columns: the bounds of
+// nb (each up to two wide of the count) where they settle which side of the
+// front height a is on, else the counts themselves.
+__device__ __forceinline__ void pair_bounds(const KP &p, const int *__restrict__ js, const int *__restrict__ nb, int pp,
+                                            int q, int col, int a, int &mn, int &mx) {
+    const int nb0 = __ldg(nb + col), nb1 = __ldg(nb + col + 1);
+    mn = min(nb0 >> 16, nb1 >> 16);
+    mx = max(nb0 & 0xffff, nb1 & 0xffff);
+    if (a + 1 >= mn && a <= mx) {
+        int c12[12];
+        load_js12(p, js, pp, q, c12);
+        range_js12(p, c12, pp, q, mn, mx);
+    }
+}
+
 // Even step, pair (x, x + 1): two liquid nodes whose 3x3 columns are liquid
 // one node above (no link crosses the phase boundary) collide as in the
 // held-solid pair kernel; two solid nodes above every neighbouring liquid
@@ -45,11 +60,12 @@ __device__ __forceinline__ void even_pair_cond(const KP &p, ST *__restrict__ F, 
                                                int x, int y, int z) {
     const int a = axial<FACE>(x, y, z);
     const int col = column<FACE>(p, x, y, z);
-    const int nb0 = __ldg(nb + col), nb1 = __ldg(nb + col + 1);
+    int mn, mx;
+    pair_bounds(p, js, nb, x, FACE == 0 ? z : y, col, a, mn, mx);
     const IX c = (IX)node_index(p, x, y, z);
-    if (a + 1 < (nb0 >> 16) && a + 1 < (nb1 >> 16)) {
+    if (a + 1 < mn) {
         even_pair_liquid<ST, IX>(p, F, G, c);
-    } else if (a > (nb0 & 0xffff) && a > (nb1 & 0xffff)) {
+    } else if (a > mx) {
         float2 g[7];
 #pragma unroll
         for (int i = 0; i < 7; ++i) g[i] = ld_pair(elem<IX>(G, c, i * p.ld));
@@ -79,21 +95,23 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_even_pair_cond(
 template <typename ST, int FACE, typename IX>
 __device__ __forceinline__ void odd_pair_cond(const KP &p, const Links *lk, ST *__restrict__ F,
                                               ST *__restrict__ G, const int *__restrict__ js,
-                                              const int *__restrict__ nb, const float *__restrict__ gpost,
+                                              const int *__restrict__ js_old, const int *__restrict__ nb,
+                                              const float *__restrict__ gpost,
                                               const float *__restrict__ thw_rd, const float *__restrict__ thw_wr,
                                               const float *__restrict__ spost, int x, int y, int z) {
     const int a = axial<FACE>(x, y, z);
     const int col = column<FACE>(p, x, y, z);
     const int q = FACE == 0 ? z : y, nq = FACE == 0 ? p.nz : p.ny;
     const bool off_qa = q >= 1 && q <= nq - 2 && a >= 1 && a <= p.H - 2;
-    const int nb0 = __ldg(nb + col), nb1 = __ldg(nb + col + 1);
-    if (off_qa && a + 1 < (nb0 >> 16) && a + 1 < (nb1 >> 16)) {
+    int mn, mx;
+    pair_bounds(p, js, nb, x, q, col, a, mn, mx);
+    if (off_qa && a + 1 < mn) {
         odd_pair_liquid<ST, FACE, IX>(p, lk, F, G, x, y, z);
         return;
     }
-    if (!(off_qa && a > (nb0 & 0xffff) && a > (nb1 & 0xffff))) {
-        odd_node<ST, FACE, true, true>(p, lk, F, G, js, nb, gpost, thw_rd, thw_wr, x, y, z, spost);
-        odd_node<ST, FACE, true, true>(p, lk, F, G, js, nb, gpost, thw_rd, thw_wr, x + 1, y, z, spost);
+    if (!(off_qa && a > mx)) {
+        odd_node<ST, FACE, true, true>(p, lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x, y, z, spost);
+        odd_node<ST, FACE, true, true>(p, lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x + 1, y, z, spost);
         return;
     }
     const IX c = (IX)node_index(p, x, y, z), c1 = c + 1;
@@ -123,12 +141,13 @@ __device__ __forceinline__ void odd_pair_cond(const KP &p, const Links *lk, ST *
 template <typename ST, int FACE, typename IX>
 __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair_cond(
     const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G, const int *__restrict__ js,
-    const int *__restrict__ nb, const float *__restrict__ gpost, const float *__restrict__ thw_rd,
+    const int *__restrict__ js_old, const int *__restrict__ nb, const float *__restrict__ gpost,
+    const float *__restrict__ thw_rd,
     const float *__restrict__ thw_wr, const __grid_constant__ Links lk, const float *__restrict__ spost) {
     step_launch_wait();
     int x, y, z;
     if (k1_pair<FACE>(p, nullptr, x, y, z))
-        odd_pair_cond<ST, FACE, IX>(p, &lk, F, G, js, nb, gpost, thw_rd, thw_wr, spost, x, y, z);
+        odd_pair_cond<ST, FACE, IX>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, spost, x, y, z);
 }
 
 // The conduction step's kernels are launched like the plain step's, with
@@ -152,10 +171,10 @@ template <typename ST, typename IX>
 static cudaError_t launch_pair_cond(const KP &p, int face, int odd, const Bufs &b, dim3 g2, dim3 blk, cudaStream_t st) {
     ST *F = (ST *)b.F, *G = (ST *)b.G;
     if (face == 0) {
-        if (odd) return launch_cond_kernel(k_odd_pair_cond<ST, 0, IX>, g2, blk, st, p, F, G, b.js, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
+        if (odd) return launch_cond_kernel(k_odd_pair_cond<ST, 0, IX>, g2, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
         else return launch_cond_kernel(k_even_pair_cond<ST, 0, IX>, g2, blk, st, p, F, G, b.js, b.nb, b.gpost, b.spost);
     } else {
-        if (odd) return launch_cond_kernel(k_odd_pair_cond<ST, 1, IX>, g2, blk, st, p, F, G, b.js, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
+        if (odd) return launch_cond_kernel(k_odd_pair_cond<ST, 1, IX>, g2, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
         else return launch_cond_kernel(k_even_pair_cond<ST, 1, IX>, g2, blk, st, p, F, G, b.js, b.nb, b.gpost, b.spost);
     }
 }
@@ -172,10 +191,10 @@ cudaError_t LaunchCond<ST>::stream_collide(const KP &p, int face, int odd, const
     }
     const dim3 grd = k1_grid(p, blk, face, p.H);
     if (face == 0) {
-        if (odd) return launch_cond_kernel(k_odd_cond<ST, 0>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
+        if (odd) return launch_cond_kernel(k_odd_cond<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
         else return launch_cond_kernel(k_even_cond<ST, 0>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, b.spost);
     } else {
-        if (odd) return launch_cond_kernel(k_odd_cond<ST, 1>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
+        if (odd) return launch_cond_kernel(k_odd_cond<ST, 1>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
         else return launch_cond_kernel(k_even_cond<ST, 1>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, b.spost);
     }
 }
@@ -183,11 +202,12 @@ cudaError_t LaunchCond<ST>::stream_collide(const KP &p, int face, int odd, const
 template <typename ST>
 cudaError_t LaunchCond<ST>::front(const KP &p, int face, int inflight, int move, const Bufs &b, cudaStream_t st) {
     const dim3 blk(b.cblk), grd = col_grid(p.ncols, b.cblk);
-    const ST *F = (const ST *)b.F, *G = (const ST *)b.G;
+    ST *F = (ST *)b.F;
+    const ST *G = (const ST *)b.G;
     if (face == 0)
-        return launch_cond_kernel(k_front_cond<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.s, b.s_next, b.gpost,
+        return launch_cond_kernel(k_front_cond<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost,
                                   b.spost, b.thw_wr, inflight, move, b.status);
-    return launch_cond_kernel(k_front_cond<ST, 1>, grd, blk, st, p, F, G, b.js, b.js_next, b.s, b.s_next, b.gpost, b.spost,
+    return launch_cond_kernel(k_front_cond<ST, 1>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.spost,
                               b.thw_wr, inflight, move, b.status);
 }
 

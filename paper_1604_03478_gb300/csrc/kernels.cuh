@@ -7,8 +7,8 @@
 //                    node per thread (k_even_pair / k_odd_pair: two
 //                    x-adjacent nodes per thread in packed FP32x2 arithmetic);
 //   k_front        : interfacial tracking, Eq. 6, one thread per column (FP64
-//                    fronts, FP32 gradient and speed);
-//   k_flip         : phase flip of the nodes the front crossed.
+//                    fronts, FP32 gradient and speed), and the phase flip of
+//                    the nodes the front crossed.
 //
 // AA pattern.  A step that starts from the natural layout (slot i of node x
 // holds f_i(x), "even") reads and writes only node x: the post-collision
@@ -23,9 +23,10 @@
 // Between an even and an odd step the post-collision values are "in flight"
 // (their streaming is deferred to the odd step).  If the front flips a node
 // there, the odd step would read the in-flight values with the new flags;
-// k_flip rewrites the two slots of every link touching a flipped node so that
-// the new-flag reads deliver exactly what the old flags (and the re-initialised
-// f = f^eq(1, 0) of a newly liquid node) prescribe.
+// flip_column moves the value of every link between a flipped node and a node
+// that was liquid to the slot where the new flags look for it, and a reader
+// takes f = f^eq(1, 0) for a node that is liquid now and was not under the
+// flags of the step before (the other of the two liquid-count buffers).
 #pragma once
 
 #include "lbm_core.cuh"
@@ -211,17 +212,67 @@ __global__ void __launch_bounds__(128) k_even_cond(const __grid_constant__ KP p,
 
 
 // -------------------------------------------------------------- odd step
+// Liquid counts of the 3x3 columns around column (pp, q), 0 outside the
+// cavity; entry (dq + 1) * 3 + dp + 1.
+__device__ __forceinline__ void load_js9(const KP &p, const int *__restrict__ js, int pp, int q, int (&js9)[9]) {
+#pragma unroll
+    for (int dq = -1; dq <= 1; ++dq)
+#pragma unroll
+        for (int dp = -1; dp <= 1; ++dp) {
+            const int p2 = pp + dp, q2 = q + dq;
+            const bool in = (unsigned)p2 < (unsigned)p.P1 && (unsigned)q2 < (unsigned)p.P2;
+            js9[(dq + 1) * 3 + dp + 1] = in ? __ldg(js + q2 * p.P1 + p2) : 0;
+        }
+}
+
 // Bit i (1..18) of the link mask: node x - e_i is inside and liquid, i.e.
 // f_i streams in from there (else halfway bounce-back).  Since x + e_i =
 // x - e_opp(i), bit opp(i) tells whether f*_i streams out to x + e_i.
+// From the counts js9 of the node's 3x3 columns and its height a.
 template <int FACE>
-__device__ __forceinline__ unsigned link_mask(const KP &p, const int *js, int x, int y, int z) {
+__device__ __forceinline__ unsigned link_mask9(const int (&js9)[9], int a) {
     unsigned m = 0;
 #pragma unroll
-    for (int i = 1; i < 19; ++i)
-        if (liquid_at<FACE>(p, js, x - ex(i), y - ey(i), z - ez(i))) m |= 1u << i;
+    for (int i = 1; i < 19; ++i) {
+        // the upstream node x - e_i: in-plane column offset and height
+        const int dp = -ex(i), dq = FACE == 0 ? -ez(i) : -ey(i), da = FACE == 0 ? -ey(i) : -ez(i);
+        const int an = a + da;
+        if (an >= 0 && an < js9[(dq + 1) * 3 + dp + 1]) m |= 1u << i;
+    }
     return m;
 }
+
+// Liquid counts of the twelve columns around those of a pair (the 3x3 columns
+// of both, pp - 1 .. pp + 2 by q - 1 .. q + 1), 0 outside the cavity; entry
+// (dq + 1) * 4 + dp + 1.
+__device__ __forceinline__ void load_js12(const KP &p, const int *__restrict__ js, int pp, int q, int (&c)[12]) {
+#pragma unroll
+    for (int dq = -1; dq <= 1; ++dq)
+#pragma unroll
+        for (int dp = -1; dp <= 2; ++dp) {
+            const int p2 = pp + dp, q2 = q + dq;
+            const bool in = (unsigned)p2 < (unsigned)p.P1 && (unsigned)q2 < (unsigned)p.P2;
+            c[(dq + 1) * 4 + dp + 1] = in ? __ldg(js + q2 * p.P1 + p2) : 0;
+        }
+}
+// Smallest (over columns inside the cavity) and largest of them.
+__device__ __forceinline__ void range_js12(const KP &p, const int (&c)[12], int pp, int q, int &mn, int &mx) {
+    mn = 1 << 15;
+    mx = 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const int dp = k % 4 - 1, dq = k / 4 - 1;
+        const bool in = (unsigned)(pp + dp) < (unsigned)p.P1 && (unsigned)(q + dq) < (unsigned)p.P2;
+        mn = in && c[k] < mn ? c[k] : mn;
+        mx = c[k] > mx ? c[k] : mx;
+    }
+}
+// The 3x3 counts (load_js9) of the pair's node `lane` (0 or 1).
+__device__ __forceinline__ void js9_of_js12(const int (&c)[12], int lane, int (&js9)[9]) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) js9[k] = lane ? c[k / 3 * 4 + k % 3 + 1] : c[k / 3 * 4 + k % 3];
+}
+
 // Bit i (1..6): node x - t_i is inside (else the link crosses a wall).
 __device__ __forceinline__ unsigned inside_mask(const KP &p, int x, int y, int z) {
     unsigned m = 0;
@@ -253,17 +304,26 @@ __device__ __forceinline__ bool xwall(int ex_up, bool xlo, bool xhi) {
 //
 // Fast path: a liquid node off the walls of the heating axis and of the
 // other in-plane axis and at least one node below the lowest first-solid
-// node of its 3x3 neighbour columns, so that every link streams except those
+// node of its 3x3 neighbour columns (by the bounds of nb, which may be two
+// low, else by the counts themselves, which the general path needs for its
+// link mask anyway), so that every link streams except those
 // across an x wall, which bounce back (no-slip for f, adiabatic for g).  The
 // x walls are taken by selects inside the fast path, so that the warps that
 // hold x = 0 or x = nx - 1 do not split between two paths.
 //
 // COND: heat conduction in the solid (see even_node).
+//
+// known: the node's 3x3 liquid counts where the caller has them, else null.
+//
+// js_old: the liquid counts the in-flight values were produced under.  A node
+// that has become liquid since (never on the fast path: the count bounds nb
+// are at most the old counts less one) starts from fh = 0.
 template <typename ST, int FACE, bool TAB = true, bool COND = false>
 __device__ __forceinline__ void odd_node(const KP &p, const Links *lk, ST *__restrict__ F, ST *__restrict__ G, const int *__restrict__ js,
-                                         const int *__restrict__ nb, const float *__restrict__ gpost,
+                                         const int *__restrict__ js_old, const int *__restrict__ nb, const float *__restrict__ gpost,
                                          const float *__restrict__ thw_rd, const float *__restrict__ thw_wr, int x,
-                                         int y, int z, const float *__restrict__ spost = nullptr) {
+                                         int y, int z, const float *__restrict__ spost = nullptr,
+                                         const int *known = nullptr) {
     const long long c = node_index(p, x, y, z);
     const int a = axial<FACE>(x, y, z);
     const int col = column<FACE>(p, x, y, z);
@@ -277,9 +337,29 @@ __device__ __forceinline__ void odd_node(const KP &p, const Links *lk, ST *__res
     ST *const Gc = G + c;
     float g[7];
     if (a < jsc) {
-        const bool fast = off_qa && a + 1 < (nbv >> 16);
+        bool fast = off_qa && a + 1 < (nbv >> 16);
         float f[19];
         unsigned lm = 0x7fffeu, im = 0x7eu;
+        if (!fast) {
+            int js9[9];
+            if (known) {
+#pragma unroll
+                for (int k = 0; k < 9; ++k) js9[k] = known[k];
+            } else {
+                load_js9(p, js, x, q, js9);
+            }
+            lm = link_mask9<FACE>(js9, a);
+            im = inside_mask(p, x, y, z);
+            // off the walls a full mask, but for the links across an x wall
+            // (which read count 0), is the interior
+            if (off_qa) {
+                unsigned need = 0x7fffeu;
+#pragma unroll
+                for (int i = 1; i < 19; ++i)
+                    if (xwall(ex(i), xlo, xhi)) need &= ~(1u << i);
+                fast = (lm & need) == need;
+            }
+        }
         if (fast) {
 #pragma unroll
             for (int i = 0; i < 19; ++i) f[i] = Store<ST>::ld(Fc + fin_off<FACE, TAB>(p, lk, i));
@@ -299,13 +379,16 @@ __device__ __forceinline__ void odd_node(const KP &p, const Links *lk, ST *__res
                     if (xwall(tx(i), xlo, xhi)) g[i] = Store<ST>::ld(Gc + i * p.ld);
             }
         } else {
-            lm = link_mask<FACE>(p, js, x, y, z);
-            im = inside_mask(p, x, y, z);
             const float th_rd = __ldg(thw_rd + col);
+            const bool was_liquid = a < __ldg(js_old + col);
             f[0] = Store<ST>::ld(Fc);
 #pragma unroll
             for (int i = 1; i < 19; ++i)  // else bounce-back: f*_opp(i) parked in slot i
                 f[i] = Store<ST>::ld(((lm >> i) & 1u) ? Fc + fin_off<FACE, TAB>(p, lk, i) : Fc + i * p.ld);
+            if (!was_liquid) {
+#pragma unroll
+                for (int i = 0; i < 19; ++i) f[i] = 0.0f;
+            }
             g[0] = Store<ST>::ld(Gc);
 #pragma unroll
             for (int i = 1; i < 7; ++i) {
@@ -373,26 +456,28 @@ __device__ __forceinline__ void odd_node(const KP &p, const Links *lk, ST *__res
 
 template <typename ST, int FACE>
 __global__ void __launch_bounds__(128, k1_min_blocks<ST>()) k_odd(const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G,
-                                             const int *__restrict__ js, const int *__restrict__ nb,
+                                             const int *__restrict__ js, const int *__restrict__ js_old,
+                                             const int *__restrict__ nb,
                                              const float *__restrict__ gpost, const float *__restrict__ thw_rd,
                                              const float *__restrict__ thw_wr, const __grid_constant__ Links lk,
                                              const int *jmax) {
     step_launch_wait();
     int x, y, z;
-    if (k1_node<FACE>(p, jmax, x, y, z)) odd_node<ST, FACE>(p, &lk, F, G, js, nb, gpost, thw_rd, thw_wr, x, y, z);
+    if (k1_node<FACE>(p, jmax, x, y, z)) odd_node<ST, FACE>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x, y, z);
 }
 
 // The odd step with heat conduction in the solid (every node updated).
 template <typename ST, int FACE>
 __global__ void __launch_bounds__(128) k_odd_cond(const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G,
-                                                  const int *__restrict__ js, const int *__restrict__ nb,
+                                                  const int *__restrict__ js, const int *__restrict__ js_old,
+                                                  const int *__restrict__ nb,
                                                   const float *__restrict__ gpost, const float *__restrict__ thw_rd,
                                                   const float *__restrict__ thw_wr, const __grid_constant__ Links lk,
                                                   const float *__restrict__ spost) {
     step_launch_wait();
     int x, y, z;
     if (k1_node<FACE>(p, nullptr, x, y, z))
-        odd_node<ST, FACE, true, true>(p, &lk, F, G, js, nb, gpost, thw_rd, thw_wr, x, y, z, spost);
+        odd_node<ST, FACE, true, true>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x, y, z, spost);
 }
 
 
@@ -541,18 +626,25 @@ __device__ __forceinline__ void odd_pair_liquid(const KP &p, const Links *lk, ST
 template <typename ST, int FACE, typename IX>
 __device__ __forceinline__ void odd_pair(const KP &p, const Links *lk, ST *__restrict__ F,
                                          ST *__restrict__ G, const int *__restrict__ js,
-                                         const int *__restrict__ nb, const float *__restrict__ gpost,
-                                         const float *__restrict__ thw_rd, const float *__restrict__ thw_wr, int x,
-                                         int y, int z) {
+                                         const int *__restrict__ js_old, const int *__restrict__ nb,
+                                         const float *__restrict__ gpost, const float *__restrict__ thw_rd,
+                                         const float *__restrict__ thw_wr, int x, int y, int z) {
     const int a = axial<FACE>(x, y, z);
     const int col = column<FACE>(p, x, y, z);
     const int q = FACE == 0 ? z : y, nq = FACE == 0 ? p.nz : p.ny;
     const bool off_qa = q >= 1 && q <= nq - 2 && a >= 1 && a <= p.H - 2;
-    const bool fast = off_qa && a + 1 < (__ldg(nb + col) >> 16) && a + 1 < (__ldg(nb + col + 1) >> 16);
-    if (!fast) {
-        odd_node<ST, FACE>(p, lk, F, G, js, nb, gpost, thw_rd, thw_wr, x, y, z);
-        odd_node<ST, FACE>(p, lk, F, G, js, nb, gpost, thw_rd, thw_wr, x + 1, y, z);
-        return;
+    const int b0 = __ldg(nb + col) >> 16, b1 = __ldg(nb + col + 1) >> 16;
+    if (!(off_qa && a + 1 < b0 && a + 1 < b1)) {
+        int c12[12], js9[9], mn, mx;
+        load_js12(p, js, x, q, c12);
+        range_js12(p, c12, x, q, mn, mx);
+        if (!(off_qa && a + 1 < mn)) {  // the bounds may be two low
+            js9_of_js12(c12, 0, js9);
+            odd_node<ST, FACE>(p, lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x, y, z, nullptr, js9);
+            js9_of_js12(c12, 1, js9);
+            odd_node<ST, FACE>(p, lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x + 1, y, z, nullptr, js9);
+            return;
+        }
     }
     odd_pair_liquid<ST, FACE, IX>(p, lk, F, G, x, y, z);
 }
@@ -560,13 +652,14 @@ __device__ __forceinline__ void odd_pair(const KP &p, const Links *lk, ST *__res
 template <typename ST, int FACE, typename IX>
 __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair(const __grid_constant__ KP p, ST *__restrict__ F,
                                                      ST *__restrict__ G, const int *__restrict__ js,
-                                                     const int *__restrict__ nb, const float *__restrict__ gpost,
+                                                     const int *__restrict__ js_old, const int *__restrict__ nb,
+                                                     const float *__restrict__ gpost,
                                                      const float *__restrict__ thw_rd,
                                                      const float *__restrict__ thw_wr,
                                                      const __grid_constant__ Links lk, const int *jmax) {
     step_launch_wait();
     int x, y, z;
-    if (k1_pair<FACE>(p, jmax, x, y, z)) odd_pair<ST, FACE, IX>(p, &lk, F, G, js, nb, gpost, thw_rd, thw_wr, x, y, z);
+    if (k1_pair<FACE>(p, jmax, x, y, z)) odd_pair<ST, FACE, IX>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x, y, z);
 }
 
 
@@ -594,8 +687,8 @@ __device__ __forceinline__ void gather_g(const KP &p, const ST *G, int x, int y,
     }
 }
 
-// Shifted pre-collision f of a liquid node, with the liquid flags js that
-// the in-flight values were produced under.
+// Shifted pre-collision f of a liquid node.  js: the liquid flags that the
+// in-flight values were produced under, or the ones after flip_column has run.
 template <typename ST, int FACE>
 __device__ __forceinline__ void gather_f(const KP &p, const ST *F, const int *js, int x, int y, int z,
                                          bool inflight, float (&f)[19]) {
@@ -610,17 +703,18 @@ __device__ __forceinline__ void gather_f(const KP &p, const ST *F, const int *js
     }
 }
 
-// Liquid counts of the 3x3 columns around column (pp, q), 0 outside the
-// cavity; entry (dq + 1) * 3 + dp + 1.
-__device__ __forceinline__ void load_js9(const KP &p, const int *__restrict__ js, int pp, int q, int (&js9)[9]) {
+// gather_f of the state between steps (flip_column has run): a node that has
+// become liquid since the in-flight values were produced (under js_old)
+// starts from fh = 0 (in the natural layout its slots hold that).
+template <typename ST, int FACE>
+__device__ __forceinline__ void gather_f_now(const KP &p, const ST *F, const int *js, const int *js_old, int x, int y,
+                                             int z, bool inflight, float (&f)[19]) {
+    if (inflight && axial<FACE>(x, y, z) >= js_old[column<FACE>(p, x, y, z)]) {
 #pragma unroll
-    for (int dq = -1; dq <= 1; ++dq)
-#pragma unroll
-        for (int dp = -1; dp <= 1; ++dp) {
-            const int p2 = pp + dp, q2 = q + dq;
-            const bool in = (unsigned)p2 < (unsigned)p.P1 && (unsigned)q2 < (unsigned)p.P2;
-            js9[(dq + 1) * 3 + dp + 1] = in ? __ldg(js + q2 * p.P1 + p2) : 0;
-        }
+        for (int i = 0; i < 19; ++i) f[i] = 0.0f;
+        return;
+    }
+    gather_f<ST, FACE>(p, F, js, x, y, z, inflight, f);
 }
 
 // gather_f in flight for the node at height a of the middle column, with
@@ -709,6 +803,76 @@ __device__ __forceinline__ float solid_gradient(int ks, int H, double sc, float 
            Y2 * (float)(sc - x1) / ((float)(x2 - sc) * (float)(x2 - x1));
 }
 
+// Bounds of the liquid counts of the 3x3 columns after a front update, from
+// the counts js9 before it (a count changes by at most one a step: a front
+// that moves half a node or more is reported as unstable), packed as
+// min << 16 | max.  The stream-collide's interior and deep-solid tests use
+// them: a bound one node wide of the true one sends a node to the general
+// path or updates a node at rest, with the same results.
+__device__ __forceinline__ int count_bounds(const KP &p, const int (&js9)[9], int pp, int q) {
+    int mn = 1 << 15, mx = 0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const int dp = k % 3 - 1, dq = k / 3 - 1;
+        const bool in = (unsigned)(pp + dp) < (unsigned)p.P1 && (unsigned)(q + dq) < (unsigned)p.P2;
+        mn = in && js9[k] < mn ? js9[k] : mn;
+        mx = js9[k] > mx ? js9[k] : mx;
+    }
+    return ((mn > 0 ? mn - 1 : 0) << 16) | (mx + 1);
+}
+
+// ------------------------------------------------------------------ flip
+// Nodes of a column between the old and the new liquid counts (jo, jn)
+// changed phase.
+// Natural layout: a newly liquid node y gets fh = 0 (f = f^eq(1, 0)).
+// In flight, for every node x = y + e_i that was liquid (liquid counts js):
+//   y newly liquid: x's population towards y bounced back under the old flags,
+//     so it waits in x's own slot i; the odd step, seeing y liquid, looks in
+//     slot opp(i) of y, so it is moved there (y's own fh = 0 is left to the
+//     readers: see odd_node, gather_f_now);
+//   y newly solid: x's population from y waits in slot opp(i) of y; the odd
+//     step, seeing y solid, looks in x's own slot i.
+// The column's own thread does this right after its front update, while other
+// columns are still reading f for their ghosts: no slot written here is one
+// that they read.  The first kind writes only slots of a node that was solid,
+// and the ghost of a column reads slots of nodes that were liquid; the second
+// writes slot i of x, which only the ghost whose source node is y reads, and
+// that is this column's, whose source has moved below y.  Flags of the new
+// state are not needed: a value moved for a node x that turns solid itself is
+// read by nothing.
+template <typename ST, int FACE>
+__device__ __forceinline__ void flip_column(const KP &p, ST *__restrict__ F, const int *__restrict__ js, bool inflight,
+                                            int col, int jo, int jn) {
+    const int lo = jo < jn ? jo : jn, hi = jo < jn ? jn : jo;
+    for (int j = lo; j < hi; ++j) {
+        int x, y, z;
+        column_node<FACE>(p, col, j, x, y, z);
+        const long long c = node_index(p, x, y, z);
+        if (!inflight) {
+            if (jo < jn) {
+#pragma unroll
+                for (int i = 0; i < 19; ++i) Store<ST>::st(F + i * p.ld + c, 0.0f);
+            }
+            continue;
+        }
+        // every load before the first store (the compiler cannot move a load
+        // above a store into the same array)
+        bool on[19];
+        float v[19];
+#pragma unroll
+        for (int i = 1; i < 19; ++i) {
+            on[i] = liquid_at<FACE>(p, js, x + ex(i), y + ey(i), z + ez(i));
+            const ST *from = jo < jn ? F + i * p.ld + (c + off19<FACE>(p, i)) : F + opp(i) * p.ld + c;
+            v[i] = on[i] ? Store<ST>::ld(from) : 0.0f;
+        }
+#pragma unroll
+        for (int i = 1; i < 19; ++i) {
+            ST *to = jo < jn ? F + opp(i) * p.ld + c : F + i * p.ld + (c + off19<FACE>(p, i));
+            if (on[i]) Store<ST>::st(to, v[i]);
+        }
+    }
+}
+
 // ------------------------------------------------------------ front (Eq. 6)
 // One thread per column.  From the state after a step (T of the liquid at
 // t + 1, front s_t): the one-sided quadratic gradient at the front, the
@@ -718,7 +882,8 @@ __device__ __forceinline__ float solid_gradient(int ks, int H, double sc, float 
 // front: g*_ghost = g^eq(T_ghost, 0) + (g*_L - g^eq(T_L, u_L)).
 // move = 0 keeps the front (used to prepare the ghost after a state upload).
 // SPEC: load the ghost's likely source node together with the gradient
-// stencil (two dependent load stages instead of three; more registers).
+// stencil (two dependent load stages instead of three; more registers), and
+// flip the column's nodes; without it the caller flips them.
 //
 // Precision: the front heights are accumulated in FP64 (s + ds, and the
 // distances from s to the stencil nodes and the ghost are FP64 differences);
@@ -734,9 +899,9 @@ __device__ __forceinline__ float solid_gradient(int ks, int H, double sc, float 
 // with T_sghost on the line through (s, Tm) and the guarded solid node (or
 // the cold wall); the rest state at Tm in a column without both phases.
 template <typename ST, int FACE, bool SPEC = true, bool COND = false>
-__device__ __forceinline__ int front_column(const KP &p, const ST *__restrict__ F, const ST *__restrict__ G,
+__device__ __forceinline__ int front_column(const KP &p, ST *__restrict__ F, const ST *__restrict__ G,
                                            const int *__restrict__ js, int *__restrict__ js_next,
-                                           const double *__restrict__ s, double *__restrict__ s_next,
+                                           int *__restrict__ nb_next, const double *__restrict__ s, double *__restrict__ s_next,
                                            float *__restrict__ gpost, const float *__restrict__ thw, int inflight,
                                            int move, int *__restrict__ status, int col,
                                            float *__restrict__ spost = nullptr) {
@@ -749,12 +914,13 @@ __device__ __forceinline__ int front_column(const KP &p, const ST *__restrict__ 
     const float Tw = thw[col];
     const int jsc = js[col];
     int js9[9];
-    if (SPEC && infl) load_js9(p, js, pp, q, js9);
+    load_js9(p, js, pp, q, js9);
     float sp = 0.0f, sq = 0.0f;
     if (move) {
         sp = 0.5f * (float)(s[q * P1 + (pp + 1 < P1 ? pp + 1 : pp)] - s[q * P1 + (pp > 0 ? pp - 1 : pp)]);
         sq = 0.5f * (float)(s[(q + 1 < P2 ? q + 1 : q) * P1 + pp] - s[(q > 0 ? q - 1 : q) * P1 + pp]);
     }
+    nb_next[col] = count_bounds(p, js9, pp, q);
     // Load stage 2: the gradient stencil of s_t and, speculatively, the node
     // below the current front, which is the ghost's source node whenever the
     // liquid count does not change (all but a few columns per step).
@@ -845,7 +1011,10 @@ __device__ __forceinline__ int front_column(const KP &p, const ST *__restrict__ 
 #pragma unroll
         for (int i = 0; i < 7; ++i) spost[(long long)i * p.ncols + col] = sg[i];
     }
-    if (jn >= H) return jn;  // fully liquid column: no ghost node
+    if (jn >= H) {  // fully liquid column: no ghost node
+        if (SPEC && move && jn != jsc) flip_column<ST, FACE>(p, F, js, infl, col, jsc, jn);
+        return jn;
+    }
     const double yg = jn + 0.5;
     const int kg = guarded_node(sn, H);
     float Tg;
@@ -905,16 +1074,22 @@ __device__ __forceinline__ int front_column(const KP &p, const ST *__restrict__ 
     }
 #pragma unroll
     for (int i = 0; i < 7; ++i) gpost[(long long)i * p.ncols + col] = gh[i];
+    if (SPEC && move && jn != jsc) flip_column<ST, FACE>(p, F, js, infl, col, jsc, jn);
     return jn;
 }
 
+// 4 blocks of 128 a multiprocessor (128 registers: 608 blocks cover a 256 x
+// 256 front at once; without the cap, 136 and 192 registers, the loop of
+// single 256^3 steps lost 2.5 us a step to a second wave).
+//
 // jmax (may be null): running maximum of the liquid counts, one atomic per
 // warp; the host reads it back now and then to bound the height of the
 // stream-collide grid (nodes two above every neighbouring count are deep
 // solid and do nothing).
 template <typename ST, int FACE>
-__global__ void __launch_bounds__(128) k_front(const __grid_constant__ KP p, const ST *__restrict__ F, const ST *__restrict__ G,
+__global__ void __launch_bounds__(128, 4) k_front(const __grid_constant__ KP p, ST *__restrict__ F, const ST *__restrict__ G,
                                                const int *__restrict__ js, int *__restrict__ js_next,
+                                               int *__restrict__ nb_next,
                                                const double *__restrict__ s, double *__restrict__ s_next,
                                                float *__restrict__ gpost, const float *__restrict__ thw,
                                                int inflight, int move, int *__restrict__ status,
@@ -922,7 +1097,7 @@ __global__ void __launch_bounds__(128) k_front(const __grid_constant__ KP p, con
     step_launch_wait();
     const int col = blockIdx.x * blockDim.x + threadIdx.x;
     int jn = -1;
-    if (col < p.ncols) jn = front_column<ST, FACE>(p, F, G, js, js_next, s, s_next, gpost, thw, inflight, move, status, col);
+    if (col < p.ncols) jn = front_column<ST, FACE>(p, F, G, js, js_next, nb_next, s, s_next, gpost, thw, inflight, move, status, col);
     // blocks are whole warps and every thread of the grid reaches this point
     const int m = __reduce_max_sync(0xffffffffu, jn);
     if (jmax && (threadIdx.x & 31) == 0 && m >= 0) atomicMax(jmax, m);
@@ -930,127 +1105,18 @@ __global__ void __launch_bounds__(128) k_front(const __grid_constant__ KP p, con
 
 // The front update with heat conduction in the solid.
 template <typename ST, int FACE>
-__global__ void __launch_bounds__(128) k_front_cond(const __grid_constant__ KP p, const ST *__restrict__ F,
+__global__ void __launch_bounds__(128) k_front_cond(const __grid_constant__ KP p, ST *__restrict__ F,
                                                     const ST *__restrict__ G, const int *__restrict__ js,
-                                                    int *__restrict__ js_next, const double *__restrict__ s,
+                                                    int *__restrict__ js_next, int *__restrict__ nb_next,
+                                                    const double *__restrict__ s,
                                                     double *__restrict__ s_next, float *__restrict__ gpost,
                                                     float *__restrict__ spost, const float *__restrict__ thw,
                                                     int inflight, int move, int *__restrict__ status) {
     step_launch_wait();
     const int col = blockIdx.x * blockDim.x + threadIdx.x;
     if (col < p.ncols)
-        front_column<ST, FACE, true, true>(p, F, G, js, js_next, s, s_next, gpost, thw, inflight, move, status, col,
+        front_column<ST, FACE, true, true>(p, F, G, js, js_next, nb_next, s, s_next, gpost, thw, inflight, move, status, col,
                                            spost);
-}
-
-
-// ------------------------------------------------------------------ flip
-// Nodes of a column between the old and the new liquid counts changed phase.
-// Natural layout: a newly liquid node gets fh = 0 (f = f^eq(1, 0)).
-// In flight: every link (x, x - e_i) touching a flipped node has its two
-// slots P = slot opp(i) of x - e_i and Q = slot i of x rewritten so that the
-// odd step's reads under the new flags deliver the values prescribed by the
-// old flags (streaming if the upstream node was liquid, bounce-back if not)
-// and zero to a newly liquid node.  A link whose two ends both flipped is
-// handled once, by the end with the lower node index.
-//
-// Every column also records the minimum and maximum of the new liquid counts
-// over its 3x3 neighbourhood (min << 16 | max) for the interior and
-// deep-solid tests of the next stream-collide.  do_flip = 0 only records.
-// The links I0 .. I0 + 8 of a flipped node c = (x, y, z) (see flip_column).
-// The 18 links of one node touch 36 distinct slots (slot i of c, slot opp(i)
-// of c - e_i), so every phase flag and slot of the nine is loaded before the
-// first store: the loads are in flight together, where a link-by-link loop
-// waits two dependent memory round trips per link (the compiler cannot move
-// a load above a store into the same array).  Same values, same stores.
-template <typename ST, int FACE, int I0>
-__device__ __forceinline__ void flip_links(const KP &p, ST *__restrict__ F, const int *__restrict__ js_old,
-                                           const int *__restrict__ js_new, int x, int y, int z, long long c,
-                                           bool lx_t, bool lx_n) {
-    bool yin[9], ly_t[9], ly_n[9], own[9];
-    long long cy[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const int i = I0 + k;
-        const int xn = x - ex(i), yn = y - ey(i), zn = z - ez(i);
-        yin[k] = inside(p, xn, yn, zn);
-        ly_t[k] = ly_n[k] = false;
-        cy[k] = 0;
-        if (yin[k]) {
-            const int cc = column<FACE>(p, xn, yn, zn), an = axial<FACE>(xn, yn, zn);
-            ly_t[k] = an < js_old[cc];
-            ly_n[k] = an < js_new[cc];
-            cy[k] = node_index(p, xn, yn, zn);
-        }
-        own[k] = !(ly_t[k] != ly_n[k] && cy[k] < c);  // else the other end owns this link
-    }
-    float P[9], Q[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const int i = I0 + k;
-        P[k] = own[k] && yin[k] ? Store<ST>::ld(F + opp(i) * p.ld + cy[k]) : 0.0f;
-        Q[k] = own[k] ? Store<ST>::ld(F + i * p.ld + c) : 0.0f;
-    }
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        if (!own[k]) continue;
-        const int i = I0 + k;
-        ST *Ps = F + opp(i) * p.ld + cy[k];
-        ST *Qs = F + i * p.ld + c;
-        const float dx = !lx_t ? 0.0f : (ly_t[k] ? P[k] : Q[k]);
-        const float dy = !ly_t[k] ? 0.0f : (lx_t ? Q[k] : P[k]);
-        if (lx_n && ly_n[k]) { Store<ST>::st(Ps, dx); Store<ST>::st(Qs, dy); }
-        else if (lx_n) Store<ST>::st(Qs, dx);
-        else if (ly_n[k]) Store<ST>::st(Ps, dy);
-    }
-}
-
-template <typename ST, int FACE>
-__device__ __forceinline__ void flip_column(const KP &p, ST *__restrict__ F, const int *__restrict__ js_old,
-                                          const int *__restrict__ js_new, int *__restrict__ nb_new, int inflight,
-                                          int do_flip, int col) {
-    {
-        const int pp = col % p.P1, q = col / p.P1;
-        int mn = 1 << 15, mx = 0;
-        for (int dq = -1; dq <= 1; ++dq)
-            for (int dp = -1; dp <= 1; ++dp) {
-                const int p2 = pp + dp, q2 = q + dq;
-                if (p2 < 0 || p2 >= p.P1 || q2 < 0 || q2 >= p.P2) continue;
-                const int v = js_new[q2 * p.P1 + p2];
-                mn = v < mn ? v : mn;
-                mx = v > mx ? v : mx;
-            }
-        nb_new[col] = (mn << 16) | mx;
-    }
-    const int jo = js_old[col], jn = js_new[col];
-    if (!do_flip || jo == jn) return;
-    const int lo = jo < jn ? jo : jn, hi = jo < jn ? jn : jo;
-    for (int j = lo; j < hi; ++j) {
-        int x, y, z;
-        column_node<FACE>(p, col, j, x, y, z);
-        const long long c = node_index(p, x, y, z);
-        const bool lx_t = j < jo, lx_n = j < jn;
-        if (!inflight) {
-            if (lx_n && !lx_t)
-                for (int i = 0; i < 19; ++i) Store<ST>::st(F + i * p.ld + c, 0.0f);
-            continue;
-        }
-        if (lx_n && !lx_t) Store<ST>::st(F + c, 0.0f);
-        flip_links<ST, FACE, 1>(p, F, js_old, js_new, x, y, z, c, lx_t, lx_n);
-        flip_links<ST, FACE, 10>(p, F, js_old, js_new, x, y, z, c, lx_t, lx_n);
-    }
-}
-
-// 4 blocks of 128 a multiprocessor (up to 128 registers: flip_links holds
-// nine links' flags and slots; 608 blocks cover a 256 x 256 front at once).
-template <typename ST, int FACE>
-__global__ void __launch_bounds__(128, 4) k_flip(const __grid_constant__ KP p, ST *__restrict__ F, const int *__restrict__ js_old,
-                                              const int *__restrict__ js_new, int *__restrict__ nb_new,
-                                              int inflight, int do_flip) {
-    step_launch_wait();
-    const int col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col >= p.ncols) return;
-    flip_column<ST, FACE>(p, F, js_old, js_new, nb_new, inflight, do_flip, col);
 }
 
 
@@ -1059,7 +1125,8 @@ __global__ void __launch_bounds__(128, 4) k_flip(const __grid_constant__ KP p, S
 // in the solid, and u = 0), natural values.
 template <typename ST, int FACE>
 __global__ void __launch_bounds__(128) k_macro(const __grid_constant__ KP p, const ST *__restrict__ F, const ST *__restrict__ G,
-                                               const int *__restrict__ js, const float *__restrict__ thw,
+                                               const int *__restrict__ js, const int *__restrict__ js_old,
+                                               const float *__restrict__ thw,
                                                int inflight, float *__restrict__ T, float *__restrict__ u) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -1071,7 +1138,7 @@ __global__ void __launch_bounds__(128) k_macro(const __grid_constant__ KP p, con
     if (a < js[col]) {
         float g[7], f[19];
         gather_g<ST, FACE>(p, G, x, y, z, inflight != 0, thw, g);
-        gather_f<ST, FACE>(p, F, js, x, y, z, inflight != 0, f);
+        gather_f_now<ST, FACE>(p, F, js, js_old, x, y, z, inflight != 0, f);
         float Th = 0.0f;
 #pragma unroll
         for (int i = 0; i < 7; ++i) Th += g[i];
@@ -1093,7 +1160,8 @@ __global__ void __launch_bounds__(128) k_macro(const __grid_constant__ KP p, con
 // rest at Tm, the value their slots would hold if they were updated.
 template <typename ST, int FACE>
 __global__ void __launch_bounds__(128) k_state_out(const __grid_constant__ KP p, const ST *__restrict__ F, const ST *__restrict__ G,
-                                                   const int *__restrict__ js, const int *__restrict__ nb,
+                                                   const int *__restrict__ js, const int *__restrict__ js_old,
+                                                   const int *__restrict__ nb,
                                                    const float *__restrict__ thw, int inflight,
                                                    float *__restrict__ fo, float *__restrict__ go) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1116,7 +1184,7 @@ __global__ void __launch_bounds__(128) k_state_out(const __grid_constant__ KP p,
     if (fo) {
         float f[19];
         const bool liq = a < js[col];
-        if (liq) gather_f<ST, FACE>(p, F, js, x, y, z, inflight != 0, f);
+        if (liq) gather_f_now<ST, FACE>(p, F, js, js_old, x, y, z, inflight != 0, f);
 #pragma unroll
         for (int i = 0; i < 19; ++i) fo[i * p.N + c] = liq ? f[i] + w19(i) : 0.0f;
     }
@@ -1194,7 +1262,8 @@ __global__ void __launch_bounds__(128) k_nusselt(const __grid_constant__ KP p, c
 // count, max |u|^2.  Fixed block and thread order: deterministic.
 template <typename ST, int FACE>
 __global__ void __launch_bounds__(256) k_totals_part(const __grid_constant__ KP p, const ST *__restrict__ F, const ST *__restrict__ G,
-                                                     const int *__restrict__ js, const float *__restrict__ thw,
+                                                     const int *__restrict__ js, const int *__restrict__ js_old,
+                                                     const float *__restrict__ thw,
                                                      int inflight, double *__restrict__ part) {
     __shared__ double sh[4][256];
     double sT = 0.0, sr = 0.0, n = 0.0, umax = 0.0;
@@ -1204,7 +1273,7 @@ __global__ void __launch_bounds__(256) k_totals_part(const __grid_constant__ KP 
         if (axial<FACE>(x, y, z) >= js[column<FACE>(p, x, y, z)]) continue;
         float g[7], f[19];
         gather_g<ST, FACE>(p, G, x, y, z, inflight != 0, thw, g);
-        gather_f<ST, FACE>(p, F, js, x, y, z, inflight != 0, f);
+        gather_f_now<ST, FACE>(p, F, js, js_old, x, y, z, inflight != 0, f);
         float Th = 0.0f, rh = 0.0f, ux = 0.0f, uy = 0.0f, uz = 0.0f;
 #pragma unroll
         for (int i = 0; i < 7; ++i) Th += g[i];

@@ -41,7 +41,6 @@ template <typename ST> struct LaunchCond {
 template <typename ST> struct Launch {
     static cudaError_t stream_collide(const KP &p, int face, int odd, const Bufs &b, dim3 blk, cudaStream_t st);
     static cudaError_t front(const KP &p, int face, int inflight, int move, const Bufs &b, cudaStream_t st);
-    static cudaError_t flip(const KP &p, int face, int inflight, int do_flip, const Bufs &b, cudaStream_t st);
     static cudaError_t macro(const KP &p, int face, int inflight, const Bufs &b, float *T, float *u, cudaStream_t st);
     static cudaError_t state_out(const KP &p, int face, int inflight, const Bufs &b, float *f, float *g, cudaStream_t st);
     static cudaError_t state_in(const KP &p, int face, const Bufs &b, const float *f, const float *g, cudaStream_t st);
@@ -51,8 +50,7 @@ template <typename ST> struct Launch {
     static cudaError_t nusselt(const KP &p, int face, int inflight, const Bufs &b, cudaStream_t st);
 };
 
-// Threads per block of the per-column kernels (front, flip and their
-// adjoints): the largest of 128, 64 and 32 that still gives two blocks per
+// Threads per block of the per-column kernels (front and its adjoints): the largest of 128, 64 and 32 that still gives two blocks per
 // SM, so that a small front (96 x 96 columns) spreads its FP64 arithmetic
 // over all SMs instead of half of them.
 inline int col_block(long long ncols, int sms) {

@@ -7,7 +7,7 @@
 
 namespace lbm {
 
-// The step's kernels (stream-collide, front, flip) are launched with
+// The step's kernels (stream-collide, front) are launched with
 // programmatic stream serialization (see step_launch_wait) when LBM_PDL.
 #ifndef LBM_PDL
 #define LBM_PDL 1
@@ -36,10 +36,10 @@ static cudaError_t launch_sc(const KP &p, int face, int odd, const Bufs &b, dim3
     const int *jm = p.skip_deep ? b.jmax : nullptr;
     ST *F = (ST *)b.F, *G = (ST *)b.G;
     if (face == 0) {
-        if (odd) return launch_step_kernel(k_odd<ST, 0>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
+        if (odd) return launch_step_kernel(k_odd<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
         else return launch_step_kernel(k_even<ST, 0, IXE>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, jm);
     } else {
-        if (odd) return launch_step_kernel(k_odd<ST, 1>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
+        if (odd) return launch_step_kernel(k_odd<ST, 1>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
         else return launch_step_kernel(k_even<ST, 1, IXE>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, jm);
     }
 }
@@ -57,10 +57,10 @@ static cudaError_t launch_sc_pair(const KP &p, int face, int odd, const Bufs &b,
     half_x.nx = p.nx / 2;
     dim3 grd = k1_grid(half_x, blk, face, b.k1_height);
     if (face == 0) {
-        if (odd) return launch_step_kernel(k_odd_pair<ST, 0, IXO>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
+        if (odd) return launch_step_kernel(k_odd_pair<ST, 0, IXO>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
         else return launch_step_kernel(k_even_pair<ST, 0, IXE>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, jm);
     } else {
-        if (odd) return launch_step_kernel(k_odd_pair<ST, 1, IXO>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
+        if (odd) return launch_step_kernel(k_odd_pair<ST, 1, IXO>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
         else return launch_step_kernel(k_even_pair<ST, 1, IXE>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, jm);
     }
 }
@@ -85,26 +85,19 @@ template <typename ST>
 cudaError_t Launch<ST>::front(const KP &p, int face, int inflight, int move, const Bufs &b, cudaStream_t st) {
     if (p.cond) return LaunchCond<ST>::front(p, face, inflight, move, b, st);
     const dim3 blk(b.cblk), grd = col_grid(p.ncols, b.cblk);
-    const ST *F = (const ST *)b.F, *G = (const ST *)b.G;
-    if (face == 0)
-        return launch_step_kernel(k_front<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.s, b.s_next, b.gpost, b.thw_wr, inflight, move, b.status, b.jmax);
-    return launch_step_kernel(k_front<ST, 1>, grd, blk, st, p, F, G, b.js, b.js_next, b.s, b.s_next, b.gpost, b.thw_wr, inflight, move, b.status, b.jmax);
-}
-
-template <typename ST>
-cudaError_t Launch<ST>::flip(const KP &p, int face, int inflight, int do_flip, const Bufs &b, cudaStream_t st) {
-    const dim3 blk(b.cblk), grd = col_grid(p.ncols, b.cblk);
     ST *F = (ST *)b.F;
-    if (face == 0) return launch_step_kernel(k_flip<ST, 0>, grd, blk, st, p, F, b.js, b.js_next, b.nb_next, inflight, do_flip);
-    return launch_step_kernel(k_flip<ST, 1>, grd, blk, st, p, F, b.js, b.js_next, b.nb_next, inflight, do_flip);
+    const ST *G = (const ST *)b.G;
+    if (face == 0)
+        return launch_step_kernel(k_front<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.thw_wr, inflight, move, b.status, b.jmax);
+    return launch_step_kernel(k_front<ST, 1>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.thw_wr, inflight, move, b.status, b.jmax);
 }
 
 template <typename ST>
 cudaError_t Launch<ST>::macro(const KP &p, int face, int inflight, const Bufs &b, float *T, float *u, cudaStream_t st) {
     dim3 blk = node_block(p), grd = node_grid(p, blk);
     const ST *F = (const ST *)b.F, *G = (const ST *)b.G;
-    if (face == 0) k_macro<ST, 0><<<grd, blk, 0, st>>>(p, F, G, b.js, b.thw_rd, inflight, T, u);
-    else k_macro<ST, 1><<<grd, blk, 0, st>>>(p, F, G, b.js, b.thw_rd, inflight, T, u);
+    if (face == 0) k_macro<ST, 0><<<grd, blk, 0, st>>>(p, F, G, b.js, b.js_next, b.thw_rd, inflight, T, u);
+    else k_macro<ST, 1><<<grd, blk, 0, st>>>(p, F, G, b.js, b.js_next, b.thw_rd, inflight, T, u);
     return cudaGetLastError();
 }
 
@@ -112,8 +105,8 @@ template <typename ST>
 cudaError_t Launch<ST>::state_out(const KP &p, int face, int inflight, const Bufs &b, float *f, float *g, cudaStream_t st) {
     dim3 blk = node_block(p), grd = node_grid(p, blk);
     const ST *F = (const ST *)b.F, *G = (const ST *)b.G;
-    if (face == 0) k_state_out<ST, 0><<<grd, blk, 0, st>>>(p, F, G, b.js, b.nb, b.thw_rd, inflight, f, g);
-    else k_state_out<ST, 1><<<grd, blk, 0, st>>>(p, F, G, b.js, b.nb, b.thw_rd, inflight, f, g);
+    if (face == 0) k_state_out<ST, 0><<<grd, blk, 0, st>>>(p, F, G, b.js, b.js_next, b.nb, b.thw_rd, inflight, f, g);
+    else k_state_out<ST, 1><<<grd, blk, 0, st>>>(p, F, G, b.js, b.js_next, b.nb, b.thw_rd, inflight, f, g);
     return cudaGetLastError();
 }
 
@@ -139,8 +132,8 @@ template <typename ST>
 cudaError_t Launch<ST>::totals(const KP &p, int face, int inflight, const Bufs &b, double *part, int nparts,
                                double t, double *out, cudaStream_t st) {
     const ST *F = (const ST *)b.F, *G = (const ST *)b.G;
-    if (face == 0) k_totals_part<ST, 0><<<nparts, 256, 0, st>>>(p, F, G, b.js, b.thw_rd, inflight, part);
-    else k_totals_part<ST, 1><<<nparts, 256, 0, st>>>(p, F, G, b.js, b.thw_rd, inflight, part);
+    if (face == 0) k_totals_part<ST, 0><<<nparts, 256, 0, st>>>(p, F, G, b.js, b.js_next, b.thw_rd, inflight, part);
+    else k_totals_part<ST, 1><<<nparts, 256, 0, st>>>(p, F, G, b.js, b.js_next, b.thw_rd, inflight, part);
     const cudaError_t e = nusselt(p, face, inflight, b, st);
     if (e != cudaSuccess) return e;
     k_totals_final<<<1, 256, 0, st>>>(part, nparts, b.s, b.nu, p.ncols, (double)p.H, t, out);

@@ -214,12 +214,12 @@ Bufs bufs(lbm_melt *h) { return bufs_at(h, h->cur, h->inflight); }
     ((h)->precision == 1 ? lbm::Launch<__half>::method(__VA_ARGS__)                  \
                          : lbm::Launch<float>::method(__VA_ARGS__))
 
-// Prepare js from s, its 3x3 bounds and the ghost nodes from the state
-// (front held, no flip).
+// Prepare js from s and the ghost nodes from the state (front held, no
+// flip), and the 3x3 bounds from the counts before (so after a new s it runs
+// twice: the second call finds both count buffers and the bounds right).
 lbm_status refresh_front(lbm_melt *h) {
     Bufs b = bufs(h);
     CK(LAUNCH(h, front, h->kp, h->face, h->inflight, 0, b, h->stream), "front refresh");
-    CK(LAUNCH(h, flip, h->kp, h->face, h->inflight, 0, b, h->stream), "neighbour bounds");
     h->cur ^= 1;
     return LBM_OK;
 }
@@ -390,7 +390,6 @@ cudaError_t enqueue_step(lbm_melt *h, int &cur, int &inflight, int height, dim3 
     inflight = !odd;
     b = bufs_at(h, cur, inflight);
     e = LAUNCH(h, front, h->kp, h->face, inflight, 1, b, st);
-    if (e == cudaSuccess) e = LAUNCH(h, flip, h->kp, h->face, inflight, 1, b, st);
     cur ^= 1;
     return e;
 }
@@ -708,7 +707,6 @@ LBM_API lbm_status lbm_melt_step(lbm_melt *h, long long n) {
         h->thw_last_prev = 0;
         b = bufs(h);
         CK(LAUNCH(h, front, h->kp, h->face, h->inflight, 1, b, h->stream), "front");
-        CK(LAUNCH(h, flip, h->kp, h->face, h->inflight, 1, b, h->stream), "flip");
         h->cur ^= 1;
         h->steps++;
         h->exec_steps++;
