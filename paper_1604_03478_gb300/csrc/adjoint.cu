@@ -398,8 +398,11 @@ __device__ __forceinline__ void adj_column(const KP &p, int col, const float *__
     // into the column (a node that is not needed is read and ignored), so
     // that no load waits behind a branch
     const bool g_on = GHOST && in.jn < H;
-    if (g_on) in.kg = guarded_node(in.sn, H);
-    if (FRONT) in.k = guarded_node(in.sc, H);
+    FrontPos fs, fc;
+    if (GHOST) fs = front_pos(in.sn, H);
+    if (FRONT) fc = front_pos(in.sc, H);
+    if (g_on) in.kg = guarded_node(fs);
+    if (FRONT) in.k = guarded_node(fc);
     const bool hasL = g_on && in.jn >= 1, hasK = g_on && in.kg >= 0;
     const bool has1 = FRONT && in.k >= 0, has0 = FRONT && in.k >= 1;
     auto node_of = [&](int j) {
@@ -459,19 +462,18 @@ __device__ __forceinline__ void adj_column(const KP &p, int col, const float *__
     if (GHOST) {
         Ls += in.slope;
         if (in.jn < H) {
-            const double sn = in.sn, yg = in.jn + 0.5;
-            const float lTG = in.lTG, dy = (float)(yg - sn);
+            const double sn = in.sn;
+            const float lTG = in.lTG, dy = ghost_distance(fs, in.jn);
             if (in.kg < 0) {
                 const float is = __fdiv_rn(1.0f, (float)sn);
                 dthw += (double)(-__fmul_rn(__fmul_rn(dy, is), lTG));
-                Ls += (double)__fmul_rn(__fmul_rn(__fsub_rn(Tm, Tw), __fmul_rn(__fmul_rn(-(float)yg, is), is)), lTG);
+                Ls += (double)__fmul_rn(__fmul_rn(__fsub_rn(Tm, Tw), __fmul_rn(__fmul_rn(-((float)in.jn + 0.5f), is), is)), lTG);
             } else {
-                const double yk = in.kg + 0.5;
-                const float id = __fdiv_rn(1.0f, (float)(sn - yk)), r = __fmul_rn(dy, id);
+                const float id = __fdiv_rn(1.0f, guarded_distance(fs)), r = __fmul_rn(dy, id);
                 const float lTk = -__fmul_rn(r, lTG);
 #pragma unroll
                 for (int i = 0; i < 7; ++i) add[1][i] = lTk;
-                Ls += (double)__fmul_rn(__fmul_rn(__fsub_rn(Tm, in.Tk), __fmul_rn(__fmul_rn(-(float)(yg - yk), id), id)),
+                Ls += (double)__fmul_rn(__fmul_rn(__fsub_rn(Tm, in.Tk), __fmul_rn(__fmul_rn(-(float)(in.jn - in.kg), id), id)),
                                         lTG);
             }
             if (in.jn >= 1) {
@@ -532,7 +534,7 @@ __device__ __forceinline__ void adj_column(const KP &p, int col, const float *__
         // test below must agree with the forward's); the derivatives through
         // reciprocals.  Operations rounded one by one here too: the kernels
         // that run this (with and without the ghost part) then agree.
-        const float G = front_gradient(k, sc, in.y0, in.y1, Tm, Tw);
+        const float G = front_gradient(k, sc, fc, in.y0, in.y1, Tm, Tw);
         float dGds, dGdy0 = 0.0f, dGdy1 = 0.0f, dGdTw = 0.0f;
         if (k < 0) {
             const float is = __fdiv_rn(1.0f, (float)sc);
@@ -540,9 +542,7 @@ __device__ __forceinline__ void adj_column(const KP &p, int col, const float *__
             dGdTw = -is;
         } else {
             const float y1 = in.y1, y0 = in.y0;
-            const double x1 = k + 0.5;
-            const double x0 = k >= 1 ? k - 0.5 : 0.0;
-            const float d1 = (float)(sc - x1), d0 = (float)(sc - x0);
+            const float d1 = guarded_distance(fc), d0 = k >= 1 ? below_distance(fc) : (float)sc;
             const float ih = k >= 1 ? 1.0f : 2.0f;  // h is 1 or 1/2
             const float i0 = __fdiv_rn(1.0f, d0), i1 = __fdiv_rn(1.0f, d1);
             dGdy0 = __fmul_rn(__fmul_rn(d1, ih), i0);
@@ -553,7 +553,7 @@ __device__ __forceinline__ void adj_column(const KP &p, int col, const float *__
         const float fac = front_slope_factor(sp, sq);
         const float v = front_speed(p, fac, G);
         const double sn = sc + (double)v;
-        if (!(sn >= 0.5) || sn > (double)H) {  // clamped: s(t) does not depend on anything
+        if (front_clamped(sn, front_pos(sn, H), H)) {  // clamped: s(t) does not depend on anything
             lams_prev[col] = 0.0;
             wp_prev[col] = 0.0;
             wq_prev[col] = 0.0;

@@ -753,6 +753,45 @@ __device__ __forceinline__ float node_T(const KP &p, const ST *G, int col, int j
     return sum_T(p, g);
 }
 
+// Where a front height s lies: n = floor(s) held to [-1, H], and fr = s - n
+// (exact; in [0, 1) for a front inside the cavity).  Every distance from s to
+// a node centre is then one exact FP64 addition of a constant to fr.  FP64
+// issues at a small fraction of the FP32 rate here (about two lanes an SM and
+// clock), and the front update spent up to forty FP64 operations and
+// conversions a column on node centres made from integers; this form has
+// about twenty, with the same values.
+struct FrontPos {
+    int n;
+    double fr;
+};
+__device__ __forceinline__ FrontPos front_pos(double s, int H) {
+    FrontPos f;
+    f.n = __double2int_rd(s);  // saturates; NaN: a value below -1
+    f.n = f.n > H ? H : (f.n < -1 ? -1 : f.n);
+    f.fr = s - (double)f.n;
+    return f;
+}
+// Highest node at least half a cell below the front (centre j + 1/2 <= s -
+// 1/2), or -1.
+__device__ __forceinline__ int guarded_node(const FrontPos &f) { return f.n >= 1 ? f.n - 1 : -1; }
+// s minus the centre of that node, and of the one below it.
+__device__ __forceinline__ float guarded_distance(const FrontPos &f) { return (float)(f.fr + 0.5); }
+__device__ __forceinline__ float below_distance(const FrontPos &f) { return (float)(f.fr + 1.5); }
+// Liquid nodes of the column: j + 1/2 < s, i.e. ceil(s - 1/2), within [0, H].
+__device__ __forceinline__ int liquid_count(const FrontPos &f, int H) {
+    const int j = f.n + (f.fr > 0.5 ? 1 : 0);
+    return j < 0 ? 0 : (j > H ? H : j);
+}
+// Whether a new front has left [1/2, H] (NaN has): the bounds are looked at
+// only where floor(s) is next to them.
+__device__ __forceinline__ bool front_clamped(double s, const FrontPos &f, int H) {
+    return f.n >= H ? s > (double)H : (f.n < 1 && !(s >= 0.5));
+}
+// Centre of the first solid node jn minus s (jn from liquid_count, below H).
+__device__ __forceinline__ float ghost_distance(const FrontPos &f, int jn) {
+    return (float)((jn == f.n ? 0.5 : 1.5) - f.fr);
+}
+
 // The Eq. 6 gradient dT/da at the front a = s (R8: the one-sided quadratic
 // through (s, Tm) and the guarded node k with the node below it, or the
 // heated wall (0, Tw) for a missing node; linear through the wall when k <
@@ -762,10 +801,11 @@ __device__ __forceinline__ float node_T(const KP &p, const ST *G, int col, int j
 // adjoint's recomputation) gets the same bits.  With h = x1 - x0,
 // d1 = s - x1, d0 = s - x0: p'(s) = (y0 d1^2 - y1 d0^2 + Tm h (d0 + d1)) /
 // (h d0 d1).
-__device__ __forceinline__ float front_gradient(int k, double sc, float y0, float y1, float Tm, float Tw) {
+__device__ __forceinline__ float front_gradient(int k, double sc, const FrontPos &f, float y0, float y1, float Tm,
+                                                float Tw) {
     if (k < 0) return __fdiv_rn(__fsub_rn(Tm, Tw), (float)sc);
-    const double x1 = k + 0.5, x0 = k >= 1 ? k - 0.5 : 0.0;
-    const float h = (float)(x1 - x0), d1 = (float)(sc - x1), d0 = (float)(sc - x0);
+    const float h = k >= 1 ? 1.0f : 0.5f;
+    const float d1 = guarded_distance(f), d0 = k >= 1 ? below_distance(f) : (float)sc;
     const float num = __fadd_rn(__fsub_rn(__fmul_rn(__fmul_rn(y0, d1), d1), __fmul_rn(__fmul_rn(y1, d0), d0)),
                                 __fmul_rn(__fmul_rn(Tm, h), __fadd_rn(d0, d1)));
     return __fdiv_rn(num, __fmul_rn(__fmul_rn(h, d0), d1));
@@ -775,12 +815,6 @@ __device__ __forceinline__ float front_slope_factor(float sp, float sq) {
 }
 __device__ __forceinline__ float front_speed(const KP &p, float fac, float G) {
     return __fmul_rn(__fmul_rn(p.coef_f, fac), -G);
-}
-
-// Highest node at least half a cell below s (centre j + 1/2 <= s - 1/2).
-__device__ __forceinline__ int guarded_node(double s, int H) {
-    int k = (int)floor(s - 1.0);
-    return k > H - 1 ? H - 1 : (k < 0 ? -1 : k);
 }
 
 // Lowest node at least half a cell above s (centre j + 1/2 >= s + 1/2, i.e.
@@ -924,7 +958,8 @@ __device__ __forceinline__ int front_column(const KP &p, ST *__restrict__ F, con
     // Load stage 2: the gradient stencil of s_t and, speculatively, the node
     // below the current front, which is the ghost's source node whenever the
     // liquid count does not change (all but a few columns per step).
-    const int k = move ? guarded_node(sc, H) : -2;
+    const FrontPos fc = front_pos(sc, H);
+    const int k = move ? guarded_node(fc) : -2;
     float y1 = 0.0f, y0 = Tw;
     if (k >= 0) {
         y1 = node_T<ST, FACE>(p, G, col, k, infl, thw);
@@ -954,18 +989,21 @@ __device__ __forceinline__ int front_column(const KP &p, ST *__restrict__ F, con
     }
     // Then Eq. 6.
     double sn = sc;
+    FrontPos fn = fc;
     if (move) {
-        const float Gr = front_gradient(k, sc, y0, y1, Tm, Tw);
+        const float Gr = front_gradient(k, sc, fc, y0, y1, Tm, Tw);
         const float v = front_speed(p, front_slope_factor(sp, sq), COND ? Gr - Gs : Gr);
         if (!isfinite(Gr) || (COND && !isfinite(Gs))) atomicOr(status, 2);
         else if (!(fabsf(v) <= 0.5f)) atomicOr(status, 1);
         sn = sc + (double)v;
-        if (!(sn >= 0.5)) sn = 0.5;  // also catches NaN
-        if (sn > (double)H) sn = (double)H;
+        fn = front_pos(sn, H);
+        if (front_clamped(sn, fn, H)) {
+            sn = fn.n >= H ? (double)H : 0.5;
+            fn = front_pos(sn, H);
+        }
     }
     s_next[col] = sn;
-    int jn = (int)ceil(sn - 0.5);
-    jn = jn < 0 ? 0 : (jn > H ? H : jn);
+    const int jn = liquid_count(fn, H);
     js_next[col] = jn;
     if (COND) {
         // the solid side's ghost populations at the last liquid node jn - 1
@@ -1015,18 +1053,18 @@ __device__ __forceinline__ int front_column(const KP &p, ST *__restrict__ F, con
         if (SPEC && move && jn != jsc) flip_column<ST, FACE>(p, F, js, infl, col, jsc, jn);
         return jn;
     }
-    const double yg = jn + 0.5;
-    const int kg = guarded_node(sn, H);
+    const int kg = guarded_node(fn);
+    const float dy = ghost_distance(fn, jn);
     float Tg;
     if (kg < 0) {
-        Tg = Tm + (Tm - Tw) * ((float)(yg - sn) / (float)sn);
+        Tg = Tm + (Tm - Tw) * (dy / (float)sn);
     } else {
         float Tk;
         if (kg == k) Tk = y1;
         else if (kg == k - 1 && k >= 1) Tk = y0;
         else if (spec && kg == L) Tk = sum_T(p, gL);
         else Tk = node_T<ST, FACE>(p, G, col, kg, infl, thw);
-        Tg = Tm + (Tm - Tk) * ((float)(yg - sn) / (float)(sn - (kg + 0.5)));
+        Tg = Tm + (Tm - Tk) * (dy / guarded_distance(fn));
     }
     // ghost populations (FP32, like the collision): rest equilibrium at the
     // ghost temperature plus the non-equilibrium part N^-1 (I - Q)(n - n^eq)
