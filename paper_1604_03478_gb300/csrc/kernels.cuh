@@ -42,6 +42,31 @@ __device__ __forceinline__ void step_launch_wait() {
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
+// What a kernel may load before step_launch_wait: whatever its immediate
+// predecessor does not write.  The predecessor let this kernel start only
+// after its own wait, so everything before the predecessor is complete.  Such
+// loads go to L2 (ld.global.cg): L1 may hold a line from before.  They and
+// the wait are volatile, so the compiler keeps their order.
+__device__ __forceinline__ int ld_l2(const int *q) {
+    int v;
+    asm volatile("ld.global.cg.s32 %0, [%1];\n" : "=r"(v) : "l"(q));
+    return v;
+}
+__device__ __forceinline__ double ld_l2(const double *q) {
+    double v;
+    asm volatile("ld.global.cg.f64 %0, [%1];\n" : "=d"(v) : "l"(q));
+    return v;
+}
+__device__ __forceinline__ float ld_l2(const float *q) {
+    float v;
+    asm volatile("ld.global.cg.f32 %0, [%1];\n" : "=f"(v) : "l"(q));
+    return v;
+}
+__device__ __forceinline__ float ld_l2(const __half *q) {
+    unsigned short v;
+    asm volatile("ld.global.cg.u16 %0, [%1];\n" : "=h"(v) : "l"(q));
+    return __half2float(__ushort_as_half(v));
+}
 
 template <int FACE> __device__ __forceinline__ long long off19(const KP &p, int i) {
     return (long long)ex(i) + (long long)ey(i) * p.nx + (long long)ez(i) * p.nx * p.ny;
@@ -170,6 +195,15 @@ __device__ __forceinline__ void even_node(const KP &p, ST *__restrict__ F, ST *_
 // written by the previous front update: nodes two or more above every
 // neighbouring count are deep solid and do nothing, so a block whose heights
 // are all >= jmax + 3 returns at once.
+// Lowest height of a block of the stream-collide grid.
+template <int FACE> __device__ __forceinline__ int k1_low() {
+    return (int)blockIdx.z * (FACE == 0 ? (int)blockDim.y : 1);
+}
+// Whether the block is past the first `early_blocks` of the grid, the ones
+// that are resident at once.
+__device__ __forceinline__ bool k1_late(int early_blocks) {
+    return (long long)(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x >= early_blocks;
+}
 template <int FACE>
 __device__ __forceinline__ bool k1_node(const KP &p, const int *jmax, int &x, int &y, int &z) {
     const int a0 = (int)blockIdx.z * (FACE == 0 ? (int)blockDim.y : 1);  // lowest height of the block
@@ -191,13 +225,60 @@ __device__ __forceinline__ bool k1_node(const KP &p, const int *jmax, int &x, in
 // blocks, no spills; forced to 8 it loses 1%).
 template <typename ST> constexpr int k1_min_blocks() { return sizeof(ST) == 2 ? 8 : 0; }
 
+// One node per thread.  These are the kernels of the smaller cavities, whose
+// step is a chain of latencies, so the blocks that find a place while the
+// front update of the step before still runs load a liquid node's
+// populations before step_launch_wait: the front update writes slots of nodes
+// that were solid only (flip_column), and a node that has just become liquid
+// takes what it wrote after the wait.  The blocks that start later
+// (early_blocks and on) find the wait over; they wait first and read the
+// flags through L1, which their neighbours on the SM have filled: with their
+// flags from L2 too, 128^3 with a thin layer ran 17.0 us a step, 96^3 18.8.
+// A step, without and with the early loads: 32^3 8.0 -> 6.5 us, 128^3 thin
+// layer 16.8 -> 16.5, 96^3 mid melt 18.6 -> 18.2, 101x75x83 19.6 -> 18.9.
 template <typename ST, int FACE, typename IX>
 __global__ void __launch_bounds__(128, k1_min_blocks<ST>()) k_even(const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G,
-                                              const int *__restrict__ js, const int *__restrict__ nb,
-                                              const float *__restrict__ gpost, const int *jmax) {
-    step_launch_wait();
-    int x, y, z;
-    if (k1_node<FACE>(p, jmax, x, y, z)) even_node<ST, FACE, IX>(p, F, G, js, nb, gpost, x, y, z);
+                                              const int *js, const int *js_old, const int *__restrict__ nb,
+                                              const float *__restrict__ gpost, const int *jmax, int early_blocks) {
+    int x = 0, y = 0, z = 0, a = 0, col = 0, jso = 0;
+    IX c = 0;
+    float f[19], g[7];
+    bool on = k1_node<FACE>(p, nullptr, x, y, z);
+    const bool late = k1_late(early_blocks);
+    if (late) step_launch_wait();
+    if (on) {
+        c = (IX)node_index(p, x, y, z);
+        a = axial<FACE>(x, y, z);
+        col = column<FACE>(p, x, y, z);
+        const int jm = jmax ? (late ? *jmax : ld_l2(jmax)) : 1 << 29;
+        jso = late ? js_old[col] : ld_l2(js_old + col);
+        on = k1_low<FACE>() < jm + 3;
+        if (a < jso) {
+#pragma unroll
+            for (int i = 0; i < 19; ++i) f[i] = ld_l2(elem<IX>(F, c, i * p.ld));
+#pragma unroll
+            for (int i = 0; i < 7; ++i) g[i] = ld_l2(elem<IX>(G, c, i * p.ld));
+        }
+    }
+    if (!late) step_launch_wait();
+    if (!on) return;
+    const int jsc = __ldg(js + col);
+    if (a < jsc) {
+        if (a >= jso) {
+#pragma unroll
+            for (int i = 0; i < 19; ++i) f[i] = ld_l2(elem<IX>(F, c, i * p.ld));
+#pragma unroll
+            for (int i = 0; i < 7; ++i) g[i] = ld_l2(elem<IX>(G, c, i * p.ld));
+        }
+        collide(p, f, g);
+#pragma unroll
+        for (int i = 0; i < 19; ++i) Store<ST>::st_stream(elem<IX>(F, c, opp(i) * p.ld), f[i]);
+    } else {
+        if (deep_solid(p, a, __ldg(nb + col))) return;
+        solid_post(p, a == jsc, gpost, col, g);
+    }
+#pragma unroll
+    for (int i = 0; i < 7; ++i) Store<ST>::st_stream(elem<IX>(G, c, opp7(i) * p.ld), g[i]);
 }
 
 // The even step with heat conduction in the solid (every node updated).
@@ -223,6 +304,16 @@ __device__ __forceinline__ void load_js9(const KP &p, const int *__restrict__ js
             const bool in = (unsigned)p2 < (unsigned)p.P1 && (unsigned)q2 < (unsigned)p.P2;
             js9[(dq + 1) * 3 + dp + 1] = in ? __ldg(js + q2 * p.P1 + p2) : 0;
         }
+}
+
+// load_js9 by loads that may stand before step_launch_wait.
+__device__ __forceinline__ void load_js9_l2(const KP &p, const int *js, int pp, int q, int (&js9)[9]) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const int p2 = pp + k % 3 - 1, q2 = q + k / 3 - 1;
+        const bool in = (unsigned)p2 < (unsigned)p.P1 && (unsigned)q2 < (unsigned)p.P2;
+        js9[k] = in ? ld_l2(js + q2 * p.P1 + p2) : 0;
+    }
 }
 
 // Bit i (1..18) of the link mask: node x - e_i is inside and liquid, i.e.
@@ -454,16 +545,144 @@ __device__ __forceinline__ void odd_node(const KP &p, const Links *lk, ST *__res
     }
 }
 
+// The odd step of one node with its loads before step_launch_wait (see
+// k_even).  A node that was liquid reads what the flags before the front
+// update prescribe (counts js_old, bounds nb_old), which no other thread
+// writes, with one exception: the slot it holds towards a node that has just
+// become liquid, which that node's thread may have written already.  Those
+// links are read again after the wait, from where flip_column moved the
+// value.  `inner`: interior under the old flags and, counts changing by at
+// most one a step, under the new ones.
+template <typename ST, int FACE>
+__device__ __forceinline__ void odd_node_early(const KP &p, const Links *lk, ST *__restrict__ F, ST *__restrict__ G,
+                                               const int *js, const int *js_old, const int *nb, const int *nb_old,
+                                               const float *__restrict__ gpost, const float *thw_rd,
+                                               const float *__restrict__ thw_wr, const int *jmax, int early_blocks,
+                                               bool on, int x, int y, int z) {
+    const long long c = on ? node_index(p, x, y, z) : 0;
+    const int a = axial<FACE>(x, y, z), col = on ? column<FACE>(p, x, y, z) : 0;
+    const int q = FACE == 0 ? z : y, nq = FACE == 0 ? p.nz : p.ny;
+    const bool off_qa = q >= 1 && q <= nq - 2 && a >= 1 && a <= p.H - 2;
+    const bool xlo = x == 0, xhi = x == p.nx - 1;
+    unsigned need = 0x7fffeu;  // the links that an interior node has
+    if (xlo | xhi) {
+#pragma unroll
+        for (int i = 1; i < 19; ++i)
+            if (xwall(ex(i), xlo, xhi)) need &= ~(1u << i);
+    }
+    ST *const Fc = F + c;
+    ST *const Gc = G + c;
+    float f[19], g[7];
+    unsigned lm = need, im = 0x7eu;
+    bool inner = false, was = false;
+    auto pull_g = [&]() {
+        const float th_rd = ld_l2(thw_rd + col);
+        g[0] = ld_l2(Gc);
+#pragma unroll
+        for (int i = 1; i < 7; ++i) {
+            const bool in = (im >> i) & 1u;
+            const float v = ld_l2(in ? Gc + lk->gin[i] : Gc + i * p.ld);
+            g[i] = in ? v : wall_value<FACE>(p, opp7(i), v, th_rd);
+        }
+    };
+    const bool late = k1_late(early_blocks);
+    if (late) step_launch_wait();
+    if (on) {
+        const int jm = jmax ? (late ? *jmax : ld_l2(jmax)) : 1 << 29;
+        const int jso = late ? js_old[col] : ld_l2(js_old + col);
+        const int nbo = late ? nb_old[col] : ld_l2(nb_old + col);
+        on = k1_low<FACE>() < jm + 3;
+        was = on && a < jso;
+        inner = was && off_qa && a + 2 < (nbo >> 16);
+        bool fast = inner;
+        if (was && !inner) {
+            int js9[9];
+            load_js9_l2(p, js_old, x, q, js9);
+            lm = link_mask9<FACE>(js9, a);
+            im = inside_mask(p, x, y, z);
+            fast = off_qa && (lm & need) == need;
+        }
+        if (was && fast) {
+#pragma unroll
+            for (int i = 0; i < 19; ++i) f[i] = ld_l2(Fc + lk->fin[i]);
+#pragma unroll
+            for (int i = 0; i < 7; ++i) g[i] = ld_l2(Gc + lk->gin[i]);
+            if (xlo | xhi) {  // across an x wall: bounce-back (see odd_node)
+#pragma unroll
+                for (int i = 1; i < 19; ++i)
+                    if (xwall(ex(i), xlo, xhi)) f[i] = ld_l2(Fc + i * p.ld);
+#pragma unroll
+                for (int i = 1; i < 7; ++i)
+                    if (xwall(tx(i), xlo, xhi)) g[i] = ld_l2(Gc + i * p.ld);
+            }
+        } else if (was) {
+            f[0] = ld_l2(Fc);
+#pragma unroll
+            for (int i = 1; i < 19; ++i) f[i] = ld_l2(((lm >> i) & 1u) ? Fc + lk->fin[i] : Fc + i * p.ld);
+            pull_g();
+        }
+    }
+    if (!late) step_launch_wait();
+    if (!on) return;
+    const int jsc = inner ? p.H : __ldg(js + col);
+    if (a < jsc) {
+        bool fast = inner;
+        if (!inner) {
+            int js9[9];
+            load_js9(p, js, x, q, js9);
+            const unsigned now = link_mask9<FACE>(js9, a);
+            if (!was) {
+                im = inside_mask(p, x, y, z);
+#pragma unroll
+                for (int i = 0; i < 19; ++i) f[i] = 0.0f;
+                pull_g();
+            } else if (now & ~lm) {
+#pragma unroll
+                for (int i = 1; i < 19; ++i)
+                    if (((now & ~lm) >> i) & 1u) f[i] = ld_l2(Fc + lk->fin[i]);
+            }
+            lm = now;
+            fast = off_qa && (lm & need) == need;
+        }
+        collide(p, f, g);
+        Store<ST>::st_stream(Fc, f[0]);
+        if (fast) {
+#pragma unroll
+            for (int i = 1; i < 19; ++i)  // towards an x wall: stays in slot opp(i)
+                Store<ST>::st_stream(xwall(-ex(i), xlo, xhi) ? Fc + opp(i) * p.ld : Fc + lk->fout[i], f[i]);
+            Store<ST>::st_stream(Gc, g[0]);
+#pragma unroll
+            for (int i = 1; i < 7; ++i)
+                Store<ST>::st_stream(xwall(-tx(i), xlo, xhi) ? Gc + opp7(i) * p.ld : Gc + lk->gout[i], g[i]);
+            return;
+        }
+#pragma unroll
+        for (int i = 1; i < 19; ++i)
+            Store<ST>::st_stream(((lm >> opp(i)) & 1u) ? Fc + lk->fout[i] : Fc + opp(i) * p.ld, f[i]);
+    } else {
+        if (deep_solid(p, a, __ldg(nb + col))) return;
+        im = inside_mask(p, x, y, z);
+        solid_post(p, a == jsc, gpost, col, g);
+    }
+    const float th_wr = __ldg(thw_wr + col);
+    Store<ST>::st_stream(Gc, g[0]);
+#pragma unroll
+    for (int i = 1; i < 7; ++i) {
+        const bool out = (im >> opp7(i)) & 1u;
+        Store<ST>::st_stream(out ? Gc + lk->gout[i] : Gc + opp7(i) * p.ld,
+                             out ? g[i] : wall_value<FACE>(p, i, g[i], th_wr));
+    }
+}
+
 template <typename ST, int FACE>
 __global__ void __launch_bounds__(128, k1_min_blocks<ST>()) k_odd(const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G,
-                                             const int *__restrict__ js, const int *__restrict__ js_old,
-                                             const int *__restrict__ nb,
-                                             const float *__restrict__ gpost, const float *__restrict__ thw_rd,
+                                             const int *js, const int *js_old, const int *nb, const int *nb_old,
+                                             const float *__restrict__ gpost, const float *thw_rd,
                                              const float *__restrict__ thw_wr, const __grid_constant__ Links lk,
-                                             const int *jmax) {
-    step_launch_wait();
-    int x, y, z;
-    if (k1_node<FACE>(p, jmax, x, y, z)) odd_node<ST, FACE>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x, y, z);
+                                             const int *jmax, int early_blocks) {
+    int x = 0, y = 0, z = 0;
+    const bool on = k1_node<FACE>(p, nullptr, x, y, z);
+    odd_node_early<ST, FACE>(p, &lk, F, G, js, js_old, nb, nb_old, gpost, thw_rd, thw_wr, jmax, early_blocks, on, x, y, z);
 }
 
 // The odd step with heat conduction in the solid (every node updated).
@@ -915,7 +1134,8 @@ __device__ __forceinline__ void flip_column(const KP &p, ST *__restrict__ F, con
 // clamped to [1/2, H], its liquid-node count, and the ghost node of the new
 // front: g*_ghost = g^eq(T_ghost, 0) + (g*_L - g^eq(T_L, u_L)).
 // move = 0 keeps the front (used to prepare the ghost after a state upload).
-// SPEC: load the ghost's likely source node together with the gradient
+// SPEC (as a kernel of its own): wait for the stream-collide once the column's
+// own data are loaded, load the ghost's likely source node together with the gradient
 // stencil (two dependent load stages instead of three; more registers), and
 // flip the column's nodes; without it the caller flips them.
 //
@@ -933,7 +1153,7 @@ __device__ __forceinline__ void flip_column(const KP &p, ST *__restrict__ F, con
 // with T_sghost on the line through (s, Tm) and the guarded solid node (or
 // the cold wall); the rest state at Tm in a column without both phases.
 template <typename ST, int FACE, bool SPEC = true, bool COND = false>
-__device__ __forceinline__ int front_column(const KP &p, ST *__restrict__ F, const ST *__restrict__ G,
+__device__ __forceinline__ int front_column(const KP &p, ST *__restrict__ F, const ST *G,
                                            const int *__restrict__ js, int *__restrict__ js_next,
                                            int *__restrict__ nb_next, const double *__restrict__ s, double *__restrict__ s_next,
                                            float *__restrict__ gpost, const float *__restrict__ thw, int inflight,
@@ -942,18 +1162,22 @@ __device__ __forceinline__ int front_column(const KP &p, ST *__restrict__ F, con
     const int P1 = p.P1, P2 = p.P2, H = p.H;
     const int pp = col % P1, q = col / P1;
     const bool infl = inflight != 0;
-    // Load stage 1: what depends on the column only.
-    const double sc = s[col];
+    // Load stage 1: what depends on the column only.  None of it is written
+    // by the stream-collide, so with SPEC it stands before the wait for it.
+    const double sc = ld_l2(s + col);
     const float Tm = p.Tm;
-    const float Tw = thw[col];
-    const int jsc = js[col];
+    const float Tw = ld_l2(thw + col);
     int js9[9];
-    load_js9(p, js, pp, q, js9);
+    load_js9_l2(p, js, pp, q, js9);
+    const int jsc = js9[4];
     float sp = 0.0f, sq = 0.0f;
     if (move) {
-        sp = 0.5f * (float)(s[q * P1 + (pp + 1 < P1 ? pp + 1 : pp)] - s[q * P1 + (pp > 0 ? pp - 1 : pp)]);
-        sq = 0.5f * (float)(s[(q + 1 < P2 ? q + 1 : q) * P1 + pp] - s[(q > 0 ? q - 1 : q) * P1 + pp]);
+        const double sp_hi = ld_l2(s + q * P1 + (pp + 1 < P1 ? pp + 1 : pp)), sp_lo = ld_l2(s + q * P1 + (pp > 0 ? pp - 1 : pp));
+        const double sq_hi = ld_l2(s + (q + 1 < P2 ? q + 1 : q) * P1 + pp), sq_lo = ld_l2(s + (q > 0 ? q - 1 : q) * P1 + pp);
+        sp = 0.5f * (float)(sp_hi - sp_lo);
+        sq = 0.5f * (float)(sq_hi - sq_lo);
     }
+    if (SPEC) step_launch_wait();
     nb_next[col] = count_bounds(p, js9, pp, q);
     // Load stage 2: the gradient stencil of s_t and, speculatively, the node
     // below the current front, which is the ghost's source node whenever the
@@ -1125,17 +1349,17 @@ __device__ __forceinline__ int front_column(const KP &p, ST *__restrict__ F, con
 // stream-collide grid (nodes two above every neighbouring count are deep
 // solid and do nothing).
 template <typename ST, int FACE>
-__global__ void __launch_bounds__(128, 4) k_front(const __grid_constant__ KP p, ST *__restrict__ F, const ST *__restrict__ G,
+__global__ void __launch_bounds__(128, 4) k_front(const __grid_constant__ KP p, ST *__restrict__ F, const ST *G,
                                                const int *__restrict__ js, int *__restrict__ js_next,
                                                int *__restrict__ nb_next,
                                                const double *__restrict__ s, double *__restrict__ s_next,
                                                float *__restrict__ gpost, const float *__restrict__ thw,
                                                int inflight, int move, int *__restrict__ status,
                                                int *__restrict__ jmax) {
-    step_launch_wait();
     const int col = blockIdx.x * blockDim.x + threadIdx.x;
     int jn = -1;
-    if (col < p.ncols) jn = front_column<ST, FACE>(p, F, G, js, js_next, nb_next, s, s_next, gpost, thw, inflight, move, status, col);
+    if (col >= p.ncols) step_launch_wait();
+    else jn = front_column<ST, FACE>(p, F, G, js, js_next, nb_next, s, s_next, gpost, thw, inflight, move, status, col);
     // blocks are whole warps and every thread of the grid reaches this point
     const int m = __reduce_max_sync(0xffffffffu, jn);
     if (jmax && (threadIdx.x & 31) == 0 && m >= 0) atomicMax(jmax, m);
@@ -1146,15 +1370,15 @@ __global__ void __launch_bounds__(128, 4) k_front(const __grid_constant__ KP p, 
 // waves, 23.3 against 16.2 us under the profiler, 353 against 348 us a step.
 template <typename ST, int FACE>
 __global__ void __launch_bounds__(128, 4) k_front_cond(const __grid_constant__ KP p, ST *__restrict__ F,
-                                                    const ST *__restrict__ G, const int *__restrict__ js,
+                                                    const ST *G, const int *__restrict__ js,
                                                     int *__restrict__ js_next, int *__restrict__ nb_next,
                                                     const double *__restrict__ s,
                                                     double *__restrict__ s_next, float *__restrict__ gpost,
                                                     float *__restrict__ spost, const float *__restrict__ thw,
                                                     int inflight, int move, int *__restrict__ status) {
-    step_launch_wait();
     const int col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col < p.ncols)
+    if (col >= p.ncols) step_launch_wait();
+    else
         front_column<ST, FACE, true, true>(p, F, G, js, js_next, nb_next, s, s_next, gpost, thw, inflight, move, status, col,
                                            spost);
 }

@@ -21,6 +21,7 @@ struct Bufs {
     int *status;
     const Links *lk;             // interior link offsets of the odd step
     int cblk;                    // threads per block of the per-column kernels (col_block)
+    int sms;                     // SMs of the device
     int *jmax;                   // running maximum of the liquid counts (k_front), or null
     int k1_height;               // the stream-collide grid covers heights < k1_height (the rest is deep solid)
     const float *thw_nu;         // heated-wall field of the last streaming (Nusselt number)

@@ -33,14 +33,16 @@ static cudaError_t launch_step_kernel(void (*kern)(KArgs...), dim3 grd, dim3 blk
 
 template <typename ST, typename IXE>
 static cudaError_t launch_sc(const KP &p, int face, int odd, const Bufs &b, dim3 grd, dim3 blk, cudaStream_t st) {
+    // blocks resident at once: 7 of 128 threads an SM (72 registers)
+    const int early = b.sms * (896 / (int)(blk.x * blk.y));
     const int *jm = p.skip_deep ? b.jmax : nullptr;
     ST *F = (ST *)b.F, *G = (ST *)b.G;
     if (face == 0) {
-        if (odd) return launch_step_kernel(k_odd<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
-        else return launch_step_kernel(k_even<ST, 0, IXE>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, jm);
+        if (odd) return launch_step_kernel(k_odd<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early);
+        else return launch_step_kernel(k_even<ST, 0, IXE>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early);
     } else {
-        if (odd) return launch_step_kernel(k_odd<ST, 1>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
-        else return launch_step_kernel(k_even<ST, 1, IXE>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, jm);
+        if (odd) return launch_step_kernel(k_odd<ST, 1>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early);
+        else return launch_step_kernel(k_even<ST, 1, IXE>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early);
     }
 }
 

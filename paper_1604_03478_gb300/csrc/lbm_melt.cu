@@ -195,6 +195,7 @@ Bufs bufs_at(lbm_melt *h, int cur, int inflight) {
     b.status = h->status_dev;
     b.lk = &h->lk;
     b.cblk = h->cblk;
+    b.sms = h->sms;
     b.jmax = h->jmax_dev;
     b.k1_height = h->kp.H;
     // the wall field of the last streaming: in flight, the one the pending

@@ -1,0 +1,41 @@
+"""GPU parity of the one-node stream-collide's two kinds of block: the ones of
+the first wave, which load before they wait for the front update, and the
+later ones.  Grids below, around and above one wave (7 blocks of 128 nodes on
+each of the SMs) against the two-nodes-per-thread kernels, which load after
+the wait, over steps in which nodes flip after even and odd steps.
+
+Tolerance: the two kernels round FP32 intermediates differently, below 3e-8
+a population and step, 26 steps: 1e-6 with all of them falling the same way."""
+import numpy as np
+import pytest
+
+from paper_1604_03478_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("face", [0, 1])
+@pytest.mark.parametrize("shape,s0", [((32, 12, 12), 4.0), ((128, 40, 40), 24.0), ((130, 66, 62), 20.0)])
+def test_early_and_late_blocks(face, shape, s0):
+    import torch
+    assert torch.cuda.is_available()
+    from paper_1604_03478_gb300 import build, Cavity
+    build.build()
+    kw = dict(face=face, Ra=1e5, Pr=0.2, Ste=0.6, Ma=0.1, s0=s0, derive=True)
+    a, b = Cavity(*shape, **kw), Cavity(*shape, **kw)
+    a.set_node_pairs(0)
+    b.set_node_pairs(1)
+    f, g, s = a.get_state()
+    s = s0 + inputs.gaussian_field(a.ncols, 0.7, 3 + face)  # fronts over several nodes
+    wall = (1.0 + inputs.gaussian_field(a.ncols, 0.05, 5)).astype(np.float32)
+    for c in (a, b):
+        c.set_state(f, g, s)
+        c.set_hot_wall(wall)
+        c.step(26)
+    (fa, ga, sa), (fb, gb, sb) = a.get_state(), b.get_state()
+    assert (np.ceil(sa - 0.5) != np.ceil(s - 0.5)).any()
+    np.testing.assert_allclose(sa, sb, atol=1e-6, rtol=0)
+    np.testing.assert_allclose(fa, fb, atol=1e-6, rtol=0)
+    np.testing.assert_allclose(ga, gb, atol=1e-6, rtol=0)
+    a.close()
+    b.close()
