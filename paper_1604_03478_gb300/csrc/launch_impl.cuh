@@ -134,11 +134,18 @@ template <typename ST>
 cudaError_t Launch<ST>::totals(const KP &p, int face, int inflight, const Bufs &b, double *part, int nparts,
                                double t, double *out, cudaStream_t st) {
     const ST *F = (const ST *)b.F, *G = (const ST *)b.G;
-    if (face == 0) k_totals_part<ST, 0><<<nparts, 256, 0, st>>>(p, F, G, b.js, b.js_next, b.thw_rd, inflight, part);
-    else k_totals_part<ST, 1><<<nparts, 256, 0, st>>>(p, F, G, b.js, b.js_next, b.thw_rd, inflight, part);
-    const cudaError_t e = nusselt(p, face, inflight, b, st);
+    const int col_tiles = (p.ncols + 255) / 256;
+    const long long tiles = (long long)col_tiles * ((p.H + kTotalsRun - 1) / kTotalsRun);
+    const int blocks = (int)(tiles < nparts ? tiles : nparts);
+    if (face == 0)
+        k_totals_part<ST, 0><<<blocks, 256, 0, st>>>(p, F, G, b.js, b.js_next, b.s, b.thw_rd, b.thw_nu, inflight,
+                                                     b.nu_scale, part);
+    else
+        k_totals_part<ST, 1><<<blocks, 256, 0, st>>>(p, F, G, b.js, b.js_next, b.s, b.thw_rd, b.thw_nu, inflight,
+                                                     b.nu_scale, part);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_totals_final<<<1, 256, 0, st>>>(part, nparts, b.s, b.nu, p.ncols, (double)p.H, t, out);
+    k_totals_final<<<1, 256, 0, st>>>(part, blocks, p.ncols, (double)p.H, t, out);
     return cudaGetLastError();
 }
 
