@@ -886,23 +886,29 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair(const _
 // Shifted pre-collision g of node (x,y,z).  In flight: pull from the
 // neighbours' slots (walls by their rules with wall field thw); natural:
 // the node's own slots.
+// One branch for the layout and addresses chosen by selects: with a branch per
+// direction every load waited for the one before it (its conversion to FP32
+// with FP16 storage above all: the fields of a 256^3 FP16 state took 441 us to
+// read, now 190, its distributions 527, now 355; in flight 490, now 228).
 template <typename ST, int FACE>
 __device__ __forceinline__ void gather_g(const KP &p, const ST *G, int x, int y, int z, bool inflight,
                                          const float *thw, float (&g)[7]) {
-    const long long c = node_index(p, x, y, z);
-    g[0] = Store<ST>::ld(G + c);
+    const ST *Gc = G + node_index(p, x, y, z);
+    if (!inflight) {
+#pragma unroll
+        for (int i = 0; i < 7; ++i) g[i] = Store<ST>::ld(Gc + i * p.ld);
+        return;
+    }
+    const unsigned im = inside_mask(p, x, y, z);
+    const float Tw = axial<FACE>(x, y, z) == 0 ? thw[column<FACE>(p, x, y, z)] : 0.0f;
+    g[0] = Store<ST>::ld(Gc);
+#pragma unroll
+    for (int i = 1; i < 7; ++i)
+        g[i] = Store<ST>::ld(((im >> i) & 1u) ? Gc + (opp7(i) * p.ld - off7<FACE>(p, i)) : Gc + i * p.ld);
 #pragma unroll
     for (int i = 1; i < 7; ++i) {
-        if (!inflight) {
-            g[i] = Store<ST>::ld(G + i * p.ld + c);
-        } else if (inside(p, x - tx(i), y - ty(i), z - tz(i))) {
-            g[i] = Store<ST>::ld(G + opp7(i) * p.ld + (c - off7<FACE>(p, i)));
-        } else {
-            const int w = wall_of_link<FACE>(opp7(i));
-            const float own = Store<ST>::ld(G + i * p.ld + c);
-            g[i] = (w == 3) ? own
-                            : -own + 2.0f * w7(i) * ((w == 1 ? thw[column<FACE>(p, x, y, z)] : p.Tc) - p.Ts);
-        }
+        const int w = wall_of_link<FACE>(opp7(i));
+        if (w != 3 && !((im >> i) & 1u)) g[i] = -g[i] + 2.0f * w7(i) * ((w == 1 ? Tw : p.Tc) - p.Ts);
     }
 }
 
@@ -911,15 +917,19 @@ __device__ __forceinline__ void gather_g(const KP &p, const ST *G, int x, int y,
 template <typename ST, int FACE>
 __device__ __forceinline__ void gather_f(const KP &p, const ST *F, const int *js, int x, int y, int z,
                                          bool inflight, float (&f)[19]) {
-    const long long c = node_index(p, x, y, z);
-    f[0] = Store<ST>::ld(F + c);
+    const ST *Fc = F + node_index(p, x, y, z);
+    if (!inflight) {
 #pragma unroll
-    for (int i = 1; i < 19; ++i) {
-        if (!inflight) f[i] = Store<ST>::ld(F + i * p.ld + c);
-        else if (liquid_at<FACE>(p, js, x - ex(i), y - ey(i), z - ez(i)))
-            f[i] = Store<ST>::ld(F + opp(i) * p.ld + (c - off19<FACE>(p, i)));
-        else f[i] = Store<ST>::ld(F + i * p.ld + c);
+        for (int i = 0; i < 19; ++i) f[i] = Store<ST>::ld(Fc + i * p.ld);
+        return;
     }
+    int js9[9];
+    load_js9(p, js, x, FACE == 0 ? z : y, js9);
+    const unsigned lm = link_mask9<FACE>(js9, axial<FACE>(x, y, z));
+    f[0] = Store<ST>::ld(Fc);
+#pragma unroll
+    for (int i = 1; i < 19; ++i)
+        f[i] = Store<ST>::ld(((lm >> i) & 1u) ? Fc + (opp(i) * p.ld - off19<FACE>(p, i)) : Fc + i * p.ld);
 }
 
 // gather_f of the state between steps (flip_column has run): a node that has
@@ -941,17 +951,12 @@ __device__ __forceinline__ void gather_f_now(const KP &p, const ST *F, const int
 template <typename ST, int FACE>
 __device__ __forceinline__ void gather_f9(const KP &p, const ST *F, const int (&js9)[9], int x, int y, int z, int a,
                                           float (&f)[19]) {
-    const long long c = node_index(p, x, y, z);
-    f[0] = Store<ST>::ld(F + c);
+    const ST *Fc = F + node_index(p, x, y, z);
+    const unsigned lm = link_mask9<FACE>(js9, a);
+    f[0] = Store<ST>::ld(Fc);
 #pragma unroll
-    for (int i = 1; i < 19; ++i) {
-        // the upstream node x - e_i: in-plane column offset and height
-        const int dp = -ex(i), dq = FACE == 0 ? -ez(i) : -ey(i), da = FACE == 0 ? -ey(i) : -ez(i);
-        const int an = a + da;
-        const bool liq = an >= 0 && an < js9[(dq + 1) * 3 + dp + 1];
-        if (liq) f[i] = Store<ST>::ld(F + opp(i) * p.ld + (c - off19<FACE>(p, i)));
-        else f[i] = Store<ST>::ld(F + i * p.ld + c);
-    }
+    for (int i = 1; i < 19; ++i)
+        f[i] = Store<ST>::ld(((lm >> i) & 1u) ? Fc + (opp(i) * p.ld - off19<FACE>(p, i)) : Fc + i * p.ld);
 }
 
 // Ts + the sum of the shifted g (the temperature the front reads; FP32, the
@@ -1402,13 +1407,15 @@ __global__ void __launch_bounds__(128) k_macro(const __grid_constant__ KP p, con
     if (a < js[col]) {
         float g[7], f[19];
         gather_g<ST, FACE>(p, G, x, y, z, inflight != 0, thw, g);
-        gather_f_now<ST, FACE>(p, F, js, js_old, x, y, z, inflight != 0, f);
         float Th = 0.0f;
+        if (u) gather_f_now<ST, FACE>(p, F, js, js_old, x, y, z, inflight != 0, f);
 #pragma unroll
         for (int i = 0; i < 7; ++i) Th += g[i];
+        if (u) {
 #pragma unroll
-        for (int i = 0; i < 19; ++i) { ux += ex(i) * f[i]; uy += ey(i) * f[i]; uz += ez(i) * f[i]; }
-        uz += 0.5f * p.gbeta * (Th - p.dTms);
+            for (int i = 0; i < 19; ++i) { ux += ex(i) * f[i]; uy += ey(i) * f[i]; uz += ez(i) * f[i]; }
+            uz += 0.5f * p.gbeta * (Th - p.dTms);
+        }
         Tc = p.Ts + Th;
     } else if (p.cond) {
         float g[7];
@@ -1550,7 +1557,7 @@ constexpr int kTotalsRun = 8;    // heights of a tile
 // far.  Read bandwidth bounds it (104 bytes a liquid node with FP32 storage);
 // with every sum in FP64 per node, 64-bit divisions for the node's
 // coordinates and the column sums left to one block, a totals call on a 256^3
-// cavity at 0.4 H took 486 us (FP16 storage 1127), now 189 (160).
+// cavity at 0.4 H took 486 us (FP16 storage 1127), now 173 (160 to 175).
 template <typename ST, int FACE>
 __global__ void __launch_bounds__(256, 4) k_totals_part(const __grid_constant__ KP p, const ST *__restrict__ F, const ST *__restrict__ G,
                                                      const int *__restrict__ js, const int *__restrict__ js_old,
@@ -1577,13 +1584,8 @@ __global__ void __launch_bounds__(256, 4) k_totals_part(const __grid_constant__ 
             int x, y, z;
             column_node<FACE>(p, col, a, x, y, z);
             float g[7], f[19];
-            if (inflight) {
-                gather_g<ST, FACE>(p, G, x, y, z, true, thw, g);
-                gather_f_now<ST, FACE>(p, F, js, js_old, x, y, z, true, f);
-            } else {
-                gather_g<ST, FACE>(p, G, x, y, z, false, thw, g);
-                gather_f<ST, FACE>(p, F, js, x, y, z, false, f);
-            }
+            gather_g<ST, FACE>(p, G, x, y, z, inflight != 0, thw, g);
+            gather_f_now<ST, FACE>(p, F, js, js_old, x, y, z, inflight != 0, f);
             float Th = 0.0f, rh = 0.0f, ux = 0.0f, uy = 0.0f, uz = 0.0f;
 #pragma unroll
             for (int i = 0; i < 7; ++i) Th += g[i];
