@@ -37,7 +37,7 @@ struct lbm_melt {
     int thw_last_prev; // set_hot_wall since the last step in the natural layout: thw_prev holds the
                        // field of the last streaming (the Nusselt number's wall value)
     double *nu_dev;    // per-column Nusselt numbers (ncols)
-    int *status_dev;
+    int *status_dev;   // the front status, and next to it the running maximum (jmax_dev): one copy reads both
     double *sum_dev;
     unsigned int *ticket;  // last-block ticket of the one-launch column sum (k_sum_once)
     double *red_part;  // scratch: per-block partials of the FP64 totals
@@ -61,7 +61,8 @@ struct lbm_melt {
     // grows by at most one node per step).
     static const int kRbRing = 32, kRbLag = 16, kRbEvery = 4;
     int *jmax_dev;
-    int *rb_val;       // pinned ring of read-backs
+    int *rb_val;       // pinned: ring of read-backs, then kFlags ints a synchronising call reads status_dev into
+    static const int kFlags = 2;
     cudaEvent_t rb_ev[kRbRing];
     long long rb_step[kRbRing];  // exec step after which each copy was taken
     long long rb_next;           // read-backs enqueued so far

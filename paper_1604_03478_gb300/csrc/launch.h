@@ -44,6 +44,7 @@ template <typename ST> struct Launch {
     static cudaError_t front(const KP &p, int face, int inflight, int move, const Bufs &b, cudaStream_t st);
     static cudaError_t macro(const KP &p, int face, int inflight, const Bufs &b, float *T, float *u, cudaStream_t st);
     static cudaError_t state_out(const KP &p, int face, int inflight, const Bufs &b, float *f, float *g, cudaStream_t st);
+    static cudaError_t set_fronts(const KP &p, const Bufs &b, const double *s_in, double *s, int *js, cudaStream_t st);
     static cudaError_t state_in(const KP &p, int face, const Bufs &b, const float *f, const float *g, cudaStream_t st);
     static cudaError_t init(const KP &p, int face, const Bufs &b, const float *Tprof, cudaStream_t st);
     static cudaError_t totals(const KP &p, int face, int inflight, const Bufs &b, double *part, int nparts,

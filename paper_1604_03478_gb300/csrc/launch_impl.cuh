@@ -113,6 +113,12 @@ cudaError_t Launch<ST>::state_out(const KP &p, int face, int inflight, const Buf
 }
 
 template <typename ST>
+cudaError_t Launch<ST>::set_fronts(const KP &p, const Bufs &b, const double *s_in, double *s, int *js, cudaStream_t st) {
+    k_set_fronts<<<col_grid(p.ncols, 128), 128, 0, st>>>(s_in, p.ncols, p.H, s, js, b.jmax);
+    return cudaGetLastError();
+}
+
+template <typename ST>
 cudaError_t Launch<ST>::state_in(const KP &p, int face, const Bufs &b, const float *f, const float *g, cudaStream_t st) {
     dim3 blk = node_block(p), grd = node_grid(p, blk);
     ST *F = (ST *)b.F, *G = (ST *)b.G;

@@ -215,9 +215,8 @@ Bufs bufs(lbm_melt *h) { return bufs_at(h, h->cur, h->inflight); }
     ((h)->precision == 1 ? lbm::Launch<__half>::method(__VA_ARGS__)                  \
                          : lbm::Launch<float>::method(__VA_ARGS__))
 
-// Prepare js from s and the ghost nodes from the state (front held, no
-// flip), and the 3x3 bounds from the counts before (so after a new s it runs
-// twice: the second call finds both count buffers and the bounds right).
+// Prepare the ghost nodes and the 3x3 count bounds from the state and its
+// liquid counts js (front held, no flip); both count buffers hold js after it.
 lbm_status refresh_front(lbm_melt *h) {
     Bufs b = bufs(h);
     CK(LAUNCH(h, front, h->kp, h->face, h->inflight, 0, b, h->stream), "front refresh");
@@ -231,13 +230,26 @@ lbm_status copy_in(lbm_melt *h, void *dst, const void *src, size_t bytes, int pt
     return LBM_OK;
 }
 
-lbm_status check_status(lbm_melt *h) {
-    int st = 0;
-    CK(cudaMemcpyAsync(&st, h->status_dev, sizeof(int), cudaMemcpyDeviceToHost, h->stream), "status read");
+// Waits for the handle's stream and reads the front status and the running
+// maximum of the liquid counts into page-locked memory on the way.
+lbm_status read_flags(lbm_melt *h) {
+    CK(cudaMemcpyAsync(h->rb_val + lbm_melt::kRbRing, h->status_dev, lbm_melt::kFlags * sizeof(int),
+                       cudaMemcpyDeviceToHost, h->stream), "status read");
     CK(cudaStreamSynchronize(h->stream), "synchronize");
+    return LBM_OK;
+}
+
+// What the status that read_flags read says.
+lbm_status status_of_flags(lbm_melt *h) {
+    const int st = h->rb_val[lbm_melt::kRbRing];
     if (st & 2) return set_err(h, LBM_ENAN, "non-finite temperature at the front");
     if (st & 1) return set_err(h, LBM_EUNSTABLE, "the front moved more than half a cell in one step");
     return LBM_OK;
+}
+
+lbm_status check_status(lbm_melt *h) {
+    const lbm_status st = read_flags(h);
+    return st == LBM_OK ? status_of_flags(h) : st;
 }
 
 void free_all(lbm_melt *h) {
@@ -254,7 +266,6 @@ void free_all(lbm_melt *h) {
     cudaFree(h->totals_dev);
     cudaFree(h->nu_dev);
     cudaFree(h->report);
-    cudaFree(h->jmax_dev);
     cudaFree(h->spost);
     if (h->rb_val) cudaFreeHost(h->rb_val);
     for (int k = 0; k < lbm_melt::kRbRing; ++k)
@@ -293,17 +304,16 @@ lbm_status k1_height(lbm_melt *h, int *out) {
     return LBM_OK;
 }
 
-// A read-back taken now, synchronously (after create and set_state, so that
-// the first steps of a run are bounded too).
-lbm_status seed_readback(lbm_melt *h) {
-    if (!h->kp.skip_deep) return LBM_OK;
+// The maximum that the last read_flags read, as a read-back of the state now
+// (after create and set_state, so that the first steps of a run are bounded
+// too).
+void seed_readback(lbm_melt *h) {
+    if (!h->kp.skip_deep) return;
     const int slot = (int)(h->rb_next % lbm_melt::kRbRing);
-    CK(cudaStreamSynchronize(h->stream), "synchronize");
-    CK(cudaMemcpy(h->rb_val + slot, h->jmax_dev, sizeof(int), cudaMemcpyDeviceToHost), "read-back");
+    h->rb_val[slot] = h->rb_val[lbm_melt::kRbRing + 1];
     h->rb_step[slot] = h->exec_steps - 1;
     h->rb_synced = h->rb_next;
     h->rb_next++;
-    return LBM_OK;
 }
 
 // After every kRbEvery-th step (or now, with force): copy the running
@@ -323,13 +333,18 @@ lbm_status jmax_readback(lbm_melt *h, bool force = false) {
 // in strides of the block size, then a tree; the block that finishes last
 // (atomic ticket) adds the partials in block order, writes the result and
 // resets the ticket.
+// copy (may be null): receives the values too.
 __global__ void k_sum_once(const double *__restrict__ v, long long n, long long chunk, double scale,
-                           double *part, unsigned int *ticket, double *__restrict__ out) {
+                           double *part, unsigned int *ticket, double *__restrict__ out, double *__restrict__ copy) {
     __shared__ double sh[256];
     __shared__ bool last;
     const long long lo = blockIdx.x * chunk, hi = lo + chunk < n ? lo + chunk : n;
     double acc = 0.0;
-    for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) acc += v[i];
+    for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+        const double x = v[i];
+        acc += x;
+        if (copy) copy[i] = x;
+    }
     sh[threadIdx.x] = acc;
     __syncthreads();
     for (int w = blockDim.x / 2; w > 0; w >>= 1) {
@@ -500,8 +515,7 @@ cudaError_t initial_state(lbm_melt *h) {
     if (e == cudaSuccess) e = cudaMemsetAsync(h->nb[1], 0, nc * 4, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->gpost, 0, 7 * nc * 4, h->stream);
     if (e == cudaSuccess && h->spost) e = cudaMemsetAsync(h->spost, 0, 7 * nc * 4, h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->status_dev, 0, sizeof(int), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->jmax_dev, 0, sizeof(int), h->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->status_dev, 0, lbm_melt::kFlags * sizeof(int), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->ticket, 0, sizeof(unsigned int), h->stream);
     if (e == cudaSuccess) {
         k_fill_d<<<nb, 256, 0, h->stream>>>(h->s[0], (long long)nc, d.s0);
@@ -521,8 +535,7 @@ cudaError_t initial_state(lbm_melt *h) {
             e = LAUNCH(h, init, p, h->face, b, Tprof_dev, h->stream);
         }
     }
-    if (e == cudaSuccess && refresh_front(h) != LBM_OK) e = cudaErrorUnknown;
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess && (refresh_front(h) != LBM_OK || read_flags(h) != LBM_OK)) e = cudaErrorUnknown;
     cudaFree(Tprof_dev);
     return e;
 }
@@ -625,7 +638,7 @@ LBM_API lbm_status lbm_melt_create(const lbm_melt_grid *grid, double Ra, double 
     // small cavities are launch bound: replay their steps from graphs
     h->graph_steps = d.N <= kGraphMaxNodes ? kGraphSteps : 0;
     h->pairs_mode = -1;
-    if (cudaMallocHost(&h->rb_val, lbm_melt::kRbRing * sizeof(int)) != cudaSuccess) return fail(LBM_ENOMEM);
+    if (cudaMallocHost(&h->rb_val, (lbm_melt::kRbRing + lbm_melt::kFlags) * sizeof(int)) != cudaSuccess) return fail(LBM_ENOMEM);
     for (int k = 0; k < lbm_melt::kRbRing; ++k)
         if (cudaEventCreateWithFlags(&h->rb_ev[k], cudaEventDisableTiming) != cudaSuccess) return fail(LBM_ECUDA);
     const size_t es = h->precision == 1 ? sizeof(__half) : sizeof(float);
@@ -635,18 +648,19 @@ LBM_API lbm_status lbm_melt_create(const lbm_melt_grid *grid, double Ra, double 
         {&h->F, nF}, {&h->G, nG}, {(void **)&h->js[0], nc * 4}, {(void **)&h->js[1], nc * 4},
         {(void **)&h->nb[0], nc * 4}, {(void **)&h->nb[1], nc * 4},
         {(void **)&h->s[0], nc * 8}, {(void **)&h->s[1], nc * 8}, {(void **)&h->gpost, 7 * nc * 4},
-        {(void **)&h->thw_cur, nc * 4}, {(void **)&h->thw_prev, nc * 4}, {(void **)&h->status_dev, 4},
+        {(void **)&h->thw_cur, nc * 4}, {(void **)&h->thw_prev, nc * 4}, {(void **)&h->status_dev, lbm_melt::kFlags * 4},
         {(void **)&h->sum_dev, 8}, {(void **)&h->ticket, 8}, {(void **)&h->red_part, kRedBlocks * 6 * 8}, {(void **)&h->totals_dev, 7 * 8},
-        {(void **)&h->jmax_dev, sizeof(int)}, {(void **)&h->nu_dev, nc * 8}};
+        {(void **)&h->nu_dev, nc * 8}};
     h->nred = kRedBlocks;
     for (auto &a : allocs) {
         cudaError_t e = cudaMalloc(a.p, a.b);
         if (e != cudaSuccess) return fail(e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA);
         h->bytes += a.b;
     }
+    h->jmax_dev = h->status_dev + 1;
     const cudaError_t e = initial_state(h);
     if (e != cudaSuccess) return fail(e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA);
-    if (seed_readback(h) != LBM_OK) return fail(LBM_ECUDA);
+    seed_readback(h);
     *out = h;
     return LBM_OK;
 }
@@ -770,21 +784,35 @@ LBM_API lbm_status lbm_melt_get_report(lbm_melt *h, double *rows, long long max_
 
 // scale * (sum of the ncols column values v), into dst on the handle's
 // stream: one launch of k_sum_once (chunks of at least 1024 columns per
-// block, fixed order), then a copy.
-lbm_status enqueue_column_sum(lbm_melt *h, const double *v, double scale, double *dst, int ptr_kind) {
+// block, fixed order), which writes a device destination itself (one aligned
+// to a double; else, and to the host, a copy).  copy (may be null): an aligned
+// device array that receives the values in the same launch.
+lbm_status enqueue_column_sum(lbm_melt *h, const double *v, double scale, double *dst, int ptr_kind,
+                              double *copy = nullptr) {
     const long long nc = h->kp.ncols;
     const long long nb = std::max<long long>(1, std::min<long long>(kRedBlocks, (nc + 1023) / 1024));
     const long long chunk = (nc + nb - 1) / nb;
-    k_sum_once<<<(int)nb, 256, 0, h->stream>>>(v, nc, chunk, scale, h->red_part, h->ticket, h->sum_dev);
+    const bool direct = ptr_kind && (size_t)dst % sizeof(double) == 0;
+    k_sum_once<<<(int)nb, 256, 0, h->stream>>>(v, nc, chunk, scale, h->red_part, h->ticket, direct ? dst : h->sum_dev,
+                                               copy);
     CK(cudaGetLastError(), "sum");
-    CK(cudaMemcpyAsync(dst, h->sum_dev, 8, ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream),
-       "copy sum");
+    if (!direct)
+        CK(cudaMemcpyAsync(dst, h->sum_dev, 8, ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream),
+           "copy sum");
     return LBM_OK;
 }
 
-// Liquid fraction = mean front height over H (Σ s / (H ncols)).
-lbm_status enqueue_liquid_fraction(lbm_melt *h, double *dst, int ptr_kind) {
-    return enqueue_column_sum(h, h->s[h->cur], 1.0 / ((double)h->kp.H * (double)h->kp.ncols), dst, ptr_kind);
+// The front S and the liquid fraction, the mean front height over H (either
+// may be null), enqueued on the handle's stream.
+lbm_status enqueue_front_out(lbm_melt *h, double *S, double *liquid_fraction, int ptr_kind) {
+    const double scale = 1.0 / ((double)h->kp.H * (double)h->kp.ncols);
+    if (S && liquid_fraction && ptr_kind && (size_t)S % sizeof(double) == 0)
+        return enqueue_column_sum(h, h->s[h->cur], scale, liquid_fraction, ptr_kind, S);
+    if (S)
+        CK(cudaMemcpyAsync(S, h->s[h->cur], (size_t)h->kp.ncols * 8,
+                           ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream), "copy S");
+    if (liquid_fraction) return enqueue_column_sum(h, h->s[h->cur], scale, liquid_fraction, ptr_kind);
+    return LBM_OK;
 }
 
 LBM_API lbm_status lbm_melt_sync(lbm_melt *h) {
@@ -795,7 +823,7 @@ LBM_API lbm_status lbm_melt_sync(lbm_melt *h) {
 LBM_API lbm_status lbm_melt_get(lbm_melt *h, float *T, float *u, double *S, double *liquid_fraction, int ptr_kind) {
     if (!h) return LBM_EINVAL;
     const KP &p = h->kp;
-    const size_t N = (size_t)p.N, nc = (size_t)p.ncols;
+    const size_t N = (size_t)p.N;
     float *Td = nullptr, *ud = nullptr;
     if (T || u) {
         if (ptr_kind) { Td = T; ud = u; }
@@ -810,24 +838,15 @@ LBM_API lbm_status lbm_melt_get(lbm_melt *h, float *T, float *u, double *S, doub
             if (u) CK(cudaMemcpyAsync(u, ud, 3 * N * 4, cudaMemcpyDeviceToHost, h->stream), "copy u");
         }
     }
-    if (S) CK(cudaMemcpyAsync(S, h->s[h->cur], nc * 8, ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                              h->stream), "copy S");
-    if (liquid_fraction) {
-        const lbm_status st = enqueue_liquid_fraction(h, liquid_fraction, ptr_kind);
-        if (st != LBM_OK) return st;
-    }
-    lbm_status st = check_status(h);
+    lbm_status st = enqueue_front_out(h, S, liquid_fraction, ptr_kind);
+    if (st == LBM_OK) st = check_status(h);
     if (!ptr_kind) { cudaFree(Td); cudaFree(ud); }
     return st;
 }
 
 LBM_API lbm_status lbm_melt_get_async(lbm_melt *h, double *S, double *liquid_fraction, int ptr_kind) {
     if (!h) return LBM_EINVAL;
-    if (S)
-        CK(cudaMemcpyAsync(S, h->s[h->cur], (size_t)h->kp.ncols * 8,
-                           ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream), "copy S");
-    if (liquid_fraction) return enqueue_liquid_fraction(h, liquid_fraction, ptr_kind);
-    return LBM_OK;
+    return enqueue_front_out(h, S, liquid_fraction, ptr_kind);
 }
 
 LBM_API lbm_status lbm_melt_get_state(lbm_melt *h, float *f, float *g, double *S, int ptr_kind) {
@@ -875,13 +894,14 @@ LBM_API lbm_status lbm_melt_set_state(lbm_melt *h, const float *f, const float *
     h->inflight = 0;
     h->thw_pending = 0;
     if (S) {
-        lbm_status st = copy_in(h, h->s[h->cur], S, nc * 8, ptr_kind);
-        if (st != LBM_OK) return st;
-        // liquid counts from the new fronts, front held; their maximum anew
-        CK(cudaMemsetAsync(h->jmax_dev, 0, sizeof(int), h->stream), "reset maximum");
-        if ((st = refresh_front(h)) != LBM_OK) return st;
-        h->rb_valid_from = h->rb_next;  // earlier copies may lie below the new counts
-        if ((st = seed_readback(h)) != LBM_OK) return st;
+        const double *s_in = S;
+        if (!ptr_kind || (size_t)S % sizeof(double)) {
+            const lbm_status st = copy_in(h, h->s[h->cur], S, nc * 8, ptr_kind);
+            if (st != LBM_OK) return st;
+            s_in = h->s[h->cur];
+        }
+        // liquid counts of the new fronts; their maximum anew
+        CK(LAUNCH(h, set_fronts, p, bufs(h), s_in, h->s[h->cur], h->js[h->cur], h->stream), "fronts in");
     }
     const float *fd = f, *gd = g;
     float *tf = nullptr, *tg = nullptr;
@@ -894,7 +914,14 @@ LBM_API lbm_status lbm_melt_set_state(lbm_melt *h, const float *f, const float *
         CK(LAUNCH(h, state_in, p, h->face, b, fd, gd, h->stream), "state in");
     }
     lbm_status st = refresh_front(h);
-    if (st == LBM_OK) st = check_status(h);
+    if (st == LBM_OK) st = read_flags(h);
+    if (st == LBM_OK) {
+        if (S) {
+            h->rb_valid_from = h->rb_next;  // earlier copies may lie below the new counts
+            seed_readback(h);
+        }
+        st = status_of_flags(h);
+    }
     cudaFree(tf);
     cudaFree(tg);
     return st;
@@ -1026,7 +1053,8 @@ LBM_API lbm_status lbm_melt_set_solid_conduction(lbm_melt *h, double ks_kl) {
     h->thw_last_prev = 0;
     const cudaError_t e = initial_state(h);
     if (e != cudaSuccess) return cuda_err(h, e, "initial state");
-    return seed_readback(h);
+    seed_readback(h);
+    return LBM_OK;
 }
 
 LBM_API lbm_status lbm_melt_set_timing(lbm_melt *h, int enable) {
@@ -1078,7 +1106,7 @@ LBM_API lbm_status lbm_melt_get_noalloc(lbm_melt *h, float *T, float *u, double 
                                         int ptr_kind) {
     if (!h) return LBM_EINVAL;
     const KP &p = h->kp;
-    const size_t N = (size_t)p.N, nc = (size_t)p.ncols;
+    const size_t N = (size_t)p.N;
     if (p.N > kNoallocMaxNodes)
         return set_err(h, LBM_EINVAL, "lbm_melt_get_noalloc stages at most %lld nodes; this cavity has %lld",
                        kNoallocMaxNodes, p.N);
@@ -1105,13 +1133,8 @@ LBM_API lbm_status lbm_melt_get_noalloc(lbm_melt *h, float *T, float *u, double 
             if (u) CK(cudaMemcpyAsync(u, ud, 3 * N * 4, cudaMemcpyDeviceToHost, h->stream), "copy u");
         }
     }
-    if (S) CK(cudaMemcpyAsync(S, h->s[h->cur], nc * 8, ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                              h->stream), "copy S");
-    if (liquid_fraction) {
-        // the handle's own reduction buffers, allocated at create: the same
-        // two-pass sum as lbm_melt_get
-        const lbm_status st = enqueue_liquid_fraction(h, liquid_fraction, ptr_kind);
-        if (st != LBM_OK) return st;
-    }
-    return check_status(h);
+    // the handle's own reduction buffers, allocated at create: the same sum
+    // as lbm_melt_get
+    const lbm_status st = enqueue_front_out(h, S, liquid_fraction, ptr_kind);
+    return st == LBM_OK ? check_status(h) : st;
 }
