@@ -46,35 +46,31 @@ namespace lbm {
 // their 3x3 ranges.  Nodes two or more above the largest liquid count of
 // their 3x3 neighbour columns are not written: the reverse sweep reads the
 // snapshot of a level only below the liquid count of that level or of the
-// level before, which differ by at most one.
+// level before, which differ by at most one.  A snapshot holds the heights
+// below the run's bound only (rows of ny_s, N_s nodes: see SnapOut).
 template <typename ST, int FACE>
 __global__ void __launch_bounds__(128) k_snapshot(const __grid_constant__ KP p, const ST *__restrict__ F, const ST *__restrict__ G,
                                                   const int *__restrict__ js, const int *__restrict__ js_old,
                                                   const int *__restrict__ nb,
                                                   const double *__restrict__ s, const float *__restrict__ thw,
-                                                  int inflight, float *__restrict__ out, double *__restrict__ out_s,
-                                                  int *__restrict__ out_js, int *__restrict__ out_nb) {
+                                                  int inflight, const __grid_constant__ SnapOut o) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
     if (x >= p.nx || y >= p.ny) return;
-    const long long c = node_index(p, x, y, z);
     const int a = axial<FACE>(x, y, z), col = column<FACE>(p, x, y, z);
     const int nbv = nb[col];
-    if (a == 0) {  // the column's front, liquid count and neighbourhood range
-        out_s[col] = s[col];
-        out_js[col] = js[col];
-        out_nb[col] = nbv;
-    }
-    if (a >= (nbv & 0xffff) + 2) return;
+    if (a == 0) snap_column(o, col, s[col], js[col], nbv);
+    if (a >= (nbv & 0xffff) + 2 || a >= o.heights) return;
     float g[7], f[19];
     gather_g<ST, FACE>(p, G, x, y, z, inflight != 0, thw, g);
     const bool liq = a < js[col];
     if (liq) gather_f_now<ST, FACE>(p, F, js, js_old, x, y, z, inflight != 0, f);
+    if (!liq) {
 #pragma unroll
-    for (int i = 0; i < 19; ++i) out[i * p.N + c] = liq ? f[i] : 0.0f;
-#pragma unroll
-    for (int i = 0; i < 7; ++i) out[(19 + i) * p.N + c] = g[i];
+        for (int i = 0; i < 19; ++i) f[i] = 0.0f;
+    }
+    snap_node(p, o, x, y, z, f, g);
 }
 
 // ------------------------------------------------- collision, transposed
@@ -736,7 +732,7 @@ struct lbm_tape {
 // The adjoint's device buffers, kept with the handle from one gradient to
 // the next (a loop of gradients of one run length allocates once): the
 // checkpoint pool of the recorded run and the work buffers of the backward,
-// by slot.  A slot is reallocated when a request's size differs; released by
+// by slot.  A slot is reallocated when a request is larger; released by
 // lbm_melt_tape_clear and lbm_melt_destroy.
 struct AdjWorkspace {
     static const int kSlots = 32;
@@ -751,12 +747,12 @@ AdjWorkspace *workspace(lbm_melt *h) {
     return (AdjWorkspace *)h->adj_ws;
 }
 
-// Device buffer of `bytes` in workspace slot k (the cached one when it has
-// that size).
+// Device buffer of at least `bytes` in workspace slot k (the cached one when
+// it is large enough).
 cudaError_t ws_alloc(lbm_melt *h, int k, size_t bytes, void **out) {
     AdjWorkspace *w = workspace(h);
     if (!w) return cudaErrorMemoryAllocation;
-    if (w->p[k] && w->b[k] == bytes) {
+    if (w->p[k] && w->b[k] >= bytes) {
         *out = w->p[k];
         return cudaSuccess;
     }
@@ -951,14 +947,16 @@ LBM_API lbm_status lbm_melt_tape_backward(lbm_melt *h, const double *seed, doubl
         if (s0 != LBM_OK) return s0;
     }
     const lbm::KP &p = h->kp;
-    const size_t N = (size_t)p.N, nc = (size_t)p.ncols;
+    const size_t nc = (size_t)p.ncols;
     const long long C = t->C;
     const dim3 blk = lbm::node_block(p);
-    const dim3 grd_all = lbm::node_grid(p, blk);
-    const size_t nblk = (size_t)grd_all.x * grd_all.y * grd_all.z;
     // Every level of the recorded run has liquid counts at most the running
     // maximum; the snapshot and the node adjoint touch nothing three or more
-    // nodes above it (deep solid), so their grids stop there.
+    // nodes above it (deep solid), so their grids stop there, and so do the
+    // snapshots and the adjoint fields: they are laid out for a cavity of
+    // those heights (pa; the walls of the other axes and the columns are the
+    // cavity's own).  With full-height buffers a gradient of 1000 steps at
+    // 96^3 with a thin layer held 18 GB and spent 7.5 ms giving them back.
     int abound = p.H;
     if (p.skip_deep) {
         int jm = 0;
@@ -967,6 +965,12 @@ LBM_API lbm_status lbm_melt_tape_backward(lbm_melt *h, const double *seed, doubl
         abound = std::min(p.H, jm + 3);
     }
     const dim3 grd = lbm::node_grid_axial(p, blk, h->face, abound);
+    const size_t nblk = (size_t)grd.x * grd.y * grd.z;
+    lbm::KP pa = p;
+    if (h->face == 0) pa.ny = abound;
+    else pa.nz = abound;
+    pa.N = (long long)pa.nx * pa.ny * pa.nz;
+    const size_t N = (size_t)pa.N;
     const int cb = h->cblk;
     const dim3 cgrid = lbm::col_grid((long long)nc, cb);
     // buffers; the snapshots of a segment twice, so that one segment's
@@ -1051,29 +1055,42 @@ LBM_API lbm_status lbm_melt_tape_backward(lbm_melt *h, const double *seed, doubl
         float *snap = snapb[b];
         double *snap_s = snap_sb[b];
         int *snap_js = snap_jsb[b], *snap_nb = snap_nbb[b];
+        auto out = [&](long long j) {
+            lbm::SnapOut o;
+            o.out = snap + (size_t)j * 26 * N;
+            o.s = snap_s + (size_t)j * nc;
+            o.js = snap_js + (size_t)j * nc;
+            o.nb = snap_nb + (size_t)j * nc;
+            o.N = pa.N;
+            o.ny = pa.ny;
+            o.heights = abound;
+            return o;
+        };
         auto snapshot = [&](long long j) {
-            float *out = snap + (size_t)j * 26 * N;
-            double *os = snap_s + (size_t)j * nc;
-            int *ojs = snap_js + (size_t)j * nc, *onb = snap_nb + (size_t)j * nc;
+            const lbm::SnapOut o = out(j);
             const int *js = h->js[cur], *jso = h->js[1 - cur], *nbv = h->nb[cur];
             const double *sv = h->s[cur];
             if (h->precision == 1) {
                 const __half *F = (const __half *)h->F, *G = (const __half *)h->G;
-                if (h->face == 0) lbm::k_snapshot<__half, 0><<<grd, blk, 0, sm>>>(p, F, G, js, jso, nbv, sv, thw, inflight, out, os, ojs, onb);
-                else lbm::k_snapshot<__half, 1><<<grd, blk, 0, sm>>>(p, F, G, js, jso, nbv, sv, thw, inflight, out, os, ojs, onb);
+                if (h->face == 0) lbm::k_snapshot<__half, 0><<<grd, blk, 0, sm>>>(p, F, G, js, jso, nbv, sv, thw, inflight, o);
+                else lbm::k_snapshot<__half, 1><<<grd, blk, 0, sm>>>(p, F, G, js, jso, nbv, sv, thw, inflight, o);
             } else {
                 const float *F = (const float *)h->F, *G = (const float *)h->G;
-                if (h->face == 0) lbm::k_snapshot<float, 0><<<grd, blk, 0, sm>>>(p, F, G, js, jso, nbv, sv, thw, inflight, out, os, ojs, onb);
-                else lbm::k_snapshot<float, 1><<<grd, blk, 0, sm>>>(p, F, G, js, jso, nbv, sv, thw, inflight, out, os, ojs, onb);
+                if (h->face == 0) lbm::k_snapshot<float, 0><<<grd, blk, 0, sm>>>(p, F, G, js, jso, nbv, sv, thw, inflight, o);
+                else lbm::k_snapshot<float, 1><<<grd, blk, 0, sm>>>(p, F, G, js, jso, nbv, sv, thw, inflight, o);
             }
             return cudaGetLastError();
         };
-        cudaError_t e = snapshot(0);
-        for (long long j = 1; j <= len && e == cudaSuccess; ++j) {
-            e = lbm_enqueue_step(h, cur, inflight, abound, sm);
-            if (e == cudaSuccess) e = snapshot(j);
+        // the snapshot of a level is written by the step that leaves it where
+        // that step can (one node per thread), else by a launch of its own
+        cudaError_t e = cudaSuccess;
+        for (long long j = 0; j < len && e == cudaSuccess; ++j) {
+            const lbm::SnapOut o = out(j);
+            const bool with = lbm_step_snapshots(h);
+            if (!with) e = snapshot(j);
+            if (e == cudaSuccess) e = lbm_enqueue_step(h, cur, inflight, abound, sm, with ? &o : nullptr);
         }
-        return e;
+        return e == cudaSuccess ? snapshot(len) : e;
     };
     // A segment's reverse sweep over its levels from snapshot set b, on
     // stream sm; it reads only the snapshots and the adjoint buffers, which
@@ -1096,20 +1113,20 @@ LBM_API lbm_status lbm_melt_tape_backward(lbm_melt *h, const double *seed, doubl
             const double *st_s_prev = j > 0 ? snap_s + (size_t)(j - 1) * nc : nullptr;
             if (h->face == 0) {
                 if (j == len - 1)
-                    lbm::k_adj_front<0><<<cgrid, cb, 0, sm>>>(p, s1, st_s, thw, lms[1], lms[0], wp[pj], wq[pj], lm[1], lthw, lcoef);
-                lbm::k_adj_node<0><<<grd, blk, 0, sm>>>(p, s0, st_js, st_nb, lm[1], lm[0], lgpost, lthw, part);
+                    lbm::k_adj_front<0><<<cgrid, cb, 0, sm>>>(pa, s1, st_s, thw, lms[1], lms[0], wp[pj], wq[pj], lm[1], lthw, lcoef);
+                lbm::k_adj_node<0><<<grd, blk, 0, sm>>>(pa, s0, st_js, st_nb, lm[1], lm[0], lgpost, lthw, part);
                 if (j > 0)
-                    lbm::k_adj_ghost_front<0><<<cgrid, cb, 0, sm>>>(p, s0, st_js, st_s, st_s_prev, thw, lgpost, lm[0], lms[0], lms[1], lthw, lsal, lgb, lcoef, wp[pj], wq[pj], wp[pm], wq[pm]);
+                    lbm::k_adj_ghost_front<0><<<cgrid, cb, 0, sm>>>(pa, s0, st_js, st_s, st_s_prev, thw, lgpost, lm[0], lms[0], lms[1], lthw, lsal, lgb, lcoef, wp[pj], wq[pj], wp[pm], wq[pm]);
                 else
-                    lbm::k_adj_ghost<0><<<cgrid, cb, 0, sm>>>(p, s0, st_js, st_s, thw, lgpost, lm[0], lms[0], lthw, lsal, lgb, wp[pj], wq[pj]);
+                    lbm::k_adj_ghost<0><<<cgrid, cb, 0, sm>>>(pa, s0, st_js, st_s, thw, lgpost, lm[0], lms[0], lthw, lsal, lgb, wp[pj], wq[pj]);
             } else {
                 if (j == len - 1)
-                    lbm::k_adj_front<1><<<cgrid, cb, 0, sm>>>(p, s1, st_s, thw, lms[1], lms[0], wp[pj], wq[pj], lm[1], lthw, lcoef);
-                lbm::k_adj_node<1><<<grd, blk, 0, sm>>>(p, s0, st_js, st_nb, lm[1], lm[0], lgpost, lthw, part);
+                    lbm::k_adj_front<1><<<cgrid, cb, 0, sm>>>(pa, s1, st_s, thw, lms[1], lms[0], wp[pj], wq[pj], lm[1], lthw, lcoef);
+                lbm::k_adj_node<1><<<grd, blk, 0, sm>>>(pa, s0, st_js, st_nb, lm[1], lm[0], lgpost, lthw, part);
                 if (j > 0)
-                    lbm::k_adj_ghost_front<1><<<cgrid, cb, 0, sm>>>(p, s0, st_js, st_s, st_s_prev, thw, lgpost, lm[0], lms[0], lms[1], lthw, lsal, lgb, lcoef, wp[pj], wq[pj], wp[pm], wq[pm]);
+                    lbm::k_adj_ghost_front<1><<<cgrid, cb, 0, sm>>>(pa, s0, st_js, st_s, st_s_prev, thw, lgpost, lm[0], lms[0], lms[1], lthw, lsal, lgb, lcoef, wp[pj], wq[pj], wp[pm], wq[pm]);
                 else
-                    lbm::k_adj_ghost<1><<<cgrid, cb, 0, sm>>>(p, s0, st_js, st_s, thw, lgpost, lm[0], lms[0], lthw, lsal, lgb, wp[pj], wq[pj]);
+                    lbm::k_adj_ghost<1><<<cgrid, cb, 0, sm>>>(pa, s0, st_js, st_s, thw, lgpost, lm[0], lms[0], lthw, lsal, lgb, wp[pj], wq[pj]);
             }
             e = cudaGetLastError();
             std::swap(lm[0], lm[1]);

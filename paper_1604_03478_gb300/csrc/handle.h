@@ -103,7 +103,12 @@ void lbm_tape_free(lbm_melt *h);
 // Enqueue one step (stream-collide, front with flip) from phase (cur, inflight)
 // on stream st, the stream-collide grid cut at `height`; advances cur and
 // inflight.  No host bookkeeping (step counters, read-backs, report rows).
-cudaError_t lbm_enqueue_step(lbm_melt *h, int &cur, int &inflight, int height, cudaStream_t st);
+// snap (may be null, else lbm_step_snapshots holds): the stream-collide also
+// writes the snapshot of the state it starts from.
+namespace lbm { struct SnapOut; }
+cudaError_t lbm_enqueue_step(lbm_melt *h, int &cur, int &inflight, int height, cudaStream_t st,
+                             const lbm::SnapOut *snap = nullptr);
+bool lbm_step_snapshots(lbm_melt *h);
 // Reads the sticky front status on the handle's stream (synchronises):
 // LBM_EUNSTABLE after a step with |ds| > 1/2, LBM_ENAN after a non-finite
 // front temperature, else LBM_OK.

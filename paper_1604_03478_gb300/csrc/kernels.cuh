@@ -29,6 +29,7 @@
 // flags of the step before (the other of the two liquid-count buffers).
 #pragma once
 
+#include "launch.h"
 #include "lbm_core.cuh"
 
 namespace lbm {
@@ -188,6 +189,26 @@ __device__ __forceinline__ void even_node(const KP &p, ST *__restrict__ F, ST *_
     for (int i = 0; i < 7; ++i) Store<ST>::st_stream(elem<IX>(G, c, opp7(i) * p.ld), g[i]);
 }
 
+// ---------------------------------------------------------- snapshots
+__device__ __forceinline__ void snap_node(const KP &p, const SnapOut &o, int x, int y, int z, const float (&f)[19],
+                                          const float (&g)[7]) {
+    float *const at = o.out + (((long long)z * o.ny + y) * p.nx + x);
+#pragma unroll
+    for (int i = 0; i < 19; ++i) at[i * o.N] = f[i];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) at[(19 + i) * o.N] = g[i];
+}
+__device__ __forceinline__ void snap_column(const SnapOut &o, int col, double s, int js, int nb) {
+    o.s[col] = s;
+    o.js[col] = js;
+    o.nb[col] = nb;
+}
+
+// The snapshot of a column's first solid node: fh = 0 and its g.
+template <typename ST, int FACE>
+__device__ __forceinline__ void snap_ghost(const KP &p, const ST *G, const float *thw, int x, int y, int z,
+                                           bool inflight, const SnapOut &o);
+
 // Stream-collide grid: blocks of blockDim.x x blockDim.y nodes of one plane
 // across the heating axis, with the height along that axis slowest
 // (blockIdx.z), so that the blocks near the heated wall are dispatched
@@ -236,10 +257,15 @@ template <typename ST> constexpr int k1_min_blocks() { return sizeof(ST) == 2 ? 
 // flags from L2 too, 128^3 with a thin layer ran 17.0 us a step, 96^3 18.8.
 // A step, without and with the early loads: 32^3 8.0 -> 6.5 us, 128^3 thin
 // layer 16.8 -> 16.5, 96^3 mid melt 18.6 -> 18.2, 101x75x83 19.6 -> 18.9.
-template <typename ST, int FACE, typename IX>
-__global__ void __launch_bounds__(128, k1_min_blocks<ST>()) k_even(const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G,
+//
+// SNAP: the snapshot of the state the step starts from (the recomputation of
+// the adjoint): the liquid nodes' populations, which the step has in
+// registers, and the first solid node's g.
+template <typename ST, int FACE, typename IX, bool SNAP>
+__global__ void __launch_bounds__(128, SNAP ? 0 : k1_min_blocks<ST>()) k_even(const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G,
                                               const int *js, const int *js_old, const int *__restrict__ nb,
-                                              const float *__restrict__ gpost, const int *jmax, int early_blocks) {
+                                              const float *__restrict__ gpost, const int *jmax, int early_blocks,
+                                              const double *s, const __grid_constant__ SnapOut snap) {
     int x = 0, y = 0, z = 0, a = 0, col = 0, jso = 0;
     IX c = 0;
     float f[19], g[7];
@@ -263,6 +289,7 @@ __global__ void __launch_bounds__(128, k1_min_blocks<ST>()) k_even(const __grid_
     if (!late) step_launch_wait();
     if (!on) return;
     const int jsc = __ldg(js + col);
+    if (SNAP && a == 0) snap_column(snap, col, s[col], jsc, nb[col]);
     if (a < jsc) {
         if (a >= jso) {
 #pragma unroll
@@ -270,11 +297,13 @@ __global__ void __launch_bounds__(128, k1_min_blocks<ST>()) k_even(const __grid_
 #pragma unroll
             for (int i = 0; i < 7; ++i) g[i] = ld_l2(elem<IX>(G, c, i * p.ld));
         }
+        if (SNAP) snap_node(p, snap, x, y, z, f, g);
         collide(p, f, g);
 #pragma unroll
         for (int i = 0; i < 19; ++i) Store<ST>::st_stream(elem<IX>(F, c, opp(i) * p.ld), f[i]);
     } else {
         if (deep_solid(p, a, __ldg(nb + col))) return;
+        if (SNAP && a == jsc) snap_ghost<ST, FACE>(p, G, nullptr, x, y, z, false, snap);
         solid_post(p, a == jsc, gpost, col, g);
     }
 #pragma unroll
@@ -553,12 +582,12 @@ __device__ __forceinline__ void odd_node(const KP &p, const Links *lk, ST *__res
 // links are read again after the wait, from where flip_column moved the
 // value.  `inner`: interior under the old flags and, counts changing by at
 // most one a step, under the new ones.
-template <typename ST, int FACE>
+template <typename ST, int FACE, bool SNAP>
 __device__ __forceinline__ void odd_node_early(const KP &p, const Links *lk, ST *__restrict__ F, ST *__restrict__ G,
                                                const int *js, const int *js_old, const int *nb, const int *nb_old,
                                                const float *__restrict__ gpost, const float *thw_rd,
                                                const float *__restrict__ thw_wr, const int *jmax, int early_blocks,
-                                               bool on, int x, int y, int z) {
+                                               bool on, int x, int y, int z, const double *s, const SnapOut &snap) {
     const long long c = on ? node_index(p, x, y, z) : 0;
     const int a = axial<FACE>(x, y, z), col = on ? column<FACE>(p, x, y, z) : 0;
     const int q = FACE == 0 ? z : y, nq = FACE == 0 ? p.nz : p.ny;
@@ -624,7 +653,8 @@ __device__ __forceinline__ void odd_node_early(const KP &p, const Links *lk, ST 
     }
     if (!late) step_launch_wait();
     if (!on) return;
-    const int jsc = inner ? p.H : __ldg(js + col);
+    const int jsc = inner && !SNAP ? p.H : __ldg(js + col);
+    if (SNAP && a == 0) snap_column(snap, col, s[col], jsc, nb[col]);
     if (a < jsc) {
         bool fast = inner;
         if (!inner) {
@@ -644,6 +674,7 @@ __device__ __forceinline__ void odd_node_early(const KP &p, const Links *lk, ST 
             lm = now;
             fast = off_qa && (lm & need) == need;
         }
+        if (SNAP) snap_node(p, snap, x, y, z, f, g);
         collide(p, f, g);
         Store<ST>::st_stream(Fc, f[0]);
         if (fast) {
@@ -662,6 +693,7 @@ __device__ __forceinline__ void odd_node_early(const KP &p, const Links *lk, ST 
     } else {
         if (deep_solid(p, a, __ldg(nb + col))) return;
         im = inside_mask(p, x, y, z);
+        if (SNAP && a == jsc) snap_ghost<ST, FACE>(p, G, thw_rd, x, y, z, true, snap);
         solid_post(p, a == jsc, gpost, col, g);
     }
     const float th_wr = __ldg(thw_wr + col);
@@ -674,15 +706,17 @@ __device__ __forceinline__ void odd_node_early(const KP &p, const Links *lk, ST 
     }
 }
 
-template <typename ST, int FACE>
-__global__ void __launch_bounds__(128, k1_min_blocks<ST>()) k_odd(const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G,
+template <typename ST, int FACE, bool SNAP>
+__global__ void __launch_bounds__(128, SNAP ? 0 : k1_min_blocks<ST>()) k_odd(const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G,
                                              const int *js, const int *js_old, const int *nb, const int *nb_old,
                                              const float *__restrict__ gpost, const float *thw_rd,
                                              const float *__restrict__ thw_wr, const __grid_constant__ Links lk,
-                                             const int *jmax, int early_blocks) {
+                                             const int *jmax, int early_blocks, const double *s,
+                                             const __grid_constant__ SnapOut snap) {
     int x = 0, y = 0, z = 0;
     const bool on = k1_node<FACE>(p, nullptr, x, y, z);
-    odd_node_early<ST, FACE>(p, &lk, F, G, js, js_old, nb, nb_old, gpost, thw_rd, thw_wr, jmax, early_blocks, on, x, y, z);
+    odd_node_early<ST, FACE, SNAP>(p, &lk, F, G, js, js_old, nb, nb_old, gpost, thw_rd, thw_wr, jmax, early_blocks, on, x, y, z, s,
+                                   snap);
 }
 
 // The odd step with heat conduction in the solid (every node updated).
@@ -914,6 +948,17 @@ __device__ __forceinline__ void gather_g(const KP &p, const ST *G, int x, int y,
 
 // Shifted pre-collision f of a liquid node.  js: the liquid flags that the
 // in-flight values were produced under, or the ones after flip_column has run.
+template <typename ST, int FACE>
+__device__ __forceinline__ void snap_ghost(const KP &p, const ST *G, const float *thw, int x, int y, int z,
+                                           bool inflight, const SnapOut &o) {
+    if (axial<FACE>(x, y, z) >= o.heights) return;
+    float f[19], g[7];
+    gather_g<ST, FACE>(p, G, x, y, z, inflight, thw, g);
+#pragma unroll
+    for (int i = 0; i < 19; ++i) f[i] = 0.0f;
+    snap_node(p, o, x, y, z, f, g);
+}
+
 template <typename ST, int FACE>
 __device__ __forceinline__ void gather_f(const KP &p, const ST *F, const int *js, int x, int y, int z,
                                          bool inflight, float (&f)[19]) {

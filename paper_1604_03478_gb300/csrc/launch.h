@@ -31,6 +31,18 @@ struct Bufs {
     int pairs;                   // stream-collide with two nodes per thread (even nx)
 };
 
+// Where a step leaves the natural-layout snapshot of the state it starts from
+// (FP32: fh of 19 directions, zero at solid nodes, then gh of 7, each of N
+// nodes in rows of nx and planes of ny rows: the heights below `heights`
+// only), and the columns' fronts, liquid counts and 3x3 bounds.
+struct SnapOut {
+    float *out;
+    double *s;
+    int *js, *nb;
+    long long N;
+    int ny, heights;
+};
+
 // The stream-collide and front kernels with heat conduction in the solid
 // (KP::cond), in a translation unit of their own (k_cond.cu); Launch
 // forwards to them.
@@ -40,7 +52,11 @@ template <typename ST> struct LaunchCond {
 };
 
 template <typename ST> struct Launch {
-    static cudaError_t stream_collide(const KP &p, int face, int odd, const Bufs &b, dim3 blk, cudaStream_t st);
+    // snap (may be null): also write the snapshot of the state the step starts
+    // from; only where snapshots(p, b).
+    static cudaError_t stream_collide(const KP &p, int face, int odd, const Bufs &b, dim3 blk, cudaStream_t st,
+                                      const SnapOut *snap = nullptr);
+    static bool snapshots(const KP &p, const Bufs &b);
     static cudaError_t front(const KP &p, int face, int inflight, int move, const Bufs &b, cudaStream_t st);
     static cudaError_t macro(const KP &p, int face, int inflight, const Bufs &b, float *T, float *u, cudaStream_t st);
     static cudaError_t state_out(const KP &p, int face, int inflight, const Bufs &b, float *f, float *g, cudaStream_t st);

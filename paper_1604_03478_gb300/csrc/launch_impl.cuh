@@ -31,18 +31,19 @@ static cudaError_t launch_step_kernel(void (*kern)(KArgs...), dim3 grd, dim3 blk
 #endif
 }
 
-template <typename ST, typename IXE>
-static cudaError_t launch_sc(const KP &p, int face, int odd, const Bufs &b, dim3 grd, dim3 blk, cudaStream_t st) {
+template <typename ST, typename IXE, bool SNAP>
+static cudaError_t launch_sc(const KP &p, int face, int odd, const Bufs &b, dim3 grd, dim3 blk, cudaStream_t st,
+                             const SnapOut &snap) {
     // blocks resident at once: 7 of 128 threads an SM (72 registers)
     const int early = b.sms * (896 / (int)(blk.x * blk.y));
     const int *jm = p.skip_deep ? b.jmax : nullptr;
     ST *F = (ST *)b.F, *G = (ST *)b.G;
     if (face == 0) {
-        if (odd) return launch_step_kernel(k_odd<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early);
-        else return launch_step_kernel(k_even<ST, 0, IXE>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early);
+        if (odd) return launch_step_kernel(k_odd<ST, 0, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early, b.s, snap);
+        else return launch_step_kernel(k_even<ST, 0, IXE, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early, b.s, snap);
     } else {
-        if (odd) return launch_step_kernel(k_odd<ST, 1>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early);
-        else return launch_step_kernel(k_even<ST, 1, IXE>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early);
+        if (odd) return launch_step_kernel(k_odd<ST, 1, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early, b.s, snap);
+        else return launch_step_kernel(k_even<ST, 1, IXE, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early, b.s, snap);
     }
 }
 
@@ -72,15 +73,22 @@ static cudaError_t launch_sc_pair(const KP &p, int face, int odd, const Bufs &b,
 // 64 bits (FP16 storage 2% faster at 256^3; the odd step ran slower with
 // 32-bit indices, 0.258 against 0.245 ms in FP32, and keeps 64-bit ones).
 template <typename ST>
-cudaError_t Launch<ST>::stream_collide(const KP &p, int face, int odd, const Bufs &b, dim3 blk, cudaStream_t st) {
+bool Launch<ST>::snapshots(const KP &p, const Bufs &b) {
+    return !p.cond && !(b.pairs && p.nx % 2 == 0) && 19LL * p.ld < (1LL << 32);
+}
+
+template <typename ST>
+cudaError_t Launch<ST>::stream_collide(const KP &p, int face, int odd, const Bufs &b, dim3 blk, cudaStream_t st,
+                                       const SnapOut *snap) {
     if (p.cond) return LaunchCond<ST>::stream_collide(p, face, odd, b, blk, st);
     if (b.pairs && p.nx % 2 == 0) {
         if (19LL * p.ld < (1LL << 32)) return launch_sc_pair<ST, unsigned, LBM_PAIR_ODD_IX>(p, face, odd, b, blk, st);
         return launch_sc_pair<ST, long long, long long>(p, face, odd, b, blk, st);
     }
     const dim3 grd = k1_grid(p, blk, face, b.k1_height);
-    if (19LL * p.ld < (1LL << 32)) return launch_sc<ST, unsigned>(p, face, odd, b, grd, blk, st);
-    return launch_sc<ST, long long>(p, face, odd, b, grd, blk, st);
+    if (snap) return launch_sc<ST, unsigned, true>(p, face, odd, b, grd, blk, st, *snap);
+    if (19LL * p.ld < (1LL << 32)) return launch_sc<ST, unsigned, false>(p, face, odd, b, grd, blk, st, SnapOut());
+    return launch_sc<ST, long long, false>(p, face, odd, b, grd, blk, st, SnapOut());
 }
 
 template <typename ST>

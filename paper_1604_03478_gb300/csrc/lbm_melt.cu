@@ -397,11 +397,12 @@ dim3 sc_block(const lbm_melt *h) {
 
 // Enqueue one step from phase (cur, inflight) on stream st with the
 // stream-collide grid cut at `height`; returns the phase after it.
-cudaError_t enqueue_step(lbm_melt *h, int &cur, int &inflight, int height, dim3 blk, cudaStream_t st) {
+cudaError_t enqueue_step(lbm_melt *h, int &cur, int &inflight, int height, dim3 blk, cudaStream_t st,
+                         const lbm::SnapOut *snap = nullptr) {
     Bufs b = bufs_at(h, cur, inflight);
     b.k1_height = height;
     const int odd = inflight;
-    cudaError_t e = LAUNCH(h, stream_collide, h->kp, h->face, odd, b, blk, st);
+    cudaError_t e = LAUNCH(h, stream_collide, h->kp, h->face, odd, b, blk, st, snap);
     if (e != cudaSuccess) return e;
     inflight = !odd;
     b = bufs_at(h, cur, inflight);
@@ -468,9 +469,12 @@ bool graph_eligible(const lbm_melt *h, long long left) {
 
 lbm_status lbm_check_status(lbm_melt *h) { return check_status(h); }
 
-cudaError_t lbm_enqueue_step(lbm_melt *h, int &cur, int &inflight, int height, cudaStream_t st) {
-    return enqueue_step(h, cur, inflight, height, sc_block(h), st);
+cudaError_t lbm_enqueue_step(lbm_melt *h, int &cur, int &inflight, int height, cudaStream_t st,
+                             const lbm::SnapOut *snap) {
+    return enqueue_step(h, cur, inflight, height, sc_block(h), st, snap);
 }
+
+bool lbm_step_snapshots(lbm_melt *h) { return LAUNCH(h, snapshots, h->kp, bufs(h)); }
 
 
 
