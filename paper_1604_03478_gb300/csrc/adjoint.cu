@@ -191,22 +191,22 @@ __device__ __forceinline__ float snap_T(const KP &p, const float *snap, int col,
 
 // The slopes s_p, s_q of column c' read the fronts of its neighbours (with a
 // mirror at the side walls); the sum of their d/d s for column col.
-__device__ __forceinline__ double slope_terms(const KP &p, const double *__restrict__ wp,
-                                              const double *__restrict__ wq, int col) {
+__device__ __forceinline__ double slope_terms(const KP &p, const double *wp,
+                                              const double *wq, int col) {
     const int P1 = p.P1, P2 = p.P2;
     const int pp = col % P1, q = col / P1;
     double acc = 0.0;
     if (P1 > 1) {
-        if (pp >= 1) acc += 0.5 * wp[col - 1];       // column pp-1 reads s[pp] as its upper neighbour
-        if (pp <= P1 - 2) acc -= 0.5 * wp[col + 1];  // column pp+1 reads s[pp] as its lower neighbour
-        if (pp == 0) acc -= 0.5 * wp[col];           // mirror: s[-1] = s[0]
-        if (pp == P1 - 1) acc += 0.5 * wp[col];      // mirror: s[P1] = s[P1-1]
+        if (pp >= 1) acc += 0.5 * ld_l2(wp + col - 1);       // column pp-1 reads s[pp] as its upper neighbour
+        if (pp <= P1 - 2) acc -= 0.5 * ld_l2(wp + col + 1);  // column pp+1 reads s[pp] as its lower neighbour
+        if (pp == 0) acc -= 0.5 * ld_l2(wp + col);           // mirror: s[-1] = s[0]
+        if (pp == P1 - 1) acc += 0.5 * ld_l2(wp + col);      // mirror: s[P1] = s[P1-1]
     }
     if (P2 > 1) {
-        if (q >= 1) acc += 0.5 * wq[col - P1];
-        if (q <= P2 - 2) acc -= 0.5 * wq[col + P1];
-        if (q == 0) acc -= 0.5 * wq[col];
-        if (q == P2 - 1) acc += 0.5 * wq[col];
+        if (q >= 1) acc += 0.5 * ld_l2(wq + col - P1);
+        if (q <= P2 - 2) acc -= 0.5 * ld_l2(wq + col + P1);
+        if (q == 0) acc -= 0.5 * ld_l2(wq + col);
+        if (q == P2 - 1) acc += 0.5 * ld_l2(wq + col);
     }
     return acc;
 }
@@ -220,9 +220,17 @@ __device__ __forceinline__ double slope_terms(const KP &p, const double *__restr
 // (ghost node) or one above the count of the level between (front terms);
 // liquid counts change by at most one per step (|ds| <= 1/2, else the run
 // stops as unstable), so both bounds lie below the skipped nodes.
+//
+// The reverse sweep is a chain of two small kernels a level (this one and the
+// column kernel), bound by their latencies.  They are launched like the
+// step's kernels (step_launch_wait): everything that does not come from the
+// kernel before (the snapshot, the counts; in the column kernel also the
+// sums and slope partials of the level above) is loaded before the wait.
+// Backward of 1000 steps at 96^3, thin layer: 18.5 -> 14.3 ms (17.2 with the
+// same kernels launched plainly); the streams' priorities changed nothing.
 template <int FACE>
 __global__ void __launch_bounds__(128) k_adj_node(const __grid_constant__ KP p, const float *__restrict__ snap, const int *__restrict__ js,
-                                                  const int *__restrict__ nb, const float *__restrict__ lam1,
+                                                  const int *__restrict__ nb, const float *lam1,
                                                   float *__restrict__ lam0, float *__restrict__ lgpost,
                                                   double *__restrict__ lthw, double *__restrict__ part) {
     __shared__ double sh[3][128];
@@ -230,14 +238,30 @@ __global__ void __launch_bounds__(128) k_adj_node(const __grid_constant__ KP p, 
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    const long long N = p.N;
+    const bool on = x < p.nx && y < p.ny;
+    const long long c = on ? node_index(p, x, y, z) : 0;
+    const int a = axial<FACE>(x, y, z), col = on ? column<FACE>(p, x, y, z) : 0;
     float dsnu = 0.0f, dsal = 0.0f, dgb = 0.0f;
-    int liquid = 0;
-    if (x < p.nx && y < p.ny) {
-        const long long c = node_index(p, x, y, z);
-        const long long N = p.N;
-        const int a = axial<FACE>(x, y, z), col = column<FACE>(p, x, y, z);
-        const int jsc = js[col];
+    float f[19], g[7];
+    int jsc = 0, nbv = 0, liquid = 0;
+    unsigned lm = 0;  // bit opp(i): x + e_i is liquid
+    if (on) {
+        int js9[9];
+        load_js9(p, js, x, FACE == 0 ? z : y, js9);
+        jsc = js9[4];
+        nbv = nb[col];
         liquid = a < jsc;
+        if (liquid) {
+#pragma unroll
+            for (int i = 0; i < 19; ++i) f[i] = snap[i * N + c];
+#pragma unroll
+            for (int i = 0; i < 7; ++i) g[i] = snap[(19 + i) * N + c];
+            lm = link_mask9<FACE>(js9, a);
+        }
+    }
+    step_launch_wait();
+    if (on) {
         // heated-wall link: the node next to the wall receives
         // -g*_opp + 2 w (Tw - Tm) along the heating axis
         if (a == 0) {
@@ -245,68 +269,56 @@ __global__ void __launch_bounds__(128) k_adj_node(const __grid_constant__ KP p, 
             lthw[col] += 2.0 * (double)w7(iin) * (double)lam1[(19 + iin) * N + c];
         }
         if (a > jsc) {
-            if (a < (nb[col] & 0xffff) + 3) {
+            if (a < (nbv & 0xffff) + 3) {
 #pragma unroll
                 for (int i = 0; i < 26; ++i) lam0[i * N + c] = 0.0f;
             }
         } else {
             // g*: every node streams g; the transpose of the pull is a gather
-            float lg[7];
+            float lg[7], lf[19];
+            const unsigned im = inside_mask(p, x, y, z);  // bit opp7(i): x + t_i is inside
             lg[0] = lam1[19 * N + c];
 #pragma unroll
             for (int i = 1; i < 7; ++i) {
-                if (inside(p, x + tx(i), y + ty(i), z + tz(i))) {
-                    lg[i] = lam1[(19 + i) * N + c + off7<FACE>(p, i)];
-                } else {
-                    const int w = wall_of_link<FACE>(i);
-                    const float v = lam1[(19 + opp7(i)) * N + c];
-                    lg[i] = w == 3 ? v : -v;
-                }
+                const bool in = (im >> opp7(i)) & 1u;
+                const float v = lam1[in ? (19 + i) * N + c + off7<FACE>(p, i) : (19 + opp7(i)) * N + c];
+                lg[i] = in || wall_of_link<FACE>(i) == 3 ? v : -v;
             }
-            if (a == jsc) {  // ghost node: its post-collision g came from the ghost rule
-#pragma unroll
-                for (int i = 0; i < 7; ++i) lgpost[(long long)i * p.ncols + col] = lg[i];
-#pragma unroll
-                for (int i = 0; i < 26; ++i) lam0[i * N + c] = 0.0f;
-            } else {
-                float lf[19], f[19], g[7], of[19], og[7];
+            if (liquid) {
                 lf[0] = lam1[c];
 #pragma unroll
-                for (int i = 1; i < 19; ++i) {
-                    if (liquid_at<FACE>(p, js, x + ex(i), y + ey(i), z + ez(i)))
-                        lf[i] = lam1[i * N + c + off19<FACE>(p, i)];
-                    else
-                        lf[i] = lam1[opp(i) * N + c];
-                }
-#pragma unroll
-                for (int i = 0; i < 19; ++i) f[i] = snap[i * N + c];
-#pragma unroll
-                for (int i = 0; i < 7; ++i) g[i] = snap[(19 + i) * N + c];
+                for (int i = 1; i < 19; ++i)
+                    lf[i] = lam1[((lm >> opp(i)) & 1u) ? i * N + c + off19<FACE>(p, i) : opp(i) * N + c];
+                float of[19], og[7];
                 collide_adjoint(p, f, g, lf, lg, of, og, dsnu, dsal, dgb);
 #pragma unroll
                 for (int i = 0; i < 19; ++i) lam0[i * N + c] = of[i];
 #pragma unroll
                 for (int i = 0; i < 7; ++i) lam0[(19 + i) * N + c] = og[i];
+            } else {  // ghost node: its post-collision g came from the ghost rule
+#pragma unroll
+                for (int i = 0; i < 7; ++i) lgpost[(long long)i * p.ncols + col] = lg[i];
+#pragma unroll
+                for (int i = 0; i < 26; ++i) lam0[i * N + c] = 0.0f;
             }
         }
     }
-    // blocks without a liquid node add nothing to the rate partials
-    if (!__syncthreads_or(liquid)) return;
+    // blocks without a liquid node add nothing to the rate partials; the sum
+    // of the block's 128 values in the order of a tree over halves, the last
+    // five levels within a warp, one warp to a value
     sh[0][tid] = dsnu;
     sh[1][tid] = dsal;
     sh[2][tid] = dgb;
-    __syncthreads();
-    for (int w = 64; w > 0; w >>= 1) {
-        if (tid < w) {
-            sh[0][tid] += sh[0][tid + w];
-            sh[1][tid] += sh[1][tid + w];
-            sh[2][tid] += sh[2][tid + w];
+    if (!__syncthreads_or(liquid)) return;
+    const int k = tid >> 5, l = tid & 31;
+    if (k < 3) {
+        double v = (sh[k][l] + sh[k][l + 64]) + (sh[k][l + 32] + sh[k][l + 96]);
+#pragma unroll
+        for (int w = 16; w > 0; w >>= 1) v += __shfl_down_sync(0xffffffffu, v, w);
+        if (l == 0) {
+            const long long b = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
+            part[b * 3 + k] += v;
         }
-        __syncthreads();
-    }
-    if (tid < 3) {
-        const long long b = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
-        part[b * 3 + tid] += sh[tid][0];
     }
 }
 
@@ -346,11 +358,11 @@ template <int FACE, bool GHOST, bool FRONT>
 __device__ __forceinline__ void adj_column(const KP &p, int col, const float *__restrict__ snap,
                                            const int *__restrict__ js, const double *__restrict__ s,
                                            const double *__restrict__ s_prev, const float *__restrict__ thw,
-                                           const float *__restrict__ lgpost, float *__restrict__ lam,
+                                           const float *lgpost, float *__restrict__ lam,
                                            double *__restrict__ lams, double *__restrict__ lams_prev,
                                            double *__restrict__ lthw, double *__restrict__ lsal,
                                            double *__restrict__ lgb, double *__restrict__ lcoef,
-                                           const double *__restrict__ wp, const double *__restrict__ wq,
+                                           const double *wp, const double *wq,
                                            double *__restrict__ wp_prev, double *__restrict__ wq_prev) {
     const int H = p.H, P1 = p.P1, P2 = p.P2;
     const long long N = p.N;
@@ -368,9 +380,9 @@ __device__ __forceinline__ void adj_column(const KP &p, int col, const float *__
     // store: the compiler cannot move a load of lam or of a per-column sum
     // above a store through another pointer, and each such wait is a
     // memory round trip of a latency-bound kernel)
-    const double lams_in = lams[col];
-    const double lsal0 = GHOST ? lsal[col] : 0.0, lgb0 = GHOST ? lgb[col] : 0.0;
-    const double lcoef0 = FRONT ? lcoef[col] : 0.0, lthw0 = lthw[col];
+    const double lams_in = ld_l2(lams + col);
+    const double lsal0 = GHOST ? ld_l2(lsal + col) : 0.0, lgb0 = GHOST ? ld_l2(lgb + col) : 0.0;
+    const double lcoef0 = FRONT ? ld_l2(lcoef + col) : 0.0;
     float lamf[19];
     // stage 1: what depends on the column only
     if (GHOST) {
@@ -378,11 +390,6 @@ __device__ __forceinline__ void adj_column(const KP &p, int col, const float *__
         in.jn = js[col];
         in.sn = s[col];
         in.lTG = 0.0f;
-#pragma unroll
-        for (int i = 0; i < 7; ++i) {
-            in.lgp[i] = lgpost[(long long)i * p.ncols + col];
-            in.lTG = __fmaf_rn(w7(i), in.lgp[i], in.lTG);
-        }
     }
     if (FRONT) {
         in.sc = s_prev[col];
@@ -414,8 +421,6 @@ __device__ __forceinline__ void adj_column(const KP &p, int col, const float *__
 #pragma unroll
         for (int i = 0; i < 19; ++i) in.fL[i] = snap[i * N + eL];
 #pragma unroll
-        for (int i = 0; i < 19; ++i) lamf[i] = lam[i * N + eL];
-#pragma unroll
         for (int i = 0; i < 7; ++i) gK[i] = snap[(19 + i) * N + eK];
     }
     if (FRONT) {
@@ -423,6 +428,15 @@ __device__ __forceinline__ void adj_column(const KP &p, int col, const float *__
         for (int i = 0; i < 7; ++i) g1[i] = snap[(19 + i) * N + e1];
 #pragma unroll
         for (int i = 0; i < 7; ++i) g0[i] = snap[(19 + i) * N + e0];
+    }
+    // stage 3, after the node kernel: what it wrote
+    if (GHOST) step_launch_wait();
+    const double lthw0 = lthw[col];
+    if (GHOST) {
+#pragma unroll
+        for (int i = 0; i < 7; ++i) in.lgp[i] = ld_l2(lgpost + (long long)i * p.ncols + col);
+#pragma unroll
+        for (int i = 0; i < 19; ++i) lamf[i] = lam[i * N + eL];
     }
     // the g adjoint of the four nodes (clamped as above)
     const long long eff[4] = {eL, eK, e1, e0};
@@ -433,6 +447,10 @@ __device__ __forceinline__ void adj_column(const KP &p, int col, const float *__
 #pragma unroll
             for (int i = 0; i < 7; ++i) base[e][i] = lam[(19 + i) * N + eff[e]];
         }
+    if (GHOST) {
+#pragma unroll
+        for (int i = 0; i < 7; ++i) in.lTG = __fmaf_rn(w7(i), in.lgp[i], in.lTG);
+    }
     // temperatures summed in the order of the forward's front update
     auto tsum = [&](const float (&g)[7]) {
         float t = 0.0f;
@@ -622,13 +640,15 @@ __global__ void __launch_bounds__(128) k_adj_front(const __grid_constant__ KP p,
 template <int FACE>
 __global__ void __launch_bounds__(128) k_adj_ghost(const __grid_constant__ KP p, const float *__restrict__ snap,
                                                    const int *__restrict__ js, const double *__restrict__ s,
-                                                   const float *__restrict__ thw, const float *__restrict__ lgpost,
+                                                   const float *__restrict__ thw, const float *lgpost,
                                                    float *__restrict__ lam0, double *__restrict__ lams0,
                                                    double *__restrict__ lthw, double *__restrict__ lsal,
-                                                   double *__restrict__ lgb, const double *__restrict__ wp,
-                                                   const double *__restrict__ wq) {
+                                                   double *__restrict__ lgb, const double *wp, const double *wq) {
     const int col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col >= p.ncols) return;
+    if (col >= p.ncols) {
+        step_launch_wait();
+        return;
+    }
     adj_column<FACE, true, false>(p, col, snap, js, s, nullptr, thw, lgpost, lam0, lams0, nullptr, lthw, lsal, lgb,
                                   nullptr, wp, wq, nullptr, nullptr);
 }
@@ -642,12 +662,15 @@ template <int FACE>
 __global__ void __launch_bounds__(128) k_adj_ghost_front(
     const __grid_constant__ KP p, const float *__restrict__ snap, const int *__restrict__ js,
     const double *__restrict__ s, const double *__restrict__ s_prev, const float *__restrict__ thw,
-    const float *__restrict__ lgpost, float *__restrict__ lam0, double *__restrict__ lams0,
+    const float *lgpost, float *__restrict__ lam0, double *__restrict__ lams0,
     double *__restrict__ lams_prev, double *__restrict__ lthw, double *__restrict__ lsal, double *__restrict__ lgb,
-    double *__restrict__ lcoef, const double *__restrict__ wp, const double *__restrict__ wq,
+    double *__restrict__ lcoef, const double *wp, const double *wq,
     double *__restrict__ wp_prev, double *__restrict__ wq_prev) {
     const int col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col >= p.ncols) return;
+    if (col >= p.ncols) {
+        step_launch_wait();
+        return;
+    }
     adj_column<FACE, true, true>(p, col, snap, js, s, s_prev, thw, lgpost, lam0, lams0, lams_prev, lthw, lsal, lgb,
                                  lcoef, wp, wq, wp_prev, wq_prev);
 }
@@ -800,6 +823,21 @@ lbm_status tape_err(lbm_melt *h, lbm_status st, const char *fmt, ...) {
             return tape_err(h, e_ == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA, "%s: %s", where,  \
                             cudaGetErrorString(e_));                                                       \
     } while (0)
+
+// Launch with programmatic stream serialization (see step_launch_wait).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grd, dim3 blk, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grd;
+    cfg.blockDim = blk;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
 
 // Layout of a checkpoint: the nine state arrays of a handle, each starting
 // on a 256-byte boundary.  Returns the total size; dev/sz/off describe them.
@@ -1112,23 +1150,26 @@ LBM_API lbm_status lbm_melt_tape_backward(lbm_melt *h, const double *seed, doubl
             const int pj = (int)(j & 1), pm = pj ^ 1;
             const double *st_s_prev = j > 0 ? snap_s + (size_t)(j - 1) * nc : nullptr;
             if (h->face == 0) {
-                if (j == len - 1)
+                if (j == len - 1) {
                     lbm::k_adj_front<0><<<cgrid, cb, 0, sm>>>(pa, s1, st_s, thw, lms[1], lms[0], wp[pj], wq[pj], lm[1], lthw, lcoef);
-                lbm::k_adj_node<0><<<grd, blk, 0, sm>>>(pa, s0, st_js, st_nb, lm[1], lm[0], lgpost, lthw, part);
-                if (j > 0)
-                    lbm::k_adj_ghost_front<0><<<cgrid, cb, 0, sm>>>(pa, s0, st_js, st_s, st_s_prev, thw, lgpost, lm[0], lms[0], lms[1], lthw, lsal, lgb, lcoef, wp[pj], wq[pj], wp[pm], wq[pm]);
-                else
-                    lbm::k_adj_ghost<0><<<cgrid, cb, 0, sm>>>(pa, s0, st_js, st_s, thw, lgpost, lm[0], lms[0], lthw, lsal, lgb, wp[pj], wq[pj]);
+                    e = cudaGetLastError();
+                }
+                if (e == cudaSuccess)
+                    e = launch_pdl(lbm::k_adj_node<0>, grd, blk, sm, pa, s0, st_js, st_nb, lm[1], lm[0], lgpost, lthw, part);
+                if (e == cudaSuccess)
+                    e = j > 0 ? launch_pdl(lbm::k_adj_ghost_front<0>, cgrid, dim3(cb), sm, pa, s0, st_js, st_s, st_s_prev, thw, lgpost, lm[0], lms[0], lms[1], lthw, lsal, lgb, lcoef, wp[pj], wq[pj], wp[pm], wq[pm])
+                              : launch_pdl(lbm::k_adj_ghost<0>, cgrid, dim3(cb), sm, pa, s0, st_js, st_s, thw, lgpost, lm[0], lms[0], lthw, lsal, lgb, wp[pj], wq[pj]);
             } else {
-                if (j == len - 1)
+                if (j == len - 1) {
                     lbm::k_adj_front<1><<<cgrid, cb, 0, sm>>>(pa, s1, st_s, thw, lms[1], lms[0], wp[pj], wq[pj], lm[1], lthw, lcoef);
-                lbm::k_adj_node<1><<<grd, blk, 0, sm>>>(pa, s0, st_js, st_nb, lm[1], lm[0], lgpost, lthw, part);
-                if (j > 0)
-                    lbm::k_adj_ghost_front<1><<<cgrid, cb, 0, sm>>>(pa, s0, st_js, st_s, st_s_prev, thw, lgpost, lm[0], lms[0], lms[1], lthw, lsal, lgb, lcoef, wp[pj], wq[pj], wp[pm], wq[pm]);
-                else
-                    lbm::k_adj_ghost<1><<<cgrid, cb, 0, sm>>>(pa, s0, st_js, st_s, thw, lgpost, lm[0], lms[0], lthw, lsal, lgb, wp[pj], wq[pj]);
+                    e = cudaGetLastError();
+                }
+                if (e == cudaSuccess)
+                    e = launch_pdl(lbm::k_adj_node<1>, grd, blk, sm, pa, s0, st_js, st_nb, lm[1], lm[0], lgpost, lthw, part);
+                if (e == cudaSuccess)
+                    e = j > 0 ? launch_pdl(lbm::k_adj_ghost_front<1>, cgrid, dim3(cb), sm, pa, s0, st_js, st_s, st_s_prev, thw, lgpost, lm[0], lms[0], lms[1], lthw, lsal, lgb, lcoef, wp[pj], wq[pj], wp[pm], wq[pm])
+                              : launch_pdl(lbm::k_adj_ghost<1>, cgrid, dim3(cb), sm, pa, s0, st_js, st_s, thw, lgpost, lm[0], lms[0], lthw, lsal, lgb, wp[pj], wq[pj]);
             }
-            e = cudaGetLastError();
             std::swap(lm[0], lm[1]);
             std::swap(lms[0], lms[1]);
         }
