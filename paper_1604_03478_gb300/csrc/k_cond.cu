@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_even_pair_cond(
     const int *__restrict__ nb, const float *__restrict__ gpost, const float *__restrict__ spost) {
     step_launch_wait();
     int x, y, z;
-    if (k1_pair<FACE>(p, nullptr, x, y, z)) even_pair_cond<ST, FACE, IX>(p, F, G, js, nb, gpost, spost, x, y, z);
+    if (k1_pair<FACE>(p, x, y, z)) even_pair_cond<ST, FACE, IX>(p, F, G, js, nb, gpost, spost, x, y, z);
 }
 
 // Odd step, pair: off the walls of the heating axis and of the other
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair_cond(
     const float *__restrict__ thw_wr, const __grid_constant__ Links lk, const float *__restrict__ spost) {
     step_launch_wait();
     int x, y, z;
-    if (k1_pair<FACE>(p, nullptr, x, y, z))
+    if (k1_pair<FACE>(p, x, y, z))
         odd_pair_cond<ST, FACE, IX>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, spost, x, y, z);
 }
 

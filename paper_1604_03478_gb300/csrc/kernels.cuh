@@ -53,6 +53,16 @@ __device__ __forceinline__ int ld_l2(const int *q) {
     asm volatile("ld.global.cg.s32 %0, [%1];\n" : "=r"(v) : "l"(q));
     return v;
 }
+__device__ __forceinline__ int2 ld_l2(const int2 *q) {
+    int2 v;
+    asm volatile("ld.global.cg.v2.s32 {%0, %1}, [%2];\n" : "=r"(v.x), "=r"(v.y) : "l"(q));
+    return v;
+}
+__device__ __forceinline__ float2 ld_l2(const float2 *q) {
+    float2 v;
+    asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "l"(q));
+    return v;
+}
 __device__ __forceinline__ double ld_l2(const double *q) {
     double v;
     asm volatile("ld.global.cg.f64 %0, [%1];\n" : "=d"(v) : "l"(q));
@@ -204,10 +214,28 @@ __device__ __forceinline__ void snap_column(const SnapOut &o, int col, double s,
     o.nb[col] = nb;
 }
 
+// A pair's (N and the pair's index are even: 8-byte aligned).
+__device__ __forceinline__ void snap_pair(const KP &p, const SnapOut &o, int x, int y, int z, const float2 (&f)[19],
+                                          const float2 (&g)[7]) {
+    float *const at = o.out + (((long long)z * o.ny + y) * p.nx + x);
+#pragma unroll
+    for (int i = 0; i < 19; ++i) *(float2 *)(at + i * o.N) = f[i];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) *(float2 *)(at + (19 + i) * o.N) = g[i];
+}
+__device__ __forceinline__ void snap_pair_columns(const SnapOut &o, int col, const double *s, const int *js,
+                                                  const int *nb) {
+    snap_column(o, col, s[col], js[col], nb[col]);
+    snap_column(o, col + 1, s[col + 1], js[col + 1], nb[col + 1]);
+}
 // The snapshot of a column's first solid node: fh = 0 and its g.
 template <typename ST, int FACE>
 __device__ __forceinline__ void snap_ghost(const KP &p, const ST *G, const float *thw, int x, int y, int z,
                                            bool inflight, const SnapOut &o);
+// The snapshot of a node that is liquid or its column's first solid one.
+template <typename ST, int FACE>
+__device__ __forceinline__ void snap_any(const KP &p, const ST *F, const ST *G, const int *js, const int *js_old,
+                                         const float *thw, int x, int y, int z, bool inflight, const SnapOut &o);
 
 // Stream-collide grid: blocks of blockDim.x x blockDim.y nodes of one plane
 // across the heating axis, with the height along that axis slowest
@@ -761,9 +789,8 @@ template <typename ST> constexpr int pair_min_blocks() {
 }
 
 template <int FACE>
-__device__ __forceinline__ bool k1_pair(const KP &p, const int *jmax, int &x, int &y, int &z) {
-    const int a0 = (int)blockIdx.z * (FACE == 0 ? (int)blockDim.y : 1);
-    if (jmax && a0 >= *jmax + 3) return false;
+__device__ __forceinline__ bool k1_pair(const KP &p, int &x, int &y, int &z) {
+    const int a0 = k1_low<FACE>();
     x = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
     if (FACE == 0) {
         y = a0 + (int)threadIdx.y;
@@ -778,22 +805,41 @@ __device__ __forceinline__ bool k1_pair(const KP &p, const int *jmax, int &x, in
 // The two adjacent populations of a pair (an aligned half2 or float2 word).
 __device__ __forceinline__ float2 ld_pair(const __half *q) { return __half22float2(*(const __half2 *)q); }
 __device__ __forceinline__ float2 ld_pair(const float *q) { return *(const float2 *)q; }
+__device__ __forceinline__ float2 ld_pair_l2(const float *q) { return ld_l2((const float2 *)q); }
+__device__ __forceinline__ float2 ld_pair_l2(const __half *q) {
+    unsigned v;
+    asm volatile("ld.global.cg.u32 %0, [%1];\n" : "=r"(v) : "l"(q));
+    return __half22float2(*(const __half2 *)&v);
+}
 __device__ __forceinline__ void st_pair(__half *q, float2 v) { __stcs((__half2 *)q, __floats2half2_rn(v.x, v.y)); }
 __device__ __forceinline__ void st_pair(float *q, float2 v) { __stcs((float2 *)q, v); }
 
-// The even step of a pair of liquid nodes (both collide, no phase test).
+// The even step of a pair of liquid nodes (both collide, no phase test): its
+// loads (EARLY: ones that may stand before step_launch_wait), then the rest.
+template <typename ST, typename IX, bool EARLY>
+__device__ __forceinline__ void even_pair_load(const KP &p, const ST *F, const ST *G, IX c, float2 (&f)[19],
+                                               float2 (&g)[7]) {
+#pragma unroll
+    for (int i = 0; i < 19; ++i)
+        f[i] = EARLY ? ld_pair_l2(elem<IX>(F, c, i * p.ld)) : ld_pair(elem<IX>(F, c, i * p.ld));
+#pragma unroll
+    for (int i = 0; i < 7; ++i)
+        g[i] = EARLY ? ld_pair_l2(elem<IX>(G, c, i * p.ld)) : ld_pair(elem<IX>(G, c, i * p.ld));
+}
 template <typename ST, typename IX>
-__device__ __forceinline__ void even_pair_liquid(const KP &p, ST *__restrict__ F, ST *__restrict__ G, IX c) {
-    float2 f[19], g[7];
-#pragma unroll
-    for (int i = 0; i < 19; ++i) f[i] = ld_pair(elem<IX>(F, c, i * p.ld));
-#pragma unroll
-    for (int i = 0; i < 7; ++i) g[i] = ld_pair(elem<IX>(G, c, i * p.ld));
+__device__ __forceinline__ void even_pair_finish(const KP &p, ST *__restrict__ F, ST *__restrict__ G, IX c,
+                                                 float2 (&f)[19], float2 (&g)[7]) {
     collide2(p, f, g);
 #pragma unroll
     for (int i = 0; i < 19; ++i) st_pair(elem<IX>(F, c, opp(i) * p.ld), f[i]);
 #pragma unroll
     for (int i = 0; i < 7; ++i) st_pair(elem<IX>(G, c, opp7(i) * p.ld), g[i]);
+}
+template <typename ST, typename IX>
+__device__ __forceinline__ void even_pair_liquid(const KP &p, ST *__restrict__ F, ST *__restrict__ G, IX c) {
+    float2 f[19], g[7];
+    even_pair_load<ST, IX, false>(p, F, G, c, f, g);
+    even_pair_finish<ST, IX>(p, F, G, c, f, g);
 }
 
 template <typename ST, int FACE, typename IX>
@@ -817,7 +863,7 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_even_pair(const 
                                                       const int *jmax) {
     step_launch_wait();
     int x, y, z;
-    if (k1_pair<FACE>(p, jmax, x, y, z)) even_pair<ST, FACE, IX>(p, F, G, js, nb, gpost, x, y, z);
+    if (k1_pair<FACE>(p, x, y, z) && !(jmax && k1_low<FACE>() >= *jmax + 3)) even_pair<ST, FACE, IX>(p, F, G, js, nb, gpost, x, y, z);
 }
 
 // The odd step of a pair on the fast path (both liquid, off the walls of the
@@ -825,31 +871,37 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_even_pair(const 
 // those across an x wall).  Links without an x component move as half2 /
 // float2 words; the others node by node, with the x walls (x0 = 0 for lane
 // x, x0 + 1 = nx - 1 for lane y) taken as in odd_node.
-template <typename ST, int FACE, typename IX>
-__device__ __forceinline__ void odd_pair_liquid(const KP &p, const Links *lk, ST *__restrict__ F,
-                                                ST *__restrict__ G, int x, int y, int z) {
+template <typename ST, int FACE, typename IX, bool EARLY>
+__device__ __forceinline__ void odd_pair_load(const KP &p, const Links *lk, const ST *F, const ST *G, int x, int y,
+                                              int z, float2 (&f)[19], float2 (&g)[7]) {
     const IX c = (IX)node_index(p, x, y, z), c1 = c + 1;
     const bool xlo = x == 0, xhi = x + 1 == p.nx - 1;
-    float2 f[19], g[7];
+    auto one = [](const ST *q) { return EARLY ? ld_l2(q) : Store<ST>::ld(q); };
 #pragma unroll
     for (int i = 0; i < 19; ++i) {
         if (ex(i) == 0) {
-            f[i] = ld_pair(elem<IX>(F, c, lk->fin[i]));
+            f[i] = EARLY ? ld_pair_l2(elem<IX>(F, c, lk->fin[i])) : ld_pair(elem<IX>(F, c, lk->fin[i]));
         } else {
             // across an x wall: bounce-back from the node's own slot i
-            f[i].x = Store<ST>::ld(elem<IX>(F, c, ex(i) > 0 && xlo ? i * p.ld : lk->fin[i]));
-            f[i].y = Store<ST>::ld(elem<IX>(F, c1, ex(i) < 0 && xhi ? i * p.ld : lk->fin[i]));
+            f[i].x = one(elem<IX>(F, c, ex(i) > 0 && xlo ? i * p.ld : lk->fin[i]));
+            f[i].y = one(elem<IX>(F, c1, ex(i) < 0 && xhi ? i * p.ld : lk->fin[i]));
         }
     }
 #pragma unroll
     for (int i = 0; i < 7; ++i) {
         if (tx(i) == 0) {
-            g[i] = ld_pair(elem<IX>(G, c, lk->gin[i]));
+            g[i] = EARLY ? ld_pair_l2(elem<IX>(G, c, lk->gin[i])) : ld_pair(elem<IX>(G, c, lk->gin[i]));
         } else {
-            g[i].x = Store<ST>::ld(elem<IX>(G, c, tx(i) > 0 && xlo ? i * p.ld : lk->gin[i]));
-            g[i].y = Store<ST>::ld(elem<IX>(G, c1, tx(i) < 0 && xhi ? i * p.ld : lk->gin[i]));
+            g[i].x = one(elem<IX>(G, c, tx(i) > 0 && xlo ? i * p.ld : lk->gin[i]));
+            g[i].y = one(elem<IX>(G, c1, tx(i) < 0 && xhi ? i * p.ld : lk->gin[i]));
         }
     }
+}
+template <typename ST, int FACE, typename IX>
+__device__ __forceinline__ void odd_pair_finish(const KP &p, const Links *lk, ST *__restrict__ F, ST *__restrict__ G,
+                                                int x, int y, int z, float2 (&f)[19], float2 (&g)[7]) {
+    const IX c = (IX)node_index(p, x, y, z), c1 = c + 1;
+    const bool xlo = x == 0, xhi = x + 1 == p.nx - 1;
     collide2(p, f, g);
 #pragma unroll
     for (int i = 0; i < 19; ++i) {
@@ -870,6 +922,13 @@ __device__ __forceinline__ void odd_pair_liquid(const KP &p, const Links *lk, ST
             Store<ST>::st_stream(elem<IX>(G, c1, tx(i) > 0 && xhi ? opp7(i) * p.ld : lk->gout[i]), g[i].y);
         }
     }
+}
+template <typename ST, int FACE, typename IX>
+__device__ __forceinline__ void odd_pair_liquid(const KP &p, const Links *lk, ST *__restrict__ F, ST *__restrict__ G,
+                                                int x, int y, int z) {
+    float2 f[19], g[7];
+    odd_pair_load<ST, FACE, IX, false>(p, lk, F, G, x, y, z, f, g);
+    odd_pair_finish<ST, FACE, IX>(p, lk, F, G, x, y, z, f, g);
 }
 
 // The odd step for a pair: both nodes on the one-node fast path (liquid, off
@@ -912,7 +971,114 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair(const _
                                                      const __grid_constant__ Links lk, const int *jmax) {
     step_launch_wait();
     int x, y, z;
-    if (k1_pair<FACE>(p, jmax, x, y, z)) odd_pair<ST, FACE, IX>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x, y, z);
+    if (k1_pair<FACE>(p, x, y, z) && !(jmax && k1_low<FACE>() >= *jmax + 3)) odd_pair<ST, FACE, IX>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x, y, z);
+}
+
+
+// The pair kernels of the middle sizes (FP32 storage, up to 160^3 nodes): the
+// first wave's pairs load before step_launch_wait, like the one-node kernels
+// (k_even, k_odd): the even step's pairs that were liquid before the front
+// update, the odd step's that are interior whatever it does.  128^3 with a
+// thin layer 15.5 -> 14.4 us a step (16.5 with one node per thread), at 0.45 H
+// 39.8 -> 37.6 (40.4).  Larger grids take the plain kernels: a first wave is
+// little of them (256^3 FP32 the same), and with FP16 storage the second set
+// of loads cost more than it hid (156.5 -> 161.7 us).
+// SNAP: see k_even; a pair that is split takes its snapshot by gathers, from
+// the slots that its nodes own in this step.
+template <typename ST, int FACE, typename IX, bool SNAP>
+__global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_even_pair_early(const __grid_constant__ KP p, ST *__restrict__ F,
+                                                      ST *__restrict__ G, const int *js, const int *js_old,
+                                                      const int *__restrict__ nb, const float *__restrict__ gpost,
+                                                      const int *jmax, int early_blocks, const double *s,
+                                                      const __grid_constant__ SnapOut snap) {
+    int x = 0, y = 0, z = 0;
+    const bool on = k1_pair<FACE>(p, x, y, z), late = k1_late(early_blocks);
+    if (late) step_launch_wait();
+    const IX c = on ? (IX)node_index(p, x, y, z) : 0;
+    const int a = axial<FACE>(x, y, z);
+    const int col = on ? column<FACE>(p, x, y, z) : 0;  // x + 1 is in column col + 1
+    float2 f[19], g[7];
+    bool low = true, loaded = false;
+    if (late) {
+        low = !jmax || k1_low<FACE>() < *jmax + 3;
+    } else {
+        const int jm = jmax ? ld_l2(jmax) : 1 << 29;
+        const int2 jo = ld_l2((const int2 *)(js_old + col));
+        low = k1_low<FACE>() < jm + 3;
+        loaded = on && low && a < jo.x && a < jo.y;
+        if (loaded) even_pair_load<ST, IX, true>(p, F, G, c, f, g);
+        step_launch_wait();
+    }
+    if (!on || !low) return;
+    if (SNAP && a == 0) snap_pair_columns(snap, col, s, js, nb);
+    if (!(a < __ldg(js + col) && a < __ldg(js + col + 1))) {
+        if (SNAP) {
+            snap_any<ST, FACE>(p, F, G, js, js_old, nullptr, x, y, z, false, snap);
+            snap_any<ST, FACE>(p, F, G, js, js_old, nullptr, x + 1, y, z, false, snap);
+        }
+        even_node<ST, FACE, IX>(p, F, G, js, nb, gpost, x, y, z);
+        even_node<ST, FACE, IX>(p, F, G, js, nb, gpost, x + 1, y, z);
+        return;
+    }
+    if (!loaded) even_pair_load<ST, IX, false>(p, F, G, c, f, g);
+    if (SNAP) snap_pair(p, snap, x, y, z, f, g);
+    even_pair_finish<ST, IX>(p, F, G, c, f, g);
+}
+
+template <typename ST, int FACE, typename IX, bool SNAP>
+__global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair_early(const __grid_constant__ KP p, ST *__restrict__ F,
+                                                     ST *__restrict__ G, const int *js, const int *js_old,
+                                                     const int *nb, const int *nb_old,
+                                                     const float *__restrict__ gpost,
+                                                     const float *__restrict__ thw_rd,
+                                                     const float *__restrict__ thw_wr,
+                                                     const __grid_constant__ Links lk, const int *jmax,
+                                                     int early_blocks, const double *s,
+                                                     const __grid_constant__ SnapOut snap) {
+    int x = 0, y = 0, z = 0;
+    const bool on = k1_pair<FACE>(p, x, y, z), late = k1_late(early_blocks);
+    if (late) step_launch_wait();
+    const int a = axial<FACE>(x, y, z);
+    const int col = on ? column<FACE>(p, x, y, z) : 0;
+    const int q = FACE == 0 ? z : y, nq = FACE == 0 ? p.nz : p.ny;
+    const bool off_qa = q >= 1 && q <= nq - 2 && a >= 1 && a <= p.H - 2;
+    float2 f[19], g[7];
+    bool low = true, loaded = false;
+    if (late) {
+        low = !jmax || k1_low<FACE>() < *jmax + 3;
+    } else {
+        const int jm = jmax ? ld_l2(jmax) : 1 << 29;
+        const int2 bo = ld_l2((const int2 *)(nb_old + col));
+        low = k1_low<FACE>() < jm + 3;
+        // interior under the counts before the front update less one, so under the new ones
+        loaded = on && low && off_qa && a + 2 < (bo.x >> 16) && a + 2 < (bo.y >> 16);
+        if (loaded) odd_pair_load<ST, FACE, IX, true>(p, &lk, F, G, x, y, z, f, g);
+        step_launch_wait();
+    }
+    if (!on || !low) return;
+    if (SNAP && a == 0) snap_pair_columns(snap, col, s, js, nb);
+    if (!loaded) {
+        const int b0 = __ldg(nb + col) >> 16, b1 = __ldg(nb + col + 1) >> 16;
+        if (!(off_qa && a + 1 < b0 && a + 1 < b1)) {
+            int c12[12], js9[9], mn, mx;
+            load_js12(p, js, x, q, c12);
+            range_js12(p, c12, x, q, mn, mx);
+            if (!(off_qa && a + 1 < mn)) {  // the bounds may be two low
+                if (SNAP) {
+                    snap_any<ST, FACE>(p, F, G, js, js_old, thw_rd, x, y, z, true, snap);
+                    snap_any<ST, FACE>(p, F, G, js, js_old, thw_rd, x + 1, y, z, true, snap);
+                }
+                js9_of_js12(c12, 0, js9);
+                odd_node<ST, FACE>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x, y, z, nullptr, js9);
+                js9_of_js12(c12, 1, js9);
+                odd_node<ST, FACE>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x + 1, y, z, nullptr, js9);
+                return;
+            }
+        }
+        odd_pair_load<ST, FACE, IX, false>(p, &lk, F, G, x, y, z, f, g);
+    }
+    if (SNAP) snap_pair(p, snap, x, y, z, f, g);
+    odd_pair_finish<ST, FACE, IX>(p, &lk, F, G, x, y, z, f, g);
 }
 
 
@@ -989,6 +1155,21 @@ __device__ __forceinline__ void gather_f_now(const KP &p, const ST *F, const int
         return;
     }
     gather_f<ST, FACE>(p, F, js, x, y, z, inflight, f);
+}
+
+template <typename ST, int FACE>
+__device__ __forceinline__ void snap_any(const KP &p, const ST *F, const ST *G, const int *js, const int *js_old,
+                                         const float *thw, int x, int y, int z, bool inflight, const SnapOut &o) {
+    const int a = axial<FACE>(x, y, z), jsc = js[column<FACE>(p, x, y, z)];
+    if (a > jsc) return;
+    if (a == jsc) {
+        snap_ghost<ST, FACE>(p, G, thw, x, y, z, inflight, o);
+        return;
+    }
+    float f[19], g[7];
+    gather_g<ST, FACE>(p, G, x, y, z, inflight, thw, g);
+    gather_f_now<ST, FACE>(p, F, js, js_old, x, y, z, inflight, f);
+    snap_node(p, o, x, y, z, f, g);
 }
 
 // gather_f in flight for the node at height a of the middle column, with

@@ -29,6 +29,7 @@ struct Bufs {
     double nu_scale;             // H / (alpha (Th - Tm))
     float *spost;                // solid-side ghost populations, 7 x ncols (heat conduction in the solid)
     int pairs;                   // stream-collide with two nodes per thread (even nx)
+    int early_pairs;             // ... with the first wave's loads before the wait (FP32 storage, middle sizes)
 };
 
 // Where a step leaves the natural-layout snapshot of the state it starts from

@@ -170,12 +170,24 @@ lbm_status cuda_err(lbm_melt *h, cudaError_t e, const char *where) {
 // Two nodes per thread in the stream-collide (an even nx): chosen for
 // cavities above 160^3, whose grids are large enough to keep the GPU busy
 // with half the threads (256^3: 0.2245 against 0.234 ms per launch in FP32,
-// 0.145 against 0.19 ms in FP16); smaller cavities with a thin liquid layer
-// are latency bound and run faster with one node per thread (96^3 adjoint
-// forward 54 against 61 ms, 128^3 convection 33 against 35 us per step).
+// 0.145 against 0.19 ms in FP16), and with FP32 storage from kPairNodes on,
+// where the early pair kernels run (us per step, two nodes against one,
+// front at 0.1, 0.25, 0.45 and 0.8 H: 112^3 12.8 / 13.5, 18.1 / 19.7, 26.5 /
+// 27.4, 47.9 / 48.9; 128^3 14.4 / 16.5, 22.3 / 23.9, 37.6 / 40.4, 65.6 / 66.3;
+// 160^3 22.0 / 24.8, 45.5 / 47.4, 73.8 / 76.3, 121.7 / 123.2), unless more
+// than a fifth of a block's lanes would idle over a row of nx / 2 (96^3, 48 of
+// 64: 12.6 / 11.3, 29.8 / 26.2).  Smaller cavities are latency bound and run
+// faster with one node per thread (48^3 8.0 / 6.4).  FP16 storage keeps one
+// below 160^3: the pairs' rounding moves stored values by an FP16 step.
+const long long kPairNodes = 110LL * 110 * 110;
 bool use_pairs(const lbm_melt *h) {
     if (h->kp.nx % 2 != 0) return false;
-    return h->pairs_mode < 0 ? h->d.N > kGraphMaxNodes : h->pairs_mode == 1;
+    if (h->pairs_mode >= 0) return h->pairs_mode == 1;
+    if (h->d.N > kGraphMaxNodes) return true;
+    if (h->precision != 0 || h->kp.cond || h->d.N < kPairNodes) return false;
+    const int half = h->kp.nx / 2, bx = lbm::block_width(half, 128);
+    const int lanes = (half + bx - 1) / bx * bx;
+    return 5 * (lanes - half) <= lanes;
 }
 
 // Buffers of a step from phase (cur, inflight) with the handle's wall fields.
@@ -206,6 +218,7 @@ Bufs bufs_at(lbm_melt *h, int cur, int inflight) {
     b.nu_scale = (double)h->kp.H / (h->d.alpha * (h->Th - h->Tm));
     b.spost = h->spost;
     b.pairs = use_pairs(h) ? 1 : 0;
+    b.early_pairs = h->d.N <= kGraphMaxNodes ? 1 : 0;
     return b;
 }
 

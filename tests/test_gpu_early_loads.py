@@ -39,3 +39,44 @@ def test_early_and_late_blocks(face, shape, s0):
     np.testing.assert_allclose(ga, gb, atol=1e-6, rtol=0)
     a.close()
     b.close()
+
+
+def _gradient(shape, kw, pairs, steps, spread):
+    from paper_1604_03478_gb300 import build, Cavity
+    build.build()
+    c = Cavity(*shape, **kw)
+    c.set_node_pairs(pairs)
+    if spread:
+        f, g, s = c.get_state()
+        c.set_state(f, g, s + inputs.gaussian_field(c.ncols, spread, 13))
+    c.set_hot_wall((1.0 + inputs.gaussian_field(c.ncols, 0.05, 11)).astype(np.float32))
+    S0 = c.get(T=False, u=False, lf=False)[2]
+    c.tape_forward(steps, 9)
+    S = c.get(T=False, u=False, lf=False)[2]
+    dth, par = c.tape_backward(inputs.gaussian_field(c.ncols, 1.0, 12))
+    c.close()
+    return S0, S, dth, par
+
+
+@pytest.mark.parametrize("face", [0, 1])
+@pytest.mark.parametrize("nx,steps", [(34, 40), (64, 37)])
+@pytest.mark.parametrize("spread", [0.0, 0.5])
+def test_gradient_with_node_pairs(face, nx, steps, spread):
+    """The adjoint's snapshots written by the pair kernels (pairs, pairs split
+    by an uneven front, first solid nodes) against those of the one-node
+    kernels.  The two forwards differ by FP32 rounding, 1e-6 of T over 40
+    steps by the bound above; the gradient is linear in such differences (the
+    runs flip the same nodes, as the equal counts say): 1e-4 of its largest
+    entry."""
+    import torch
+    assert torch.cuda.is_available()
+    shape = (nx, 20, 14) if face == 0 else (nx, 14, 20)
+    kw = dict(face=face, Ra=5e4, Pr=0.3, Ste=0.8, Ma=0.15, s0=3.3, derive=True)
+    S0, Sa, da, pa = _gradient(shape, kw, 0, steps, spread)
+    _, Sb, db, pb = _gradient(shape, kw, 1, steps, spread)
+    np.testing.assert_array_equal(np.ceil(Sa - 0.5), np.ceil(Sb - 0.5))
+    if spread:
+        assert (np.ceil(Sa - 0.5) != np.ceil(S0 - 0.5)).any()  # nodes flipped
+    assert np.abs(da - db).max() <= 1e-4 * np.abs(da).max()
+    for k in pa:
+        assert abs(pa[k] - pb[k]) <= 1e-4 * max(abs(pa[k]), 1e-12)
