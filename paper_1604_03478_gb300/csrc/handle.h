@@ -63,6 +63,8 @@ struct lbm_melt {
     int *jmax_dev;
     int *rb_val;       // pinned: ring of read-backs, then kFlags ints a synchronising call reads status_dev into
     static const int kFlags = 2;
+    static const int kHostOut = 8;
+    double *host_out;  // pinned (behind rb_val): small results of the synchronising calls, written by the kernels
     cudaEvent_t rb_ev[kRbRing];
     long long rb_step[kRbRing];  // exec step after which each copy was taken
     long long rb_next;           // read-backs enqueued so far

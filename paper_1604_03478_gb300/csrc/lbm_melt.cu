@@ -237,6 +237,31 @@ lbm_status refresh_front(lbm_melt *h) {
     return LBM_OK;
 }
 
+// The address by which a kernel reaches p, a device pointer (ptr_kind 1) or
+// page-locked host memory, aligned to `align` bytes; null for other host
+// memory.  A copy between two kernels costs the stream several microseconds
+// however small it is; GB300 reads and writes page-locked memory from a
+// kernel at link speed.
+template <typename T> T *kernel_view(T *p, int ptr_kind, size_t align) {
+    if (!p || (size_t)p % align) return nullptr;
+    if (ptr_kind) return p;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    return a.type == cudaMemoryTypeHost ? (T *)a.devicePointer : nullptr;
+}
+
+// A new heated-wall field, the old one kept in prev where that is not null.
+__global__ void k_set_wall(const float *__restrict__ src, float *cur, float *prev, long long n) {
+    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const float v = src[i];
+    if (prev) prev[i] = cur[i];
+    cur[i] = v;
+}
+
 lbm_status copy_in(lbm_melt *h, void *dst, const void *src, size_t bytes, int ptr_kind) {
     CK(cudaMemcpyAsync(dst, src, bytes, ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream),
        "copy in");
@@ -655,7 +680,10 @@ LBM_API lbm_status lbm_melt_create(const lbm_melt_grid *grid, double Ra, double 
     // small cavities are launch bound: replay their steps from graphs
     h->graph_steps = d.N <= kGraphMaxNodes ? kGraphSteps : 0;
     h->pairs_mode = -1;
-    if (cudaMallocHost(&h->rb_val, (lbm_melt::kRbRing + lbm_melt::kFlags) * sizeof(int)) != cudaSuccess) return fail(LBM_ENOMEM);
+    const size_t rb_bytes = ((lbm_melt::kRbRing + lbm_melt::kFlags) * sizeof(int) + 127) / 128 * 128;
+    if (cudaMallocHost(&h->rb_val, rb_bytes + lbm_melt::kHostOut * sizeof(double)) != cudaSuccess)
+        return fail(LBM_ENOMEM);
+    h->host_out = (double *)((unsigned char *)h->rb_val + rb_bytes);
     for (int k = 0; k < lbm_melt::kRbRing; ++k)
         if (cudaEventCreateWithFlags(&h->rb_ev[k], cudaEventDisableTiming) != cudaSuccess) return fail(LBM_ECUDA);
     const size_t es = h->precision == 1 ? sizeof(__half) : sizeof(float);
@@ -757,11 +785,14 @@ LBM_API lbm_status lbm_melt_step(lbm_melt *h, long long n) {
 LBM_API lbm_status lbm_melt_totals(lbm_melt *h, double *out, int ptr_kind) {
     if (!h || !out) return LBM_EINVAL;
     Bufs b = bufs(h);
-    CK(LAUNCH(h, totals, h->kp, h->face, h->inflight, b, h->red_part, h->nred, -1.0, h->totals_dev, h->stream),
-       "totals");
-    CK(cudaMemcpyAsync(out, h->totals_dev, 7 * 8, ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                       h->stream), "copy totals");
-    return check_status(h);
+    double *const view = ptr_kind ? kernel_view(out, 1, sizeof(double)) : h->host_out;
+    CK(LAUNCH(h, totals, h->kp, h->face, h->inflight, b, h->red_part, h->nred, -1.0, view ? view : h->totals_dev,
+              h->stream), "totals");
+    if (!view) CK(cudaMemcpyAsync(out, h->totals_dev, 7 * 8, cudaMemcpyDeviceToDevice, h->stream), "copy totals");
+    const lbm_status st = read_flags(h);
+    if (st != LBM_OK) return st;
+    if (!ptr_kind) std::memcpy(out, h->host_out, 7 * 8);
+    return status_of_flags(h);
 }
 
 LBM_API lbm_status lbm_melt_set_report(lbm_melt *h, long long every, long long capacity) {
@@ -801,17 +832,16 @@ LBM_API lbm_status lbm_melt_get_report(lbm_melt *h, double *rows, long long max_
 
 // scale * (sum of the ncols column values v), into dst on the handle's
 // stream: one launch of k_sum_once (chunks of at least 1024 columns per
-// block, fixed order), which writes a device destination itself (one aligned
-// to a double; else, and to the host, a copy).  copy (may be null): an aligned
-// device array that receives the values in the same launch.
+// block, fixed order), which writes a destination that kernels reach itself
+// (else a copy).  copy (may be null): receives the values in the same launch.
 lbm_status enqueue_column_sum(lbm_melt *h, const double *v, double scale, double *dst, int ptr_kind,
                               double *copy = nullptr) {
     const long long nc = h->kp.ncols;
     const long long nb = std::max<long long>(1, std::min<long long>(kRedBlocks, (nc + 1023) / 1024));
     const long long chunk = (nc + nb - 1) / nb;
-    const bool direct = ptr_kind && (size_t)dst % sizeof(double) == 0;
-    k_sum_once<<<(int)nb, 256, 0, h->stream>>>(v, nc, chunk, scale, h->red_part, h->ticket, direct ? dst : h->sum_dev,
-                                               copy);
+    double *const direct = kernel_view(dst, ptr_kind, sizeof(double));
+    k_sum_once<<<(int)nb, 256, 0, h->stream>>>(v, nc, chunk, scale, h->red_part, h->ticket,
+                                               direct ? direct : h->sum_dev, copy);
     CK(cudaGetLastError(), "sum");
     if (!direct)
         CK(cudaMemcpyAsync(dst, h->sum_dev, 8, ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream),
@@ -823,13 +853,23 @@ lbm_status enqueue_column_sum(lbm_melt *h, const double *v, double scale, double
 // may be null), enqueued on the handle's stream.
 lbm_status enqueue_front_out(lbm_melt *h, double *S, double *liquid_fraction, int ptr_kind) {
     const double scale = 1.0 / ((double)h->kp.H * (double)h->kp.ncols);
-    if (S && liquid_fraction && ptr_kind && (size_t)S % sizeof(double) == 0)
-        return enqueue_column_sum(h, h->s[h->cur], scale, liquid_fraction, ptr_kind, S);
-    if (S)
+    double *const view = liquid_fraction ? kernel_view(S, ptr_kind, sizeof(double)) : nullptr;
+    if (S && !view)
         CK(cudaMemcpyAsync(S, h->s[h->cur], (size_t)h->kp.ncols * 8,
                            ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream), "copy S");
-    if (liquid_fraction) return enqueue_column_sum(h, h->s[h->cur], scale, liquid_fraction, ptr_kind);
+    if (liquid_fraction) return enqueue_column_sum(h, h->s[h->cur], scale, liquid_fraction, ptr_kind, view);
     return LBM_OK;
+}
+
+// The same for a call that synchronises: a liquid fraction for the host goes
+// through the handle's page-locked memory.  Then the status.
+lbm_status front_out_sync(lbm_melt *h, double *S, double *liquid_fraction, int ptr_kind) {
+    double *const lf = liquid_fraction && !ptr_kind ? h->host_out : liquid_fraction;
+    lbm_status st = enqueue_front_out(h, S, lf, ptr_kind);
+    if (st == LBM_OK) st = read_flags(h);
+    if (st != LBM_OK) return st;
+    if (lf != liquid_fraction) *liquid_fraction = *lf;
+    return status_of_flags(h);
 }
 
 LBM_API lbm_status lbm_melt_sync(lbm_melt *h) {
@@ -855,8 +895,7 @@ LBM_API lbm_status lbm_melt_get(lbm_melt *h, float *T, float *u, double *S, doub
             if (u) CK(cudaMemcpyAsync(u, ud, 3 * N * 4, cudaMemcpyDeviceToHost, h->stream), "copy u");
         }
     }
-    lbm_status st = enqueue_front_out(h, S, liquid_fraction, ptr_kind);
-    if (st == LBM_OK) st = check_status(h);
+    const lbm_status st = front_out_sync(h, S, liquid_fraction, ptr_kind);
     if (!ptr_kind) { cudaFree(Td); cudaFree(ud); }
     return st;
 }
@@ -947,19 +986,23 @@ LBM_API lbm_status lbm_melt_set_state(lbm_melt *h, const float *f, const float *
 LBM_API lbm_status lbm_melt_set_hot_wall(lbm_melt *h, const float *T_h_field, int ptr_kind) {
     if (!h || !T_h_field) return LBM_EINVAL;
     const size_t nc = (size_t)h->kp.ncols;
-    if (h->inflight && !h->thw_pending) {
-        // the pending odd step must still read the walls with the field of
-        // the step that produced the in-flight values
+    // In flight, the pending odd step must still read the walls with the
+    // field of the step that produced the in-flight values; in the natural
+    // layout, the field of the last streaming is kept for the Nusselt number
+    // until the next step (an even one, which reads no wall).
+    const bool keep = h->inflight ? !h->thw_pending : !h->thw_last_prev;
+    const float *const src = kernel_view(T_h_field, ptr_kind, sizeof(float));
+    if (src) {
+        k_set_wall<<<(int)((nc + 255) / 256), 256, 0, h->stream>>>(src, h->thw_cur, keep ? h->thw_prev : nullptr,
+                                                                   (long long)nc);
+        CK(cudaGetLastError(), "set wall");
+    } else if (keep) {
         CK(cudaMemcpyAsync(h->thw_prev, h->thw_cur, nc * 4, cudaMemcpyDeviceToDevice, h->stream), "copy wall");
-        h->thw_pending = 1;
-    } else if (!h->inflight && !h->thw_last_prev) {
-        // keep the field of the last streaming for the Nusselt number until
-        // the next step (the next step, an even one, reads no wall)
-        CK(cudaMemcpyAsync(h->thw_prev, h->thw_cur, nc * 4, cudaMemcpyDeviceToDevice, h->stream), "copy wall");
-        h->thw_last_prev = 1;
     }
+    if (h->inflight) h->thw_pending = 1;
+    else h->thw_last_prev = 1;
     h->thw_gen++;
-    return copy_in(h, h->thw_cur, T_h_field, nc * 4, ptr_kind);
+    return src ? LBM_OK : copy_in(h, h->thw_cur, T_h_field, nc * 4, ptr_kind);
 }
 
 LBM_API lbm_status lbm_melt_get_nusselt(lbm_melt *h, double *Nu, double *Nu_mean, int ptr_kind) {
@@ -971,11 +1014,15 @@ LBM_API lbm_status lbm_melt_get_nusselt(lbm_melt *h, double *Nu, double *Nu_mean
             CK(cudaMemcpyAsync(Nu, h->nu_dev, (size_t)h->kp.ncols * 8,
                                ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream), "copy Nu");
         if (Nu_mean) {
-            const lbm_status st = enqueue_column_sum(h, h->nu_dev, 1.0 / (double)h->kp.ncols, Nu_mean, ptr_kind);
+            const lbm_status st = enqueue_column_sum(h, h->nu_dev, 1.0 / (double)h->kp.ncols,
+                                                     ptr_kind ? Nu_mean : h->host_out, ptr_kind);
             if (st != LBM_OK) return st;
         }
     }
-    return check_status(h);
+    const lbm_status st = read_flags(h);
+    if (st != LBM_OK) return st;
+    if (Nu_mean && !ptr_kind) *Nu_mean = *h->host_out;
+    return status_of_flags(h);
 }
 
 LBM_API lbm_status lbm_melt_get_info(lbm_melt *h, lbm_melt_info *info) {
@@ -1152,6 +1199,5 @@ LBM_API lbm_status lbm_melt_get_noalloc(lbm_melt *h, float *T, float *u, double 
     }
     // the handle's own reduction buffers, allocated at create: the same sum
     // as lbm_melt_get
-    const lbm_status st = enqueue_front_out(h, S, liquid_fraction, ptr_kind);
-    return st == LBM_OK ? check_status(h) : st;
+    return front_out_sync(h, S, liquid_fraction, ptr_kind);
 }
