@@ -336,10 +336,12 @@ lbm_status lbm_melt_tape_clear(lbm_melt *h);
    A batch of independent cavities of uneven sizes and parameters advanced in
    lockstep by one persistent kernel launch per run of steps: each step covers
    the nodes of all cavities (fused stream-collide), then all their columns
-   (front update, Eq. 6), then the phase flips, separated by grid-wide
+   (front update, Eq. 6, then the phase flips), separated by grid-wide
    barriers whose waits are bounded (an exhausted wait ends the launch;
-   lbm_ensemble_sync then returns LBM_ETIMEOUT).  The launch is captured once
-   in a CUDA graph (graph_steps steps per replay) and replayed. */
+   lbm_ensemble_sync then returns LBM_ETIMEOUT).  A run of fewer than about 64
+   steps is one launch; a longer one replays a launch of the largest multiple
+   of graph_steps up to 64 (or of graph_steps, where that is more) steps,
+   captured once in a CUDA graph. */
 typedef struct lbm_ensemble lbm_ensemble;
 
 /* One member cavity: the arguments of lbm_melt_create. */
@@ -361,8 +363,10 @@ lbm_status lbm_ensemble_step(lbm_ensemble *e, long long nsteps);
 
 /* Launch shape: threads per block (64, 128 or 256; a block covers an x-y
    tile of one cavity), nodes per thread in the stream-collide phase (1, 2,
-   4 or 8 consecutive z-planes) and steps per graph replay (even, >= 2).  The grid
-   is the co-resident maximum for that shape. */
+   4 or 8 consecutive z-planes) and the unit of the steps per graph replay
+   (even, >= 2).  The grid is the co-resident maximum for that shape.  Until it
+   is called: 256 threads and one node for an ensemble that fits two such
+   items a block, else 128 and two, and 8 steps. */
 lbm_status lbm_ensemble_set_launch(lbm_ensemble *e, int block, int nodes_per_thread, int graph_steps);
 
 /* Bound of a barrier wait, in polls (default 2^24, about a second). */
@@ -375,10 +379,10 @@ lbm_status lbm_ensemble_set_barrier_timeout(lbm_ensemble *e, long long max_spins
 lbm_status lbm_ensemble_inject_barrier_fault(lbm_ensemble *e, int block);
 
 /* Phase timers of the persistent kernel: block 0 reads the GPU's global
-   timer each time it leaves a grid barrier, so a step splits into the fused
-   stream-collide of every cavity (phase 1), the front update of every column
-   (Eq. 6, phase 2) and the phase flip (phase 3), each with the barrier that
-   ends it.  us_per_step (3 doubles, may be NULL): the mean microseconds per
+   timer each time it leaves a grid barrier and between its front updates and
+   its flips, so a step splits into the fused stream-collide of every cavity
+   (phase 1, with its barrier), the front update of every column (Eq. 6, phase
+   2) and the phase flip (phase 3, with the barrier that ends both).  us_per_step (3 doubles, may be NULL): the mean microseconds per
    step of each phase since the ensemble was created or last reset; steps
    (may be NULL): the steps timed.  reset != 0 zeroes the timers after the
    read.  Synchronizes the ensemble's stream (call it between steps, not

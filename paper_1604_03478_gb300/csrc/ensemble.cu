@@ -5,13 +5,13 @@
 // The launch walks a work list: per step, phase 1 covers every node of every
 // cavity in items of (block size x nodes per thread) nodes, handed out one
 // by one from an atomic counter (fused stream-collide, Eqs. 1-5), phase 2
-// every column of every cavity in
-// items of one block (front update, Eq. 6), phase 3 the same columns (phase
-// flip).  Phases are separated by a grid-wide barrier; the launch is
-// cooperative (all blocks resident) and every barrier wait is bounded: a
-// block that waits too long raises an error flag and the whole launch
-// returns, which the host reports as LBM_ETIMEOUT.  The launch (with the
-// barrier reset) is captured once in a CUDA graph and replayed.
+// every column of every cavity in items of one block (front update, Eq. 6),
+// phase 3 the same columns (phase flip, by the threads of phase 2).  A
+// grid-wide barrier ends phases 1 and 3; the launch is cooperative (all
+// blocks resident) and every barrier wait is bounded: a block that waits too
+// long raises an error flag and the whole launch returns, which the host
+// reports as LBM_ETIMEOUT.  Long runs replay the launch (with the barrier
+// reset) from a CUDA graph captured once.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -113,6 +113,15 @@ void fill_desc(lbm_melt *h, CavDesc &d, int block) {
     d.status = h->status_dev;
     d.jmax = h->jmax_dev;
     d.cut = h->kp.skip_deep;
+}
+
+// Steps of one launch (and of one graph replay): a multiple of graph_steps of
+// about 64.  A launch costs the stream some 20 us besides its steps (8 steps
+// a launch: 31.8 us a step for eight cavities of 20 to 47 nodes an edge, 64:
+// 30.6).
+long long launch_steps(const lbm_ensemble *e) {
+    const long long G = e->graph_steps;
+    return G >= 64 ? G : 64 / G * G;
 }
 
 // Work-list prefix sums and the co-resident grid for the launch shape.
@@ -248,8 +257,21 @@ LBM_API lbm_status lbm_ensemble_create(int n, const lbm_melt_case *cases, void *
     if (cudaMalloc(&e->bar_dev, 16 * sizeof(unsigned int)) != cudaSuccess ||
         cudaMemset(e->bar_dev, 0, 16 * sizeof(unsigned int)) != cudaSuccess)
         return fail(LBM_ENOMEM);
+    // A small ensemble, whose nodes are at most two items of 256 a resident
+    // block, takes 256 threads and one plane an item: each item's latency
+    // counts there (eight cavities of 20 to 47 nodes an edge: 27.0 us a step
+    // against 31.8 with 128 and two planes); a larger one the other shape
+    // (20 cavities of 48 to 128: 326 against 368).
+    e->block = 256;
+    e->K = 1;
     refresh_desc(e);
     if (plan(e) != LBM_OK) return fail(LBM_ECUDA);
+    if (e->items[n] > 2LL * e->grid) {
+        e->block = 128;
+        e->K = 2;
+        refresh_desc(e);
+        if (plan(e) != LBM_OK) return fail(LBM_ECUDA);
+    }
     if (cudaStreamSynchronize(e->stream) != cudaSuccess) return fail(LBM_ECUDA);
     *out = e;
     return LBM_OK;
@@ -304,7 +326,7 @@ LBM_API lbm_status lbm_ensemble_step(lbm_ensemble *e, long long nsteps) {
     ECK(cudaStreamWaitEvent(e->stream, e->ev_in, 0), "wait");
     if (!desc_current(e)) refresh_desc(e);
     long long left = nsteps;
-    const long long G = e->graph_steps;
+    const long long G = launch_steps(e);
     if (left >= G) {
         if (!e->graph) {
             cudaGraph_t g;

@@ -60,23 +60,25 @@ struct EnsWork {
     long long item_begin[kMaxCavities + 1];  // prefix sums of node items
     long long col_begin[kMaxCavities + 1];   // prefix sums of column items
     CavDesc desc[kMaxCavities];
-    unsigned int *bar;            // {arrived, generation, timed out, -, item counters (2 x u64),
+    unsigned int *bar;            // {arrivals, -, timed out, -, item counters (2 x u64),
                                   //  phase times in ns and steps (4 x u64)}
     long long max_spins;
     int skip_arrival_block;       // fault injection for tests: this block never arrives (-1: none)
 };
 
 // Grid-wide barrier with a bounded wait.  Returns false once any block has
-// given up (then every block leaves the launch).
-__device__ __forceinline__ bool grid_barrier(const EnsWork &w, unsigned int nblocks) {
+// given up (then every block leaves the launch).  Arrivals are counted on
+// across the barriers of a launch, and a block waits for the count of the
+// barrier's last arrival: an arrival needs no answer and the last one no
+// second flag (with a count reset and a generation a barrier took the last
+// block two more round trips to memory).
+__device__ __forceinline__ bool grid_barrier(const EnsWork &w, unsigned int target) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         ok = 1;
         volatile unsigned int *vb = w.bar;
-        if (vb[2]) {
-            ok = 0;
-        } else if ((int)blockIdx.x == w.skip_arrival_block) {
+        if ((int)blockIdx.x == w.skip_arrival_block) {
             // injected fault: this block does not arrive; it waits like the
             // others so that every block leaves through the timeout
             long long spins = 0;
@@ -84,24 +86,18 @@ __device__ __forceinline__ bool grid_barrier(const EnsWork &w, unsigned int nblo
             atomicExch(w.bar + 2, 1u);
             ok = 0;
         } else {
-            const unsigned int gen = vb[1];
             __threadfence();
-            const unsigned int arrived = atomicAdd(w.bar, 1u) + 1u;
-            if (arrived == nblocks) {
-                atomicExch(w.bar, 0u);
-                __threadfence();
-                atomicAdd(w.bar + 1, 1u);
-            } else {
-                long long spins = 0;
-                while (vb[1] == gen) {
-                    if (vb[2] || ++spins > w.max_spins) {
-                        atomicExch(w.bar + 2, 1u);
-                        ok = 0;
-                        break;
-                    }
-                    __nanosleep(64);
+            atomicAdd(w.bar, 1u);
+            long long spins = 0;
+            while ((int)(vb[0] - target) < 0) {
+                if (vb[2] || ++spins > w.max_spins) {
+                    atomicExch(w.bar + 2, 1u);
+                    ok = 0;
+                    break;
                 }
+                __nanosleep(32);
             }
+            if (vb[2]) ok = 0;
             __threadfence();
         }
     }
@@ -167,14 +163,15 @@ template <typename ST, int K>
 __global__ void ENS_BOUNDS k_ensemble(const __grid_constant__ EnsWork w, int nsteps) {
     const long long items1 = w.item_begin[w.ncav], items2 = w.col_begin[w.ncav];
     __shared__ int top[kMaxCavities];  // per cavity: first height at which every node is deep solid
-    __shared__ long long next;         // first item of the block's next chunk
+    __shared__ long long next;         // the block's next item
     // per-step item counters (alternating), zeroed with the barrier words
     unsigned long long *ctr = reinterpret_cast<unsigned long long *>(w.bar + 4);
-    constexpr int kChunk = 1;  // measured: 1, 2, 4 items -> 19.3, 18.7, 18.5 k MLUPS
+    unsigned int arrivals = 0;         // of the barriers so far
     int kc = 0;  // cavity of the block's last item (items are handed out in increasing order)
-    // Block 0 times the phases on the global timer: each phase ends when
-    // block 0 leaves the grid barrier after it (accumulated, with the step
-    // count, in the barrier words 8..15 for lbm_ensemble_phase_times).
+    // Block 0 times the phases on the global timer: phases 1 and 3 end
+    // when block 0 leaves the grid barrier after them, phase 2 with its last
+    // column (accumulated, with the step count, in the barrier words 8..15 for
+    // lbm_ensemble_phase_times).
     unsigned long long *phase_ns = reinterpret_cast<unsigned long long *>(w.bar + 8);
     const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
     unsigned long long tp = timer ? global_ns() : 0ull;
@@ -184,31 +181,30 @@ __global__ void ENS_BOUNDS k_ensemble(const __grid_constant__ EnsWork w, int nst
             const CavDesc &d = w.desc[k];
             top[k] = d.cut ? *(volatile int *)d.jmax + 3 : 1 << 30;
         }
-        if (threadIdx.x == 0) next = (long long)atomicAdd(ctr + (t & 1), (unsigned long long)kChunk);
         __syncthreads();
         // phase 1: fused stream-collide of every node of every cavity; an
         // item is one (1 << bxs) x by tile of K consecutive z-planes; tiles
-        // wholly above the liquid (deep solid) are skipped.  Blocks take
-        // chunks of kChunk items from the step's counter (tiles differ in
-        // work: deep-solid ones are skipped), asking for the next chunk
-        // before working on the current one.
-        for (long long base = next; base < items1; base = next) {
+        // wholly above the liquid (deep solid) are skipped.  A block's first
+        // item is its own number, the others come one at a time from the
+        // step's counter (tiles differ in work: deep-solid ones are skipped;
+        // chunks of 2 or 4 were slower), asked for before the current one is
+        // worked on.
+        for (long long it = blockIdx.x; it < items1; it = next) {
             __syncthreads();  // every thread has read `next`
-            if (threadIdx.x == 0) next = (long long)atomicAdd(ctr + (t & 1), (unsigned long long)kChunk);
-            const long long stop = base + kChunk < items1 ? base + kChunk : items1;
-            for (long long it = base; it < stop; ++it) {
+            if (threadIdx.x == 0) next = gridDim.x + (long long)atomicAdd(ctr + (t & 1), 1ull);
+            [&]() {
             if (it >= w.item_begin[kc + 1]) kc += find_cavity(w.item_begin + kc, w.ncav - kc, it);
             const int k = kc;
             const CavDesc &d = w.desc[k];
             const int li = (int)(it - w.item_begin[k]);
             const int zc = li / d.gxy, r = li - zc * d.gxy;
             const int iy = r / d.gx, ix = r - iy * d.gx;
-            if ((d.face == 0 ? iy * d.by : zc * K) >= top[k]) continue;
+            if ((d.face == 0 ? iy * d.by : zc * K) >= top[k]) return;
             const int cur = d.cur0 ^ (t & 1), odd = d.inflight0 ^ (t & 1);
             const float *trd = t == 0 ? d.thw_rd0 : d.thw;
             const int x = (ix << d.bxs) + (threadIdx.x & ((1 << d.bxs) - 1));
             const int y = iy * d.by + (threadIdx.x >> d.bxs);
-            if (x >= d.p.nx || y >= d.p.ny) continue;
+            if (x >= d.p.nx || y >= d.p.ny) return;
 #pragma unroll 1
             for (int j = 0; j < K; ++j) {
                 const int z = zc * K + j;
@@ -221,13 +217,13 @@ __global__ void ENS_BOUNDS k_ensemble(const __grid_constant__ EnsWork w, int nst
                     else ens_even<ST, 1>(d, cur, x, y, z);
                 }
             }
-            }
-            __syncthreads();  // `next` holds the following chunk
+            }();
+            __syncthreads();  // `next` holds the following item
         }
         // the other counter serves the next step; it was last used by the
         // step before, which every block has left
         if (blockIdx.x == 0 && threadIdx.x == 0) ctr[(t + 1) & 1] = 0ull;
-        if (!grid_barrier(w, gridDim.x)) return;
+        if (!grid_barrier(w, arrivals += gridDim.x)) return;
         if (timer) { const unsigned long long tn = global_ns(); phase_ns[0] += tn - tp; tp = tn; }
         // phase 2: front update (Eq. 6) of every column; phase 3: flip of the
         // columns whose liquid count changed, by the thread that updated
@@ -263,7 +259,7 @@ __global__ void ENS_BOUNDS k_ensemble(const __grid_constant__ EnsWork w, int nst
             const int m = __reduce_max_sync(0xffffffffu, jn);  // an item is one cavity's columns: whole warps
             if ((threadIdx.x & 31) == 0 && m >= 0) atomicMax(d.jmax, m);
         }
-        if (!grid_barrier(w, gridDim.x)) return;
+        if (!grid_barrier(w, arrivals += gridDim.x)) return;
         if (timer) {
             const unsigned long long tn = global_ns();
             phase_ns[2] += tn - tp;

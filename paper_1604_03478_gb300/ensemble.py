@@ -71,8 +71,8 @@ class Ensemble:
 
     def phase_times(self, reset=False):
         """Mean microseconds per step of the stream-collide, front and flip
-        phases (each with its closing grid barrier) since creation or the
-        last reset, and the number of steps timed."""
+        phases (the first and the last with the grid barrier that closes
+        them) since creation or the last reset, and the number of steps timed."""
         us = (C.c_double * 3)()
         n = C.c_longlong()
         self._check(_abi.load().lbm_ensemble_phase_times(self._h, 1 if reset else 0, us, C.byref(n)))
