@@ -250,9 +250,8 @@ lbm_status lbm_melt_set_graph_steps(lbm_melt *h, int steps);
 
 /* Nodes per thread of the stream-collide (the same method and results up to
    FP32 rounding): -1 (default) chooses two for cavities above 160^3 nodes
-   with an even nx, and with FP32 storage (no conduction in the solid) above
-   110^3 unless a row of nx / 2 leaves more than a fifth of a block's lanes
-   idle, and one otherwise; 0 one node per thread; 1 two nodes per
+   with an even nx, and with FP32 storage (no conduction in the solid) from
+   120^3 on, and one otherwise; 0 one node per thread; 1 two nodes per
    thread (x-adjacent nodes as the two lanes of packed FP32x2 arithmetic,
    their populations moved as float2/half2 words where aligned; needs an
    even nx, else LBM_EINVAL).  Two nodes

@@ -17,7 +17,7 @@ import os
 from . import build as _build
 
 CACHE = os.path.join(_build.BUILD, "autotune.json")
-CAVITY_SHAPES = ((128, 1), (64, 2), (32, 4))
+CAVITY_SHAPES = ((0, 0), (128, 1), (64, 2), (32, 4))  # (0, 0): the default
 ENSEMBLE_SHAPES = ((64, 2), (128, 1), (128, 2), (128, 4), (128, 8), (256, 1), (256, 2), (256, 4))
 
 

@@ -78,13 +78,13 @@ __device__ __forceinline__ void even_pair_cond(const KP &p, ST *__restrict__ F, 
     }
 }
 
-template <typename ST, int FACE, typename IX>
+template <typename ST, int FACE, typename IX, int LIN>
 __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_even_pair_cond(
     const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G, const int *__restrict__ js,
     const int *__restrict__ nb, const float *__restrict__ gpost, const float *__restrict__ spost) {
     step_launch_wait();
     int x, y, z;
-    if (k1_pair<FACE>(p, x, y, z)) even_pair_cond<ST, FACE, IX>(p, F, G, js, nb, gpost, spost, x, y, z);
+    if (k1_pair<FACE, LIN>(p, x, y, z)) even_pair_cond<ST, FACE, IX>(p, F, G, js, nb, gpost, spost, x, y, z);
 }
 
 // Odd step, pair: off the walls of the heating axis and of the other
@@ -138,7 +138,7 @@ __device__ __forceinline__ void odd_pair_cond(const KP &p, const Links *lk, ST *
     }
 }
 
-template <typename ST, int FACE, typename IX>
+template <typename ST, int FACE, typename IX, int LIN>
 __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair_cond(
     const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G, const int *__restrict__ js,
     const int *__restrict__ js_old, const int *__restrict__ nb, const float *__restrict__ gpost,
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair_cond(
     const float *__restrict__ thw_wr, const __grid_constant__ Links lk, const float *__restrict__ spost) {
     step_launch_wait();
     int x, y, z;
-    if (k1_pair<FACE>(p, x, y, z))
+    if (k1_pair<FACE, LIN>(p, x, y, z))
         odd_pair_cond<ST, FACE, IX>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, spost, x, y, z);
 }
 
@@ -167,15 +167,15 @@ static cudaError_t launch_cond_kernel(void (*kern)(KArgs...), dim3 grd, dim3 blk
 }
 
 // Two nodes per thread, element indices in IX (32 bits whenever all fit).
-template <typename ST, typename IX>
+template <typename ST, typename IX, int LIN>
 static cudaError_t launch_pair_cond(const KP &p, int face, int odd, const Bufs &b, dim3 g2, dim3 blk, cudaStream_t st) {
     ST *F = (ST *)b.F, *G = (ST *)b.G;
     if (face == 0) {
-        if (odd) return launch_cond_kernel(k_odd_pair_cond<ST, 0, IX>, g2, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
-        else return launch_cond_kernel(k_even_pair_cond<ST, 0, IX>, g2, blk, st, p, F, G, b.js, b.nb, b.gpost, b.spost);
+        if (odd) return launch_cond_kernel(k_odd_pair_cond<ST, 0, IX, LIN>, g2, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
+        else return launch_cond_kernel(k_even_pair_cond<ST, 0, IX, LIN>, g2, blk, st, p, F, G, b.js, b.nb, b.gpost, b.spost);
     } else {
-        if (odd) return launch_cond_kernel(k_odd_pair_cond<ST, 1, IX>, g2, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
-        else return launch_cond_kernel(k_even_pair_cond<ST, 1, IX>, g2, blk, st, p, F, G, b.js, b.nb, b.gpost, b.spost);
+        if (odd) return launch_cond_kernel(k_odd_pair_cond<ST, 1, IX, LIN>, g2, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
+        else return launch_cond_kernel(k_even_pair_cond<ST, 1, IX, LIN>, g2, blk, st, p, F, G, b.js, b.nb, b.gpost, b.spost);
     }
 }
 
@@ -185,11 +185,13 @@ cudaError_t LaunchCond<ST>::stream_collide(const KP &p, int face, int odd, const
     if (b.pairs && p.nx % 2 == 0) {
         KP half_x = p;
         half_x.nx = p.nx / 2;
-        const dim3 g2 = k1_grid(half_x, blk, face, p.H);
-        if (19LL * p.ld < (1LL << 32)) return launch_pair_cond<ST, unsigned>(p, face, odd, b, g2, blk, st);
-        return launch_pair_cond<ST, long long>(p, face, odd, b, g2, blk, st);
+        const bool narrow = 19LL * p.ld < (1LL << 32), line = b.linear && narrow;
+        const dim3 g2 = k1_grid(half_x, blk, face, p.H, line);
+        if (line) return launch_pair_cond<ST, unsigned, 1>(p, face, odd, b, g2, blk, st);
+        if (narrow) return launch_pair_cond<ST, unsigned, 0>(p, face, odd, b, g2, blk, st);
+        return launch_pair_cond<ST, long long, 0>(p, face, odd, b, g2, blk, st);
     }
-    const dim3 grd = k1_grid(p, blk, face, p.H);
+    const dim3 grd = k1_grid(p, blk, face, p.H, b.linear);
     if (face == 0) {
         if (odd) return launch_cond_kernel(k_odd_cond<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
         else return launch_cond_kernel(k_even_cond<ST, 0>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, b.spost);

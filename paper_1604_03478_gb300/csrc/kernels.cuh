@@ -244,6 +244,11 @@ __device__ __forceinline__ void snap_any(const KP &p, const ST *F, const ST *G, 
 // written by the previous front update: nodes two or more above every
 // neighbouring count are deep solid and do nothing, so a block whose heights
 // are all >= jmax + 3 returns at once.
+// A grid of one block row (gridDim.y == blockDim.y == 1) is linear instead:
+// consecutive threads take consecutive columns of one height, across the ends
+// of rows, so that no lane idles whatever nx is (k1_linear in launch.h says
+// when).
+__device__ __forceinline__ bool k1_is_linear() { return gridDim.y == 1 && blockDim.y == 1; }
 // Lowest height of a block of the stream-collide grid.
 template <int FACE> __device__ __forceinline__ int k1_low() {
     return (int)blockIdx.z * (FACE == 0 ? (int)blockDim.y : 1);
@@ -258,6 +263,13 @@ __device__ __forceinline__ bool k1_node(const KP &p, const int *jmax, int &x, in
     const int a0 = (int)blockIdx.z * (FACE == 0 ? (int)blockDim.y : 1);  // lowest height of the block
     if (jmax && a0 >= *jmax + 3) return false;
     x = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (k1_is_linear()) {
+        const int q = (int)((unsigned)x / (unsigned)p.nx);
+        x -= q * p.nx;
+        y = FACE == 0 ? a0 : q;
+        z = FACE == 0 ? q : a0;
+        return q < p.P2 && a0 < p.H;
+    }
     if (FACE == 0) {
         y = a0 + (int)threadIdx.y;
         z = (int)blockIdx.y;
@@ -788,10 +800,19 @@ template <typename ST> constexpr int pair_min_blocks() {
     return sizeof(ST) == 2 ? LBM_PAIR_MIN_BLOCKS : LBM_PAIR_MIN_BLOCKS_F32;
 }
 
-template <int FACE>
+// LIN: 0 rows, 1 columns in a line (known at compile time: with FP16 storage
+// the test alone cost spills, 156.5 -> 162 us at 256^3).
+template <int FACE, int LIN>
 __device__ __forceinline__ bool k1_pair(const KP &p, int &x, int &y, int &z) {
     const int a0 = k1_low<FACE>();
     x = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (LIN) {  // x / nx and x % nx of an even nx: whole pairs
+        const int q = (int)((unsigned)x / (unsigned)p.nx);
+        x -= q * p.nx;
+        y = FACE == 0 ? a0 : q;
+        z = FACE == 0 ? q : a0;
+        return q < p.P2 && a0 < p.H;
+    }
     if (FACE == 0) {
         y = a0 + (int)threadIdx.y;
         z = (int)blockIdx.y;
@@ -856,14 +877,14 @@ __device__ __forceinline__ void even_pair(const KP &p, ST *__restrict__ F, ST *_
     }
 }
 
-template <typename ST, int FACE, typename IX>
+template <typename ST, int FACE, typename IX, int LIN>
 __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_even_pair(const __grid_constant__ KP p, ST *__restrict__ F,
                                                       ST *__restrict__ G, const int *__restrict__ js,
                                                       const int *__restrict__ nb, const float *__restrict__ gpost,
                                                       const int *jmax) {
     step_launch_wait();
     int x, y, z;
-    if (k1_pair<FACE>(p, x, y, z) && !(jmax && k1_low<FACE>() >= *jmax + 3)) even_pair<ST, FACE, IX>(p, F, G, js, nb, gpost, x, y, z);
+    if (k1_pair<FACE, LIN>(p, x, y, z) && !(jmax && k1_low<FACE>() >= *jmax + 3)) even_pair<ST, FACE, IX>(p, F, G, js, nb, gpost, x, y, z);
 }
 
 // The odd step of a pair on the fast path (both liquid, off the walls of the
@@ -961,7 +982,7 @@ __device__ __forceinline__ void odd_pair(const KP &p, const Links *lk, ST *__res
     odd_pair_liquid<ST, FACE, IX>(p, lk, F, G, x, y, z);
 }
 
-template <typename ST, int FACE, typename IX>
+template <typename ST, int FACE, typename IX, int LIN>
 __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair(const __grid_constant__ KP p, ST *__restrict__ F,
                                                      ST *__restrict__ G, const int *__restrict__ js,
                                                      const int *__restrict__ js_old, const int *__restrict__ nb,
@@ -971,7 +992,7 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair(const _
                                                      const __grid_constant__ Links lk, const int *jmax) {
     step_launch_wait();
     int x, y, z;
-    if (k1_pair<FACE>(p, x, y, z) && !(jmax && k1_low<FACE>() >= *jmax + 3)) odd_pair<ST, FACE, IX>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x, y, z);
+    if (k1_pair<FACE, LIN>(p, x, y, z) && !(jmax && k1_low<FACE>() >= *jmax + 3)) odd_pair<ST, FACE, IX>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x, y, z);
 }
 
 
@@ -985,14 +1006,14 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair(const _
 // of loads cost more than it hid (156.5 -> 161.7 us).
 // SNAP: see k_even; a pair that is split takes its snapshot by gathers, from
 // the slots that its nodes own in this step.
-template <typename ST, int FACE, typename IX, bool SNAP>
+template <typename ST, int FACE, typename IX, int LIN, bool SNAP>
 __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_even_pair_early(const __grid_constant__ KP p, ST *__restrict__ F,
                                                       ST *__restrict__ G, const int *js, const int *js_old,
                                                       const int *__restrict__ nb, const float *__restrict__ gpost,
                                                       const int *jmax, int early_blocks, const double *s,
                                                       const __grid_constant__ SnapOut snap) {
     int x = 0, y = 0, z = 0;
-    const bool on = k1_pair<FACE>(p, x, y, z), late = k1_late(early_blocks);
+    const bool on = k1_pair<FACE, LIN>(p, x, y, z), late = k1_late(early_blocks);
     if (late) step_launch_wait();
     const IX c = on ? (IX)node_index(p, x, y, z) : 0;
     const int a = axial<FACE>(x, y, z);
@@ -1025,7 +1046,7 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_even_pair_early(
     even_pair_finish<ST, IX>(p, F, G, c, f, g);
 }
 
-template <typename ST, int FACE, typename IX, bool SNAP>
+template <typename ST, int FACE, typename IX, int LIN, bool SNAP>
 __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair_early(const __grid_constant__ KP p, ST *__restrict__ F,
                                                      ST *__restrict__ G, const int *js, const int *js_old,
                                                      const int *nb, const int *nb_old,
@@ -1036,7 +1057,7 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair_early(c
                                                      int early_blocks, const double *s,
                                                      const __grid_constant__ SnapOut snap) {
     int x = 0, y = 0, z = 0;
-    const bool on = k1_pair<FACE>(p, x, y, z), late = k1_late(early_blocks);
+    const bool on = k1_pair<FACE, LIN>(p, x, y, z), late = k1_late(early_blocks);
     if (late) step_launch_wait();
     const int a = axial<FACE>(x, y, z);
     const int col = on ? column<FACE>(p, x, y, z) : 0;

@@ -29,6 +29,7 @@ struct Bufs {
     double nu_scale;             // H / (alpha (Th - Tm))
     float *spost;                // solid-side ghost populations, 7 x ncols (heat conduction in the solid)
     int pairs;                   // stream-collide with two nodes per thread (even nx)
+    int linear;                  // stream-collide blocks of consecutive columns (k1_linear)
     int early_pairs;             // ... with the first wave's loads before the wait (FP32 storage, middle sizes)
 };
 
@@ -95,6 +96,17 @@ inline int block_width(int nx, int block) {
     }
     return best;
 }
+// Whether rows of nxt threads (nx, or nx / 2 with two nodes per thread) leave
+// lanes idle in the fitted width: then the stream-collide's blocks take
+// consecutive columns instead.  Us per step, rows against columns, front at
+// 0.5 H: 71^3 13.7 / 12.6, 101x75x83 18.3 / 16.9, 100^3 24.4 / 22.0, 160^3 (80
+// pairs a row) 81.1 / 78.3, 200^3 166.8 / 159.2, 200^3 with a conducting solid
+// 196 / 186, FP16 100^3 22.0 / 19.4.  Rows that fit keep their blocks (FP16
+// 160^3 55.0 / 56.9, 256^3 162 / 171; FP32 the same either way).
+inline bool k1_linear(int nxt, int widest) {
+    const int bx = block_width(nxt, widest);
+    return nxt % bx != 0;
+}
 inline dim3 node_block(const KP &p) {
     const int bx = block_width(p.nx, 128);
     return dim3(bx, 128 / bx, 1);
@@ -104,7 +116,13 @@ inline dim3 node_grid(const KP &p, dim3 b) {
 }
 // Grid of the stream-collide (k1_node): x tiles, the in-plane tiles, then
 // the heights along the heating axis (slowest).
-inline dim3 k1_grid(const KP &p, dim3 b, int face, int height) {
+// Linear: blocks of 128 consecutive columns (b.x; pairs of them with p.nx
+// halved), whatever rows they lie in.
+inline dim3 k1_grid(const KP &p, dim3 b, int face, int height, int linear) {
+    if (linear) {
+        if (height < 1) height = 1;
+        return dim3((unsigned)(((long long)p.nx * p.P2 + b.x - 1) / b.x), 1, height < p.H ? height : p.H);
+    }
     const unsigned gx = (p.nx + b.x - 1) / b.x;
     if (height < 1) height = 1;
     if (face == 0) {

@@ -50,43 +50,43 @@ static cudaError_t launch_sc(const KP &p, int face, int odd, const Bufs &b, dim3
 #ifndef LBM_PAIR_ODD_IX
 #define LBM_PAIR_ODD_IX unsigned
 #endif
-template <typename ST, typename IX, bool SNAP>
+template <typename ST, typename IX, int LIN, bool SNAP>
 static cudaError_t launch_sc_pair_early(const KP &p, int face, int odd, const Bufs &b, dim3 grd, dim3 blk,
                                         cudaStream_t st, const SnapOut &snap) {
     const int early = b.sms * (pair_min_blocks<ST>() * 128 / (int)(blk.x * blk.y));  // blocks resident at once
     const int *jm = p.skip_deep ? b.jmax : nullptr;
     ST *F = (ST *)b.F, *G = (ST *)b.G;
     if (face == 0) {
-        if (odd) return launch_step_kernel(k_odd_pair_early<ST, 0, IX, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early, b.s, snap);
-        else return launch_step_kernel(k_even_pair_early<ST, 0, IX, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early, b.s, snap);
+        if (odd) return launch_step_kernel(k_odd_pair_early<ST, 0, IX, LIN, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early, b.s, snap);
+        else return launch_step_kernel(k_even_pair_early<ST, 0, IX, LIN, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early, b.s, snap);
     } else {
-        if (odd) return launch_step_kernel(k_odd_pair_early<ST, 1, IX, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early, b.s, snap);
-        else return launch_step_kernel(k_even_pair_early<ST, 1, IX, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early, b.s, snap);
+        if (odd) return launch_step_kernel(k_odd_pair_early<ST, 1, IX, LIN, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early, b.s, snap);
+        else return launch_step_kernel(k_even_pair_early<ST, 1, IX, LIN, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early, b.s, snap);
     }
 }
 
 // An even nx: two nodes per thread (k_even_pair / k_odd_pair, or their early
 // forms), the grid's x extent covering nx / 2 threads.
-template <typename ST, typename IXE, typename IXO>
+template <typename ST, typename IXE, typename IXO, int LIN>
 static cudaError_t launch_sc_pair(const KP &p, int face, int odd, const Bufs &b, dim3 blk, cudaStream_t st,
                                   const SnapOut *snap) {
     const int *jm = p.skip_deep ? b.jmax : nullptr;
     ST *F = (ST *)b.F, *G = (ST *)b.G;
     KP half_x = p;
     half_x.nx = p.nx / 2;
-    dim3 grd = k1_grid(half_x, blk, face, b.k1_height);
+    const dim3 grd = k1_grid(half_x, blk, face, b.k1_height, LIN);
     if constexpr (sizeof(ST) == 4 && sizeof(IXE) == 4) {
         if (b.early_pairs) {
-            if (snap) return launch_sc_pair_early<ST, IXE, true>(p, face, odd, b, grd, blk, st, *snap);
-            return launch_sc_pair_early<ST, IXE, false>(p, face, odd, b, grd, blk, st, SnapOut());
+            if (snap) return launch_sc_pair_early<ST, IXE, LIN, true>(p, face, odd, b, grd, blk, st, *snap);
+            return launch_sc_pair_early<ST, IXE, LIN, false>(p, face, odd, b, grd, blk, st, SnapOut());
         }
     }
     if (face == 0) {
-        if (odd) return launch_step_kernel(k_odd_pair<ST, 0, IXO>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
-        else return launch_step_kernel(k_even_pair<ST, 0, IXE>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, jm);
+        if (odd) return launch_step_kernel(k_odd_pair<ST, 0, IXO, LIN>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
+        else return launch_step_kernel(k_even_pair<ST, 0, IXE, LIN>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, jm);
     } else {
-        if (odd) return launch_step_kernel(k_odd_pair<ST, 1, IXO>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
-        else return launch_step_kernel(k_even_pair<ST, 1, IXE>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, jm);
+        if (odd) return launch_step_kernel(k_odd_pair<ST, 1, IXO, LIN>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
+        else return launch_step_kernel(k_even_pair<ST, 1, IXE, LIN>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, jm);
     }
 }
 
@@ -105,10 +105,13 @@ cudaError_t Launch<ST>::stream_collide(const KP &p, int face, int odd, const Buf
                                        const SnapOut *snap) {
     if (p.cond) return LaunchCond<ST>::stream_collide(p, face, odd, b, blk, st);
     if (b.pairs && p.nx % 2 == 0) {
-        if (19LL * p.ld < (1LL << 32)) return launch_sc_pair<ST, unsigned, LBM_PAIR_ODD_IX>(p, face, odd, b, blk, st, snap);
-        return launch_sc_pair<ST, long long, long long>(p, face, odd, b, blk, st, nullptr);
+        if (19LL * p.ld < (1LL << 32)) {
+            if (b.linear) return launch_sc_pair<ST, unsigned, LBM_PAIR_ODD_IX, 1>(p, face, odd, b, blk, st, snap);
+            return launch_sc_pair<ST, unsigned, LBM_PAIR_ODD_IX, 0>(p, face, odd, b, blk, st, snap);
+        }
+        return launch_sc_pair<ST, long long, long long, 0>(p, face, odd, b, blk, st, nullptr);
     }
-    const dim3 grd = k1_grid(p, blk, face, b.k1_height);
+    const dim3 grd = k1_grid(p, blk, face, b.k1_height, b.linear);
     if (snap) return launch_sc<ST, unsigned, true>(p, face, odd, b, grd, blk, st, *snap);
     if (19LL * p.ld < (1LL << 32)) return launch_sc<ST, unsigned, false>(p, face, odd, b, grd, blk, st, SnapOut());
     return launch_sc<ST, long long, false>(p, face, odd, b, grd, blk, st, SnapOut());

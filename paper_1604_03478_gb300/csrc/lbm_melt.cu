@@ -172,23 +172,20 @@ lbm_status cuda_err(lbm_melt *h, cudaError_t e, const char *where) {
 // with half the threads (256^3: 0.2245 against 0.234 ms per launch in FP32,
 // 0.145 against 0.19 ms in FP16), and with FP32 storage from kPairNodes on,
 // where the early pair kernels run (us per step, two nodes against one,
-// front at 0.1, 0.25, 0.45 and 0.8 H: 112^3 12.8 / 13.5, 18.1 / 19.7, 26.5 /
-// 27.4, 47.9 / 48.9; 128^3 14.4 / 16.5, 22.3 / 23.9, 37.6 / 40.4, 65.6 / 66.3;
-// 160^3 22.0 / 24.8, 45.5 / 47.4, 73.8 / 76.3, 121.7 / 123.2), unless more
-// than a fifth of a block's lanes would idle over a row of nx / 2 (96^3, 48 of
-// 64: 12.6 / 11.3, 29.8 / 26.2).  Smaller cavities are latency bound and run
-// faster with one node per thread (48^3 8.0 / 6.4).  FP16 storage keeps one
-// below 160^3: the pairs' rounding moves stored values by an FP16 step.
-const long long kPairNodes = 110LL * 110 * 110;
+// front at 0.15 and 0.5 H: 128^3 17.0 / 18.3 and 44.2 / 45.8, 160^3 26.7 /
+// 31.2 and 78.3 / 83.5; 112^3 15.2 / 15.0 and 29.8 / 29.3, 100^3 12.9 / 12.7
+// and 23.9 / 22.0, 48^3 9.4 / 6.8).  Smaller cavities are latency bound and run
+// faster with one node per thread.  FP16 storage keeps one below 160^3: the
+// pairs' rounding moves stored values by an FP16 step.
+const long long kPairNodes = 120LL * 120 * 120;
 bool use_pairs(const lbm_melt *h) {
     if (h->kp.nx % 2 != 0) return false;
     if (h->pairs_mode >= 0) return h->pairs_mode == 1;
     if (h->d.N > kGraphMaxNodes) return true;
-    if (h->precision != 0 || h->kp.cond || h->d.N < kPairNodes) return false;
-    const int half = h->kp.nx / 2, bx = lbm::block_width(half, 128);
-    const int lanes = (half + bx - 1) / bx * bx;
-    return 5 * (lanes - half) <= lanes;
+    return h->precision == 0 && !h->kp.cond && h->d.N >= kPairNodes;
 }
+
+bool sc_linear(const lbm_melt *h);
 
 // Buffers of a step from phase (cur, inflight) with the handle's wall fields.
 Bufs bufs_at(lbm_melt *h, int cur, int inflight) {
@@ -218,6 +215,7 @@ Bufs bufs_at(lbm_melt *h, int cur, int inflight) {
     b.nu_scale = (double)h->kp.H / (h->d.alpha * (h->Th - h->Tm));
     b.spost = h->spost;
     b.pairs = use_pairs(h) ? 1 : 0;
+    b.linear = sc_linear(h) ? 1 : 0;
     b.early_pairs = h->d.N <= kGraphMaxNodes ? 1 : 0;
     return b;
 }
@@ -421,13 +419,20 @@ __global__ void k_fill_d(double *p, long long n, double v) {
     if (i < n) p[i] = v;
 }
 
-// Launch shape of the stream-collide.
+// Columns in a line (k1_linear) where rows would leave lanes idle.
+bool sc_linear(const lbm_melt *h) {
+    if (h->bx) return false;
+    return use_pairs(h) ? lbm::k1_linear(h->kp.nx / 2, h->precision == 1 ? 64 : 128) : lbm::k1_linear(h->kp.nx, 128);
+}
+
 // Launch shape of the stream-collide: the caller's (lbm_melt_set_launch),
-// else 128 threads x-major, the width fitted to the threads of a row (nx / 2
-// with two nodes per thread; at most 64 wide with FP16 pairs, 0.141 against
-// 0.145 ms at 256^3 with 128).
+// else 128 threads, over consecutive columns where rows do not fit, x-major
+// with the width fitted to the threads of a row where they do (nx / 2 with
+// two nodes per thread; at most 64 wide with FP16 pairs, 0.141 against 0.145
+// ms at 256^3 with 128).
 dim3 sc_block(const lbm_melt *h) {
     if (h->bx) return dim3(h->bx, h->by, 1);
+    if (sc_linear(h)) return dim3(128, 1, 1);
     if (!use_pairs(h)) return lbm::node_block(h->kp);
     const int bx = lbm::block_width(h->kp.nx / 2, h->precision == 1 ? 64 : 128);
     return dim3(bx, 128 / bx, 1);

@@ -80,3 +80,34 @@ def test_gradient_with_node_pairs(face, nx, steps, spread):
     assert np.abs(da - db).max() <= 1e-4 * np.abs(da).max()
     for k in pa:
         assert abs(pa[k] - pb[k]) <= 1e-4 * max(abs(pa[k]), 1e-12)
+
+
+@pytest.mark.parametrize("face", [0, 1])
+@pytest.mark.parametrize("nx,pairs,solid", [(1, 0, 0), (5, 0, 0), (33, 0, 0), (71, 0, 1), (130, 0, 0), (6, 1, 0),
+                                            (38, 1, 0), (70, 1, 1), (140, 1, 0)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_columns_in_a_line(face, nx, pairs, solid, precision):
+    """Stream-collide blocks of consecutive columns (rows that leave lanes
+    idle) against blocks of rows: the same threads do the same arithmetic, so
+    the states are the same bits."""
+    import torch
+    assert torch.cuda.is_available()
+    from paper_1604_03478_gb300 import build, Cavity
+    build.build()
+    shape = (nx, 11, 7) if face == 0 else (nx, 7, 11)
+    kw = dict(face=face, precision=precision, Ra=5e4, Pr=0.3, Ste=0.8, Ma=0.15, s0=4.2, derive=True)
+    if solid:
+        kw.update(solid=1, ks_kl=0.7, Tc=-0.2)
+    out = []
+    for rows in (False, True):
+        c = Cavity(*shape, **kw)
+        c.set_node_pairs(pairs)
+        if rows:
+            c.set_launch(32, 2)
+        f, g, s = c.get_state()
+        c.set_state(f, g, s + inputs.uniform(c.ncols, -1.2, 1.2, 17))
+        c.step(19)
+        out.append(c.get_state())
+        c.close()
+    for a, b in zip(*out):
+        np.testing.assert_array_equal(a, b)
