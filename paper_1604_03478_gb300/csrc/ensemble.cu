@@ -41,7 +41,7 @@ struct lbm_ensemble {
     cudaStream_t stream;  // own non-blocking stream: capturable, unlike the legacy default stream
     cudaEvent_t ev_in, ev_out;
     int precision;
-    int block, K, grid;
+    int block, K, grid, linear;
     long long max_spins;
     unsigned int *bar_dev;
     long long items[lbm::kMaxCavities + 1], cols[lbm::kMaxCavities + 1];
@@ -100,6 +100,7 @@ void fill_desc(lbm_melt *h, CavDesc &d, int block) {
     tile(h->kp, block, d.bxs, d.by);
     d.gx = (h->kp.nx + (1 << d.bxs) - 1) >> d.bxs;
     d.gxy = d.gx * ((h->kp.ny + d.by - 1) / d.by);
+    d.cblk = (int)((h->kp.ncols + block - 1) / block);
     d.p = h->kp;
     d.face = h->face;
     d.cur0 = h->cur;
@@ -126,15 +127,28 @@ long long launch_steps(const lbm_ensemble *e) {
 
 // Work-list prefix sums and the co-resident grid for the launch shape.
 lbm_status plan(lbm_ensemble *e) {
+    // Tiles unless they leave a tenth of the lanes idle over all members: then
+    // blocks of consecutive columns.  Us per step, tiles against columns: eight
+    // cavities of edges 20 to 47 31.1 / 25.3, four of 20 to 81 29.6 / 24.6; with
+    // few lanes idle 20 of 48 to 128 322 / 327, 48 of 48 to 160 1189 / 1229.
+    long long lanes = 0, nodes = 0;
+    for (lbm_melt *h : e->cav) {
+        int bxs, by;
+        tile(h->kp, e->block, bxs, by);
+        const long long bx = 1LL << bxs;
+        lanes += (h->kp.nx + bx - 1) / bx * bx * ((h->kp.ny + by - 1) / by * by) * h->kp.nz;
+        nodes += h->kp.N;
+    }
+    e->linear = 10 * lanes > 11 * nodes ? 1 : 0;
     e->items[0] = e->cols[0] = 0;
     for (int k = 0; k < e->n; ++k) {
         const lbm::KP &p = e->cav[k]->kp;
         int bxs, by;
         tile(p, e->block, bxs, by);
         const long long gx = (p.nx + (1 << bxs) - 1) >> bxs, gy = (p.ny + by - 1) / by;
-        const long long gz = (p.nz + e->K - 1) / e->K;
-        e->items[k + 1] = e->items[k] + gx * gy * gz;
-        e->cols[k + 1] = e->cols[k] + (p.ncols + e->block - 1) / e->block;
+        const long long cblk = (p.ncols + e->block - 1) / e->block;
+        e->items[k + 1] = e->items[k] + (e->linear ? cblk * ((p.H + e->K - 1) / e->K) : gx * gy * ((p.nz + e->K - 1) / e->K));
+        e->cols[k + 1] = e->cols[k] + cblk;
     }
     int dev = 0, sms = 0, per_sm = 0;
     ECK(cudaGetDevice(&dev), "device");
@@ -164,7 +178,7 @@ lbm_status launch(lbm_ensemble *e, int nsteps, int skip_block) {
     EnsWork *w = new (std::nothrow) EnsWork();
     if (!w) return LBM_ENOMEM;
     w->ncav = e->n;
-    w->nodes_per_item = e->block * e->K;
+    w->linear = e->linear;
     for (int k = 0; k <= e->n; ++k) {
         w->item_begin[k] = e->items[k];
         w->col_begin[k] = e->cols[k];
@@ -259,8 +273,8 @@ LBM_API lbm_status lbm_ensemble_create(int n, const lbm_melt_case *cases, void *
         return fail(LBM_ENOMEM);
     // A small ensemble, whose nodes are at most two items of 256 a resident
     // block, takes 256 threads and one plane an item: each item's latency
-    // counts there (eight cavities of 20 to 47 nodes an edge: 27.0 us a step
-    // against 31.8 with 128 and two planes); a larger one the other shape
+    // counts there (eight cavities of 20 to 47 nodes an edge: 24.9 us a step
+    // against 28 with 128 and two planes); a larger one the other shape
     // (20 cavities of 48 to 128: 326 against 368).
     e->block = 256;
     e->K = 1;

@@ -41,6 +41,7 @@ struct CavDesc {
     KP p;
     int face, cur0, inflight0;
     int bxs, by, gx, gxy;         // tile: 1 << bxs by by threads; tiles per row and per plane
+    int cblk;                     // blocks of consecutive columns that cover the cavity
     void *F, *G;
     int *js[2], *nb[2];
     double *s[2];
@@ -56,7 +57,7 @@ struct CavDesc {
 constexpr int kMaxCavities = 64;
 struct EnsWork {
     int ncav;
-    int nodes_per_item;
+    int linear;                                // items are consecutive columns, not tiles
     long long item_begin[kMaxCavities + 1];  // prefix sums of node items
     long long col_begin[kMaxCavities + 1];   // prefix sums of column items
     CavDesc desc[kMaxCavities];
@@ -183,8 +184,9 @@ __global__ void ENS_BOUNDS k_ensemble(const __grid_constant__ EnsWork w, int nst
         }
         __syncthreads();
         // phase 1: fused stream-collide of every node of every cavity; an
-        // item is one (1 << bxs) x by tile of K consecutive z-planes; tiles
-        // wholly above the liquid (deep solid) are skipped.  A block's first
+        // item is one (1 << bxs) x by tile of K consecutive z-planes, or (where
+        // tiles would leave lanes idle) one block of consecutive columns by K
+        // heights; items wholly above the liquid (deep solid) are skipped.  A block's first
         // item is its own number, the others come one at a time from the
         // step's counter (tiles differ in work: deep-solid ones are skipped;
         // chunks of 2 or 4 were slower), asked for before the current one is
@@ -197,18 +199,29 @@ __global__ void ENS_BOUNDS k_ensemble(const __grid_constant__ EnsWork w, int nst
             const int k = kc;
             const CavDesc &d = w.desc[k];
             const int li = (int)(it - w.item_begin[k]);
-            const int zc = li / d.gxy, r = li - zc * d.gxy;
-            const int iy = r / d.gx, ix = r - iy * d.gx;
-            if ((d.face == 0 ? iy * d.by : zc * K) >= top[k]) return;
             const int cur = d.cur0 ^ (t & 1), odd = d.inflight0 ^ (t & 1);
             const float *trd = t == 0 ? d.thw_rd0 : d.thw;
-            const int x = (ix << d.bxs) + (threadIdx.x & ((1 << d.bxs) - 1));
-            const int y = iy * d.by + (threadIdx.x >> d.bxs);
-            if (x >= d.p.nx || y >= d.p.ny) return;
+            int x, y, z, dy = 0;  // and dz = 1 - dy from one of the K nodes to the next
+            if (w.linear) {
+                const int ac = li / d.cblk, col = (li - ac * d.cblk) * (int)blockDim.x + (int)threadIdx.x;
+                const int a0 = ac * K;
+                if (a0 >= top[k] || col >= d.p.ncols) return;
+                const int q = (int)((unsigned)col / (unsigned)d.p.nx);
+                x = col - q * d.p.nx;
+                dy = d.face == 0;
+                y = dy ? a0 : q;
+                z = dy ? q : a0;
+            } else {
+                const int zc = li / d.gxy, r = li - zc * d.gxy;
+                const int iy = r / d.gx, ix = r - iy * d.gx;
+                if ((d.face == 0 ? iy * d.by : zc * K) >= top[k]) return;
+                x = (ix << d.bxs) + (threadIdx.x & ((1 << d.bxs) - 1));
+                y = iy * d.by + (threadIdx.x >> d.bxs);
+                z = zc * K;
+                if (x >= d.p.nx || y >= d.p.ny) return;
+            }
 #pragma unroll 1
-            for (int j = 0; j < K; ++j) {
-                const int z = zc * K + j;
-                if (z >= d.p.nz) break;
+            for (int j = 0; j < K && y < d.p.ny && z < d.p.nz; ++j, y += dy, z += 1 - dy) {
                 if (d.face == 0) {
                     if (odd) ens_odd<ST, 0>(d, cur, trd, x, y, z);
                     else ens_even<ST, 0>(d, cur, x, y, z);
