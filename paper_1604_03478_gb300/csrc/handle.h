@@ -54,14 +54,19 @@ struct lbm_melt {
     int sms;           // SMs of the device
     // Running maximum of the liquid counts, kept by k_front on the device;
     // stream-collide blocks at heights >= it + 3 (all deep solid) return at
-    // once.  It is also copied every kRbEvery steps into a ring of pinned
-    // slots; before a stream-collide the host takes the newest copy at least
-    // kRbLag steps old (waiting for it only when it runs that far ahead of
-    // the device) and launches no block above it + its age + 2 (a count
-    // grows by at most one node per step).
+    // once.  k_front raises a copy in page-locked memory with it, and the host
+    // records an event every kRbEvery steps (an ensemble member, whose counts
+    // the persistent kernel also raises, copies the maximum into a ring of
+    // pinned slots instead); before a stream-collide the host takes the newest
+    // event at least kRbLag steps old (waiting for it only when it runs that
+    // far ahead of the device) and launches no block above the maximum it
+    // then reads + the event's age + 2 (a count grows by at most one node per
+    // step).
     static const int kRbRing = 32, kRbLag = 16, kRbEvery = 4;
     int *jmax_dev;
-    int *rb_val;       // pinned: ring of read-backs, then kFlags ints a synchronising call reads status_dev into
+    int *rb_val;       // pinned: ring of read-backs, kFlags ints a synchronising call reads status_dev into, and
+                       // the running maximum that k_front raises (at kRbTop)
+    static const int kRbTop = kRbRing + 2;
     static const int kFlags = 2;
     static const int kHostOut = 8;
     double *host_out;  // pinned (behind rb_val): small results of the synchronising calls, written by the kernels

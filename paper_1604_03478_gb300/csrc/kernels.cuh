@@ -1596,10 +1596,12 @@ __device__ __forceinline__ int front_column(const KP &p, ST *__restrict__ F, con
 // 256 front at once; without the cap, 136 and 192 registers, the loop of
 // single 256^3 steps lost 2.5 us a step to a second wave).
 //
-// jmax (may be null): running maximum of the liquid counts, one atomic per
-// warp; the host reads it back now and then to bound the height of the
-// stream-collide grid (nodes two above every neighbouring count are deep
-// solid and do nothing).
+// jmax (may be null): running maximum of the liquid counts.  A warp whose
+// columns exceed it (few do: a count grows by one now and then) raises it with
+// an atomic, and its copy in page-locked host memory, jmax_host (may be null),
+// which the host reads now and then to bound the height of the stream-collide
+// grid (nodes two above every neighbouring count are deep solid and do
+// nothing).
 template <typename ST, int FACE>
 __global__ void __launch_bounds__(128, 4) k_front(const __grid_constant__ KP p, ST *__restrict__ F, const ST *G,
                                                const int *__restrict__ js, int *__restrict__ js_next,
@@ -1607,14 +1609,18 @@ __global__ void __launch_bounds__(128, 4) k_front(const __grid_constant__ KP p, 
                                                const double *__restrict__ s, double *__restrict__ s_next,
                                                float *__restrict__ gpost, const float *__restrict__ thw,
                                                int inflight, int move, int *__restrict__ status,
-                                               int *__restrict__ jmax) {
+                                               int *jmax, int *jmax_host) {
     const int col = blockIdx.x * blockDim.x + threadIdx.x;
     int jn = -1;
+    const int top = jmax ? ld_l2(jmax) : 1 << 30;  // of the steps before
     if (col >= p.ncols) step_launch_wait();
     else jn = front_column<ST, FACE>(p, F, G, js, js_next, nb_next, s, s_next, gpost, thw, inflight, move, status, col);
     // blocks are whole warps and every thread of the grid reaches this point
     const int m = __reduce_max_sync(0xffffffffu, jn);
-    if (jmax && (threadIdx.x & 31) == 0 && m >= 0) atomicMax(jmax, m);
+    if ((threadIdx.x & 31) == 0 && m > top) {
+        atomicMax(jmax, m);
+        if (jmax_host) atomicMax_system(jmax_host, m);
+    }
 }
 
 // The front update with heat conduction in the solid.  4 blocks of 128 an SM

@@ -23,6 +23,7 @@ struct Bufs {
     int cblk;                    // threads per block of the per-column kernels (col_block)
     int sms;                     // SMs of the device
     int *jmax;                   // running maximum of the liquid counts (k_front), or null
+    int *jmax_host;              // its copy in page-locked host memory (device address), or null
     int k1_height;               // the stream-collide grid covers heights < k1_height (the rest is deep solid)
     const float *thw_nu;         // heated-wall field of the last streaming (Nusselt number)
     double *nu;                  // per-column Nusselt numbers (ncols)

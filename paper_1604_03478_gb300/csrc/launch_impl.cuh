@@ -124,8 +124,8 @@ cudaError_t Launch<ST>::front(const KP &p, int face, int inflight, int move, con
     ST *F = (ST *)b.F;
     const ST *G = (const ST *)b.G;
     if (face == 0)
-        return launch_step_kernel(k_front<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.thw_wr, inflight, move, b.status, b.jmax);
-    return launch_step_kernel(k_front<ST, 1>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.thw_wr, inflight, move, b.status, b.jmax);
+        return launch_step_kernel(k_front<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.thw_wr, inflight, move, b.status, b.jmax, b.jmax_host);
+    return launch_step_kernel(k_front<ST, 1>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.thw_wr, inflight, move, b.status, b.jmax, b.jmax_host);
 }
 
 template <typename ST>

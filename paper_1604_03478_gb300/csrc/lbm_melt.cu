@@ -206,6 +206,7 @@ Bufs bufs_at(lbm_melt *h, int cur, int inflight) {
     b.cblk = h->cblk;
     b.sms = h->sms;
     b.jmax = h->jmax_dev;
+    b.jmax_host = h->member ? nullptr : h->rb_val + lbm_melt::kRbTop;
     b.k1_height = h->kp.H;
     // the wall field of the last streaming: in flight, the one the pending
     // reads will apply; in the natural layout, the one the last odd step
@@ -331,9 +332,11 @@ lbm_status k1_height(lbm_melt *h, int *out) {
             CK(cudaEventSynchronize(h->rb_ev[slot]), "read-back wait");
             h->rb_synced = k;
         }
-        // the copy followed step rb_step (0-based): counts of the state the
-        // coming step reads exceed it by at most the steps in between
-        const long long b = (long long)h->rb_val[slot] + (h->exec_steps - h->rb_step[slot] - 1) + 3;
+        // the event (or copy) followed step rb_step (0-based): counts of the
+        // state the coming step reads exceed the maximum then, or a later
+        // one, by at most the steps in between
+        const int top = h->member ? h->rb_val[slot] : *(volatile int *)(h->rb_val + lbm_melt::kRbTop);
+        const long long b = (long long)top + (h->exec_steps - h->rb_step[slot] - 1) + 3;
         *out = b < H ? (int)b : H;
         return LBM_OK;
     }
@@ -346,18 +349,18 @@ lbm_status k1_height(lbm_melt *h, int *out) {
 void seed_readback(lbm_melt *h) {
     if (!h->kp.skip_deep) return;
     const int slot = (int)(h->rb_next % lbm_melt::kRbRing);
-    h->rb_val[slot] = h->rb_val[lbm_melt::kRbRing + 1];
+    h->rb_val[slot] = h->rb_val[lbm_melt::kRbTop] = h->rb_val[lbm_melt::kRbRing + 1];
     h->rb_step[slot] = h->exec_steps - 1;
     h->rb_synced = h->rb_next;
     h->rb_next++;
 }
 
-// After every kRbEvery-th step (or now, with force): copy the running
-// maximum into the next ring slot.
+// After every kRbEvery-th step (or now, with force): the next read-back.
 lbm_status jmax_readback(lbm_melt *h, bool force = false) {
     if (!h->kp.skip_deep || (!force && h->exec_steps % lbm_melt::kRbEvery)) return LBM_OK;
     const int slot = (int)(h->rb_next % lbm_melt::kRbRing);
-    CK(cudaMemcpyAsync(h->rb_val + slot, h->jmax_dev, sizeof(int), cudaMemcpyDeviceToHost, h->stream), "read-back");
+    if (h->member)
+        CK(cudaMemcpyAsync(h->rb_val + slot, h->jmax_dev, sizeof(int), cudaMemcpyDeviceToHost, h->stream), "read-back");
     CK(cudaEventRecord(h->rb_ev[slot], h->stream), "read-back event");
     h->rb_step[slot] = h->exec_steps - 1;
     h->rb_next++;
@@ -685,7 +688,7 @@ LBM_API lbm_status lbm_melt_create(const lbm_melt_grid *grid, double Ra, double 
     // small cavities are launch bound: replay their steps from graphs
     h->graph_steps = d.N <= kGraphMaxNodes ? kGraphSteps : 0;
     h->pairs_mode = -1;
-    const size_t rb_bytes = ((lbm_melt::kRbRing + lbm_melt::kFlags) * sizeof(int) + 127) / 128 * 128;
+    const size_t rb_bytes = ((lbm_melt::kRbTop + 1) * sizeof(int) + 127) / 128 * 128;
     if (cudaMallocHost(&h->rb_val, rb_bytes + lbm_melt::kHostOut * sizeof(double)) != cudaSuccess)
         return fail(LBM_ENOMEM);
     h->host_out = (double *)((unsigned char *)h->rb_val + rb_bytes);
