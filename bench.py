@@ -875,7 +875,7 @@ def run_gpu(args):
                 "d2h_bytes_per_step": ncols * 8 + 8, "steps": e2e_steps,
                 "read_back": "lbm_melt_get_async into alternating page-locked buffers, one sync at the end",
                 "synchronous_value": e2e_sync_value},
-        "gpu_launches": 3 * args.steps,
+        "gpu_launches": 2 * args.steps,
         "clocks": clk.summary(),
         "all_node_mlups": (units / n_liq) * (n ** 3) / (ms_max * 1e-3) / 1e6,
     }
