@@ -858,6 +858,7 @@ size_t state_layout(const lbm_melt *h, void *dev[9], size_t sz[9], size_t off[9]
 
 // copy the handle's state to (dir = 0) or from (dir = 1) a checkpoint buffer
 lbm_status move_state(lbm_melt *h, unsigned char *buf, int dir) {
+    if (dir) h->plain_next = 1;
     void *dev[9];
     size_t sz[9], off[9];
     state_layout(h, dev, sz, off);
@@ -874,6 +875,7 @@ lbm_status move_state(lbm_melt *h, unsigned char *buf, int dir) {
 // `boff` of the checkpoint); else the whole state.
 lbm_status move_checkpoint(lbm_melt *h, unsigned char *buf, size_t boff, int dir) {
     if (!h->kp.skip_deep) return move_state(h, buf, dir);
+    if (dir) h->plain_next = 1;
     void *dev[9];
     size_t sz[9], off[9];
     state_layout(h, dev, sz, off);

@@ -210,6 +210,7 @@ void advance_handles(lbm_ensemble *e, long long n) {
         if (n & 1) { h->cur ^= 1; h->inflight ^= 1; }
         if (n > 0) { h->thw_pending = 0; h->thw_last_prev = 0; }
         h->exec_steps += n;  // the launch kept the running maximum: host read-backs stay bounds
+        h->plain_next = 1;
     }
     e->steps += n;
 }

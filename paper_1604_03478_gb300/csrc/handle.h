@@ -52,6 +52,7 @@ struct lbm_melt {
     int bx, by;        // block shape of the per-node kernels (0: default)
     int cblk;          // threads per block of the per-column kernels
     int sms;           // SMs of the device
+    int plain_next;    // the stream's last work wrote what the step's kernels load early: the next one is launched plainly
     // Running maximum of the liquid counts, kept by k_front on the device;
     // stream-collide blocks at heights >= it + 3 (all deep solid) return at
     // once.  k_front raises a copy in page-locked memory with it, and the host

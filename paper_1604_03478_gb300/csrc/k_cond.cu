@@ -151,9 +151,10 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair_cond(
 }
 
 // The conduction step's kernels are launched like the plain step's, with
-// programmatic stream serialization (see step_launch_wait).
+// programmatic stream serialization (see step_launch_wait), or plainly (see
+// launch_step_kernel).
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_cond_kernel(void (*kern)(KArgs...), dim3 grd, dim3 blk, cudaStream_t st, Args... args) {
+static cudaError_t launch_cond_kernel(void (*kern)(KArgs...), dim3 grd, dim3 blk, cudaStream_t st, int plain, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grd;
     cfg.blockDim = blk;
@@ -162,7 +163,7 @@ static cudaError_t launch_cond_kernel(void (*kern)(KArgs...), dim3 grd, dim3 blk
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = plain ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
@@ -171,11 +172,11 @@ template <typename ST, typename IX, int LIN>
 static cudaError_t launch_pair_cond(const KP &p, int face, int odd, const Bufs &b, dim3 g2, dim3 blk, cudaStream_t st) {
     ST *F = (ST *)b.F, *G = (ST *)b.G;
     if (face == 0) {
-        if (odd) return launch_cond_kernel(k_odd_pair_cond<ST, 0, IX, LIN>, g2, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
-        else return launch_cond_kernel(k_even_pair_cond<ST, 0, IX, LIN>, g2, blk, st, p, F, G, b.js, b.nb, b.gpost, b.spost);
+        if (odd) return launch_cond_kernel(k_odd_pair_cond<ST, 0, IX, LIN>, g2, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
+        else return launch_cond_kernel(k_even_pair_cond<ST, 0, IX, LIN>, g2, blk, st, b.plain, p, F, G, b.js, b.nb, b.gpost, b.spost);
     } else {
-        if (odd) return launch_cond_kernel(k_odd_pair_cond<ST, 1, IX, LIN>, g2, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
-        else return launch_cond_kernel(k_even_pair_cond<ST, 1, IX, LIN>, g2, blk, st, p, F, G, b.js, b.nb, b.gpost, b.spost);
+        if (odd) return launch_cond_kernel(k_odd_pair_cond<ST, 1, IX, LIN>, g2, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
+        else return launch_cond_kernel(k_even_pair_cond<ST, 1, IX, LIN>, g2, blk, st, b.plain, p, F, G, b.js, b.nb, b.gpost, b.spost);
     }
 }
 
@@ -193,11 +194,11 @@ cudaError_t LaunchCond<ST>::stream_collide(const KP &p, int face, int odd, const
     }
     const dim3 grd = k1_grid(p, blk, face, p.H, b.linear);
     if (face == 0) {
-        if (odd) return launch_cond_kernel(k_odd_cond<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
-        else return launch_cond_kernel(k_even_cond<ST, 0>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, b.spost);
+        if (odd) return launch_cond_kernel(k_odd_cond<ST, 0>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
+        else return launch_cond_kernel(k_even_cond<ST, 0>, grd, blk, st, b.plain, p, F, G, b.js, b.nb, b.gpost, b.spost);
     } else {
-        if (odd) return launch_cond_kernel(k_odd_cond<ST, 1>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
-        else return launch_cond_kernel(k_even_cond<ST, 1>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, b.spost);
+        if (odd) return launch_cond_kernel(k_odd_cond<ST, 1>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
+        else return launch_cond_kernel(k_even_cond<ST, 1>, grd, blk, st, b.plain, p, F, G, b.js, b.nb, b.gpost, b.spost);
     }
 }
 
@@ -207,9 +208,9 @@ cudaError_t LaunchCond<ST>::front(const KP &p, int face, int inflight, int move,
     ST *F = (ST *)b.F;
     const ST *G = (const ST *)b.G;
     if (face == 0)
-        return launch_cond_kernel(k_front_cond<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost,
+        return launch_cond_kernel(k_front_cond<ST, 0>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost,
                                   b.spost, b.thw_wr, inflight, move, b.status);
-    return launch_cond_kernel(k_front_cond<ST, 1>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.spost,
+    return launch_cond_kernel(k_front_cond<ST, 1>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.spost,
                               b.thw_wr, inflight, move, b.status);
 }
 

@@ -32,6 +32,7 @@ struct Bufs {
     int pairs;                   // stream-collide with two nodes per thread (even nx)
     int linear;                  // stream-collide blocks of consecutive columns (k1_linear)
     int early_pairs;             // ... with the first wave's loads before the wait (FP32 storage, middle sizes)
+    int plain;                   // launch without programmatic serialization (launch_step_kernel)
 };
 
 // Where a step leaves the natural-layout snapshot of the state it starts from

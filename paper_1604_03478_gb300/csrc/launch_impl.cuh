@@ -8,12 +8,16 @@
 namespace lbm {
 
 // The step's kernels (stream-collide, front) are launched with
-// programmatic stream serialization (see step_launch_wait) when LBM_PDL.
+// programmatic stream serialization (see step_launch_wait) when LBM_PDL, but
+// plainly (`plain`) after a kernel that is not one of them and writes what
+// this one loads before its wait (a wall field, fronts, a restored state):
+// such a kernel lets its successor start when its blocks have returned, which
+// does not order its stores before loads that no wait precedes.
 #ifndef LBM_PDL
 #define LBM_PDL 1
 #endif
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_step_kernel(void (*kern)(KArgs...), dim3 grd, dim3 blk, cudaStream_t st, Args... args) {
+static cudaError_t launch_step_kernel(void (*kern)(KArgs...), dim3 grd, dim3 blk, cudaStream_t st, int plain, Args... args) {
 #if LBM_PDL
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grd;
@@ -23,7 +27,7 @@ static cudaError_t launch_step_kernel(void (*kern)(KArgs...), dim3 grd, dim3 blk
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = plain ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, kern, args...);
 #else
     kern<<<grd, blk, 0, st>>>(args...);
@@ -39,11 +43,11 @@ static cudaError_t launch_sc(const KP &p, int face, int odd, const Bufs &b, dim3
     const int *jm = p.skip_deep ? b.jmax : nullptr;
     ST *F = (ST *)b.F, *G = (ST *)b.G;
     if (face == 0) {
-        if (odd) return launch_step_kernel(k_odd<ST, 0, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early, b.s, snap);
-        else return launch_step_kernel(k_even<ST, 0, IXE, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early, b.s, snap);
+        if (odd) return launch_step_kernel(k_odd<ST, 0, SNAP>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early, b.s, snap);
+        else return launch_step_kernel(k_even<ST, 0, IXE, SNAP>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early, b.s, snap);
     } else {
-        if (odd) return launch_step_kernel(k_odd<ST, 1, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early, b.s, snap);
-        else return launch_step_kernel(k_even<ST, 1, IXE, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early, b.s, snap);
+        if (odd) return launch_step_kernel(k_odd<ST, 1, SNAP>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early, b.s, snap);
+        else return launch_step_kernel(k_even<ST, 1, IXE, SNAP>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early, b.s, snap);
     }
 }
 
@@ -57,11 +61,11 @@ static cudaError_t launch_sc_pair_early(const KP &p, int face, int odd, const Bu
     const int *jm = p.skip_deep ? b.jmax : nullptr;
     ST *F = (ST *)b.F, *G = (ST *)b.G;
     if (face == 0) {
-        if (odd) return launch_step_kernel(k_odd_pair_early<ST, 0, IX, LIN, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early, b.s, snap);
-        else return launch_step_kernel(k_even_pair_early<ST, 0, IX, LIN, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early, b.s, snap);
+        if (odd) return launch_step_kernel(k_odd_pair_early<ST, 0, IX, LIN, SNAP>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early, b.s, snap);
+        else return launch_step_kernel(k_even_pair_early<ST, 0, IX, LIN, SNAP>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early, b.s, snap);
     } else {
-        if (odd) return launch_step_kernel(k_odd_pair_early<ST, 1, IX, LIN, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early, b.s, snap);
-        else return launch_step_kernel(k_even_pair_early<ST, 1, IX, LIN, SNAP>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early, b.s, snap);
+        if (odd) return launch_step_kernel(k_odd_pair_early<ST, 1, IX, LIN, SNAP>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.nb_next, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm, early, b.s, snap);
+        else return launch_step_kernel(k_even_pair_early<ST, 1, IX, LIN, SNAP>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, jm, early, b.s, snap);
     }
 }
 
@@ -82,11 +86,11 @@ static cudaError_t launch_sc_pair(const KP &p, int face, int odd, const Bufs &b,
         }
     }
     if (face == 0) {
-        if (odd) return launch_step_kernel(k_odd_pair<ST, 0, IXO, LIN>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
-        else return launch_step_kernel(k_even_pair<ST, 0, IXE, LIN>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, jm);
+        if (odd) return launch_step_kernel(k_odd_pair<ST, 0, IXO, LIN>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
+        else return launch_step_kernel(k_even_pair<ST, 0, IXE, LIN>, grd, blk, st, b.plain, p, F, G, b.js, b.nb, b.gpost, jm);
     } else {
-        if (odd) return launch_step_kernel(k_odd_pair<ST, 1, IXO, LIN>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
-        else return launch_step_kernel(k_even_pair<ST, 1, IXE, LIN>, grd, blk, st, p, F, G, b.js, b.nb, b.gpost, jm);
+        if (odd) return launch_step_kernel(k_odd_pair<ST, 1, IXO, LIN>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, jm);
+        else return launch_step_kernel(k_even_pair<ST, 1, IXE, LIN>, grd, blk, st, b.plain, p, F, G, b.js, b.nb, b.gpost, jm);
     }
 }
 
@@ -124,8 +128,8 @@ cudaError_t Launch<ST>::front(const KP &p, int face, int inflight, int move, con
     ST *F = (ST *)b.F;
     const ST *G = (const ST *)b.G;
     if (face == 0)
-        return launch_step_kernel(k_front<ST, 0>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.thw_wr, inflight, move, b.status, b.jmax, b.jmax_host);
-    return launch_step_kernel(k_front<ST, 1>, grd, blk, st, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.thw_wr, inflight, move, b.status, b.jmax, b.jmax_host);
+        return launch_step_kernel(k_front<ST, 0>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.thw_wr, inflight, move, b.status, b.jmax, b.jmax_host);
+    return launch_step_kernel(k_front<ST, 1>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.thw_wr, inflight, move, b.status, b.jmax, b.jmax_host);
 }
 
 template <typename ST>

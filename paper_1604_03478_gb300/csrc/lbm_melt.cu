@@ -207,6 +207,7 @@ Bufs bufs_at(lbm_melt *h, int cur, int inflight) {
     b.sms = h->sms;
     b.jmax = h->jmax_dev;
     b.jmax_host = h->member ? nullptr : h->rb_val + lbm_melt::kRbTop;
+    b.plain = 0;
     b.k1_height = h->kp.H;
     // the wall field of the last streaming: in flight, the one the pending
     // reads will apply; in the natural layout, the one the last odd step
@@ -231,6 +232,7 @@ Bufs bufs(lbm_melt *h) { return bufs_at(h, h->cur, h->inflight); }
 // liquid counts js (front held, no flip); both count buffers hold js after it.
 lbm_status refresh_front(lbm_melt *h) {
     Bufs b = bufs(h);
+    b.plain = 1;
     CK(LAUNCH(h, front, h->kp, h->face, h->inflight, 0, b, h->stream), "front refresh");
     h->cur ^= 1;
     return LBM_OK;
@@ -447,6 +449,8 @@ cudaError_t enqueue_step(lbm_melt *h, int &cur, int &inflight, int height, dim3 
                          const lbm::SnapOut *snap = nullptr) {
     Bufs b = bufs_at(h, cur, inflight);
     b.k1_height = height;
+    b.plain = h->plain_next;
+    h->plain_next = 0;
     const int odd = inflight;
     cudaError_t e = LAUNCH(h, stream_collide, h->kp, h->face, odd, b, blk, st, snap);
     if (e != cudaSuccess) return e;
@@ -578,6 +582,7 @@ cudaError_t initial_state(lbm_melt *h) {
         h->cur = 0;
         h->inflight = 0;
         Bufs b = bufs(h);
+        b.plain = 1;
         e = LAUNCH(h, front, p, h->face, 0, 0, b, h->stream);
         if (e == cudaSuccess) {
             h->cur = 1;
@@ -768,6 +773,8 @@ LBM_API lbm_status lbm_melt_step(lbm_melt *h, long long n) {
             h->ev_used += 2;
             CK(cudaEventRecord(evp[0], h->stream), "event record");
         }
+        b.plain = h->plain_next;
+        h->plain_next = 0;
         CK(LAUNCH(h, stream_collide, h->kp, h->face, odd, b, blk, h->stream), "stream-collide");
         if (evp) CK(cudaEventRecord(evp[1], h->stream), "event record");
         h->inflight = !odd;
@@ -1010,6 +1017,7 @@ LBM_API lbm_status lbm_melt_set_hot_wall(lbm_melt *h, const float *T_h_field, in
     if (h->inflight) h->thw_pending = 1;
     else h->thw_last_prev = 1;
     h->thw_gen++;
+    h->plain_next = 1;
     return src ? LBM_OK : copy_in(h, h->thw_cur, T_h_field, nc * 4, ptr_kind);
 }
 
