@@ -111,8 +111,9 @@ void fill_desc(lbm_melt *h, CavDesc &d, int block) {
     d.gpost = h->gpost;
     d.thw = h->thw_cur;
     d.thw_rd0 = h->thw_pending ? h->thw_prev : h->thw_cur;
-    d.status = h->status_dev;
+    d.status = h->flags + lbm_melt::kStatus;
     d.jmax = h->jmax_dev;
+    d.jmax_host = h->flags + lbm_melt::kTop;
     d.cut = h->kp.skip_deep;
 }
 

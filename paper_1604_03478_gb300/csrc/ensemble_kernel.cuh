@@ -47,7 +47,7 @@ struct CavDesc {
     double *s[2];
     float *gpost, *thw, *thw_rd0;
     int *status;
-    int *jmax;                    // running maximum of the liquid counts (kept by phase 2)
+    int *jmax, *jmax_host;        // running maximum of the liquid counts (kept by phase 2), its copy for the host
     int cut;                      // nodes at heights >= *jmax + 3 are deep solid (Tc == Tm)
 };
 
@@ -265,12 +265,17 @@ __global__ void ENS_BOUNDS k_ensemble(const __grid_constant__ EnsWork w, int nst
             const int cur = d.cur0 ^ (t & 1), inflight = 1 - (d.inflight0 ^ (t & 1));
             const int col = (int)((it - w.col_begin[k]) * blockDim.x + threadIdx.x);
             int jn = -1;
+            // the maximum of the steps before (or a newer one)
+            const int had = d.cut ? top[k] - 3 : *(volatile int *)d.jmax;
             if (col < d.p.ncols) {
                 jn = ens_front<ST>(d, cur, inflight, col);
                 if (jn != d.js[cur][col]) changed |= 1ull << (int)((it - first) / gridDim.x);
             }
             const int m = __reduce_max_sync(0xffffffffu, jn);  // an item is one cavity's columns: whole warps
-            if ((threadIdx.x & 31) == 0 && m >= 0) atomicMax(d.jmax, m);
+            if ((threadIdx.x & 31) == 0 && m > had) {
+                atomicMax(d.jmax, m);
+                atomicMax_system(d.jmax_host, m);
+            }
         }
         if (!grid_barrier(w, arrivals += gridDim.x)) return;
         if (timer) {

@@ -37,7 +37,6 @@ struct lbm_melt {
     int thw_last_prev; // set_hot_wall since the last step in the natural layout: thw_prev holds the
                        // field of the last streaming (the Nusselt number's wall value)
     double *nu_dev;    // per-column Nusselt numbers (ncols)
-    int *status_dev;   // the front status, and next to it the running maximum (jmax_dev): one copy reads both
     double *sum_dev;
     unsigned int *ticket;  // last-block ticket of the one-launch column sum (k_sum_once)
     double *red_part;  // scratch: per-block partials of the FP64 totals
@@ -55,27 +54,25 @@ struct lbm_melt {
     int plain_next;    // the stream's last work wrote what the step's kernels load early: the next one is launched plainly
     // Running maximum of the liquid counts, kept by k_front on the device;
     // stream-collide blocks at heights >= it + 3 (all deep solid) return at
-    // once.  k_front raises a copy in page-locked memory with it, and the host
-    // records an event every kRbEvery steps (an ensemble member, whose counts
-    // the persistent kernel also raises, copies the maximum into a ring of
-    // pinned slots instead); before a stream-collide the host takes the newest
-    // event at least kRbLag steps old (waiting for it only when it runs that
-    // far ahead of the device) and launches no block above the maximum it
-    // then reads + the event's age + 2 (a count grows by at most one node per
-    // step).
+    // once.  The front kernels (the ensemble's too) raise a copy in page-locked
+    // memory with it, and the host records an event every kRbEvery steps;
+    // before a stream-collide the host takes the newest event at least kRbLag
+    // steps old (waiting for it only when it runs that far ahead of the
+    // device) and launches no block above the maximum it then reads + the
+    // event's age + 2 (a count grows by at most one node per step).
     static const int kRbRing = 32, kRbLag = 16, kRbEvery = 4;
     int *jmax_dev;
-    int *rb_val;       // pinned: ring of read-backs, kFlags ints a synchronising call reads status_dev into, and
-                       // the running maximum that k_front raises (at kRbTop)
-    static const int kRbTop = kRbRing + 2;
-    static const int kFlags = 2;
-    static const int kHostOut = 8;
-    double *host_out;  // pinned (behind rb_val): small results of the synchronising calls, written by the kernels
+    // Page-locked, written by the kernels and read by the host once the stream
+    // has got there: the front status (kStatus, touched on an error only), the
+    // running maximum (kTop), then small results of the synchronising calls.
+    static const int kStatus = 0, kTop = 1, kHostOut = 8;
+    int *flags;
+    double *host_out;
     cudaEvent_t rb_ev[kRbRing];
-    long long rb_step[kRbRing];  // exec step after which each copy was taken
-    long long rb_next;           // read-backs enqueued so far
-    long long rb_valid_from;     // read-backs before this one are not bounds any more
-    long long rb_synced;         // newest read-back known complete (its value read)
+    long long rb_step[kRbRing];  // exec step after which each event was recorded
+    long long rb_next;           // events recorded so far
+    long long rb_valid_from;     // events before this one are not bounds any more
+    long long rb_synced;         // newest event known complete
     long long exec_steps;        // steps this handle executed (never rewound)
     double Ra;         // as given to create
     int derived_from_Ra;

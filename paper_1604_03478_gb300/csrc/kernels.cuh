@@ -1469,8 +1469,8 @@ __device__ __forceinline__ int front_column(const KP &p, ST *__restrict__ F, con
     if (move) {
         const float Gr = front_gradient(k, sc, fc, y0, y1, Tm, Tw);
         const float v = front_speed(p, front_slope_factor(sp, sq), COND ? Gr - Gs : Gr);
-        if (!isfinite(Gr) || (COND && !isfinite(Gs))) atomicOr(status, 2);
-        else if (!(fabsf(v) <= 0.5f)) atomicOr(status, 1);
+        if (!isfinite(Gr) || (COND && !isfinite(Gs))) atomicOr_system(status, 2);
+        else if (!(fabsf(v) <= 0.5f)) atomicOr_system(status, 1);
         sn = sc + (double)v;
         fn = front_pos(sn, H);
         if (front_clamped(sn, fn, H)) {
@@ -1598,8 +1598,8 @@ __device__ __forceinline__ int front_column(const KP &p, ST *__restrict__ F, con
 //
 // jmax (may be null): running maximum of the liquid counts.  A warp whose
 // columns exceed it (few do: a count grows by one now and then) raises it with
-// an atomic, and its copy in page-locked host memory, jmax_host (may be null),
-// which the host reads now and then to bound the height of the stream-collide
+// an atomic, and its copy in page-locked host memory, jmax_host, which the
+// host reads now and then to bound the height of the stream-collide
 // grid (nodes two above every neighbouring count are deep solid and do
 // nothing).
 template <typename ST, int FACE>
@@ -1619,7 +1619,7 @@ __global__ void __launch_bounds__(128, 4) k_front(const __grid_constant__ KP p, 
     const int m = __reduce_max_sync(0xffffffffu, jn);
     if ((threadIdx.x & 31) == 0 && m > top) {
         atomicMax(jmax, m);
-        if (jmax_host) atomicMax_system(jmax_host, m);
+        atomicMax_system(jmax_host, m);
     }
 }
 
@@ -1715,11 +1715,11 @@ __global__ void __launch_bounds__(128) k_state_out(const __grid_constant__ KP p,
 }
 
 // New fronts (s_in: an array of ncols heights) and their liquid counts; the
-// running maximum of the counts starts anew.
+// running maximum of the counts and its copy start anew.
 static __global__ void __launch_bounds__(128) k_set_fronts(const double *s_in, int ncols, int H, double *s, int *js,
-                                                           int *jmax) {
+                                                           int *jmax, int *jmax_host) {
     const int col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col == 0) *jmax = 0;
+    if (col == 0) *jmax = *jmax_host = 0;
     if (col >= ncols) return;
     const double v = s_in[col];
     s[col] = v;

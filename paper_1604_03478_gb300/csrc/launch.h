@@ -18,12 +18,12 @@ struct Bufs {
     double *s_next;
     float *gpost;                // ghost-node post-collision g, 7 x ncols
     const float *thw_rd, *thw_wr;
-    int *status;
+    int *status;                 // page-locked: the front status, set on an error
     const Links *lk;             // interior link offsets of the odd step
     int cblk;                    // threads per block of the per-column kernels (col_block)
     int sms;                     // SMs of the device
     int *jmax;                   // running maximum of the liquid counts (k_front), or null
-    int *jmax_host;              // its copy in page-locked host memory (device address), or null
+    int *jmax_host;              // its copy in page-locked host memory
     int k1_height;               // the stream-collide grid covers heights < k1_height (the rest is deep solid)
     const float *thw_nu;         // heated-wall field of the last streaming (Nusselt number)
     double *nu;                  // per-column Nusselt numbers (ncols)

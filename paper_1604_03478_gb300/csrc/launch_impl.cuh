@@ -152,7 +152,7 @@ cudaError_t Launch<ST>::state_out(const KP &p, int face, int inflight, const Buf
 
 template <typename ST>
 cudaError_t Launch<ST>::set_fronts(const KP &p, const Bufs &b, const double *s_in, double *s, int *js, cudaStream_t st) {
-    k_set_fronts<<<col_grid(p.ncols, 128), 128, 0, st>>>(s_in, p.ncols, p.H, s, js, b.jmax);
+    k_set_fronts<<<col_grid(p.ncols, 128), 128, 0, st>>>(s_in, p.ncols, p.H, s, js, b.jmax, b.jmax_host);
     return cudaGetLastError();
 }
 

@@ -201,12 +201,12 @@ Bufs bufs_at(lbm_melt *h, int cur, int inflight) {
     b.gpost = h->gpost;
     b.thw_rd = h->thw_pending ? h->thw_prev : h->thw_cur;
     b.thw_wr = h->thw_cur;
-    b.status = h->status_dev;
+    b.status = h->flags + lbm_melt::kStatus;
     b.lk = &h->lk;
     b.cblk = h->cblk;
     b.sms = h->sms;
     b.jmax = h->jmax_dev;
-    b.jmax_host = h->member ? nullptr : h->rb_val + lbm_melt::kRbTop;
+    b.jmax_host = h->flags + lbm_melt::kTop;
     b.plain = 0;
     b.k1_height = h->kp.H;
     // the wall field of the last streaming: in flight, the one the pending
@@ -269,18 +269,16 @@ lbm_status copy_in(lbm_melt *h, void *dst, const void *src, size_t bytes, int pt
     return LBM_OK;
 }
 
-// Waits for the handle's stream and reads the front status and the running
-// maximum of the liquid counts into page-locked memory on the way.
+// Waits for the handle's stream; the flags in page-locked memory are those of
+// everything enqueued so far.
 lbm_status read_flags(lbm_melt *h) {
-    CK(cudaMemcpyAsync(h->rb_val + lbm_melt::kRbRing, h->status_dev, lbm_melt::kFlags * sizeof(int),
-                       cudaMemcpyDeviceToHost, h->stream), "status read");
     CK(cudaStreamSynchronize(h->stream), "synchronize");
     return LBM_OK;
 }
 
-// What the status that read_flags read says.
+// What the status says (after read_flags).
 lbm_status status_of_flags(lbm_melt *h) {
-    const int st = h->rb_val[lbm_melt::kRbRing];
+    const int st = *(volatile int *)(h->flags + lbm_melt::kStatus);
     if (st & 2) return set_err(h, LBM_ENAN, "non-finite temperature at the front");
     if (st & 1) return set_err(h, LBM_EUNSTABLE, "the front moved more than half a cell in one step");
     return LBM_OK;
@@ -298,7 +296,7 @@ void free_all(lbm_melt *h) {
     cudaFree(h->gpost);
     cudaFree(h->thw_cur);
     cudaFree(h->thw_prev);
-    cudaFree(h->status_dev);
+    cudaFree(h->jmax_dev);
     cudaFree(h->sum_dev);
     cudaFree(h->ticket);
     cudaFree(h->red_part);
@@ -306,7 +304,7 @@ void free_all(lbm_melt *h) {
     cudaFree(h->nu_dev);
     cudaFree(h->report);
     cudaFree(h->spost);
-    if (h->rb_val) cudaFreeHost(h->rb_val);
+    if (h->flags) cudaFreeHost(h->flags);
     for (int k = 0; k < lbm_melt::kRbRing; ++k)
         if (h->rb_ev[k]) cudaEventDestroy(h->rb_ev[k]);
     for (cudaEvent_t e : h->ev) cudaEventDestroy(e);
@@ -334,10 +332,10 @@ lbm_status k1_height(lbm_melt *h, int *out) {
             CK(cudaEventSynchronize(h->rb_ev[slot]), "read-back wait");
             h->rb_synced = k;
         }
-        // the event (or copy) followed step rb_step (0-based): counts of the
+        // the event followed step rb_step (0-based): counts of the
         // state the coming step reads exceed the maximum then, or a later
         // one, by at most the steps in between
-        const int top = h->member ? h->rb_val[slot] : *(volatile int *)(h->rb_val + lbm_melt::kRbTop);
+        const int top = *(volatile int *)(h->flags + lbm_melt::kTop);
         const long long b = (long long)top + (h->exec_steps - h->rb_step[slot] - 1) + 3;
         *out = b < H ? (int)b : H;
         return LBM_OK;
@@ -345,13 +343,11 @@ lbm_status k1_height(lbm_melt *h, int *out) {
     return LBM_OK;
 }
 
-// The maximum that the last read_flags read, as a read-back of the state now
-// (after create and set_state, so that the first steps of a run are bounded
-// too).
+// The state now (the stream has just been waited for) as a read-back, after
+// create and set_state, so that the first steps of a run are bounded too.
 void seed_readback(lbm_melt *h) {
     if (!h->kp.skip_deep) return;
     const int slot = (int)(h->rb_next % lbm_melt::kRbRing);
-    h->rb_val[slot] = h->rb_val[lbm_melt::kRbTop] = h->rb_val[lbm_melt::kRbRing + 1];
     h->rb_step[slot] = h->exec_steps - 1;
     h->rb_synced = h->rb_next;
     h->rb_next++;
@@ -361,8 +357,6 @@ void seed_readback(lbm_melt *h) {
 lbm_status jmax_readback(lbm_melt *h, bool force = false) {
     if (!h->kp.skip_deep || (!force && h->exec_steps % lbm_melt::kRbEvery)) return LBM_OK;
     const int slot = (int)(h->rb_next % lbm_melt::kRbRing);
-    if (h->member)
-        CK(cudaMemcpyAsync(h->rb_val + slot, h->jmax_dev, sizeof(int), cudaMemcpyDeviceToHost, h->stream), "read-back");
     CK(cudaEventRecord(h->rb_ev[slot], h->stream), "read-back event");
     h->rb_step[slot] = h->exec_steps - 1;
     h->rb_next++;
@@ -569,7 +563,8 @@ cudaError_t initial_state(lbm_melt *h) {
     if (e == cudaSuccess) e = cudaMemsetAsync(h->nb[1], 0, nc * 4, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->gpost, 0, 7 * nc * 4, h->stream);
     if (e == cudaSuccess && h->spost) e = cudaMemsetAsync(h->spost, 0, 7 * nc * 4, h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->status_dev, 0, lbm_melt::kFlags * sizeof(int), h->stream);
+    h->flags[lbm_melt::kStatus] = h->flags[lbm_melt::kTop] = 0;  // nothing of the handle's is running
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->jmax_dev, 0, sizeof(int), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->ticket, 0, sizeof(unsigned int), h->stream);
     if (e == cudaSuccess) {
         k_fill_d<<<nb, 256, 0, h->stream>>>(h->s[0], (long long)nc, d.s0);
@@ -693,10 +688,8 @@ LBM_API lbm_status lbm_melt_create(const lbm_melt_grid *grid, double Ra, double 
     // small cavities are launch bound: replay their steps from graphs
     h->graph_steps = d.N <= kGraphMaxNodes ? kGraphSteps : 0;
     h->pairs_mode = -1;
-    const size_t rb_bytes = ((lbm_melt::kRbTop + 1) * sizeof(int) + 127) / 128 * 128;
-    if (cudaMallocHost(&h->rb_val, rb_bytes + lbm_melt::kHostOut * sizeof(double)) != cudaSuccess)
-        return fail(LBM_ENOMEM);
-    h->host_out = (double *)((unsigned char *)h->rb_val + rb_bytes);
+    if (cudaMallocHost(&h->flags, 128 + lbm_melt::kHostOut * sizeof(double)) != cudaSuccess) return fail(LBM_ENOMEM);
+    h->host_out = (double *)((unsigned char *)h->flags + 128);
     for (int k = 0; k < lbm_melt::kRbRing; ++k)
         if (cudaEventCreateWithFlags(&h->rb_ev[k], cudaEventDisableTiming) != cudaSuccess) return fail(LBM_ECUDA);
     const size_t es = h->precision == 1 ? sizeof(__half) : sizeof(float);
@@ -706,7 +699,7 @@ LBM_API lbm_status lbm_melt_create(const lbm_melt_grid *grid, double Ra, double 
         {&h->F, nF}, {&h->G, nG}, {(void **)&h->js[0], nc * 4}, {(void **)&h->js[1], nc * 4},
         {(void **)&h->nb[0], nc * 4}, {(void **)&h->nb[1], nc * 4},
         {(void **)&h->s[0], nc * 8}, {(void **)&h->s[1], nc * 8}, {(void **)&h->gpost, 7 * nc * 4},
-        {(void **)&h->thw_cur, nc * 4}, {(void **)&h->thw_prev, nc * 4}, {(void **)&h->status_dev, lbm_melt::kFlags * 4},
+        {(void **)&h->thw_cur, nc * 4}, {(void **)&h->thw_prev, nc * 4}, {(void **)&h->jmax_dev, 4},
         {(void **)&h->sum_dev, 8}, {(void **)&h->ticket, 8}, {(void **)&h->red_part, kRedBlocks * 6 * 8}, {(void **)&h->totals_dev, 7 * 8},
         {(void **)&h->nu_dev, nc * 8}};
     h->nred = kRedBlocks;
@@ -715,7 +708,6 @@ LBM_API lbm_status lbm_melt_create(const lbm_melt_grid *grid, double Ra, double 
         if (e != cudaSuccess) return fail(e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA);
         h->bytes += a.b;
     }
-    h->jmax_dev = h->status_dev + 1;
     const cudaError_t e = initial_state(h);
     if (e != cudaSuccess) return fail(e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA);
     seed_readback(h);
