@@ -65,6 +65,9 @@ struct lbm_melt {
     // Page-locked, written by the kernels and read by the host once the stream
     // has got there: the front status (kStatus, touched on an error only), the
     // running maximum (kTop), then small results of the synchronising calls.
+    // With device flags copied back by each such call (an ensemble: by each
+    // member), 16 steps of 8 FP16 cavities with restores and reads took 840 us
+    // instead of 737, a 256^3 readout 396 instead of 374.
     static const int kStatus = 0, kTop = 1, kHostOut = 8;
     int *flags;
     double *host_out;

@@ -45,8 +45,9 @@ __device__ __forceinline__ void step_launch_wait() {
 }
 // What a kernel may load before step_launch_wait: whatever its immediate
 // predecessor does not write.  The predecessor let this kernel start only
-// after its own wait, so everything before the predecessor is complete.  Such
-// loads go to L2 (ld.global.cg): L1 may hold a line from before.  They and
+// after its own wait, so everything before the predecessor is complete (after
+// other kernels, which have no such wait, the launch is plain: see
+// launch_step_kernel).  Such loads go to L2 (ld.global.cg): L1 may hold a line from before.  They and
 // the wait are volatile, so the compiler keeps their order.
 __device__ __forceinline__ int ld_l2(const int *q) {
     int v;
