@@ -312,7 +312,8 @@ void lbm_melt_destroy(lbm_melt *h);
    dL/d(g beta)} (coef = alpha Ste / (Th - Tm), the Eq. 6 factor; dL/dRa
    chains these through the parameter map of lbm_melt_derive).  Segments are
    recomputed from their checkpoints with one snapshot per step, then
-   reversed; the handle is back in its final state afterwards.  Synchronises.
+   reversed; the handle is back in the state it had before the call (the run's
+   final one, or whatever was stepped to or uploaded since).  Synchronises.
    Returns LBM_EUNSTABLE (or LBM_ENAN) without computing anything when the
    front status of the handle is flagged: the reverse sweep relies on fronts
    that moved at most half a node per step; and LBM_EINVAL when the

@@ -739,6 +739,13 @@ __global__ void __launch_bounds__(256) k_ckpt_move(const __grid_constant__ KP p,
     }
 }
 
+// Raises the running maximum liquid count and its copy in page-locked host
+// memory (written together, as by the front kernels) to a recorded run's.
+__global__ void k_raise_top(const int *top, int *jmax, int *jmax_host) {
+    atomicMax(jmax, *top);
+    atomicMax_system(jmax_host, *top);
+}
+
 }  // namespace lbm
 
 // ------------------------------------------------------------------ tape
@@ -750,6 +757,7 @@ struct lbm_tape {
     std::vector<void *> ck;          // device checkpoints, one per segment (in the workspace's pool)
     std::vector<int> ck_cur, ck_inflight;
     std::vector<long long> ck_steps;
+    int *top;                        // device: the running maximum liquid count at the end of the run
 };
 
 // The adjoint's device buffers, kept with the handle from one gradient to
@@ -946,12 +954,13 @@ LBM_API lbm_status lbm_melt_tape_forward(lbm_melt *h, long long steps, long long
     t->ck_bytes = t->ck_bound_off + 256;  // + the recorded height bound
     void *pool = nullptr;
     {
-        const cudaError_t e = ws_alloc(h, kSlotCheckpoints, (size_t)t->nseg * t->ck_bytes, &pool);
+        const cudaError_t e = ws_alloc(h, kSlotCheckpoints, (size_t)t->nseg * t->ck_bytes + 256, &pool);
         if (e != cudaSuccess) {
             free_tape(h);
             return tape_err(h, LBM_ENOMEM, "%lld checkpoints: %s", t->nseg, cudaGetErrorString(e));
         }
     }
+    t->top = (int *)((unsigned char *)pool + (size_t)t->nseg * t->ck_bytes);
     for (long long sgm = 0; sgm < t->nseg; ++sgm) {
         void *buf = (unsigned char *)pool + (size_t)sgm * t->ck_bytes;
         t->ck.push_back(buf);
@@ -964,6 +973,8 @@ LBM_API lbm_status lbm_melt_tape_forward(lbm_melt *h, long long steps, long long
         st = lbm_melt_step(h, n);
         if (st != LBM_OK) return st;
     }
+    // the handle's own maximum starts anew with the next uploaded state
+    TCK(cudaMemcpyAsync(t->top, h->jmax_dev, sizeof(int), cudaMemcpyDeviceToDevice, h->stream), "liquid-count maximum");
     return LBM_OK;
 }
 
@@ -990,8 +1001,9 @@ LBM_API lbm_status lbm_melt_tape_backward(lbm_melt *h, const double *seed, doubl
     const size_t nc = (size_t)p.ncols;
     const long long C = t->C;
     const dim3 blk = lbm::node_block(p);
-    // Every level of the recorded run has liquid counts at most the running
-    // maximum; the snapshot and the node adjoint touch nothing three or more
+    // Every level of the recorded run has liquid counts at most its running
+    // maximum (the handle's may be lower: a state uploaded since starts it
+    // anew); the snapshot and the node adjoint touch nothing three or more
     // nodes above it (deep solid), so their grids stop there, and so do the
     // snapshots and the adjoint fields: they are laid out for a cavity of
     // those heights (pa; the walls of the other axes and the columns are the
@@ -1000,7 +1012,7 @@ LBM_API lbm_status lbm_melt_tape_backward(lbm_melt *h, const double *seed, doubl
     int abound = p.H;
     if (p.skip_deep) {
         int jm = 0;
-        if (cudaMemcpy(&jm, h->jmax_dev, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+        if (cudaMemcpy(&jm, t->top, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
             return tape_err(h, LBM_ECUDA, "liquid-count maximum");
         abound = std::min(p.H, jm + 3);
     }
@@ -1084,6 +1096,9 @@ LBM_API lbm_status lbm_melt_tape_backward(lbm_melt *h, const double *seed, doubl
         BCK(cudaMemsetAsync(snap_jsb[1], 0, (size_t)(C + 1) * nc * 4, h->stream), "zero");
         BCK(cudaMemsetAsync(snap_nbb[1], 0, (size_t)(C + 1) * nc * 4, h->stream), "zero");
     }
+    // the recomputed steps cut their grids at the handle's maximum
+    lbm::k_raise_top<<<1, 1, 0, h->stream>>>(t->top, h->jmax_dev, h->flags + lbm_melt::kTop);
+    BCK(cudaGetLastError(), "liquid-count maximum");
     BCK(cudaMemcpyAsync(lams[1], seed, nc * 8, ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                         h->stream), "seed");
     // A segment's recomputation: snapshot of its first level, then the
