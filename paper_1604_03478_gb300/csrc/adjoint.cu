@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(128) k_adj_node(const __grid_constant__ KP p, 
     unsigned lm = 0;  // bit opp(i): x + e_i is liquid
     if (on) {
         int js9[9];
-        load_js9(p, js, x, FACE == 0 ? z : y, js9);
+        load_js9<true>(p, js, x, FACE == 0 ? z : y, js9);
         jsc = js9[4];
         nbv = nb[col];
         liquid = a < jsc;

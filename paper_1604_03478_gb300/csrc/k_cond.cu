@@ -36,9 +36,9 @@ __device__ __forceinline__ void collide_solid2(const KP &p, float2 (&g)[7]) {
 // Smallest and largest liquid count of the pair's 3x3 columns: the bounds of
 // nb (each up to two wide of the count) where they settle which side of the
 // front height a is on, else the counts themselves.
-__device__ __forceinline__ void pair_bounds(const KP &p, const int *__restrict__ js, const int *__restrict__ nb, int pp,
+__device__ __forceinline__ void pair_bounds(const KP &p, const int *js, const int *nb, int pp,
                                             int q, int col, int a, int &mn, int &mx) {
-    const int nb0 = __ldg(nb + col), nb1 = __ldg(nb + col + 1);
+    const int nb0 = nb[col], nb1 = nb[col + 1];
     mn = min(nb0 >> 16, nb1 >> 16);
     mx = max(nb0 & 0xffff, nb1 & 0xffff);
     if (a + 1 >= mn && a <= mx) {
@@ -55,8 +55,8 @@ __device__ __forceinline__ void pair_bounds(const KP &p, const int *__restrict__
 // the one-node conduction code node by node.
 template <typename ST, int FACE, typename IX>
 __device__ __forceinline__ void even_pair_cond(const KP &p, ST *__restrict__ F, ST *__restrict__ G,
-                                               const int *__restrict__ js, const int *__restrict__ nb,
-                                               const float *__restrict__ gpost, const float *__restrict__ spost,
+                                               const int *js, const int *nb,
+                                               const float *gpost, const float *spost,
                                                int x, int y, int z) {
     const int a = axial<FACE>(x, y, z);
     const int col = column<FACE>(p, x, y, z);
@@ -80,8 +80,8 @@ __device__ __forceinline__ void even_pair_cond(const KP &p, ST *__restrict__ F, 
 
 template <typename ST, int FACE, typename IX, int LIN>
 __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_even_pair_cond(
-    const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G, const int *__restrict__ js,
-    const int *__restrict__ nb, const float *__restrict__ gpost, const float *__restrict__ spost) {
+    const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G, const int *js,
+    const int *nb, const float *gpost, const float *spost) {
     step_launch_wait();
     int x, y, z;
     if (k1_pair<FACE, LIN>(p, x, y, z)) even_pair_cond<ST, FACE, IX>(p, F, G, js, nb, gpost, spost, x, y, z);
@@ -94,11 +94,11 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_even_pair_cond(
 // other pair the one-node conduction code.
 template <typename ST, int FACE, typename IX>
 __device__ __forceinline__ void odd_pair_cond(const KP &p, const Links *lk, ST *__restrict__ F,
-                                              ST *__restrict__ G, const int *__restrict__ js,
-                                              const int *__restrict__ js_old, const int *__restrict__ nb,
-                                              const float *__restrict__ gpost,
+                                              ST *__restrict__ G, const int *js,
+                                              const int *js_old, const int *nb,
+                                              const float *gpost,
                                               const float *__restrict__ thw_rd, const float *__restrict__ thw_wr,
-                                              const float *__restrict__ spost, int x, int y, int z) {
+                                              const float *spost, int x, int y, int z) {
     const int a = axial<FACE>(x, y, z);
     const int col = column<FACE>(p, x, y, z);
     const int q = FACE == 0 ? z : y, nq = FACE == 0 ? p.nz : p.ny;
@@ -140,10 +140,10 @@ __device__ __forceinline__ void odd_pair_cond(const KP &p, const Links *lk, ST *
 
 template <typename ST, int FACE, typename IX, int LIN>
 __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair_cond(
-    const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G, const int *__restrict__ js,
-    const int *__restrict__ js_old, const int *__restrict__ nb, const float *__restrict__ gpost,
+    const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G, const int *js,
+    const int *js_old, const int *nb, const float *gpost,
     const float *__restrict__ thw_rd,
-    const float *__restrict__ thw_wr, const __grid_constant__ Links lk, const float *__restrict__ spost) {
+    const float *__restrict__ thw_wr, const __grid_constant__ Links lk, const float *spost) {
     step_launch_wait();
     int x, y, z;
     if (k1_pair<FACE, LIN>(p, x, y, z))

@@ -49,6 +49,12 @@ __device__ __forceinline__ void step_launch_wait() {
 // other kernels, which have no such wait, the launch is plain: see
 // launch_step_kernel).  Such loads go to L2 (ld.global.cg): L1 may hold a line from before.  They and
 // the wait are volatile, so the compiler keeps their order.
+// After the wait, what the front update writes (js, nb, gpost, spost) is read
+// by ordinary loads: never by __ldg and never through a const __restrict__
+// parameter, which allow the non-coherent path and promise that nobody writes
+// it while the grid lives, and its early blocks live while the front update
+// still writes.  The same holds for the ensemble's kernel, which writes them
+// itself.
 __device__ __forceinline__ int ld_l2(const int *q) {
     int v;
     asm volatile("ld.global.cg.s32 %0, [%1];\n" : "=r"(v) : "l"(q));
@@ -116,7 +122,7 @@ __device__ __forceinline__ ST *elem(ST *base, IX c, long long off) {
 // at rest at Tm (gh = w (Tm - Ts), zero with FP32 storage).
 __device__ __forceinline__ void solid_post(const KP &p, bool ghost, const float *gpost, int col, float (&g)[7]) {
 #pragma unroll
-    for (int i = 0; i < 7; ++i) g[i] = ghost ? __ldg(gpost + (long long)i * p.ncols + col) : w7(i) * p.dTms;
+    for (int i = 0; i < 7; ++i) g[i] = ghost ? gpost[(long long)i * p.ncols + col] : w7(i) * p.dTms;
 }
 
 // A solid node at least two nodes above its column's first solid node and
@@ -133,13 +139,13 @@ __device__ __forceinline__ bool deep_solid(const KP &p, int a, int nbv) {
 // Bit i (1..6): the D3Q7 link leaving node x along t_i ends inside the
 // cavity on a node of the other phase (liq: x is liquid).
 template <int FACE>
-__device__ __forceinline__ unsigned other_phase7(const KP &p, const int *__restrict__ js, int x, int y, int z,
+__device__ __forceinline__ unsigned other_phase7(const KP &p, const int *js, int x, int y, int z,
                                                  bool liq) {
     unsigned m = 0;
 #pragma unroll
     for (int i = 1; i < 7; ++i) {
         const int xn = x + tx(i), yn = y + ty(i), zn = z + tz(i);
-        if (inside(p, xn, yn, zn) && (axial<FACE>(xn, yn, zn) < __ldg(js + column<FACE>(p, xn, yn, zn))) != liq)
+        if (inside(p, xn, yn, zn) && (axial<FACE>(xn, yn, zn) < js[column<FACE>(p, xn, yn, zn)]) != liq)
             m |= 1u << i;
     }
     return m;
@@ -151,11 +157,11 @@ __device__ __forceinline__ unsigned other_phase7(const KP &p, const int *__restr
 // when x is that ghost (ghost: the first solid node towards the liquid, with
 // the liquid side's ghost populations gbuf; the last liquid node towards the
 // solid, with the solid side's), else the rest state at Tm.
-__device__ __forceinline__ void cross_phase(const KP &p, unsigned other, bool ghost, const float *__restrict__ gbuf,
+__device__ __forceinline__ void cross_phase(const KP &p, unsigned other, bool ghost, const float *gbuf,
                                             int col, float (&g)[7]) {
 #pragma unroll
     for (int i = 1; i < 7; ++i)
-        if ((other >> i) & 1u) g[i] = ghost ? __ldg(gbuf + (long long)i * p.ncols + col) : w7(i) * p.dTms;
+        if ((other >> i) & 1u) g[i] = ghost ? gbuf[(long long)i * p.ncols + col] : w7(i) * p.dTms;
 }
 
 // ------------------------------------------------------------- even step
@@ -163,13 +169,13 @@ __device__ __forceinline__ void cross_phase(const KP &p, unsigned other, bool gh
 // and the links across the phase boundary carry the ghost or rest values of
 // cross_phase; spost holds the solid side's ghost populations).
 template <typename ST, int FACE, typename IX = long long, bool COND = false>
-__device__ __forceinline__ void even_node(const KP &p, ST *__restrict__ F, ST *__restrict__ G, const int *__restrict__ js,
-                                          const int *__restrict__ nb, const float *__restrict__ gpost, int x, int y,
-                                          int z, const float *__restrict__ spost = nullptr) {
+__device__ __forceinline__ void even_node(const KP &p, ST *__restrict__ F, ST *__restrict__ G, const int *js,
+                                          const int *nb, const float *gpost, int x, int y,
+                                          int z, const float *spost = nullptr) {
     const IX c = (IX)node_index(p, x, y, z);
     const int a = axial<FACE>(x, y, z);
     const int col = column<FACE>(p, x, y, z);
-    const int jsc = __ldg(js + col);
+    const int jsc = js[col];
     float g[7];
     if (a < jsc) {
         float f[19];
@@ -180,7 +186,7 @@ __device__ __forceinline__ void even_node(const KP &p, ST *__restrict__ F, ST *_
         collide(p, f, g);
 #pragma unroll
         for (int i = 0; i < 19; ++i) Store<ST>::st_stream(elem<IX>(F, c, opp(i) * p.ld), f[i]);
-        if (COND && a + 1 >= (__ldg(nb + col) >> 16)) {
+        if (COND && a + 1 >= (nb[col] >> 16)) {
             const unsigned other = other_phase7<FACE>(p, js, x, y, z, true);
             if (other) cross_phase(p, other, a == jsc - 1, spost, col, g);
         }
@@ -188,12 +194,12 @@ __device__ __forceinline__ void even_node(const KP &p, ST *__restrict__ F, ST *_
 #pragma unroll
         for (int i = 0; i < 7; ++i) g[i] = Store<ST>::ld(elem<IX>(G, c, i * p.ld));
         collide_solid(p, g);
-        if (a <= (__ldg(nb + col) & 0xffff)) {
+        if (a <= (nb[col] & 0xffff)) {
             const unsigned other = other_phase7<FACE>(p, js, x, y, z, false);
             if (other) cross_phase(p, other, a == jsc, gpost, col, g);
         }
     } else {
-        if (deep_solid(p, a, __ldg(nb + col))) return;
+        if (deep_solid(p, a, nb[col])) return;
         solid_post(p, a == jsc, gpost, col, g);
     }
 #pragma unroll
@@ -304,8 +310,8 @@ template <typename ST> constexpr int k1_min_blocks() { return sizeof(ST) == 2 ? 
 // registers, and the first solid node's g.
 template <typename ST, int FACE, typename IX, bool SNAP>
 __global__ void __launch_bounds__(128, SNAP ? 0 : k1_min_blocks<ST>()) k_even(const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G,
-                                              const int *js, const int *js_old, const int *__restrict__ nb,
-                                              const float *__restrict__ gpost, const int *jmax, int early_blocks,
+                                              const int *js, const int *js_old, const int *nb,
+                                              const float *gpost, const int *jmax, int early_blocks,
                                               const double *s, const __grid_constant__ SnapOut snap) {
     int x = 0, y = 0, z = 0, a = 0, col = 0, jso = 0;
     IX c = 0;
@@ -329,7 +335,7 @@ __global__ void __launch_bounds__(128, SNAP ? 0 : k1_min_blocks<ST>()) k_even(co
     }
     if (!late) step_launch_wait();
     if (!on) return;
-    const int jsc = __ldg(js + col);
+    const int jsc = js[col];
     if (SNAP && a == 0) snap_column(snap, col, s[col], jsc, nb[col]);
     if (a < jsc) {
         if (a >= jso) {
@@ -343,7 +349,7 @@ __global__ void __launch_bounds__(128, SNAP ? 0 : k1_min_blocks<ST>()) k_even(co
 #pragma unroll
         for (int i = 0; i < 19; ++i) Store<ST>::st_stream(elem<IX>(F, c, opp(i) * p.ld), f[i]);
     } else {
-        if (deep_solid(p, a, __ldg(nb + col))) return;
+        if (deep_solid(p, a, nb[col])) return;
         if (SNAP && a == jsc) snap_ghost<ST, FACE>(p, G, nullptr, x, y, z, false, snap);
         solid_post(p, a == jsc, gpost, col, g);
     }
@@ -354,8 +360,8 @@ __global__ void __launch_bounds__(128, SNAP ? 0 : k1_min_blocks<ST>()) k_even(co
 // The even step with heat conduction in the solid (every node updated).
 template <typename ST, int FACE>
 __global__ void __launch_bounds__(128) k_even_cond(const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G,
-                                                   const int *__restrict__ js, const int *__restrict__ nb,
-                                                   const float *__restrict__ gpost, const float *__restrict__ spost) {
+                                                   const int *js, const int *nb,
+                                                   const float *gpost, const float *spost) {
     step_launch_wait();
     int x, y, z;
     if (k1_node<FACE>(p, nullptr, x, y, z)) even_node<ST, FACE, long long, true>(p, F, G, js, nb, gpost, x, y, z, spost);
@@ -364,15 +370,19 @@ __global__ void __launch_bounds__(128) k_even_cond(const __grid_constant__ KP p,
 
 // -------------------------------------------------------------- odd step
 // Liquid counts of the 3x3 columns around column (pp, q), 0 outside the
-// cavity; entry (dq + 1) * 3 + dp + 1.
-__device__ __forceinline__ void load_js9(const KP &p, const int *__restrict__ js, int pp, int q, int (&js9)[9]) {
+// cavity; entry (dq + 1) * 3 + dp + 1.  FIXED: in a kernel during which nobody
+// writes them (read-outs, the adjoint's node kernel), through the read-only
+// path (fields and totals of a 256^3 state 376 us, else 390).  The front update
+// of a lone cavity is one too, not the ensemble's (SPEC, see front_column).
+template <bool FIXED = false>
+__device__ __forceinline__ void load_js9(const KP &p, const int *js, int pp, int q, int (&js9)[9]) {
 #pragma unroll
     for (int dq = -1; dq <= 1; ++dq)
 #pragma unroll
         for (int dp = -1; dp <= 1; ++dp) {
             const int p2 = pp + dp, q2 = q + dq;
             const bool in = (unsigned)p2 < (unsigned)p.P1 && (unsigned)q2 < (unsigned)p.P2;
-            js9[(dq + 1) * 3 + dp + 1] = in ? __ldg(js + q2 * p.P1 + p2) : 0;
+            js9[(dq + 1) * 3 + dp + 1] = in ? (FIXED ? __ldg(js + q2 * p.P1 + p2) : js[q2 * p.P1 + p2]) : 0;
         }
 }
 
@@ -406,14 +416,14 @@ __device__ __forceinline__ unsigned link_mask9(const int (&js9)[9], int a) {
 // Liquid counts of the twelve columns around those of a pair (the 3x3 columns
 // of both, pp - 1 .. pp + 2 by q - 1 .. q + 1), 0 outside the cavity; entry
 // (dq + 1) * 4 + dp + 1.
-__device__ __forceinline__ void load_js12(const KP &p, const int *__restrict__ js, int pp, int q, int (&c)[12]) {
+__device__ __forceinline__ void load_js12(const KP &p, const int *js, int pp, int q, int (&c)[12]) {
 #pragma unroll
     for (int dq = -1; dq <= 1; ++dq)
 #pragma unroll
         for (int dp = -1; dp <= 2; ++dp) {
             const int p2 = pp + dp, q2 = q + dq;
             const bool in = (unsigned)p2 < (unsigned)p.P1 && (unsigned)q2 < (unsigned)p.P2;
-            c[(dq + 1) * 4 + dp + 1] = in ? __ldg(js + q2 * p.P1 + p2) : 0;
+            c[(dq + 1) * 4 + dp + 1] = in ? js[q2 * p.P1 + p2] : 0;
         }
 }
 // Smallest (over columns inside the cavity) and largest of them.
@@ -480,16 +490,16 @@ __device__ __forceinline__ bool xwall(int ex_up, bool xlo, bool xhi) {
 // that has become liquid since (never on the fast path: the count bounds nb
 // are at most the old counts less one) starts from fh = 0.
 template <typename ST, int FACE, bool TAB = true, bool COND = false>
-__device__ __forceinline__ void odd_node(const KP &p, const Links *lk, ST *__restrict__ F, ST *__restrict__ G, const int *__restrict__ js,
-                                         const int *__restrict__ js_old, const int *__restrict__ nb, const float *__restrict__ gpost,
+__device__ __forceinline__ void odd_node(const KP &p, const Links *lk, ST *__restrict__ F, ST *__restrict__ G, const int *js,
+                                         const int *js_old, const int *nb, const float *gpost,
                                          const float *__restrict__ thw_rd, const float *__restrict__ thw_wr, int x,
-                                         int y, int z, const float *__restrict__ spost = nullptr,
+                                         int y, int z, const float *spost = nullptr,
                                          const int *known = nullptr) {
     const long long c = node_index(p, x, y, z);
     const int a = axial<FACE>(x, y, z);
     const int col = column<FACE>(p, x, y, z);
-    const int jsc = __ldg(js + col);
-    const int nbv = __ldg(nb + col);
+    const int jsc = js[col];
+    const int nbv = nb[col];
     const int q = FACE == 0 ? z : y, nq = FACE == 0 ? p.nz : p.ny;
     const bool off_qa = q >= 1 && q <= nq - 2 && a >= 1 && a <= p.H - 2;
     const bool off_walls = off_qa && x >= 1 && x <= p.nx - 2;
@@ -541,7 +551,7 @@ __device__ __forceinline__ void odd_node(const KP &p, const Links *lk, ST *__res
             }
         } else {
             const float th_rd = __ldg(thw_rd + col);
-            const bool was_liquid = a < __ldg(js_old + col);
+            const bool was_liquid = a < js_old[col];
             f[0] = Store<ST>::ld(Fc);
 #pragma unroll
             for (int i = 1; i < 19; ++i)  // else bounce-back: f*_opp(i) parked in slot i
@@ -626,7 +636,7 @@ __device__ __forceinline__ void odd_node(const KP &p, const Links *lk, ST *__res
 template <typename ST, int FACE, bool SNAP>
 __device__ __forceinline__ void odd_node_early(const KP &p, const Links *lk, ST *__restrict__ F, ST *__restrict__ G,
                                                const int *js, const int *js_old, const int *nb, const int *nb_old,
-                                               const float *__restrict__ gpost, const float *thw_rd,
+                                               const float *gpost, const float *thw_rd,
                                                const float *__restrict__ thw_wr, const int *jmax, int early_blocks,
                                                bool on, int x, int y, int z, const double *s, const SnapOut &snap) {
     const long long c = on ? node_index(p, x, y, z) : 0;
@@ -694,7 +704,7 @@ __device__ __forceinline__ void odd_node_early(const KP &p, const Links *lk, ST 
     }
     if (!late) step_launch_wait();
     if (!on) return;
-    const int jsc = inner && !SNAP ? p.H : __ldg(js + col);
+    const int jsc = inner && !SNAP ? p.H : js[col];
     if (SNAP && a == 0) snap_column(snap, col, s[col], jsc, nb[col]);
     if (a < jsc) {
         bool fast = inner;
@@ -732,7 +742,7 @@ __device__ __forceinline__ void odd_node_early(const KP &p, const Links *lk, ST 
         for (int i = 1; i < 19; ++i)
             Store<ST>::st_stream(((lm >> opp(i)) & 1u) ? Fc + lk->fout[i] : Fc + opp(i) * p.ld, f[i]);
     } else {
-        if (deep_solid(p, a, __ldg(nb + col))) return;
+        if (deep_solid(p, a, nb[col])) return;
         im = inside_mask(p, x, y, z);
         if (SNAP && a == jsc) snap_ghost<ST, FACE>(p, G, thw_rd, x, y, z, true, snap);
         solid_post(p, a == jsc, gpost, col, g);
@@ -750,7 +760,7 @@ __device__ __forceinline__ void odd_node_early(const KP &p, const Links *lk, ST 
 template <typename ST, int FACE, bool SNAP>
 __global__ void __launch_bounds__(128, SNAP ? 0 : k1_min_blocks<ST>()) k_odd(const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G,
                                              const int *js, const int *js_old, const int *nb, const int *nb_old,
-                                             const float *__restrict__ gpost, const float *thw_rd,
+                                             const float *gpost, const float *thw_rd,
                                              const float *__restrict__ thw_wr, const __grid_constant__ Links lk,
                                              const int *jmax, int early_blocks, const double *s,
                                              const __grid_constant__ SnapOut snap) {
@@ -763,11 +773,11 @@ __global__ void __launch_bounds__(128, SNAP ? 0 : k1_min_blocks<ST>()) k_odd(con
 // The odd step with heat conduction in the solid (every node updated).
 template <typename ST, int FACE>
 __global__ void __launch_bounds__(128) k_odd_cond(const __grid_constant__ KP p, ST *__restrict__ F, ST *__restrict__ G,
-                                                  const int *__restrict__ js, const int *__restrict__ js_old,
-                                                  const int *__restrict__ nb,
-                                                  const float *__restrict__ gpost, const float *__restrict__ thw_rd,
+                                                  const int *js, const int *js_old,
+                                                  const int *nb,
+                                                  const float *gpost, const float *__restrict__ thw_rd,
                                                   const float *__restrict__ thw_wr, const __grid_constant__ Links lk,
-                                                  const float *__restrict__ spost) {
+                                                  const float *spost) {
     step_launch_wait();
     int x, y, z;
     if (k1_node<FACE>(p, nullptr, x, y, z))
@@ -866,11 +876,11 @@ __device__ __forceinline__ void even_pair_liquid(const KP &p, ST *__restrict__ F
 
 template <typename ST, int FACE, typename IX>
 __device__ __forceinline__ void even_pair(const KP &p, ST *__restrict__ F, ST *__restrict__ G,
-                                          const int *__restrict__ js, const int *__restrict__ nb,
-                                          const float *__restrict__ gpost, int x, int y, int z) {
+                                          const int *js, const int *nb,
+                                          const float *gpost, int x, int y, int z) {
     const int a = axial<FACE>(x, y, z);
     const int col = column<FACE>(p, x, y, z);  // x + 1 is in column col + 1
-    if (a < __ldg(js + col) && a < __ldg(js + col + 1)) {
+    if (a < js[col] && a < js[col + 1]) {
         even_pair_liquid<ST, IX>(p, F, G, (IX)node_index(p, x, y, z));
     } else {
         even_node<ST, FACE, IX>(p, F, G, js, nb, gpost, x, y, z);
@@ -880,8 +890,8 @@ __device__ __forceinline__ void even_pair(const KP &p, ST *__restrict__ F, ST *_
 
 template <typename ST, int FACE, typename IX, int LIN>
 __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_even_pair(const __grid_constant__ KP p, ST *__restrict__ F,
-                                                      ST *__restrict__ G, const int *__restrict__ js,
-                                                      const int *__restrict__ nb, const float *__restrict__ gpost,
+                                                      ST *__restrict__ G, const int *js,
+                                                      const int *nb, const float *gpost,
                                                       const int *jmax) {
     step_launch_wait();
     int x, y, z;
@@ -959,15 +969,15 @@ __device__ __forceinline__ void odd_pair_liquid(const KP &p, const Links *lk, ST
 // odd_pair_liquid, any other pair the one-node code node by node.
 template <typename ST, int FACE, typename IX>
 __device__ __forceinline__ void odd_pair(const KP &p, const Links *lk, ST *__restrict__ F,
-                                         ST *__restrict__ G, const int *__restrict__ js,
-                                         const int *__restrict__ js_old, const int *__restrict__ nb,
-                                         const float *__restrict__ gpost, const float *__restrict__ thw_rd,
+                                         ST *__restrict__ G, const int *js,
+                                         const int *js_old, const int *nb,
+                                         const float *gpost, const float *__restrict__ thw_rd,
                                          const float *__restrict__ thw_wr, int x, int y, int z) {
     const int a = axial<FACE>(x, y, z);
     const int col = column<FACE>(p, x, y, z);
     const int q = FACE == 0 ? z : y, nq = FACE == 0 ? p.nz : p.ny;
     const bool off_qa = q >= 1 && q <= nq - 2 && a >= 1 && a <= p.H - 2;
-    const int b0 = __ldg(nb + col) >> 16, b1 = __ldg(nb + col + 1) >> 16;
+    const int b0 = nb[col] >> 16, b1 = nb[col + 1] >> 16;
     if (!(off_qa && a + 1 < b0 && a + 1 < b1)) {
         int c12[12], js9[9], mn, mx;
         load_js12(p, js, x, q, c12);
@@ -985,9 +995,9 @@ __device__ __forceinline__ void odd_pair(const KP &p, const Links *lk, ST *__res
 
 template <typename ST, int FACE, typename IX, int LIN>
 __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair(const __grid_constant__ KP p, ST *__restrict__ F,
-                                                     ST *__restrict__ G, const int *__restrict__ js,
-                                                     const int *__restrict__ js_old, const int *__restrict__ nb,
-                                                     const float *__restrict__ gpost,
+                                                     ST *__restrict__ G, const int *js,
+                                                     const int *js_old, const int *nb,
+                                                     const float *gpost,
                                                      const float *__restrict__ thw_rd,
                                                      const float *__restrict__ thw_wr,
                                                      const __grid_constant__ Links lk, const int *jmax) {
@@ -1010,7 +1020,7 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair(const _
 template <typename ST, int FACE, typename IX, int LIN, bool SNAP>
 __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_even_pair_early(const __grid_constant__ KP p, ST *__restrict__ F,
                                                       ST *__restrict__ G, const int *js, const int *js_old,
-                                                      const int *__restrict__ nb, const float *__restrict__ gpost,
+                                                      const int *nb, const float *gpost,
                                                       const int *jmax, int early_blocks, const double *s,
                                                       const __grid_constant__ SnapOut snap) {
     int x = 0, y = 0, z = 0;
@@ -1033,7 +1043,7 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_even_pair_early(
     }
     if (!on || !low) return;
     if (SNAP && a == 0) snap_pair_columns(snap, col, s, js, nb);
-    if (!(a < __ldg(js + col) && a < __ldg(js + col + 1))) {
+    if (!(a < js[col] && a < js[col + 1])) {
         if (SNAP) {
             snap_any<ST, FACE>(p, F, G, js, js_old, nullptr, x, y, z, false, snap);
             snap_any<ST, FACE>(p, F, G, js, js_old, nullptr, x + 1, y, z, false, snap);
@@ -1051,7 +1061,7 @@ template <typename ST, int FACE, typename IX, int LIN, bool SNAP>
 __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair_early(const __grid_constant__ KP p, ST *__restrict__ F,
                                                      ST *__restrict__ G, const int *js, const int *js_old,
                                                      const int *nb, const int *nb_old,
-                                                     const float *__restrict__ gpost,
+                                                     const float *gpost,
                                                      const float *__restrict__ thw_rd,
                                                      const float *__restrict__ thw_wr,
                                                      const __grid_constant__ Links lk, const int *jmax,
@@ -1080,7 +1090,7 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair_early(c
     if (!on || !low) return;
     if (SNAP && a == 0) snap_pair_columns(snap, col, s, js, nb);
     if (!loaded) {
-        const int b0 = __ldg(nb + col) >> 16, b1 = __ldg(nb + col + 1) >> 16;
+        const int b0 = nb[col] >> 16, b1 = nb[col + 1] >> 16;
         if (!(off_qa && a + 1 < b0 && a + 1 < b1)) {
             int c12[12], js9[9], mn, mx;
             load_js12(p, js, x, q, c12);
@@ -1147,7 +1157,7 @@ __device__ __forceinline__ void snap_ghost(const KP &p, const ST *G, const float
     snap_node(p, o, x, y, z, f, g);
 }
 
-template <typename ST, int FACE>
+template <typename ST, int FACE, bool FIXED = false>
 __device__ __forceinline__ void gather_f(const KP &p, const ST *F, const int *js, int x, int y, int z,
                                          bool inflight, float (&f)[19]) {
     const ST *Fc = F + node_index(p, x, y, z);
@@ -1157,7 +1167,7 @@ __device__ __forceinline__ void gather_f(const KP &p, const ST *F, const int *js
         return;
     }
     int js9[9];
-    load_js9(p, js, x, FACE == 0 ? z : y, js9);
+    load_js9<FIXED>(p, js, x, FACE == 0 ? z : y, js9);
     const unsigned lm = link_mask9<FACE>(js9, axial<FACE>(x, y, z));
     f[0] = Store<ST>::ld(Fc);
 #pragma unroll
@@ -1167,8 +1177,9 @@ __device__ __forceinline__ void gather_f(const KP &p, const ST *F, const int *js
 
 // gather_f of the state between steps (flip_column has run): a node that has
 // become liquid since the in-flight values were produced (under js_old)
-// starts from fh = 0 (in the natural layout its slots hold that).
-template <typename ST, int FACE>
+// starts from fh = 0 (in the natural layout its slots hold that).  FIXED: see
+// load_js9.
+template <typename ST, int FACE, bool FIXED = true>
 __device__ __forceinline__ void gather_f_now(const KP &p, const ST *F, const int *js, const int *js_old, int x, int y,
                                              int z, bool inflight, float (&f)[19]) {
     if (inflight && axial<FACE>(x, y, z) >= js_old[column<FACE>(p, x, y, z)]) {
@@ -1176,7 +1187,7 @@ __device__ __forceinline__ void gather_f_now(const KP &p, const ST *F, const int
         for (int i = 0; i < 19; ++i) f[i] = 0.0f;
         return;
     }
-    gather_f<ST, FACE>(p, F, js, x, y, z, inflight, f);
+    gather_f<ST, FACE, FIXED>(p, F, js, x, y, z, inflight, f);
 }
 
 template <typename ST, int FACE>
@@ -1190,7 +1201,7 @@ __device__ __forceinline__ void snap_any(const KP &p, const ST *F, const ST *G, 
     }
     float f[19], g[7];
     gather_g<ST, FACE>(p, G, x, y, z, inflight, thw, g);
-    gather_f_now<ST, FACE>(p, F, js, js_old, x, y, z, inflight, f);
+    gather_f_now<ST, FACE, false>(p, F, js, js_old, x, y, z, inflight, f);
     snap_node(p, o, x, y, z, f, g);
 }
 
@@ -1347,7 +1358,7 @@ __device__ __forceinline__ int count_bounds(const KP &p, const int (&js9)[9], in
 // state are not needed: a value moved for a node x that turns solid itself is
 // read by nothing.
 template <typename ST, int FACE>
-__device__ __forceinline__ void flip_column(const KP &p, ST *__restrict__ F, const int *__restrict__ js, bool inflight,
+__device__ __forceinline__ void flip_column(const KP &p, ST *__restrict__ F, const int *js, bool inflight,
                                             int col, int jo, int jn) {
     const int lo = jo < jn ? jo : jn, hi = jo < jn ? jn : jo;
     for (int j = lo; j < hi; ++j) {
@@ -1450,7 +1461,7 @@ __device__ __forceinline__ int front_column(const KP &p, ST *__restrict__ F, con
         column_node<FACE>(p, col, L, x, y, z);
         gather_g<ST, FACE>(p, G, x, y, z, infl, thw, gL);
         if (infl) gather_f9<ST, FACE>(p, F, js9, x, y, z, L, fL);
-        else gather_f<ST, FACE>(p, F, js, x, y, z, false, fL);
+        else gather_f<ST, FACE, SPEC>(p, F, js, x, y, z, false, fL);
     }
     // The solid side of the front (conduction in the solid, a column with a
     // solid node): temperatures of the guarded solid node and the one above.
@@ -1560,7 +1571,7 @@ __device__ __forceinline__ int front_column(const KP &p, ST *__restrict__ F, con
 #pragma unroll
                 for (int i = 0; i < 19; ++i) fL[i] = 0.0f;
             } else {
-                gather_f<ST, FACE>(p, F, js, x, y, z, infl, fL);
+                gather_f<ST, FACE, SPEC>(p, F, js, x, y, z, infl, fL);
             }
         }
         float Th = 0.0f, jx = 0.0f, jy = 0.0f, jz = 0.0f;

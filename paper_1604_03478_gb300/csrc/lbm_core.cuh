@@ -667,7 +667,7 @@ __device__ __forceinline__ bool inside(const KP &p, int x, int y, int z) {
     return (unsigned)x < (unsigned)p.nx && (unsigned)y < (unsigned)p.ny && (unsigned)z < (unsigned)p.nz;
 }
 template <int FACE> __device__ __forceinline__ bool liquid_at(const KP &p, const int *js, int x, int y, int z) {
-    return inside(p, x, y, z) && axial<FACE>(x, y, z) < __ldg(js + column<FACE>(p, x, y, z));
+    return inside(p, x, y, z) && axial<FACE>(x, y, z) < js[column<FACE>(p, x, y, z)];
 }
 
 // Wall crossed by the D3Q7 link that leaves node (x,y,z) along direction i
