@@ -51,7 +51,11 @@ struct lbm_melt {
     int bx, by;        // block shape of the per-node kernels (0: default)
     int cblk;          // threads per block of the per-column kernels
     int sms;           // SMs of the device
-    int plain_next;    // the stream's last work wrote what the step's kernels load early: the next one is launched plainly
+    // The stream's last work wrote what the step's kernels load early: the next
+    // one is launched plainly (take_plain).  plain_capture: the capture whose
+    // first step already was.
+    int plain_next;
+    unsigned long long plain_capture;
     // Running maximum of the liquid counts, kept by k_front on the device;
     // stream-collide blocks at heights >= it + 3 (all deep solid) return at
     // once.  The front kernels (the ensemble's too) raise a copy in page-locked

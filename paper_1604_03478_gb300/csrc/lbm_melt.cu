@@ -437,14 +437,33 @@ dim3 sc_block(const lbm_melt *h) {
     return dim3(bx, 128 / bx, 1);
 }
 
+// Whether the step launched now on st is the one that plain_next asks for.  A
+// step that is only captured leaves plain_next to the next one that runs: what
+// was written is still the stream's last work.
+int take_plain(lbm_melt *h, cudaStream_t st) {
+    if (!h->plain_next) return 0;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(st, &cs, &id) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 1;
+    }
+    if (cs == cudaStreamCaptureStatusNone) {
+        h->plain_next = 0;
+        return 1;
+    }
+    if (id == h->plain_capture) return 0;
+    h->plain_capture = id;
+    return 1;
+}
+
 // Enqueue one step from phase (cur, inflight) on stream st with the
 // stream-collide grid cut at `height`; returns the phase after it.
 cudaError_t enqueue_step(lbm_melt *h, int &cur, int &inflight, int height, dim3 blk, cudaStream_t st,
                          const lbm::SnapOut *snap = nullptr) {
     Bufs b = bufs_at(h, cur, inflight);
     b.k1_height = height;
-    b.plain = h->plain_next;
-    h->plain_next = 0;
+    b.plain = take_plain(h, st);
     const int odd = inflight;
     cudaError_t e = LAUNCH(h, stream_collide, h->kp, h->face, odd, b, blk, st, snap);
     if (e != cudaSuccess) return e;
@@ -765,8 +784,7 @@ LBM_API lbm_status lbm_melt_step(lbm_melt *h, long long n) {
             h->ev_used += 2;
             CK(cudaEventRecord(evp[0], h->stream), "event record");
         }
-        b.plain = h->plain_next;
-        h->plain_next = 0;
+        b.plain = take_plain(h, h->stream);
         CK(LAUNCH(h, stream_collide, h->kp, h->face, odd, b, blk, h->stream), "stream-collide");
         if (evp) CK(cudaEventRecord(evp[1], h->stream), "event record");
         h->inflight = !odd;
@@ -1010,6 +1028,7 @@ LBM_API lbm_status lbm_melt_set_hot_wall(lbm_melt *h, const float *T_h_field, in
     else h->thw_last_prev = 1;
     h->thw_gen++;
     h->plain_next = 1;
+    h->plain_capture = 0;
     return src ? LBM_OK : copy_in(h, h->thw_cur, T_h_field, nc * 4, ptr_kind);
 }
 
