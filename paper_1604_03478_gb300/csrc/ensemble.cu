@@ -343,6 +343,21 @@ LBM_API lbm_status lbm_ensemble_step(lbm_ensemble *e, long long nsteps) {
     if (!desc_current(e)) refresh_desc(e);
     long long left = nsteps;
     const long long G = launch_steps(e);
+    // A wall changed in flight is read in its old form by the first step only
+    // (thw_rd0), and every launch of the same descriptors takes that form at
+    // its own first step: where there will be several, the remainder (or one
+    // launch) goes first, and the others start from the new walls.
+    bool pending = false;
+    for (const lbm_melt *h : e->cav) pending = pending || h->thw_pending;
+    if (pending && left > G) {
+        const long long first = left % G ? left % G : G;
+        lbm_status st = launch(e, (int)first, -1);
+        if (st != LBM_OK) return st;
+        advance_handles(e, first);
+        refresh_desc(e);
+        left -= first;
+        nsteps -= first;
+    }
     if (left >= G) {
         if (!e->graph) {
             cudaGraph_t g;
