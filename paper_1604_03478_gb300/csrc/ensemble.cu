@@ -43,7 +43,8 @@ struct lbm_ensemble {
     int precision;
     int block, K, grid, linear;
     long long max_spins;
-    unsigned int *bar_dev;
+    unsigned int *bar_dev;   // the launch's barrier words (8), the phase timers (8), kTimedOut
+    int reported;            // a timeout was reported by lbm_ensemble_sync: the next launch clears it
     long long items[lbm::kMaxCavities + 1], cols[lbm::kMaxCavities + 1];
     std::vector<CavDesc> desc;
     cudaGraphExec_t graph;
@@ -53,6 +54,10 @@ struct lbm_ensemble {
 };
 
 namespace {
+
+// Word of bar_dev that a launch which timed out leaves set (its own word goes
+// with the next launch's reset), until lbm_ensemble_sync has reported it.
+const int kTimedOut = 16, kBarWords = 24;
 
 lbm_status ens_err(lbm_ensemble *e, lbm_status st, const char *fmt, ...) {
     if (e) {
@@ -186,6 +191,7 @@ lbm_status launch(lbm_ensemble *e, int nsteps, int skip_block) {
     }
     for (int k = 0; k < e->n; ++k) w->desc[k] = e->desc[k];
     w->bar = e->bar_dev;
+    w->timed_out = e->bar_dev + kTimedOut;
     w->max_spins = e->max_spins;
     w->skip_arrival_block = skip_block;
     void *args[] = {w, &nsteps};
@@ -269,9 +275,10 @@ LBM_API lbm_status lbm_ensemble_create(int n, const lbm_melt_case *cases, void *
         if (k == 0) e->precision = h->precision;
         else if (h->precision != e->precision) return fail(LBM_EINVAL);
     }
-    // 8 barrier words, then the phase timers (4 x u64), zeroed here only
-    if (cudaMalloc(&e->bar_dev, 16 * sizeof(unsigned int)) != cudaSuccess ||
-        cudaMemset(e->bar_dev, 0, 16 * sizeof(unsigned int)) != cudaSuccess)
+    // 8 barrier words, then the phase timers (4 x u64), zeroed here only, and
+    // the timeout of any launch so far
+    if (cudaMalloc(&e->bar_dev, kBarWords * sizeof(unsigned int)) != cudaSuccess ||
+        cudaMemset(e->bar_dev, 0, kBarWords * sizeof(unsigned int)) != cudaSuccess)
         return fail(LBM_ENOMEM);
     // A small ensemble, whose nodes are at most two items of 256 a resident
     // block, takes 256 threads and one plane an item: each item's latency
@@ -341,6 +348,10 @@ LBM_API lbm_status lbm_ensemble_step(lbm_ensemble *e, long long nsteps) {
     ECK(cudaEventRecord(e->ev_in, e->user), "event");
     ECK(cudaStreamWaitEvent(e->stream, e->ev_in, 0), "wait");
     if (!desc_current(e)) refresh_desc(e);
+    if (e->reported) {
+        ECK(cudaMemsetAsync(e->bar_dev + kTimedOut, 0, sizeof(unsigned int), e->stream), "barrier reset");
+        e->reported = 0;
+    }
     long long left = nsteps;
     const long long G = launch_steps(e);
     // A wall changed in flight is read in its old form by the first step only
@@ -403,10 +414,12 @@ LBM_API lbm_status lbm_ensemble_inject_barrier_fault(lbm_ensemble *e, int block)
 
 LBM_API lbm_status lbm_ensemble_sync(lbm_ensemble *e) {
     if (!e) return LBM_EINVAL;
-    unsigned int bar[3] = {0, 0, 0};
-    ECK(cudaMemcpyAsync(bar, e->bar_dev, sizeof bar, cudaMemcpyDeviceToHost, e->stream), "barrier read");
+    unsigned int timed_out = 0;
+    ECK(cudaMemcpyAsync(&timed_out, e->bar_dev + kTimedOut, sizeof timed_out, cudaMemcpyDeviceToHost, e->stream),
+        "barrier read");
     ECK(cudaStreamSynchronize(e->stream), "synchronize");
-    if (bar[2]) return ens_err(e, LBM_ETIMEOUT, "a grid-barrier wait gave up (bounded spin exhausted)");
+    if (timed_out) e->reported = 1;
+    if (timed_out) return ens_err(e, LBM_ETIMEOUT, "a grid-barrier wait gave up (bounded spin exhausted)");
     for (int k = 0; k < e->n; ++k) {
         lbm_status st = lbm_melt_sync(e->cav[k]);
         if (st != LBM_OK) return ens_err(e, st, "cavity %d: %s", k, lbm_melt_last_error(e->cav[k]));

@@ -63,6 +63,7 @@ struct EnsWork {
     CavDesc desc[kMaxCavities];
     unsigned int *bar;            // {arrivals, -, timed out, -, item counters (2 x u64),
                                   //  phase times in ns and steps (4 x u64)}
+    unsigned int *timed_out;      // set with bar[2], which the next launch resets
     long long max_spins;
     int skip_arrival_block;       // fault injection for tests: this block never arrives (-1: none)
 };
@@ -84,6 +85,7 @@ __device__ __forceinline__ bool grid_barrier(const EnsWork &w, unsigned int targ
             // others so that every block leaves through the timeout
             long long spins = 0;
             while (!vb[2] && ++spins <= w.max_spins) __nanosleep(256);
+            atomicExch(w.timed_out, 1u);
             atomicExch(w.bar + 2, 1u);
             ok = 0;
         } else {
@@ -92,6 +94,7 @@ __device__ __forceinline__ bool grid_barrier(const EnsWork &w, unsigned int targ
             long long spins = 0;
             while ((int)(vb[0] - target) < 0) {
                 if (vb[2] || ++spins > w.max_spins) {
+                    atomicExch(w.timed_out, 1u);
                     atomicExch(w.bar + 2, 1u);
                     ok = 0;
                     break;
