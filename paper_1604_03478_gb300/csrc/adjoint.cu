@@ -794,6 +794,7 @@ cudaError_t ws_alloc(lbm_melt *h, int k, size_t bytes, void **out) {
     }
     const cudaError_t e = cudaMalloc(&w->p[k], bytes);
     if (e != cudaSuccess) {
+        (void)cudaGetLastError();  // else the next launch would report it
         w->p[k] = nullptr;
         *out = nullptr;
         return e;
@@ -817,6 +818,7 @@ void free_workspace(lbm_melt *h) {
 const int kSlotCheckpoints = 0, kSlotBackward = 1;
 
 lbm_status tape_err(lbm_melt *h, lbm_status st, const char *fmt, ...) {
+    if (st == LBM_ECUDA || st == LBM_ENOMEM) (void)cudaGetLastError();
     va_list ap;
     va_start(ap, fmt);
     vsnprintf(h->err, sizeof h->err, fmt, ap);

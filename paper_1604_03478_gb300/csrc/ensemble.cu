@@ -60,6 +60,7 @@ namespace {
 const int kTimedOut = 16, kBarWords = 24;
 
 lbm_status ens_err(lbm_ensemble *e, lbm_status st, const char *fmt, ...) {
+    if (st == LBM_ECUDA || st == LBM_ENOMEM) (void)cudaGetLastError();  // else the next launch would report it
     if (e) {
         va_list ap;
         va_start(ap, fmt);
@@ -248,6 +249,7 @@ LBM_API lbm_status lbm_ensemble_create(int n, const lbm_melt_case *cases, void *
     e->graph_steps = 8;
     e->desc.resize(n);
     auto fail = [&](lbm_status st) {
+        (void)cudaGetLastError();
         for (lbm_melt *h : e->cav) lbm_melt_destroy(h);
         cudaFree(e->bar_dev);
         if (e->ev_in) cudaEventDestroy(e->ev_in);

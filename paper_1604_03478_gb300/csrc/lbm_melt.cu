@@ -156,7 +156,11 @@ lbm_status set_err(lbm_melt *h, lbm_status st, const char *fmt, ...) {
     return st;
 }
 
+// A failed call's message.  The runtime also keeps the error for the next
+// cudaGetLastError, where a launch that went well would report it: taken away
+// here (an error that lost the context stays).
 lbm_status cuda_err(lbm_melt *h, cudaError_t e, const char *where) {
+    (void)cudaGetLastError();
     return set_err(h, e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA, "%s: %s", where,
                    cudaGetErrorString(e));
 }
@@ -694,7 +698,12 @@ LBM_API lbm_status lbm_melt_create(const lbm_melt_grid *grid, double Ra, double 
             h->lk.gout[i] = i * p.ld + off;
         }
     }
-    auto fail = [&](lbm_status s) { free_all(h); delete h; return s; };
+    auto fail = [&](lbm_status s) {
+        (void)cudaGetLastError();  // see cuda_err
+        free_all(h);
+        delete h;
+        return s;
+    };
     if (cudaGetDevice(&h->device) != cudaSuccess) return fail(LBM_ECUDA);
     {
         int sms = 0;
