@@ -267,6 +267,17 @@ __global__ void k_set_wall(const float *__restrict__ src, float *cur, float *pre
     cur[i] = v;
 }
 
+// Device memory of one call, given back when the call returns (cudaFree waits
+// for the work that uses it).
+struct DeviceScratch {
+    float *p = nullptr;
+    cudaError_t alloc(size_t bytes) { return cudaMalloc(&p, bytes); }
+    ~DeviceScratch() { cudaFree(p); }
+    DeviceScratch() = default;
+    DeviceScratch(const DeviceScratch &) = delete;
+    DeviceScratch &operator=(const DeviceScratch &) = delete;
+};
+
 lbm_status copy_in(lbm_melt *h, void *dst, const void *src, size_t bytes, int ptr_kind) {
     CK(cudaMemcpyAsync(dst, src, bytes, ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream),
        "copy in");
@@ -916,11 +927,14 @@ LBM_API lbm_status lbm_melt_get(lbm_melt *h, float *T, float *u, double *S, doub
     const KP &p = h->kp;
     const size_t N = (size_t)p.N;
     float *Td = nullptr, *ud = nullptr;
+    DeviceScratch down_T, down_u;
     if (T || u) {
         if (ptr_kind) { Td = T; ud = u; }
         else {
-            if (T) CK(cudaMalloc(&Td, N * 4), "alloc T");
-            if (u) CK(cudaMalloc(&ud, 3 * N * 4), "alloc u");
+            if (T) CK(down_T.alloc(N * 4), "alloc T");
+            if (u) CK(down_u.alloc(3 * N * 4), "alloc u");
+            Td = down_T.p;
+            ud = down_u.p;
         }
         Bufs b = bufs(h);
         CK(LAUNCH(h, macro, p, h->face, h->inflight, b, Td, ud, h->stream), "macro");
@@ -929,9 +943,7 @@ LBM_API lbm_status lbm_melt_get(lbm_melt *h, float *T, float *u, double *S, doub
             if (u) CK(cudaMemcpyAsync(u, ud, 3 * N * 4, cudaMemcpyDeviceToHost, h->stream), "copy u");
         }
     }
-    const lbm_status st = front_out_sync(h, S, liquid_fraction, ptr_kind);
-    if (!ptr_kind) { cudaFree(Td); cudaFree(ud); }
-    return st;
+    return front_out_sync(h, S, liquid_fraction, ptr_kind);
 }
 
 LBM_API lbm_status lbm_melt_get_async(lbm_melt *h, double *S, double *liquid_fraction, int ptr_kind) {
@@ -944,11 +956,14 @@ LBM_API lbm_status lbm_melt_get_state(lbm_melt *h, float *f, float *g, double *S
     const KP &p = h->kp;
     const size_t N = (size_t)p.N, nc = (size_t)p.ncols;
     float *fd = nullptr, *gd = nullptr;
+    DeviceScratch down_f, down_g;
     if (f || g) {
         if (ptr_kind) { fd = f; gd = g; }
         else {
-            if (f) CK(cudaMalloc(&fd, 19 * N * 4), "alloc f");
-            if (g) CK(cudaMalloc(&gd, 7 * N * 4), "alloc g");
+            if (f) CK(down_f.alloc(19 * N * 4), "alloc f");
+            if (g) CK(down_g.alloc(7 * N * 4), "alloc g");
+            fd = down_f.p;
+            gd = down_g.p;
         }
         Bufs b = bufs(h);
         CK(LAUNCH(h, state_out, p, h->face, h->inflight, b, fd, gd, h->stream), "state out");
@@ -959,9 +974,7 @@ LBM_API lbm_status lbm_melt_get_state(lbm_melt *h, float *f, float *g, double *S
     }
     if (S) CK(cudaMemcpyAsync(S, h->s[h->cur], nc * 8, ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                               h->stream), "copy S");
-    lbm_status st = check_status(h);
-    if (!ptr_kind) { cudaFree(fd); cudaFree(gd); }
-    return st;
+    return check_status(h);
 }
 
 LBM_API lbm_status lbm_melt_set_state(lbm_melt *h, const float *f, const float *g, const double *S, int ptr_kind) {
@@ -969,17 +982,26 @@ LBM_API lbm_status lbm_melt_set_state(lbm_melt *h, const float *f, const float *
     if (S && (!f || !g)) return set_err(h, LBM_EINVAL, "a new front needs f and g too");
     const KP &p = h->kp;
     const size_t N = (size_t)p.N, nc = (size_t)p.ncols;
-    // Bring the layout to natural first, so that kept parts stay valid.
-    if (h->inflight && (!f || !g)) {
-        float *fd = nullptr, *gd = nullptr;
-        CK(cudaMalloc(&fd, 19 * N * 4), "alloc f");
-        CK(cudaMalloc(&gd, 7 * N * 4), "alloc g");
+    // Every buffer and upload before anything of the state is touched: a call
+    // that fails for lack of memory leaves the handle as it was.
+    const bool relayout = h->inflight && (!f || !g);
+    DeviceScratch kept_f, kept_g, up_f, up_g;
+    if (relayout && !f) CK(kept_f.alloc(19 * N * 4), "alloc f");
+    if (relayout && !g) CK(kept_g.alloc(7 * N * 4), "alloc g");
+    const float *fd = f, *gd = g;
+    if (!ptr_kind) {
+        if (f) CK(up_f.alloc(19 * N * 4), "alloc f");
+        if (g) CK(up_g.alloc(7 * N * 4), "alloc g");
+        if (f) CK(cudaMemcpyAsync(up_f.p, f, 19 * N * 4, cudaMemcpyHostToDevice, h->stream), "copy f");
+        if (g) CK(cudaMemcpyAsync(up_g.p, g, 7 * N * 4, cudaMemcpyHostToDevice, h->stream), "copy g");
+        fd = up_f.p;
+        gd = up_g.p;
+    }
+    // Bring the parts that are kept to the natural layout.
+    if (relayout) {
         Bufs b = bufs(h);
-        CK(LAUNCH(h, state_out, p, h->face, 1, b, fd, gd, h->stream), "state out");
-        CK(LAUNCH(h, state_in, p, h->face, b, fd, gd, h->stream), "state in");
-        CK(cudaStreamSynchronize(h->stream), "synchronize");
-        cudaFree(fd);
-        cudaFree(gd);
+        CK(LAUNCH(h, state_out, p, h->face, 1, b, kept_f.p, kept_g.p, h->stream), "state out");
+        CK(LAUNCH(h, state_in, p, h->face, b, kept_f.p, kept_g.p, h->stream), "state in");
     }
     h->inflight = 0;
     h->thw_pending = 0;
@@ -991,13 +1013,8 @@ LBM_API lbm_status lbm_melt_set_state(lbm_melt *h, const float *f, const float *
             s_in = h->s[h->cur];
         }
         // liquid counts of the new fronts; their maximum anew
+        h->rb_valid_from = h->rb_next;  // earlier read-backs may lie below the new counts
         CK(LAUNCH(h, set_fronts, p, bufs(h), s_in, h->s[h->cur], h->js[h->cur], h->stream), "fronts in");
-    }
-    const float *fd = f, *gd = g;
-    float *tf = nullptr, *tg = nullptr;
-    if (!ptr_kind) {
-        if (f) { CK(cudaMalloc(&tf, 19 * N * 4), "alloc f"); CK(cudaMemcpyAsync(tf, f, 19 * N * 4, cudaMemcpyHostToDevice, h->stream), "copy f"); fd = tf; }
-        if (g) { CK(cudaMalloc(&tg, 7 * N * 4), "alloc g"); CK(cudaMemcpyAsync(tg, g, 7 * N * 4, cudaMemcpyHostToDevice, h->stream), "copy g"); gd = tg; }
     }
     if (f || g) {
         Bufs b = bufs(h);
@@ -1006,14 +1023,9 @@ LBM_API lbm_status lbm_melt_set_state(lbm_melt *h, const float *f, const float *
     lbm_status st = refresh_front(h);
     if (st == LBM_OK) st = read_flags(h);
     if (st == LBM_OK) {
-        if (S) {
-            h->rb_valid_from = h->rb_next;  // earlier copies may lie below the new counts
-            seed_readback(h);
-        }
+        if (S) seed_readback(h);
         st = status_of_flags(h);
     }
-    cudaFree(tf);
-    cudaFree(tg);
     return st;
 }
 

@@ -44,3 +44,32 @@ def test_the_call_after_a_failed_one_succeeds():
     del held
     torch.cuda.empty_cache()
     c.close()
+
+
+@pytest.mark.parametrize("leave", [0.8, 1.2])  # f takes 0.93 GiB, g 0.34 GiB
+def test_a_failed_upload_changes_nothing(leave):
+    """The call gives back what it had allocated, and the cavity steps on like
+    one that was never asked."""
+    import torch
+    from paper_1604_03478_gb300 import _abi, LbmError
+    out = []
+    for fail in (False, True):
+        c = _cavity()
+        c.step(7)
+        if fail:
+            f, g = np.zeros((19, c.N), np.float32), np.zeros((7, c.N), np.float32)
+            c.get()
+            held = _hold(int(leave * GB))
+            free = torch.cuda.mem_get_info()[0]
+            for call in (lambda: c.set_state(f, g, np.full(c.ncols, 1.0)), c.get_state):
+                with pytest.raises(LbmError) as ei:
+                    call()
+                assert ei.value.status == _abi.LBM_ENOMEM
+                assert torch.cuda.mem_get_info()[0] == free
+            del held
+            torch.cuda.empty_cache()
+        c.step(30)
+        out.append(c.get()[:3] + (c.totals()["n_liquid"],))
+        c.close()
+    for a, b in zip(*out):
+        np.testing.assert_array_equal(a, b)
