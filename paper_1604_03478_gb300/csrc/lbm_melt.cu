@@ -242,20 +242,27 @@ lbm_status refresh_front(lbm_melt *h) {
     return LBM_OK;
 }
 
-// The address by which a kernel reaches p, a device pointer (ptr_kind 1) or
-// page-locked host memory, aligned to `align` bytes; null for other host
-// memory.  A copy between two kernels costs the stream several microseconds
+// The address by which a kernel reaches the n elements at p, a device pointer
+// (ptr_kind 1) or page-locked host memory, aligned to its type; null for other
+// host memory, for an array that is page-locked at one end only too (a copy
+// then says what it makes of it).  A copy between two kernels costs the stream several microseconds
 // however small it is; GB300 reads and writes page-locked memory from a
 // kernel at link speed.
-template <typename T> T *kernel_view(T *p, int ptr_kind, size_t align) {
-    if (!p || (size_t)p % align) return nullptr;
+template <typename T> T *kernel_view(T *p, int ptr_kind, size_t n) {
+    if (!p || (size_t)p % sizeof(T)) return nullptr;
     if (ptr_kind) return p;
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return nullptr;
+    const unsigned char *const ends[2] = {(const unsigned char *)p, (const unsigned char *)(p + n) - 1};
+    unsigned char *dev[2];
+    for (int k = 0; k < 2; ++k) {
+        cudaPointerAttributes a;
+        if (cudaPointerGetAttributes(&a, ends[k]) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return nullptr;
+        }
+        if (a.type != cudaMemoryTypeHost || !a.devicePointer) return nullptr;
+        dev[k] = (unsigned char *)a.devicePointer;
     }
-    return a.type == cudaMemoryTypeHost ? (T *)a.devicePointer : nullptr;
+    return dev[1] - dev[0] == ends[1] - ends[0] ? (T *)dev[0] : nullptr;
 }
 
 // A new heated-wall field, the old one kept in prev where that is not null.
@@ -830,7 +837,7 @@ LBM_API lbm_status lbm_melt_step(lbm_melt *h, long long n) {
 LBM_API lbm_status lbm_melt_totals(lbm_melt *h, double *out, int ptr_kind) {
     if (!h || !out) return LBM_EINVAL;
     Bufs b = bufs(h);
-    double *const view = ptr_kind ? kernel_view(out, 1, sizeof(double)) : h->host_out;
+    double *const view = ptr_kind ? kernel_view(out, 1, 7) : h->host_out;
     CK(LAUNCH(h, totals, h->kp, h->face, h->inflight, b, h->red_part, h->nred, -1.0, view ? view : h->totals_dev,
               h->stream), "totals");
     if (!view) CK(cudaMemcpyAsync(out, h->totals_dev, 7 * 8, cudaMemcpyDeviceToDevice, h->stream), "copy totals");
@@ -884,7 +891,7 @@ lbm_status enqueue_column_sum(lbm_melt *h, const double *v, double scale, double
     const long long nc = h->kp.ncols;
     const long long nb = std::max<long long>(1, std::min<long long>(kRedBlocks, (nc + 1023) / 1024));
     const long long chunk = (nc + nb - 1) / nb;
-    double *const direct = kernel_view(dst, ptr_kind, sizeof(double));
+    double *const direct = kernel_view(dst, ptr_kind, 1);
     k_sum_once<<<(int)nb, 256, 0, h->stream>>>(v, nc, chunk, scale, h->red_part, h->ticket,
                                                direct ? direct : h->sum_dev, copy);
     CK(cudaGetLastError(), "sum");
@@ -898,7 +905,7 @@ lbm_status enqueue_column_sum(lbm_melt *h, const double *v, double scale, double
 // may be null), enqueued on the handle's stream.
 lbm_status enqueue_front_out(lbm_melt *h, double *S, double *liquid_fraction, int ptr_kind) {
     const double scale = 1.0 / ((double)h->kp.H * (double)h->kp.ncols);
-    double *const view = liquid_fraction ? kernel_view(S, ptr_kind, sizeof(double)) : nullptr;
+    double *const view = liquid_fraction ? kernel_view(S, ptr_kind, (size_t)h->kp.ncols) : nullptr;
     if (S && !view)
         CK(cudaMemcpyAsync(S, h->s[h->cur], (size_t)h->kp.ncols * 8,
                            ptr_kind ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream), "copy S");
@@ -1037,7 +1044,7 @@ LBM_API lbm_status lbm_melt_set_hot_wall(lbm_melt *h, const float *T_h_field, in
     // layout, the field of the last streaming is kept for the Nusselt number
     // until the next step (an even one, which reads no wall).
     const bool keep = h->inflight ? !h->thw_pending : !h->thw_last_prev;
-    const float *const src = kernel_view(T_h_field, ptr_kind, sizeof(float));
+    const float *const src = kernel_view(T_h_field, ptr_kind, nc);
     if (src) {
         k_set_wall<<<(int)((nc + 255) / 256), 256, 0, h->stream>>>(src, h->thw_cur, keep ? h->thw_prev : nullptr,
                                                                    (long long)nc);
