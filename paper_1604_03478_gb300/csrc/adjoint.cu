@@ -763,8 +763,10 @@ struct lbm_tape {
 // The adjoint's device buffers, kept with the handle from one gradient to
 // the next (a loop of gradients of one run length allocates once): the
 // checkpoint pool of the recorded run and the work buffers of the backward,
-// by slot.  A slot is reallocated when a request is larger; released by
-// lbm_melt_tape_clear and lbm_melt_destroy.
+// by slot.  The checkpoint pool has the size of the recorded run; a work
+// buffer is kept while it is large enough (the height bound of one run is
+// seldom that of the next) and memory is not short (trim_workspace).  Released
+// by lbm_melt_tape_clear and lbm_melt_destroy.
 struct AdjWorkspace {
     static const int kSlots = 32;
     void *p[kSlots] = {};
@@ -778,12 +780,12 @@ AdjWorkspace *workspace(lbm_melt *h) {
     return (AdjWorkspace *)h->adj_ws;
 }
 
-// Device buffer of at least `bytes` in workspace slot k (the cached one when
-// it is large enough).
-cudaError_t ws_alloc(lbm_melt *h, int k, size_t bytes, void **out) {
+// Device buffer of at least `bytes` in workspace slot k: the cached one when
+// it is large enough (exact: when it has that size).
+cudaError_t ws_alloc(lbm_melt *h, int k, size_t bytes, void **out, bool exact = false) {
     AdjWorkspace *w = workspace(h);
     if (!w) return cudaErrorMemoryAllocation;
-    if (w->p[k] && w->b[k] >= bytes) {
+    if (w->p[k] && (exact ? w->b[k] == bytes : w->b[k] >= bytes)) {
         *out = w->p[k];
         return cudaSuccess;
     }
@@ -816,6 +818,21 @@ void free_workspace(lbm_melt *h) {
 
 // Workspace slots: 0 the checkpoint pool, 1.. the backward's buffers.
 const int kSlotCheckpoints = 0, kSlotBackward = 1;
+
+// Gives back the backward's buffers that are larger than what is asked for
+// (want: bytes by slot); true if there were any.
+bool trim_workspace(lbm_melt *h, const size_t (&want)[AdjWorkspace::kSlots]) {
+    AdjWorkspace *w = workspace(h);
+    bool any = false;
+    for (int k = kSlotBackward; w && k < AdjWorkspace::kSlots; ++k)
+        if (w->p[k] && w->b[k] > want[k]) {
+            cudaFree(w->p[k]);
+            w->p[k] = nullptr;
+            w->b[k] = 0;
+            any = true;
+        }
+    return any;
+}
 
 lbm_status tape_err(lbm_melt *h, lbm_status st, const char *fmt, ...) {
     if (st == LBM_ECUDA || st == LBM_ENOMEM) (void)cudaGetLastError();
@@ -956,7 +973,9 @@ LBM_API lbm_status lbm_melt_tape_forward(lbm_melt *h, long long steps, long long
     t->ck_bytes = t->ck_bound_off + 256;  // + the recorded height bound
     void *pool = nullptr;
     {
-        const cudaError_t e = ws_alloc(h, kSlotCheckpoints, (size_t)t->nseg * t->ck_bytes + 256, &pool);
+        const size_t bytes = (size_t)t->nseg * t->ck_bytes + 256, none[AdjWorkspace::kSlots] = {};
+        cudaError_t e = ws_alloc(h, kSlotCheckpoints, bytes, &pool, true);
+        if (e != cudaSuccess && trim_workspace(h, none)) e = ws_alloc(h, kSlotCheckpoints, bytes, &pool, true);
         if (e != cudaSuccess) {
             free_tape(h);
             return tape_err(h, LBM_ENOMEM, "%lld checkpoints: %s", t->nseg, cudaGetErrorString(e));
@@ -1051,31 +1070,38 @@ LBM_API lbm_status lbm_melt_tape_backward(lbm_melt *h, const double *seed, doubl
     // an error they are released
     auto cleanup = [&]() {};
     const int nal = (int)(sizeof al / sizeof al[0]);
-    for (int k = 0; k < nal; ++k) {
-        cudaError_t e = ws_alloc(h, kSlotBackward + k, al[k].b, al[k].p);
-        if (e != cudaSuccess) {
-            free_workspace(h);
-            return tape_err(h, LBM_ENOMEM, "adjoint buffers: %s", cudaGetErrorString(e));
-        }
-    }
     // the second snapshot set if the device has room for it (else the
     // segments run one after another through the first)
-    int nsets = 2;
-    {
-        const int k2 = kSlotBackward + nal;
-        if (ws_alloc(h, k2, (size_t)(C + 1) * 26 * N * 4, (void **)&snapb[1]) != cudaSuccess ||
-            ws_alloc(h, k2 + 1, (size_t)(C + 1) * nc * 8, (void **)&snap_sb[1]) != cudaSuccess ||
-            ws_alloc(h, k2 + 2, (size_t)(C + 1) * nc * 4, (void **)&snap_jsb[1]) != cudaSuccess ||
-            ws_alloc(h, k2 + 3, (size_t)(C + 1) * nc * 4, (void **)&snap_nbb[1]) != cudaSuccess) {
-            (void)cudaGetLastError();
-            AdjWorkspace *w = workspace(h);
-            for (int k = k2; k < k2 + 4; ++k)
-                if (w->p[k]) { cudaFree(w->p[k]); w->p[k] = nullptr; w->b[k] = 0; }
-            snapb[1] = nullptr;
-            snap_sb[1] = nullptr;
-            snap_jsb[1] = nullptr;
-            snap_nbb[1] = nullptr;
-            nsets = 1;
+    Alloc second[] = {{(void **)&snapb[1], (size_t)(C + 1) * 26 * N * 4}, {(void **)&snap_sb[1], (size_t)(C + 1) * nc * 8},
+                      {(void **)&snap_jsb[1], (size_t)(C + 1) * nc * 4}, {(void **)&snap_nbb[1], (size_t)(C + 1) * nc * 4}};
+    const int k2 = kSlotBackward + nal;
+    cudaError_t first_error = cudaSuccess;
+    auto reserve = [&]() {  // how many snapshot sets there is room for
+        for (int k = 0; k < nal; ++k)
+            if ((first_error = ws_alloc(h, kSlotBackward + k, al[k].b, al[k].p)) != cudaSuccess) return 0;
+        for (int k = 0; k < 4; ++k)
+            if (ws_alloc(h, k2 + k, second[k].b, second[k].p) != cudaSuccess) return 1;
+        return 2;
+    };
+    int nsets = reserve();
+    if (nsets < 2) {
+        // larger buffers kept from other runs may be what is in the way
+        size_t want[AdjWorkspace::kSlots] = {};
+        for (int k = 0; k < nal; ++k) want[kSlotBackward + k] = al[k].b;
+        for (int k = 0; k < 4; ++k) want[k2 + k] = second[k].b;
+        if (trim_workspace(h, want)) nsets = reserve();
+    }
+    if (nsets == 0) {
+        free_workspace(h);
+        return tape_err(h, LBM_ENOMEM, "adjoint buffers: %s", cudaGetErrorString(first_error));
+    }
+    if (nsets == 1) {
+        AdjWorkspace *w = workspace(h);
+        for (int k = 0; k < 4; ++k) {
+            if (w->p[k2 + k]) cudaFree(w->p[k2 + k]);
+            w->p[k2 + k] = nullptr;
+            w->b[k2 + k] = 0;
+            *second[k].p = nullptr;
         }
     }
 #define BCK(call, where)                                                             \
