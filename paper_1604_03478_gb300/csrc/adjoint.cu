@@ -1092,7 +1092,10 @@ LBM_API lbm_status lbm_melt_tape_backward(lbm_melt *h, const double *seed, doubl
         if (trim_workspace(h, want)) nsets = reserve();
     }
     if (nsets == 0) {
-        free_workspace(h);
+        // the recorded run's checkpoints stay: the caller may make room and
+        // ask again
+        const size_t none[AdjWorkspace::kSlots] = {};
+        trim_workspace(h, none);
         return tape_err(h, LBM_ENOMEM, "adjoint buffers: %s", cudaGetErrorString(first_error));
     }
     if (nsets == 1) {

@@ -53,3 +53,26 @@ def test_buffers_of_the_run_before(order):
     del held
     torch.cuda.empty_cache()
     c.close()
+
+
+def test_backward_after_one_without_room():
+    """A backward without room for its buffers says so and keeps the recorded
+    run: asked again with room, it gives the gradient."""
+    import torch
+    from paper_1604_03478_gb300 import _abi, LbmError
+    c, start, seed = _setup()
+    c.tape_forward(STEPS, STEPS)
+    want = c.tape_backward(seed)
+    c.tape_clear()
+    c.set_state(*start)
+    c.tape_forward(STEPS, STEPS)
+    held = _hold(int(0.5 * GB))  # the snapshots take 0.85 GiB
+    with pytest.raises(LbmError) as ei:
+        c.tape_backward(seed)
+    assert ei.value.status == _abi.LBM_ENOMEM
+    del held
+    torch.cuda.empty_cache()
+    got = c.tape_backward(seed)
+    np.testing.assert_array_equal(got[0], want[0])
+    assert got[1] == want[1]
+    c.close()
