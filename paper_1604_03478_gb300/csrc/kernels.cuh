@@ -861,7 +861,7 @@ __device__ __forceinline__ void even_pair_load(const KP &p, const ST *F, const S
 template <typename ST, typename IX>
 __device__ __forceinline__ void even_pair_finish(const KP &p, ST *__restrict__ F, ST *__restrict__ G, IX c,
                                                  float2 (&f)[19], float2 (&g)[7]) {
-    collide2(p, f, g);
+    collide2<sizeof(ST) == 4>(p, f, g);
 #pragma unroll
     for (int i = 0; i < 19; ++i) st_pair(elem<IX>(F, c, opp(i) * p.ld), f[i]);
 #pragma unroll
@@ -934,7 +934,7 @@ __device__ __forceinline__ void odd_pair_finish(const KP &p, const Links *lk, ST
                                                 int x, int y, int z, float2 (&f)[19], float2 (&g)[7]) {
     const IX c = (IX)node_index(p, x, y, z), c1 = c + 1;
     const bool xlo = x == 0, xhi = x + 1 == p.nx - 1;
-    collide2(p, f, g);
+    collide2<sizeof(ST) == 4>(p, f, g);
 #pragma unroll
     for (int i = 0; i < 19; ++i) {
         if (ex(i) == 0) {
