@@ -279,7 +279,7 @@ __global__ void k_set_wall(const float *__restrict__ src, float *cur, float *pre
 struct DeviceScratch {
     float *p = nullptr;
     cudaError_t alloc(size_t bytes) { return cudaMalloc(&p, bytes); }
-    ~DeviceScratch() { cudaFree(p); }
+    ~DeviceScratch() { if (p) cudaFree(p); }
     DeviceScratch() = default;
     DeviceScratch(const DeviceScratch &) = delete;
     DeviceScratch &operator=(const DeviceScratch &) = delete;
