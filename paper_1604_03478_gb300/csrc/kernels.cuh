@@ -1813,6 +1813,27 @@ __global__ void __launch_bounds__(128) k_nusselt(const __grid_constant__ KP p, c
 }
 
 // ------------------------------------------------------ FP64 reductions
+// A sum of FP32 values held as three floats: the error of every addition
+// (Knuth's two-sum, exact) goes on to the next, so the sum carries some 72
+// bits, more than FP64.  FP64 issues at a small fraction of the FP32 rate
+// here: with two FP64 sums a node a totals call on a convecting 256^3 state at 0.4 H
+// took 165.6 us, with these 150.3 (in flight 198; two floats, which hold only
+// 48 bits, 150.4 and 193).
+struct TripleSum {
+    float a = 0.0f, b = 0.0f, c = 0.0f;
+    static __device__ __forceinline__ float two_sum(float &s, float v) {
+        const float t = __fadd_rn(s, v), z = __fsub_rn(t, s);
+        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v, z));
+        s = t;
+        return e;
+    }
+    __device__ __forceinline__ void add(float v) { c = __fadd_rn(c, two_sum(b, two_sum(a, v))); }
+    __device__ __forceinline__ double value() const {
+        const double tail = (double)b + (double)c;
+        return isfinite(tail) ? (double)a + tail : (double)a;  // an infinite a leaves NaN behind
+    }
+};
+
 constexpr int kTotals = 6;       // partials of a block
 constexpr int kTotalsRun = 8;    // heights of a tile
 // Block partials of the liquid-node totals: sum (T - Tm), sum (rho - 1),
@@ -1820,12 +1841,10 @@ constexpr int kTotalsRun = 8;    // heights of a tile
 // walk over tiles of 256 columns by kTotalsRun heights in a fixed order:
 // deterministic.  max |u|^2 is taken in FP64, as is, of the nodes whose FP32
 // value comes within its rounding (below 4e-7 relative) of the maximum so
-// far.  The sums are FP64 throughout (sums of FP32 pairs hold 48 bits).
-// Read bandwidth bounds it (104 bytes a liquid node with FP32 storage);
+// far.  Read bandwidth bounds it (104 bytes a liquid node with FP32 storage);
 // with every |u|^2 and count in FP64 too, 64-bit divisions for the node's
 // coordinates and the column sums left to one block, a totals call on a 256^3
-// cavity at 0.4 H took 486 us (FP16 storage 1127), now 146, in flight 186 (125, 186);
-// pairs of FP32 values instead of FP64 sums gained nothing (145, 184).
+// cavity at 0.4 H took 486 us (FP16 storage 1127), now 150 (138), in flight 198.
 template <typename ST, int FACE>
 __global__ void __launch_bounds__(256, 4) k_totals_part(const __grid_constant__ KP p, const ST *__restrict__ F, const ST *__restrict__ G,
                                                      const int *__restrict__ js, const int *__restrict__ js_old,
@@ -1833,7 +1852,8 @@ __global__ void __launch_bounds__(256, 4) k_totals_part(const __grid_constant__ 
                                                      const float *__restrict__ thw_nu, int inflight, double nu_scale,
                                                      double *__restrict__ part) {
     __shared__ double sh[kTotals][256];
-    double sT = 0.0, sr = 0.0, ss = 0.0, sn = 0.0, umax = 0.0;
+    TripleSum sT, sr;
+    double ss = 0.0, sn = 0.0, umax = 0.0;
     float ufloor = 0.0f;  // nodes with an FP32 |u|^2 below it are not the maximum
     int n = 0;
     const int ctiles = (p.ncols + 255) / 256, atiles = (p.H + kTotalsRun - 1) / kTotalsRun;
@@ -1859,8 +1879,8 @@ __global__ void __launch_bounds__(256, 4) k_totals_part(const __grid_constant__ 
 #pragma unroll
             for (int i = 0; i < 19; ++i) { rh += f[i]; ux += ex(i) * f[i]; uy += ey(i) * f[i]; uz += ez(i) * f[i]; }
             uz += 0.5f * p.gbeta * (Th - p.dTms);
-            sT += Th - p.dTms;
-            sr += rh;
+            sT.add(Th - p.dTms);
+            sr.add(rh);
             ++n;
             if (ux * ux + uy * uy + uz * uz >= ufloor) {
                 const double u2 = (double)ux * ux + (double)uy * uy + (double)uz * uz;
@@ -1871,7 +1891,7 @@ __global__ void __launch_bounds__(256, 4) k_totals_part(const __grid_constant__ 
             }
         }
     }
-    const double v[kTotals] = {sT, sr, (double)n, umax, ss, sn};
+    const double v[kTotals] = {sT.value(), sr.value(), (double)n, umax, ss, sn};
 #pragma unroll
     for (int k = 0; k < kTotals; ++k) sh[k][threadIdx.x] = v[k];
     __syncthreads();
