@@ -102,7 +102,7 @@ struct lbm_melt {
     cudaStream_t cap_stream;     // private stream the graphs are captured on
     struct StepGraph {
         cudaGraphExec_t exec;
-        int height, bx, by;
+        int height, bx, by, linear;
     } graphs[2][2];              // [cur][inflight]
     std::vector<cudaEvent_t> ev;  // start/stop pairs of timed launches
     size_t ev_used;

@@ -498,14 +498,16 @@ cudaError_t enqueue_step(lbm_melt *h, int &cur, int &inflight, int height, dim3 
 
 // The graph of graph_steps steps from the handle's phase with the
 // stream-collide grid cut at `height` or higher: the cached one when it was
-// captured for this phase and block shape at a height from `height` to
+// captured for this phase, block shape and layout at a height from `height` to
 // height + 32, else a new capture (heights rounded up to a multiple of 8).
 // The replays are bit-identical to single steps: the extra blocks of a
 // higher grid find only deep solid nodes and return at once.
 lbm_status step_graph(lbm_melt *h, int height, cudaGraphExec_t *out) {
     const dim3 blk = sc_block(h);
     lbm_melt::StepGraph &g = h->graphs[h->cur][h->inflight];
-    if (g.exec && g.bx == (int)blk.x && g.by == (int)blk.y && g.height >= height && g.height <= height + 32) {
+    const int linear = sc_linear(h) ? 1 : 0;  // blocks of 128 columns and rows of 128 have one shape
+    if (g.exec && g.bx == (int)blk.x && g.by == (int)blk.y && g.linear == linear && g.height >= height &&
+        g.height <= height + 32) {
         *out = g.exec;
         return LBM_OK;
     }
@@ -536,6 +538,7 @@ lbm_status step_graph(lbm_melt *h, int height, cudaGraphExec_t *out) {
     g.height = hc;
     g.bx = (int)blk.x;
     g.by = (int)blk.y;
+    g.linear = linear;
     *out = g.exec;
     return LBM_OK;
 }
