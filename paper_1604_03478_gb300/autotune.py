@@ -2,15 +2,19 @@
 caches the choice as JSON (one file per machine, next to the built library).
 
 Two searches:
-  * single cavity: the (bx, by) block shape of the stream-collide kernels,
-    per (cavity edge lengths, precision);
-  * ensemble: (threads per block, nodes per thread) of the persistent kernel,
-    per (number of cavities, total nodes, precision).
+  * single cavity: the (bx, by) block shape of the stream-collide kernels;
+  * ensemble: (threads per block, nodes per thread) of the persistent kernel.
+An entry is for the device, what the choice depends on (edge lengths, heated
+face, storage, nodes per thread, conduction in the solid; for an ensemble its
+members' edges and faces) and the library's sources: shapes measured with other
+kernels, or before the default was one of the candidates, are measured anew.
 Timing is by CUDA events on the handle's stream; the state advances while
 tuning (tune before the run you care about, or on a scratch copy).
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import os
 
@@ -24,6 +28,25 @@ ENSEMBLE_SHAPES = ((64, 2), (128, 1), (128, 2), (128, 4), (128, 8), (256, 1), (2
 def _device_key():
     import torch
     return torch.cuda.get_device_name()
+
+
+@functools.lru_cache(maxsize=None)
+def _code_key():
+    h = hashlib.sha1()
+    for path in sorted(_build._deps()):
+        with open(path, "rb") as fh:
+            h.update(fh.read())
+    return h.hexdigest()[:12]
+
+
+def _cavity_key(cav):
+    return "cavity|%s|%s|face%d|p%d|pairs%d|solid%d|%s" % (
+        _device_key(), "x".join(map(str, cav.shape)), cav.face, cav.precision, cav.node_pairs, cav.solid, _code_key())
+
+
+def _ensemble_key(ens):
+    members = hashlib.sha1(repr(ens.dims).encode()).hexdigest()[:12]
+    return "ensemble|%s|n%d|%s|p%d|%s" % (_device_key(), ens.n, members, ens.precision, _code_key())
 
 
 def _load():
@@ -56,9 +79,9 @@ def _time(step, sync, steps, stream):
 
 
 def tune_cavity(cav, steps=20, shapes=CAVITY_SHAPES, use_cache=True):
-    """Best (bx, by) for this cavity's size and precision; applied to cav."""
+    """Best (bx, by) for this cavity; applied to cav."""
     import torch
-    key = "cavity|%s|%s|p%d" % (_device_key(), "x".join(map(str, cav.shape)), cav.grid.precision)
+    key = _cavity_key(cav)
     cache = _load()
     if use_cache and key in cache:
         bx, by = cache[key]["shape"]
@@ -80,9 +103,7 @@ def tune_cavity(cav, steps=20, shapes=CAVITY_SHAPES, use_cache=True):
 def tune_ensemble(ens, steps=8, shapes=ENSEMBLE_SHAPES, use_cache=True, graph_steps=8):
     """Best (block, nodes per thread) of the persistent kernel; applied."""
     import torch
-    info = ens.info()
-    prec = ens.member(0).grid.precision if hasattr(ens.member(0), "grid") else 0
-    key = "ensemble|%s|n%d|%d|p%d" % (_device_key(), ens.n, info["nodes"], prec)
+    key = _ensemble_key(ens)
     cache = _load()
     if use_cache and key in cache:
         b, k = cache[key]["shape"]

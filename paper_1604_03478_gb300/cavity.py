@@ -54,6 +54,8 @@ class Cavity:
     (lbm_melt_set_solid_conduction).
     """
 
+    node_pairs, solid = -1, 0  # as set_node_pairs and set_solid_conduction left them
+
     def __init__(self, nx, ny, nz, face=0, precision=0, Ra=0.0, Pr=1.0, Ste=0.1, Th=1.0, Tc=0.0, Tm=0.0,
                  Ma=0.1, s0=1.0, s_nu=1.0, s_alpha=1.0, derive=False, stream=None, solid=0, ks_kl=1.0,
                  **rates):
@@ -73,6 +75,7 @@ class Cavity:
         self.shape = (nz, ny, nx)
         self.N = nx * ny * nz
         self.face = face
+        self.precision = precision
         self.H = ny if face == 0 else nz
         self.cols_shape = (nz, nx) if face == 0 else (ny, nx)
         self.ncols = self.cols_shape[0] * self.cols_shape[1]
@@ -80,7 +83,7 @@ class Cavity:
             self.set_solid_conduction(ks_kl)
 
     @classmethod
-    def _member(cls, handle, nx, ny, nz, face):
+    def _member(cls, handle, nx, ny, nz, face, precision):
         """View of a cavity owned by an ensemble (never destroyed here)."""
         obj = cls.__new__(cls)
         obj._h = C.c_void_p(handle)
@@ -88,6 +91,7 @@ class Cavity:
         obj.shape = (nz, ny, nx)
         obj.N = nx * ny * nz
         obj.face = face
+        obj.precision = precision
         obj.H = ny if face == 0 else nz
         obj.cols_shape = (nz, nx) if face == 0 else (ny, nx)
         obj.ncols = obj.cols_shape[0] * obj.cols_shape[1]
@@ -212,11 +216,13 @@ class Cavity:
         """Nodes per thread of the stream-collide: -1 choose, 0 one, 1 two
         (lbm_melt_set_node_pairs)."""
         self._check(_abi.load().lbm_melt_set_node_pairs(self._h, int(mode)))
+        self.node_pairs = int(mode)
 
     def set_solid_conduction(self, ks_kl):
         """Heat conduction in the solid with k_s / k_l = ks_kl (0: off);
         before the first step, re-initialises the state."""
         self._check(_abi.load().lbm_melt_set_solid_conduction(self._h, float(ks_kl)))
+        self.solid = 1 if ks_kl else 0
 
     def set_graph_steps(self, steps):
         """Steps per CUDA-graph replay in step() (0: step by step)."""

@@ -18,7 +18,8 @@ class Ensemble:
             import torch
             stream = torch.cuda.current_stream().cuda_stream
         arr = (_abi.lbm_melt_case * len(cases))()
-        self._dims = []
+        self.dims = []  # (nx, ny, nz, face) of each member
+        self.precision = cases[0].get("precision", 0) if cases else 0  # of all members
         for k, c in enumerate(cases):
             c = dict(c)
             nx, ny, nz = c.pop("nx"), c.pop("ny"), c.pop("nz")
@@ -36,7 +37,7 @@ class Ensemble:
             arr[k].Tm = c.pop("Tm", 0.0)
             if c:
                 raise TypeError("unknown case keys: %s" % sorted(c))
-            self._dims.append((nx, ny, nz, face))
+            self.dims.append((nx, ny, nz, face))
         h = C.c_void_p()
         st = L.lbm_ensemble_create(len(cases), arr, C.c_void_p(stream), C.byref(h))
         if st != 0:
@@ -82,8 +83,8 @@ class Ensemble:
         h = _abi.load().lbm_ensemble_member(self._h, int(i))
         if not h:
             raise IndexError(i)
-        nx, ny, nz, face = self._dims[i]
-        return Cavity._member(h, nx, ny, nz, face)
+        nx, ny, nz, face = self.dims[i]
+        return Cavity._member(h, nx, ny, nz, face, self.precision)
 
     def close(self):
         if getattr(self, "_h", None):
