@@ -121,11 +121,11 @@ lbm_status lbm_melt_create(const lbm_melt_grid *grid, double Ra, double Pr, doub
 /* Advance n >= 0 time steps (Eqs. 1-6 per step: stream-collide, front
    update, phase flip).  Asynchronous, with one exception: with Tc == Tm the
    stream-collide grid stops above the liquid (deep solid nodes have no
-   work), at a height taken from a copy of the running maximum liquid count
-   that the device posts every 4 steps; before a step the host uses the newest
-   copy already complete, else waits for one 16 steps old.  So the host blocks
-   only while it is more than ~16 steps ahead of the device (no effect on the
-   results). */
+   work), at a height taken from the running maximum liquid count, which the
+   device raises in page-locked memory.  The host marks every fourth step;
+   before a step it goes by the newest mark that the device is known to have
+   passed, else waits for one 16 steps old.  So the host blocks only while it
+   is more than ~16 steps ahead of the device (no effect on the results). */
 lbm_status lbm_melt_step(lbm_melt *h, long long n);
 
 /* Macroscopic outputs, any of them NULL to skip: T per node (solid nodes
@@ -193,7 +193,8 @@ lbm_status lbm_melt_set_hot_wall(lbm_melt *h, const float *T_h_field, int ptr_ki
    liquid nodes, out[4] max |u| over liquid nodes, out[5] sum of S over
    columns, out[6] mean Nusselt number over the heated wall (as
    lbm_melt_get_nusselt).  The heat content relative to solid at Tm is
-   out[1] + (Th - Tm) / Ste * out[5].  Deterministic (fixed reduction order).
+   out[1] + (Th - Tm) / Ste * out[5].  Deterministic (fixed reduction order);
+   the sums of FP32 values carry FP64's precision or more at every stage.
    Synchronises. */
 lbm_status lbm_melt_totals(lbm_melt *h, double *out, int ptr_kind);
 
@@ -237,7 +238,7 @@ lbm_status lbm_melt_set_timing(lbm_melt *h, int enable);
 lbm_status lbm_melt_kernel_time(lbm_melt *h, double *ms, long long *launches, int reset);
 
 /* Replay lbm_melt_step's steps from CUDA graphs of `steps` steps each (0:
-   launch every step on its own).  A step is three kernels; on a small
+   launch every step on its own).  A step is two kernels; on a small
    cavity the host's launches take longer than the GPU's work, so by default
    cavities of at most 160^3 nodes replay 16 steps per graph and larger ones
    launch step by step.  A graph is captured once per starting phase of the
@@ -362,14 +363,17 @@ lbm_status lbm_ensemble_create(int n, const lbm_melt_case *cases, void *cuda_str
 lbm_status lbm_ensemble_step(lbm_ensemble *e, long long nsteps);
 
 /* Launch shape: threads per block (64, 128 or 256; a block covers an x-y
-   tile of one cavity), nodes per thread in the stream-collide phase (1, 2,
-   4 or 8 consecutive z-planes) and the unit of the steps per graph replay
+   tile of one cavity, or, in an ensemble whose tiles would leave a tenth of
+   the lanes idle, a run of consecutive columns), nodes per thread in the
+   stream-collide phase (1, 2, 4 or 8 consecutive z-planes, or heights of the
+   columns) and the unit of the steps per graph replay
    (even, >= 2).  The grid is the co-resident maximum for that shape.  Until it
    is called: 256 threads and one node for an ensemble that fits two such
    items a block, else 128 and two, and 8 steps. */
 lbm_status lbm_ensemble_set_launch(lbm_ensemble *e, int block, int nodes_per_thread, int graph_steps);
 
-/* Bound of a barrier wait, in polls (default 2^24, about a second). */
+/* Bound of a barrier wait, in polls (default 2^24; a poll takes 0.32 to 0.37
+   us, so more than five seconds). */
 lbm_status lbm_ensemble_set_barrier_timeout(lbm_ensemble *e, long long max_spins);
 
 /* Test hook for failure detection: one step in which block `block` never
@@ -390,7 +394,8 @@ lbm_status lbm_ensemble_inject_barrier_fault(lbm_ensemble *e, int block);
    the read fails. */
 lbm_status lbm_ensemble_phase_times(lbm_ensemble *e, int reset, double *us_per_step, long long *steps);
 
-/* Wait for the ensemble; report a barrier timeout or a member's error. */
+/* Wait for the ensemble; report a barrier timeout (of any launch since the
+   last report) or a member's error. */
 lbm_status lbm_ensemble_sync(lbm_ensemble *e);
 
 /* Member i as a cavity handle (for lbm_melt_get, _totals, _set_hot_wall ...;

@@ -851,21 +851,6 @@ lbm_status tape_err(lbm_melt *h, lbm_status st, const char *fmt, ...) {
                             cudaGetErrorString(e_));                                                       \
     } while (0)
 
-// Launch with programmatic stream serialization (see step_launch_wait).
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grd, dim3 blk, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grd;
-    cfg.blockDim = blk;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
-}
-
 // Layout of a checkpoint: the nine state arrays of a handle, each starting
 // on a 256-byte boundary.  Returns the total size; dev/sz/off describe them.
 size_t state_layout(const lbm_melt *h, void *dev[9], size_t sz[9], size_t off[9]) {
@@ -1168,7 +1153,8 @@ LBM_API lbm_status lbm_melt_tape_backward(lbm_melt *h, const double *seed, doubl
             return cudaGetLastError();
         };
         // the snapshot of a level is written by the step that leaves it where
-        // that step can (one node per thread), else by a launch of its own
+        // that step can (one node per thread, or the early pair kernels), else
+        // by a launch of its own
         cudaError_t e = cudaSuccess;
         for (long long j = 0; j < len && e == cudaSuccess; ++j) {
             const lbm::SnapOut o = out(j);
@@ -1203,20 +1189,20 @@ LBM_API lbm_status lbm_melt_tape_backward(lbm_melt *h, const double *seed, doubl
                     e = cudaGetLastError();
                 }
                 if (e == cudaSuccess)
-                    e = launch_pdl(lbm::k_adj_node<0>, grd, blk, sm, pa, s0, st_js, st_nb, lm[1], lm[0], lgpost, lthw, part);
+                    e = lbm::launch_step_kernel(lbm::k_adj_node<0>, grd, blk, sm, 0, pa, s0, st_js, st_nb, lm[1], lm[0], lgpost, lthw, part);
                 if (e == cudaSuccess)
-                    e = j > 0 ? launch_pdl(lbm::k_adj_ghost_front<0>, cgrid, dim3(cb), sm, pa, s0, st_js, st_s, st_s_prev, thw, lgpost, lm[0], lms[0], lms[1], lthw, lsal, lgb, lcoef, wp[pj], wq[pj], wp[pm], wq[pm])
-                              : launch_pdl(lbm::k_adj_ghost<0>, cgrid, dim3(cb), sm, pa, s0, st_js, st_s, thw, lgpost, lm[0], lms[0], lthw, lsal, lgb, wp[pj], wq[pj]);
+                    e = j > 0 ? lbm::launch_step_kernel(lbm::k_adj_ghost_front<0>, cgrid, dim3(cb), sm, 0, pa, s0, st_js, st_s, st_s_prev, thw, lgpost, lm[0], lms[0], lms[1], lthw, lsal, lgb, lcoef, wp[pj], wq[pj], wp[pm], wq[pm])
+                              : lbm::launch_step_kernel(lbm::k_adj_ghost<0>, cgrid, dim3(cb), sm, 0, pa, s0, st_js, st_s, thw, lgpost, lm[0], lms[0], lthw, lsal, lgb, wp[pj], wq[pj]);
             } else {
                 if (j == len - 1) {
                     lbm::k_adj_front<1><<<cgrid, cb, 0, sm>>>(pa, s1, st_s, thw, lms[1], lms[0], wp[pj], wq[pj], lm[1], lthw, lcoef);
                     e = cudaGetLastError();
                 }
                 if (e == cudaSuccess)
-                    e = launch_pdl(lbm::k_adj_node<1>, grd, blk, sm, pa, s0, st_js, st_nb, lm[1], lm[0], lgpost, lthw, part);
+                    e = lbm::launch_step_kernel(lbm::k_adj_node<1>, grd, blk, sm, 0, pa, s0, st_js, st_nb, lm[1], lm[0], lgpost, lthw, part);
                 if (e == cudaSuccess)
-                    e = j > 0 ? launch_pdl(lbm::k_adj_ghost_front<1>, cgrid, dim3(cb), sm, pa, s0, st_js, st_s, st_s_prev, thw, lgpost, lm[0], lms[0], lms[1], lthw, lsal, lgb, lcoef, wp[pj], wq[pj], wp[pm], wq[pm])
-                              : launch_pdl(lbm::k_adj_ghost<1>, cgrid, dim3(cb), sm, pa, s0, st_js, st_s, thw, lgpost, lm[0], lms[0], lthw, lsal, lgb, wp[pj], wq[pj]);
+                    e = j > 0 ? lbm::launch_step_kernel(lbm::k_adj_ghost_front<1>, cgrid, dim3(cb), sm, 0, pa, s0, st_js, st_s, st_s_prev, thw, lgpost, lm[0], lms[0], lms[1], lthw, lsal, lgb, lcoef, wp[pj], wq[pj], wp[pm], wq[pm])
+                              : lbm::launch_step_kernel(lbm::k_adj_ghost<1>, cgrid, dim3(cb), sm, 0, pa, s0, st_js, st_s, thw, lgpost, lm[0], lms[0], lthw, lsal, lgb, wp[pj], wq[pj]);
             }
             std::swap(lm[0], lm[1]);
             std::swap(lms[0], lms[1]);

@@ -245,7 +245,7 @@ LBM_API lbm_status lbm_ensemble_create(int n, const lbm_melt_case *cases, void *
     e->user = (cudaStream_t)cuda_stream;
     e->block = 128;
     e->K = 2;
-    e->max_spins = 1LL << 24;  // with 64 ns sleeps: about a second
+    e->max_spins = 1LL << 24;  // polls of 0.32 to 0.37 us with their 32 ns sleeps: more than five seconds
     e->graph_steps = 8;
     e->desc.resize(n);
     auto fail = [&](lbm_status st) {

@@ -150,33 +150,16 @@ __global__ void __launch_bounds__(128, pair_min_blocks<ST>()) k_odd_pair_cond(
         odd_pair_cond<ST, FACE, IX>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, spost, x, y, z);
 }
 
-// The conduction step's kernels are launched like the plain step's, with
-// programmatic stream serialization (see step_launch_wait), or plainly (see
-// launch_step_kernel).
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_cond_kernel(void (*kern)(KArgs...), dim3 grd, dim3 blk, cudaStream_t st, int plain, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grd;
-    cfg.blockDim = blk;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = plain ? 0 : 1;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 // Two nodes per thread, element indices in IX (32 bits whenever all fit).
 template <typename ST, typename IX, int LIN>
 static cudaError_t launch_pair_cond(const KP &p, int face, int odd, const Bufs &b, dim3 g2, dim3 blk, cudaStream_t st) {
     ST *F = (ST *)b.F, *G = (ST *)b.G;
     if (face == 0) {
-        if (odd) return launch_cond_kernel(k_odd_pair_cond<ST, 0, IX, LIN>, g2, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
-        else return launch_cond_kernel(k_even_pair_cond<ST, 0, IX, LIN>, g2, blk, st, b.plain, p, F, G, b.js, b.nb, b.gpost, b.spost);
+        if (odd) return launch_step_kernel(k_odd_pair_cond<ST, 0, IX, LIN>, g2, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
+        else return launch_step_kernel(k_even_pair_cond<ST, 0, IX, LIN>, g2, blk, st, b.plain, p, F, G, b.js, b.nb, b.gpost, b.spost);
     } else {
-        if (odd) return launch_cond_kernel(k_odd_pair_cond<ST, 1, IX, LIN>, g2, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
-        else return launch_cond_kernel(k_even_pair_cond<ST, 1, IX, LIN>, g2, blk, st, b.plain, p, F, G, b.js, b.nb, b.gpost, b.spost);
+        if (odd) return launch_step_kernel(k_odd_pair_cond<ST, 1, IX, LIN>, g2, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
+        else return launch_step_kernel(k_even_pair_cond<ST, 1, IX, LIN>, g2, blk, st, b.plain, p, F, G, b.js, b.nb, b.gpost, b.spost);
     }
 }
 
@@ -194,11 +177,11 @@ cudaError_t LaunchCond<ST>::stream_collide(const KP &p, int face, int odd, const
     }
     const dim3 grd = k1_grid(p, blk, face, p.H, b.linear);
     if (face == 0) {
-        if (odd) return launch_cond_kernel(k_odd_cond<ST, 0>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
-        else return launch_cond_kernel(k_even_cond<ST, 0>, grd, blk, st, b.plain, p, F, G, b.js, b.nb, b.gpost, b.spost);
+        if (odd) return launch_step_kernel(k_odd_cond<ST, 0>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
+        else return launch_step_kernel(k_even_cond<ST, 0>, grd, blk, st, b.plain, p, F, G, b.js, b.nb, b.gpost, b.spost);
     } else {
-        if (odd) return launch_cond_kernel(k_odd_cond<ST, 1>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
-        else return launch_cond_kernel(k_even_cond<ST, 1>, grd, blk, st, b.plain, p, F, G, b.js, b.nb, b.gpost, b.spost);
+        if (odd) return launch_step_kernel(k_odd_cond<ST, 1>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb, b.gpost, b.thw_rd, b.thw_wr, *b.lk, b.spost);
+        else return launch_step_kernel(k_even_cond<ST, 1>, grd, blk, st, b.plain, p, F, G, b.js, b.nb, b.gpost, b.spost);
     }
 }
 
@@ -208,9 +191,9 @@ cudaError_t LaunchCond<ST>::front(const KP &p, int face, int inflight, int move,
     ST *F = (ST *)b.F;
     const ST *G = (const ST *)b.G;
     if (face == 0)
-        return launch_cond_kernel(k_front_cond<ST, 0>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost,
+        return launch_step_kernel(k_front_cond<ST, 0>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost,
                                   b.spost, b.thw_wr, inflight, move, b.status);
-    return launch_cond_kernel(k_front_cond<ST, 1>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.spost,
+    return launch_step_kernel(k_front_cond<ST, 1>, grd, blk, st, b.plain, p, F, G, b.js, b.js_next, b.nb_next, b.s, b.s_next, b.gpost, b.spost,
                               b.thw_wr, inflight, move, b.status);
 }
 

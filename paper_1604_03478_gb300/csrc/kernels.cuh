@@ -43,6 +43,26 @@ __device__ __forceinline__ void step_launch_wait() {
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
+// How the kernels that call step_launch_wait are launched (the step's, the
+// adjoint's): with programmatic stream serialization, but plainly (`plain`)
+// after a kernel that is not one of them and writes what this one loads before
+// its wait (a wall field, fronts, a restored state): such a kernel lets its
+// successor start when its blocks have returned, which does not order its
+// stores before loads that no wait precedes.
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_step_kernel(void (*kern)(KArgs...), dim3 grd, dim3 blk, cudaStream_t st, int plain, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grd;
+    cfg.blockDim = blk;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = plain ? 0 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
 // What a kernel may load before step_launch_wait: whatever its immediate
 // predecessor does not write.  The predecessor let this kernel start only
 // after its own wait, so everything before the predecessor is complete (after
@@ -266,9 +286,8 @@ __device__ __forceinline__ bool k1_late(int early_blocks) {
     return (long long)(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x >= early_blocks;
 }
 template <int FACE>
-__device__ __forceinline__ bool k1_node(const KP &p, const int *jmax, int &x, int &y, int &z) {
-    const int a0 = (int)blockIdx.z * (FACE == 0 ? (int)blockDim.y : 1);  // lowest height of the block
-    if (jmax && a0 >= *jmax + 3) return false;
+__device__ __forceinline__ bool k1_node(const KP &p, int &x, int &y, int &z) {
+    const int a0 = k1_low<FACE>();
     x = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     if (k1_is_linear()) {
         const int q = (int)((unsigned)x / (unsigned)p.nx);
@@ -316,7 +335,7 @@ __global__ void __launch_bounds__(128, SNAP ? 0 : k1_min_blocks<ST>()) k_even(co
     int x = 0, y = 0, z = 0, a = 0, col = 0, jso = 0;
     IX c = 0;
     float f[19], g[7];
-    bool on = k1_node<FACE>(p, nullptr, x, y, z);
+    bool on = k1_node<FACE>(p, x, y, z);
     const bool late = k1_late(early_blocks);
     if (late) step_launch_wait();
     if (on) {
@@ -364,7 +383,7 @@ __global__ void __launch_bounds__(128) k_even_cond(const __grid_constant__ KP p,
                                                    const float *gpost, const float *spost) {
     step_launch_wait();
     int x, y, z;
-    if (k1_node<FACE>(p, nullptr, x, y, z)) even_node<ST, FACE, long long, true>(p, F, G, js, nb, gpost, x, y, z, spost);
+    if (k1_node<FACE>(p, x, y, z)) even_node<ST, FACE, long long, true>(p, F, G, js, nb, gpost, x, y, z, spost);
 }
 
 
@@ -765,7 +784,7 @@ __global__ void __launch_bounds__(128, SNAP ? 0 : k1_min_blocks<ST>()) k_odd(con
                                              const int *jmax, int early_blocks, const double *s,
                                              const __grid_constant__ SnapOut snap) {
     int x = 0, y = 0, z = 0;
-    const bool on = k1_node<FACE>(p, nullptr, x, y, z);
+    const bool on = k1_node<FACE>(p, x, y, z);
     odd_node_early<ST, FACE, SNAP>(p, &lk, F, G, js, js_old, nb, nb_old, gpost, thw_rd, thw_wr, jmax, early_blocks, on, x, y, z, s,
                                    snap);
 }
@@ -780,7 +799,7 @@ __global__ void __launch_bounds__(128) k_odd_cond(const __grid_constant__ KP p, 
                                                   const float *spost) {
     step_launch_wait();
     int x, y, z;
-    if (k1_node<FACE>(p, nullptr, x, y, z))
+    if (k1_node<FACE>(p, x, y, z))
         odd_node<ST, FACE, true, true>(p, &lk, F, G, js, js_old, nb, gpost, thw_rd, thw_wr, x, y, z, spost);
 }
 
@@ -1144,8 +1163,6 @@ __device__ __forceinline__ void gather_g(const KP &p, const ST *G, int x, int y,
     }
 }
 
-// Shifted pre-collision f of a liquid node.  js: the liquid flags that the
-// in-flight values were produced under, or the ones after flip_column has run.
 template <typename ST, int FACE>
 __device__ __forceinline__ void snap_ghost(const KP &p, const ST *G, const float *thw, int x, int y, int z,
                                            bool inflight, const SnapOut &o) {
@@ -1157,6 +1174,8 @@ __device__ __forceinline__ void snap_ghost(const KP &p, const ST *G, const float
     snap_node(p, o, x, y, z, f, g);
 }
 
+// Shifted pre-collision f of a liquid node.  js: the liquid flags that the
+// in-flight values were produced under, or the ones after flip_column has run.
 template <typename ST, int FACE, bool FIXED = false>
 __device__ __forceinline__ void gather_f(const KP &p, const ST *F, const int *js, int x, int y, int z,
                                          bool inflight, float (&f)[19]) {

@@ -7,34 +7,6 @@
 
 namespace lbm {
 
-// The step's kernels (stream-collide, front) are launched with
-// programmatic stream serialization (see step_launch_wait) when LBM_PDL, but
-// plainly (`plain`) after a kernel that is not one of them and writes what
-// this one loads before its wait (a wall field, fronts, a restored state):
-// such a kernel lets its successor start when its blocks have returned, which
-// does not order its stores before loads that no wait precedes.
-#ifndef LBM_PDL
-#define LBM_PDL 1
-#endif
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_step_kernel(void (*kern)(KArgs...), dim3 grd, dim3 blk, cudaStream_t st, int plain, Args... args) {
-#if LBM_PDL
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grd;
-    cfg.blockDim = blk;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = plain ? 0 : 1;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
-#else
-    kern<<<grd, blk, 0, st>>>(args...);
-    return cudaGetLastError();
-#endif
-}
-
 template <typename ST, typename IXE, bool SNAP>
 static cudaError_t launch_sc(const KP &p, int face, int odd, const Bufs &b, dim3 grd, dim3 blk, cudaStream_t st,
                              const SnapOut &snap) {

@@ -28,8 +28,12 @@ namespace {
 const double CS2T = 0.25;  // D3Q7 pseudo sound speed squared (w0 = 1/4)
 const int kRedBlocks = 608;  // partial blocks of the FP64 totals (4 per SM of a GB300)
 // Step graphs: steps per replay, and the largest cavity that uses them by
-// default (a 160^3 step takes about as long on the GPU as its three launches
-// take the host; larger cavities are bound by the GPU).
+// default (drawn where a step of three launches took the host as long as the
+// GPU; larger cavities are bound by the GPU).  With two launches a step the
+// host keeps up on its own, replays against single steps in us a step: FP32
+// 96^3 10.0 / 9.0 at 0.1 H and 17.7 / 16.8 at 0.5 H, 160^3 17.6 / 17.0 and
+// 72.3 / 72.1, FP16 160^3 64.8 / 61.1; a replay takes one launch
+// of the host's for 32.
 const int kGraphSteps = 16;
 const long long kGraphMaxNodes = 160LL * 160 * 160;
 
@@ -291,14 +295,14 @@ lbm_status copy_in(lbm_melt *h, void *dst, const void *src, size_t bytes, int pt
     return LBM_OK;
 }
 
-// Waits for the handle's stream; the flags in page-locked memory are those of
-// everything enqueued so far.
-lbm_status read_flags(lbm_melt *h) {
+// Waits for the handle's stream; the flags in page-locked memory are then those
+// of everything enqueued so far.
+lbm_status wait_stream(lbm_melt *h) {
     CK(cudaStreamSynchronize(h->stream), "synchronize");
     return LBM_OK;
 }
 
-// What the status says (after read_flags).
+// What the status says (after wait_stream).
 lbm_status status_of_flags(lbm_melt *h) {
     const int st = *(volatile int *)(h->flags + lbm_melt::kStatus);
     if (st & 2) return set_err(h, LBM_ENAN, "non-finite temperature at the front");
@@ -307,7 +311,7 @@ lbm_status status_of_flags(lbm_melt *h) {
 }
 
 lbm_status check_status(lbm_melt *h) {
-    const lbm_status st = read_flags(h);
+    const lbm_status st = wait_stream(h);
     return st == LBM_OK ? status_of_flags(h) : st;
 }
 
@@ -629,7 +633,7 @@ cudaError_t initial_state(lbm_melt *h) {
             e = LAUNCH(h, init, p, h->face, b, Tprof_dev, h->stream);
         }
     }
-    if (e == cudaSuccess && (refresh_front(h) != LBM_OK || read_flags(h) != LBM_OK)) e = cudaErrorUnknown;
+    if (e == cudaSuccess && (refresh_front(h) != LBM_OK || wait_stream(h) != LBM_OK)) e = cudaErrorUnknown;
     cudaFree(Tprof_dev);
     return e;
 }
@@ -844,7 +848,7 @@ LBM_API lbm_status lbm_melt_totals(lbm_melt *h, double *out, int ptr_kind) {
     CK(LAUNCH(h, totals, h->kp, h->face, h->inflight, b, h->red_part, h->nred, -1.0, view ? view : h->totals_dev,
               h->stream), "totals");
     if (!view) CK(cudaMemcpyAsync(out, h->totals_dev, 7 * 8, cudaMemcpyDeviceToDevice, h->stream), "copy totals");
-    const lbm_status st = read_flags(h);
+    const lbm_status st = wait_stream(h);
     if (st != LBM_OK) return st;
     if (!ptr_kind) std::memcpy(out, h->host_out, 7 * 8);
     return status_of_flags(h);
@@ -921,7 +925,7 @@ lbm_status enqueue_front_out(lbm_melt *h, double *S, double *liquid_fraction, in
 lbm_status front_out_sync(lbm_melt *h, double *S, double *liquid_fraction, int ptr_kind) {
     double *const lf = liquid_fraction && !ptr_kind ? h->host_out : liquid_fraction;
     lbm_status st = enqueue_front_out(h, S, lf, ptr_kind);
-    if (st == LBM_OK) st = read_flags(h);
+    if (st == LBM_OK) st = wait_stream(h);
     if (st != LBM_OK) return st;
     if (lf != liquid_fraction) *liquid_fraction = *lf;
     return status_of_flags(h);
@@ -1031,7 +1035,7 @@ LBM_API lbm_status lbm_melt_set_state(lbm_melt *h, const float *f, const float *
         CK(LAUNCH(h, state_in, p, h->face, b, fd, gd, h->stream), "state in");
     }
     lbm_status st = refresh_front(h);
-    if (st == LBM_OK) st = read_flags(h);
+    if (st == LBM_OK) st = wait_stream(h);
     if (st == LBM_OK) {
         if (S) seed_readback(h);
         st = status_of_flags(h);
@@ -1077,7 +1081,7 @@ LBM_API lbm_status lbm_melt_get_nusselt(lbm_melt *h, double *Nu, double *Nu_mean
             if (st != LBM_OK) return st;
         }
     }
-    const lbm_status st = read_flags(h);
+    const lbm_status st = wait_stream(h);
     if (st != LBM_OK) return st;
     if (Nu_mean && !ptr_kind) *Nu_mean = *h->host_out;
     return status_of_flags(h);
