@@ -974,13 +974,19 @@ LBM_API lbm_status lbm_melt_tape_forward(lbm_melt *h, long long steps, long long
         t->ck_inflight.push_back(h->inflight);
         t->ck_steps.push_back(h->steps);
         lbm_status st = move_checkpoint(h, (unsigned char *)buf, t->ck_bound_off, 0);
-        if (st != LBM_OK) return st;
         const long long n = std::min(ckpt_every, steps - sgm * ckpt_every);
-        st = lbm_melt_step(h, n);
-        if (st != LBM_OK) return st;
+        if (st == LBM_OK) st = lbm_melt_step(h, n);
+        if (st != LBM_OK) {  // not a recorded run
+            free_tape(h);
+            return st;
+        }
     }
     // the handle's own maximum starts anew with the next uploaded state
-    TCK(cudaMemcpyAsync(t->top, h->jmax_dev, sizeof(int), cudaMemcpyDeviceToDevice, h->stream), "liquid-count maximum");
+    const cudaError_t e = cudaMemcpyAsync(t->top, h->jmax_dev, sizeof(int), cudaMemcpyDeviceToDevice, h->stream);
+    if (e != cudaSuccess) {
+        free_tape(h);
+        return tape_err(h, LBM_ECUDA, "liquid-count maximum: %s", cudaGetErrorString(e));
+    }
     return LBM_OK;
 }
 
